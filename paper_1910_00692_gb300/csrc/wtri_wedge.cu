@@ -339,7 +339,8 @@ int ws_prepare(const wtri_graph* g, const WsScratch& W, cudaStream_t s) {
 
 size_t ws_bytes(const wtri_graph* g) {
     const int64_t n = g->d.n, m = g->d.m, tiles = (n + CT - 1) / CT;
-    return 16 * (size_t)m + 8 * (size_t)n + 16 * (size_t)n + 16 * (size_t)tiles + 4 * 256;
+    const size_t b = 16 * (size_t)m + 8 * (size_t)n + 16 * (size_t)n + 16 * (size_t)tiles + 4 * 256;
+    return (b + 255) & ~(size_t)255;  // what follows in the same block starts aligned
 }
 
 WsScratch ws_carve(const wtri_graph* g, char* p) {
@@ -401,7 +402,7 @@ int run_wedge_topk(const wtri_graph* g, int32_t k, int64_t nsamples, uint64_t se
     while (tcap < 2 * (uint64_t)nsamples) tcap <<= 1;
     const uint32_t cap = (uint32_t)std::min<int64_t>(std::max<int64_t>(nsamples, k), (int64_t(1) << 31) - 1);
     const size_t wsb = ws_bytes(g) + 512;
-    const size_t qb = 256 + (size_t)cap * 24 + 256 + 16 * sizeof(LongItem);
+    const size_t qb = 256 + (size_t)cap * 24 + 512 + 16 * sizeof(LongItem);
     const size_t hb = 8 * (size_t)tcap;
     void* buf = nullptr;
     if (cudaMallocAsync(&buf, wsb + qb + hb, s) != cudaSuccess) {
@@ -416,6 +417,7 @@ int run_wedge_topk(const wtri_graph* g, int32_t k, int64_t nsamples, uint64_t se
     p += 256;
     q.ckey = (unsigned long long*)p;
     p += (size_t)cap * 8;
+    p = (char*)(((uintptr_t)p + 15) & ~(uintptr_t)15);  // 16-byte triples: cap may be odd
     q.ctri = (int4*)p;
     p += (size_t)cap * 16;
     p = (char*)(((uintptr_t)p + 255) & ~(uintptr_t)255);

@@ -58,3 +58,16 @@ def test_wedge_errors(graphs):
     assert ei.value.code == -1
     tris, _ = wt.wedge_topk(d, 1.0, 10, 0, 1)
     assert tris.shape[0] == 0
+
+
+@pytest.mark.parametrize("n,k,nsamples", [(2001, 10, 2000), (2000, 10, 2001), (2001, 11, 2001), (2001, 1001, 1)])
+def test_wedge_topk_odd_sizes(n, k, nsamples):
+    """Odd vertex and sample counts: every scratch array keeps its alignment."""
+    g = synth.scaled_mid_graph(n, 20_000, seed=12)
+    d = wt.build_csr(g.n, g.u, g.v, g.w)
+    try:
+        want = oracle.wedge_topk(g.n, g.u, g.v, g.w, 1.0, k, nsamples, 7)
+        tris, wts = wt.wedge_topk(d, 1.0, k, nsamples, 7)
+        assert_topk_equal(tris, wts, want, 1.0, f"n={n} k={k} s={nsamples}")
+    finally:
+        d.free()
