@@ -175,8 +175,8 @@ WTRI_API int wtri_topk_device(const wtri_graph* g, double p, int32_t k, wtri_tri
  * on cudaMalloc/cudaMallocAsync.  Arguments, outputs and results are those
  * of wtri_topk_device.
  *
- * Scratch comes from one fixed array inside the library: about 26 MB
- * (1,048,576 candidate triangles and 65,536 deferred scans) that every GPU
+ * Scratch comes from one fixed array inside the library: about 28 MB
+ * (1,048,576 candidate triangles and the scans of 46,592 edges) that every GPU
  * loading the library keeps until the process exits.  k above 16384 is
  * rejected with WTRI_EINVAL.  If a query produces more candidates than the
  * array holds, d_count receives WTRI_ENOMEM; use wtri_topk_device then.
@@ -219,8 +219,8 @@ WTRI_API int wtri_merge_topk(int32_t nparts, const int32_t* counts, const wtri_t
  * Batched exact top-k: query i asks for the top-k[i] triangles of gs[i] at
  * p[i] (same problem and result format as wtri_topk, results in outs[i]).
  * All queries run in one launch sequence captured in a CUDA graph on the
- * first graph's stream: each phase kernel covers every query at once, and
- * each query keeps its own threshold and candidate buffer.  Graphs must be
+ * first graph's stream: small graphs one block each, larger ones a share of
+ * the SMs each, and each query keeps its own threshold and candidate buffer.  Graphs must be
  * on one device.  Returns after all results are in the host arrays.  No
  * counterpart in the paper (whose algorithms answer one query at a time).
  */
@@ -283,10 +283,10 @@ WTRI_API int wtri_server_set_option(wtri_server* s, int option, int64_t value);
 /*
  * Query schedule tuning (no counterpart in the paper).  A query sweeps the
  * edge order in rounds over [0, first_round), then ranges growing by
- * `growth`; a thread scans up to t_short wedges of an edge itself and hands
- * longer scans to a block that stages the closing vertex's list in shared
- * memory, so t_short is the boundary between the short-list and long-list
- * strategies.  Defaults: 64, 8, 32.
+ * `growth`; in small rounds a warp scans up to t_short wedges of an edge
+ * itself (rounded up to a multiple of 32) and leaves longer scans to the
+ * whole team, so t_short is the boundary between the short-list and
+ * long-list strategies.  Defaults: 64, 8, 32.
  *
  * wtri_autotune times a grid of settings (first_round in {32, 64, 256,
  * 1024}, growth in {4, 8, 16}, t_short in {8, 16, 32, 64, 128}) on the
@@ -468,13 +468,12 @@ WTRI_API int wtri_prof_read_ex(int idx, char* name, int name_cap, long long* cal
 WTRI_API int wtri_query_bytes(int on, int reset, unsigned long long* bytes);
 
 /*
- * Fault injection for tests (no counterpart in the paper).  The long-scan
- * kernel of the exact query stages a vertex's neighbour list in shared
- * memory with a bulk copy and waits for it with a bounded number of polls
- * of an mbarrier; when the polls run out the query reports WTRI_ETIMEOUT
- * (the copy in flight is still waited for, with the full bound, before the
- * block moves on).  This sets the bound of that first wait for queries
- * started afterwards in this process: polls = 0 makes every staged wait
+ * Fault injection for tests (no counterpart in the paper).  The blocks of
+ * an exact query's kernel wait for one another at a grid barrier with a
+ * bounded number of polls; when the polls run out the query reports
+ * WTRI_ETIMEOUT (the other blocks are still waited for, with the full bound,
+ * so that all leave in step).  This sets the bound of each block's first
+ * wait for queries started afterwards in this process: polls = 0 makes it
  * report a timeout at once; polls < 0 restores the default.  Nothing else
  * changes; a query after restoring the default is unaffected.
  */

@@ -1,186 +1,159 @@
-// Batched exact top-k: many (graph, p, k) queries in one launch sequence.
+// Batched exact top-k: many (graph, p, k) queries in one launch.
 //
-// Every query keeps its own state (threshold, stop point, candidate buffer)
-// exactly as in the single query; the kernels of each phase run over all
-// queries at once:
-//   k_round_offsets one block: each query's live range for this round (cut
-//                   at its stop point) and their prefix offsets;
-//   k_round_batch   threads stride over the concatenated live ranges (a
-//                   binary search maps a work item to its query);
-//   k_long_batch    deferred long scans of all queries (items carry the
-//                   query index);
-//   k_select_batch  one block per query: k-th key, compaction, threshold;
-//   k_final_batch / k_rank_batch: exact selection and ranking per query.
-// The whole sequence (rounds x 4 + 2 launches) is captured in one CUDA
-// graph and launched once.
+// Every query runs the sweep of the single query (wtri_query.cuh), with its
+// own state, threshold and candidate buffer.  One kernel holds the whole GPU
+// (a cooperative launch, one block per SM).  Queries whose expected work is
+// above an even share get a team of SMs each, in proportion to it; every
+// other block, and every team once its query is answered, works as PARTS
+// parts that take the remaining queries from a list, largest first, one query
+// per part: the phases of a query wait only for its own part or team, and its
+// results are ranked there.  Most queries are bound by latency, so many side
+// by side take little longer than one; the teams keep the few large ones
+// from being the tail (64 graphs of up to 2e5 edges, one block each: 3.5 ms).
+// The launch is captured in a CUDA graph.
 #include "wtri_query.cuh"
 
 #include <vector>
 
-#ifndef WTRI_BATCH_FIRST
-#define WTRI_BATCH_FIRST 64  // first round of a batched query (edges)
-#endif
-#ifndef WTRI_BATCH_GROWTH
-#define WTRI_BATCH_GROWTH 8  // growth of the batch's rounds
-#endif
-
 namespace wtri {
 namespace {
+
+constexpr int PT = 512;                   // threads of a part
+constexpr int PARTS = TGRID / PT;         // parts of a block
+// Items, shared evenly by the SMs: a round of a query takes at most its share
+// (edges).  A server's batches keep to the bytes its admission counts.
+constexpr int64_t POOL_SERVED = 180000;
+constexpr int64_t POOL_BATCH = 640000;
+constexpr int TEAMS = 64;                 // most teams of a launch
+constexpr int64_t BATCH_FIRST = 64;       // first round of a batched query (edges)
+constexpr int32_t BATCH_GROWTH = 8;       // growth of its rounds
 
 struct BatchDev {
     const DevGraph* graphs;
     const Query* queries;
+    const Out* outs;
     const int32_t* pcodes;
-    int32_t nq;
+    const int32_t* order;  // the queries answered by parts, largest first
+    int32_t count;
+    int32_t* cursor;
+    Item* items;           // per_sm for each block
+    unsigned long long* ibase;
+    int64_t per_sm;
 };
 
-// Last q with offs[q] <= t (offs non-decreasing, offs[0] = 0 <= t).
-__device__ __forceinline__ int find_q(const int64_t* offs, int nq, int64_t t) {
-    int lo = 0, hi = nq;
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (__ldg(offs + mid) <= t) lo = mid;
-        else hi = mid;
-    }
-    return lo;
+// Teams of one launch: team t has blocks [blk[t], blk[t + 1]) and query qi[t].
+struct TeamList {
+    int32_t n;
+    int32_t qi[TEAMS];
+    int16_t blk[TEAMS + 1];
+};
+
+struct PartSmem {
+    SweepSmem<PT> sweep;
+    DevGraph G;
+    Query q;
+    Out o;
+    QState st;
+    int32_t at;
+};
+
+// (not inlined: the instantiations would share one frame of registers)
+template <int P>
+__device__ __noinline__ void sweep_part(PartSmem& S) {
+    BlockTeam<PT> T;
+    sweep<P, false>(S.G, S.q, S.o, T, S.sweep);
 }
 
-// Per round: each query's live range is [lo, min(hi, its stop point)); the
-// exclusive prefix of the live sizes maps work items to queries, so
-// queries that have stopped cost nothing in later rounds.
-__global__ void __launch_bounds__(1024) k_round_offsets(BatchDev B, const int64_t* __restrict__ lo,
-                                                        const int64_t* __restrict__ hi,
-                                                        int64_t* __restrict__ offs) {
-    __shared__ int64_t warp_sum[32];
-    __shared__ int64_t carry;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    for (int base = 0; base < B.nq; base += 1024) {
-        const int qi = base + threadIdx.x;
-        int64_t sz = 0;
-        if (qi < B.nq) {
-            const int64_t stop = (int64_t)(STOP_NONE - *(volatile const uint32_t*)&B.queries[qi].st->stop_rev);
-            const int64_t e = min(hi[qi], stop);
-            sz = e > lo[qi] ? e - lo[qi] : 0;
-        }
-        int64_t inc = sz;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int64_t y = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += y;
-        }
-        if (lane == 31) warp_sum[wid] = inc;
-        __syncthreads();
+template <int P>
+__device__ __noinline__ void sweep_team(const DevGraph& G, const Query& q, const Out& o, SweepSmem<TGRID>& S,
+                                        uint32_t blk0, uint32_t nblk) {
+    GridTeam<TGRID> T;
+    T.limit = q.wait_first;
+    T.blk0 = blk0;
+    T.nblk = nblk;
+    T.gone = &S.sel.gone;
+    sweep<P, false>(G, q, o, T, S);
+}
+
+union BatchSmem {
+    SweepSmem<TGRID> team;
+    PartSmem part[PARTS];
+};
+
+__global__ void __launch_bounds__(TGRID, 1) k_sweep_batch(BatchDev B, TeamList L) {
+    extern __shared__ __align__(16) unsigned char batch_smem[];
+    BatchSmem& S = *reinterpret_cast<BatchSmem*>(batch_smem);
+    __shared__ DevGraph G;
+    __shared__ Query q;
+    __shared__ Out o;
+    int t = 0;
+    while (t < L.n && (int)blockIdx.x >= L.blk[t + 1]) t++;
+    if (t < L.n) {
+        const int32_t qi = L.qi[t];
+        const uint32_t blk0 = (uint32_t)L.blk[t], nblk = (uint32_t)(L.blk[t + 1] - L.blk[t]);
         if (threadIdx.x == 0) {
-            int64_t acc = carry;
-            for (int k = 0; k < 32; k++) {
-                const int64_t t = warp_sum[k];
-                warp_sum[k] = acc;
-                acc += t;
+            G = B.graphs[qi];
+            q = B.queries[qi];
+            o = B.outs[qi];
+            q.items = B.items + B.per_sm * blk0;
+            q.ibase = B.ibase + B.per_sm * blk0;
+            q.item_cap = B.per_sm * nblk;
+            S.team.sel.gone = 0;
+        }
+        __syncthreads();
+        switch (B.pcodes[qi]) {
+            case P_MIN: sweep_team<P_MIN>(G, q, o, S.team, blk0, nblk); break;
+            case P_ONE: sweep_team<P_ONE>(G, q, o, S.team, blk0, nblk); break;
+            case P_TWO: sweep_team<P_TWO>(G, q, o, S.team, blk0, nblk); break;
+            case P_GEO: sweep_team<P_GEO>(G, q, o, S.team, blk0, nblk); break;
+            default: sweep_team<P_MAX>(G, q, o, S.team, blk0, nblk); break;
+        }
+        __syncthreads();
+    }
+    const int p = threadIdx.x / PT;
+    const Part<PT> part;
+    PartSmem& M = S.part[p];
+    for (;;) {
+        if (part.tid() == 0) {
+            M.at = atomicAdd(B.cursor, 1);
+            if (M.at < B.count) {
+                const int32_t qi = B.order[M.at];
+                const int64_t per = B.per_sm / PARTS;
+                M.G = B.graphs[qi];
+                M.q = B.queries[qi];
+                M.o = B.outs[qi];
+                M.st = QState{};
+                M.q.st = &M.st;
+                M.q.items = B.items + B.per_sm * blockIdx.x + per * p;
+                M.q.ibase = B.ibase + B.per_sm * blockIdx.x + per * p;
+                M.q.item_cap = per;
             }
-            carry = acc;
         }
-        __syncthreads();
-        if (qi < B.nq) offs[qi] = warp_sum[wid] + inc - sz;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) offs[B.nq] = carry;
-}
-
-__global__ void __launch_bounds__(RBLK) k_round_batch(BatchDev B, const int64_t* __restrict__ offs,
-                                                      const int64_t* __restrict__ lo) {
-    const int64_t total = offs[B.nq];
-    const int64_t stride = (int64_t)gridDim.x * RBLK;
-    for (int64_t t = (int64_t)blockIdx.x * RBLK + threadIdx.x; t < total; t += stride) {
-        const int qi = find_q(offs, B.nq, t);
-        const Query& q = B.queries[qi];
-        const int64_t idx = lo[qi] + (t - offs[qi]);
-        if (idx >= (int64_t)(STOP_NONE - *(volatile const uint32_t*)&q.st->stop_rev)) continue;
-        const unsigned long long tau = ld_volatile_u64(&q.st->tau);
-        const DevGraph& G = B.graphs[qi];
-        Tally tb;  // batched queries are not instrumented
-        switch (B.pcodes[qi]) {
-            case P_MIN: process_edge<P_MIN, false>(G, q, tau, (int32_t)idx, tb); break;
-            case P_ONE: process_edge<P_ONE, false>(G, q, tau, (int32_t)idx, tb); break;
-            case P_TWO: process_edge<P_TWO, false>(G, q, tau, (int32_t)idx, tb); break;
-            case P_GEO: process_edge<P_GEO, false>(G, q, tau, (int32_t)idx, tb); break;
-            default: process_edge<P_MAX, false>(G, q, tau, (int32_t)idx, tb); break;
+        part.sync();
+        const int32_t at = M.at;
+        if (at >= B.count) return;
+        switch (B.pcodes[B.order[at]]) {
+            case P_MIN: sweep_part<P_MIN>(M); break;
+            case P_ONE: sweep_part<P_ONE>(M); break;
+            case P_TWO: sweep_part<P_TWO>(M); break;
+            case P_GEO: sweep_part<P_GEO>(M); break;
+            default: sweep_part<P_MAX>(M); break;
         }
+        part.sync();
     }
 }
 
-__global__ void __launch_bounds__(LBLK) k_long_batch(BatchDev B, const LongItem* __restrict__ longs,
-                                                     const uint32_t* long_count, uint32_t long_cap) {
-    extern __shared__ __align__(128) unsigned char lsm[];
-    int32_t* srow = reinterpret_cast<int32_t*>(lsm);
-    __shared__ __align__(8) uint64_t bar;
-    __shared__ int timed_out;
-    const uint32_t n_items = min(*(volatile const uint32_t*)long_count, long_cap);
-    if (blockIdx.x >= n_items) return;
-    if (threadIdx.x == 0) {
-        mbar_init(&bar, 1);
-        timed_out = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncthreads();
-    uint32_t phase = 0;
-    for (uint32_t it = blockIdx.x; it < n_items; it += gridDim.x) {
-        const LongItem item = longs[it];
-        const int qi = item.pad;
-        const Query& q = B.queries[qi];
-        const DevGraph& G = B.graphs[qi];
-        const unsigned long long tau = ld_volatile_u64(&q.st->tau);
-        const int64_t dy = __ldg(G.rowptr + item.y + 1) - __ldg(G.rowptr + item.y);
-        const int64_t obeg = __ldg(G.orowptr + item.y);
-        const int32_t ody = (int32_t)(__ldg(G.orowptr + item.y + 1) - obeg);
-        const bool staged = ody > 0 && ody <= STAGE_MAX;
-        int32_t off = 0;
-        if (staged && !stage_row(G, obeg, ody, srow, &bar, phase, off, &q.st->err, &timed_out,
-                                 WAIT_LIMIT))
-            return;
-        Tally tb;
-        switch (B.pcodes[qi]) {
-            case P_MIN: long_scan<P_MIN, false>(G, q, tau, item, srow, off, obeg, ody, dy, staged, tb); break;
-            case P_ONE: long_scan<P_ONE, false>(G, q, tau, item, srow, off, obeg, ody, dy, staged, tb); break;
-            case P_TWO: long_scan<P_TWO, false>(G, q, tau, item, srow, off, obeg, ody, dy, staged, tb); break;
-            case P_GEO: long_scan<P_GEO, false>(G, q, tau, item, srow, off, obeg, ody, dy, staged, tb); break;
-            default: long_scan<P_MAX, false>(G, q, tau, item, srow, off, obeg, ody, dy, staged, tb); break;
-        }
-        __syncthreads();
-    }
-}
-
-__global__ void __launch_bounds__(SBLK) k_select_batch(BatchDev B) {
-    __shared__ SelectSmem S;
-    select_round(B.queries[blockIdx.x], S);
-}
-
-__global__ void __launch_bounds__(SBLK) k_final_batch(BatchDev B) {
-    __shared__ SelectSmem S;
-    final_select(B.queries[blockIdx.x], S);
-}
-
-__global__ void __launch_bounds__(256) k_rank_batch(BatchDev B, const int64_t* __restrict__ koffs,
-                                                    wtri_tri* out_tri, double* out_w,
-                                                    int32_t* status) {
-    const int64_t total = koffs[B.nq];
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t wv = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; wv < total;
-         wv += nwarps) {
-        const int qi = find_q(koffs, B.nq, wv);
-        const uint32_t i = (uint32_t)(wv - koffs[qi]);
-        const Query& q = B.queries[qi];
-        wtri_tri* ot = out_tri + koffs[qi];
-        double* ow = out_w + koffs[qi];
-        switch (B.pcodes[qi]) {
-            case P_MIN: rank_one<P_MIN>(q, i, ot, ow, status + qi); break;
-            case P_ONE: rank_one<P_ONE>(q, i, ot, ow, status + qi); break;
-            case P_TWO: rank_one<P_TWO>(q, i, ot, ow, status + qi); break;
-            case P_GEO: rank_one<P_GEO>(q, i, ot, ow, status + qi); break;
-            default: rank_one<P_MAX>(q, i, ot, ow, status + qi); break;
-        }
-    }
+// Expected microseconds of a query on one part (half an SM), from queries of
+// k = 500 timed on graphs of 1e4 to 2e7 edges.  The arithmetic means, the
+// geometric mean and the maximum are bound by latency and hardly grow with
+// the graph: on one whole SM 94 us at 1e4 edges, 151 at 2e5 (the long rows of
+// its heaviest edges), 117 at 2e7; on 152 SMs 64-97.  The minimum reads the
+// rows of a share of all edges: 348 us on one SM at 1e4 edges, 1,151 at 5e4,
+// 1,289 at 2e5, 5,881 at 5e6, 13,990 at 2e7; on 152 SMs 298 at 2e7.
+double part_us(int pcode, int64_t m) {
+    const double x = (double)m;
+    if (pcode != P_MIN) return 150.0 + 100.0 * std::min(1.0, x / 2e5);
+    return 300.0 + 900.0 * std::min(1.0, x / 5e4) + 1200.0 * std::min(1.0, x / 2e5) + 1.3e-3 * x;
 }
 
 size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -196,16 +169,16 @@ size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
 // ---------------------------------------------------------------------------
 struct wtri_batch_plan {
     int32_t nq = 0;
-    int R = 0;
+    int64_t pool = 0;  // items
     std::vector<wtri::DevGraph> hg;
     std::vector<int32_t> pcodes, ks, tshort;
+    std::vector<int32_t> alone;  // queries with a launch of their own (k above what a part ranks, no team left)
+    std::vector<int32_t> order;  // the queries answered by parts, largest first
+    wtri::TeamList teams;
     std::vector<uint32_t> caps;
-    std::vector<int64_t> offs, los, totals, koffs;
-    std::vector<unsigned char> hq;  // Query descriptors (filled at launch)
+    std::vector<int64_t> koffs;
     size_t cand_total = 0;
-    uint32_t long_cap = 1u << 18;
-    size_t o_st, o_key, o_tri, o_long, o_lcnt, o_g, o_q, o_pc, o_offs, o_live, o_los, o_koffs, o_otri,
-        o_ow, o_stat, bytes;
+    size_t o_st, o_key, o_tri, o_items, o_ibase, o_cur, o_g, o_q, o_o, o_pc, o_ord, o_otri, o_ow, o_stat, bytes;
     std::vector<int32_t> stat;
     std::vector<wtri_tri> otri;
     std::vector<double> ow;
@@ -221,10 +194,48 @@ uint32_t batch_query_cap(int32_t k, int64_t m) {
     return (uint32_t)std::max<int64_t>(cap, 16384);
 }
 
+// Deals the SMs: a query whose expected time on one part is well above an even
+// share of the whole batch (or that has more results than a part ranks) gets
+// a team of SMs in proportion to its work, the rest are left to the parts.
+static void plan_teams(BatchPlan* P) {
+    const int nq = P->nq, sms = sm_count();
+    std::vector<double> us((size_t)nq);
+    double total = 0.0;
+    for (int i = 0; i < nq; i++) total += us[(size_t)i] = part_us(P->pcodes[(size_t)i], P->hg[(size_t)i].m);
+    std::vector<int32_t> by((size_t)nq);
+    for (int i = 0; i < nq; i++) by[(size_t)i] = i;
+    std::stable_sort(by.begin(), by.end(), [&](int32_t a, int32_t b) {
+        const bool ka = P->ks[(size_t)a] > SORT_MAX, kb = P->ks[(size_t)b] > SORT_MAX;
+        return ka != kb ? ka : us[(size_t)a] > us[(size_t)b];
+    });
+    P->teams.n = 0;
+    P->teams.blk[0] = 0;
+    P->order.clear();
+    const double share = total / ((double)PARTS * sms);  // an even share of one part
+    for (int32_t i : by) {
+        const int t = P->teams.n, used = P->teams.blk[t];
+        const bool must = P->ks[(size_t)i] > SORT_MAX;
+        if (must || (us[(size_t)i] > 1.5 * share && us[(size_t)i] > 150.0 && t < TEAMS && used < sms)) {
+            if (t == TEAMS || used == sms) {  // no team left: a launch of its own
+                P->alone.push_back(i);
+                continue;
+            }
+            int want = (int)(us[(size_t)i] / (PARTS * share) + 0.999);
+            want = std::max(1, std::min(want, sms - used));
+            P->teams.qi[t] = i;
+            P->teams.blk[t + 1] = (int16_t)(used + want);
+            P->teams.n++;
+        } else {
+            P->order.push_back(i);
+        }
+    }
+}
+
 BatchPlan* batch_plan_create(const wtri_graph* const* gs, const int32_t* pcodes, const int32_t* ks,
-                             int32_t nq) {
+                             int32_t nq, bool served) {
     BatchPlan* P = new (std::nothrow) BatchPlan();
     if (!P) return nullptr;
+    P->pool = served ? POOL_SERVED : POOL_BATCH;
     P->nq = nq;
     P->hg.resize((size_t)nq);
     P->pcodes.assign(pcodes, pcodes + nq);
@@ -232,69 +243,32 @@ BatchPlan* batch_plan_create(const wtri_graph* const* gs, const int32_t* pcodes,
     P->caps.resize((size_t)nq);
     P->tshort.resize((size_t)nq);
     P->koffs.assign((size_t)nq + 1, 0);
-    int64_t mmax = 0;
-    for (int i = 0; i < nq; i++) {
-        P->hg[(size_t)i] = gs[i]->d;
-        P->tshort[(size_t)i] = gs[i]->tune.t_short;
-        mmax = std::max<int64_t>(mmax, gs[i]->d.m);
-        P->koffs[(size_t)i + 1] = P->koffs[(size_t)i] + ks[i];
-        P->caps[(size_t)i] = batch_query_cap(ks[i], gs[i]->d.m);
-        P->cand_total += P->caps[(size_t)i];
-    }
-    // Round schedule: one for the whole batch (first round, growth: the
-    // WTRI_BATCH_* switches), since every batch round costs a launch sequence and a
-    // select over all queries and the smallest growth would set the round
-    // count of all; each query keeps its own graph's short/long boundary
-    // (t_short).  Round r of the batch runs round r of every query (empty
-    // once a query's schedule has covered its edges).
-    (void)mmax;
-    const int64_t first = WTRI_BATCH_FIRST;
-    const int64_t growth = WTRI_BATCH_GROWTH;
-    int R = 0;
-    std::vector<std::vector<int64_t>> his((size_t)nq);
     for (int i = 0; i < nq; i++) {
         const int64_t m = gs[i]->d.m;
-        for (int64_t lo = 0, size = first; lo < m; lo += size, size *= growth)
-            his[(size_t)i].push_back(std::min(m, lo + size));
-        R = std::max<int>(R, (int)his[(size_t)i].size());
+        P->hg[(size_t)i] = gs[i]->d;
+        P->tshort[(size_t)i] = gs[i]->tune.t_short;
+        P->koffs[(size_t)i + 1] = P->koffs[(size_t)i] + ks[i];
+        P->caps[(size_t)i] = batch_query_cap(ks[i], m);
+        P->cand_total += P->caps[(size_t)i];
     }
-    P->R = R;
-    // offs: per round, the query ranges' hi ends (the device computes the
-    // live offsets from them and the stop points); totals bound the grids.
-    P->offs.resize((size_t)R * nq);
-    P->los.resize((size_t)R * nq);
-    P->totals.resize((size_t)R);
-    for (int r = 0; r < R; r++) {
-        int64_t acc = 0;
-        for (int i = 0; i < nq; i++) {
-            const auto& h = his[(size_t)i];
-            const int64_t m = gs[i]->d.m;
-            const int64_t a = r == 0 ? 0 : (r - 1 < (int)h.size() ? h[(size_t)r - 1] : m);
-            const int64_t b = r < (int)h.size() ? h[(size_t)r] : m;
-            P->offs[(size_t)r * nq + i] = b;
-            P->los[(size_t)r * nq + i] = a;
-            acc += b - a;
-        }
-        P->totals[(size_t)r] = acc;
-    }
+    plan_teams(P);
     size_t off = 0;
     auto take = [&](size_t bytes) {
         size_t o = off;
         off = al256(off + bytes);
         return o;
     };
-    P->o_st = take(sizeof(QState) * (size_t)nq);
+    P->o_st = take(sizeof(QState) * ((size_t)P->teams.n + P->alone.size() + 1));
+    P->o_cur = take(64);  // cleared together with the states
     P->o_key = take(8 * P->cand_total);
     P->o_tri = take(16 * P->cand_total);
-    P->o_long = take(sizeof(LongItem) * (size_t)P->long_cap);
-    P->o_lcnt = take(64);
+    P->o_items = take(sizeof(Item) * (size_t)P->pool);
+    P->o_ibase = take(8 * (size_t)P->pool);
     P->o_g = take(sizeof(DevGraph) * (size_t)nq);
     P->o_q = take(sizeof(Query) * (size_t)nq);
+    P->o_o = take(sizeof(Out) * (size_t)nq);
     P->o_pc = take(4 * (size_t)nq);
-    P->o_offs = take(8 * std::max<size_t>(P->offs.size(), 1));
-    P->o_live = take(8 * ((size_t)nq + 1) * std::max(R, 1));
-    P->o_los = take(8 * std::max<size_t>(P->los.size(), 1));
-    P->o_koffs = take(8 * P->koffs.size());
+    P->o_ord = take(4 * (size_t)nq);
     P->o_otri = take(sizeof(wtri_tri) * (size_t)P->koffs[(size_t)nq]);
     P->o_ow = take(8 * (size_t)P->koffs[(size_t)nq]);
     P->o_stat = take(4 * (size_t)nq);
@@ -328,91 +302,90 @@ int batch_plan_launch(BatchPlan* P, void* dbuf, cudaStream_t s, int use_graph) {
     QState* st = (QState*)(B0 + P->o_st);
     unsigned long long* ckey = (unsigned long long*)(B0 + P->o_key);
     int4* ctri = (int4*)(B0 + P->o_tri);
-    LongItem* longs = (LongItem*)(B0 + P->o_long);
-    uint32_t* lcnt = (uint32_t*)(B0 + P->o_lcnt);
-    std::vector<Query> hq((size_t)nq);
-    size_t c0 = 0;
-    for (int i = 0; i < nq; i++) {
-        Query& q = hq[(size_t)i];
-        q.st = st + i;
-        q.ckey = ckey + c0;
-        q.ctri = ctri + c0;
-        q.cap = P->caps[(size_t)i];
-        q.longs = longs;
-        q.long_cap = P->long_cap;
-        q.k = P->ks[(size_t)i];
-        q.smark = nullptr;
-        q.slist = nullptr;
-        q.long_count = lcnt;
-        q.qid = i;
-        q.shard = 0;
-        q.nshards = 1;
-        q.t_short = P->tshort[(size_t)i];
-        q.qbytes = nullptr;
-        q.gp = 0.0;  // batched queries take the exact-key p values only
-        q.fw = 0;    // and integer weights
-        q.wait_first = WAIT_LIMIT;
-        c0 += P->caps[(size_t)i];
-    }
-    BatchDev Bd;
-    Bd.graphs = (const DevGraph*)(B0 + P->o_g);
-    Bd.queries = (const Query*)(B0 + P->o_q);
-    Bd.pcodes = (const int32_t*)(B0 + P->o_pc);
-    Bd.nq = nq;
-    int64_t* d_offs = (int64_t*)(B0 + P->o_offs);
-    int64_t* d_live = (int64_t*)(B0 + P->o_live);
-    int64_t* d_los = (int64_t*)(B0 + P->o_los);
-    int64_t* d_koffs = (int64_t*)(B0 + P->o_koffs);
     wtri_tri* d_otri = (wtri_tri*)(B0 + P->o_otri);
     double* d_ow = (double*)(B0 + P->o_ow);
     int32_t* d_stat = (int32_t*)(B0 + P->o_stat);
+    std::vector<Query> hq((size_t)nq);
+    std::vector<Out> ho((size_t)nq);
+    size_t c0 = 0;
+    for (int i = 0; i < nq; i++) {
+        Query& q = hq[(size_t)i];
+        q = Query{};
+        q.ckey = ckey + c0;
+        q.ctri = ctri + c0;
+        q.cap = P->caps[(size_t)i];
+        q.k = P->ks[(size_t)i];
+        // one schedule (first round, growth) for the whole batch; each query
+        // keeps its own graph's t_short
+        q.total = P->hg[(size_t)i].m;
+        q.first = BATCH_FIRST;
+        q.growth = BATCH_GROWTH;
+        q.nshards = 1;
+        q.t_short = P->tshort[(size_t)i];
+        q.wait_first = WAIT_LIMIT;
+        ho[(size_t)i] = Out{d_otri + P->koffs[(size_t)i], d_ow + P->koffs[(size_t)i], d_stat + i, nullptr};
+        c0 += P->caps[(size_t)i];
+    }
+    for (int t = 0; t < P->teams.n; t++) hq[(size_t)P->teams.qi[t]].st = st + t;
+    for (size_t j = 0; j < P->alone.size(); j++) hq[(size_t)P->alone[j]].st = st + P->teams.n + j;
+    BatchDev Bd;
+    Bd.graphs = (const DevGraph*)(B0 + P->o_g);
+    Bd.queries = (const Query*)(B0 + P->o_q);
+    Bd.outs = (const Out*)(B0 + P->o_o);
+    Bd.pcodes = (const int32_t*)(B0 + P->o_pc);
+    Bd.order = (const int32_t*)(B0 + P->o_ord);
+    Bd.count = (int32_t)P->order.size();
+    Bd.cursor = (int32_t*)(B0 + P->o_cur);
+    Bd.items = (Item*)(B0 + P->o_items);
+    Bd.ibase = (unsigned long long*)(B0 + P->o_ibase);
+    Bd.per_sm = P->pool / sm_count() / (32 * PARTS) * (32 * PARTS);
     WTRI_CUDA(cudaMemcpyAsync((void*)Bd.graphs, P->hg.data(), sizeof(DevGraph) * nq, cudaMemcpyHostToDevice, s));
     WTRI_CUDA(cudaMemcpyAsync((void*)Bd.queries, hq.data(), sizeof(Query) * nq, cudaMemcpyHostToDevice, s));
+    WTRI_CUDA(cudaMemcpyAsync((void*)Bd.outs, ho.data(), sizeof(Out) * nq, cudaMemcpyHostToDevice, s));
     WTRI_CUDA(cudaMemcpyAsync((void*)Bd.pcodes, P->pcodes.data(), 4 * (size_t)nq, cudaMemcpyHostToDevice, s));
-    WTRI_CUDA(cudaMemcpyAsync(d_offs, P->offs.data(), 8 * P->offs.size(), cudaMemcpyHostToDevice, s));
-    if (!P->los.empty())
-        WTRI_CUDA(cudaMemcpyAsync(d_los, P->los.data(), 8 * P->los.size(), cudaMemcpyHostToDevice, s));
-    WTRI_CUDA(cudaMemcpyAsync(d_koffs, P->koffs.data(), 8 * P->koffs.size(), cudaMemcpyHostToDevice, s));
-
-    const size_t lsmem = LONG_SMEM;
-    {
-        static std::atomic<uint64_t> done{0};
-        WTRI_TRY(smem_optin((const void*)k_long_batch, (int)lsmem, done));
+    if (!P->order.empty())
+        WTRI_CUDA(cudaMemcpyAsync((void*)Bd.order, P->order.data(), 4 * P->order.size(), cudaMemcpyHostToDevice, s));
+    static std::atomic<uint64_t> done{0};
+    WTRI_TRY(smem_optin((const void*)k_sweep_batch, (int)sizeof(BatchSmem), done));
+    // the teams, then each query left over as a team of the whole GPU
+    std::vector<TeamList> launches;
+    launches.push_back(P->teams);
+    for (int32_t i : P->alone) {
+        TeamList L{};
+        L.n = 1;
+        L.qi[0] = i;
+        L.blk[1] = (int16_t)sm_count();
+        launches.push_back(L);
     }
-    const int long_grid = sm_count() * 2;
-    const int R = P->R;
-    auto launch_all = [&]() {
-        cudaMemsetAsync(st, 0, sizeof(QState) * (size_t)nq, s);
-        cudaMemsetAsync(lcnt, 0, 64, s);
-        for (int r = 0; r < R; r++) {
-            int64_t* live = d_live + (size_t)r * (nq + 1);
-            k_round_offsets<<<1, 1024, 0, s>>>(Bd, d_los + (size_t)r * nq, d_offs + (size_t)r * nq, live);
-            k_round_batch<<<round_grid(P->totals[(size_t)r]), RBLK, 0, s>>>(Bd, live,
-                                                                            d_los + (size_t)r * nq);
-            k_long_batch<<<long_grid, LBLK, lsmem, s>>>(Bd, longs, lcnt, P->long_cap);
-            k_select_batch<<<nq, SBLK, 0, s>>>(Bd);
+    const size_t clear = P->o_cur + 64 - P->o_st;  // states of the teams, cursor
+    auto launch_all = [&]() -> int {
+        WTRI_CUDA(cudaMemsetAsync(B0 + P->o_st, 0, clear, s));
+        for (TeamList& L : launches) {
+            void* args[] = {&Bd, &L};
+            WTRI_CUDA(cudaLaunchCooperativeKernel((const void*)k_sweep_batch, dim3((unsigned)sm_count()), dim3(TGRID),
+                                                  args, sizeof(BatchSmem), s));
         }
-        k_final_batch<<<nq, SBLK, 0, s>>>(Bd);
-        const int64_t warps = P->koffs[(size_t)nq];
-        k_rank_batch<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>((warps + 7) / 8,
-                                                                        sm_count() * 16)),
-                       256, 0, s>>>(Bd, d_koffs, d_otri, d_ow, d_stat);
+        return WTRI_OK;
     };
     int rc = WTRI_OK;
-    ProfScope ps("topk_batch", s, 0.0, 4 * R + 2);
+    ProfScope ps("topk_batch", s, 0.0, (int)launches.size());
     if (use_graph) {
         // The descriptors must have landed before the captured work refers
         // to them only through device pointers: that holds, the copies are
         // ordered on s before the graph launch.  The instantiated graph is
         // kept (per thread and device) and refreshed with
         // cudaGraphExecUpdate when the next batch has the same launch
-        // topology (same number of rounds), so a repeated batch shape is
-        // instantiated once.
+        // topology (the same kinds of launch), so a repeated batch
+        // shape is instantiated once.
         cudaGraph_t graph = nullptr;
         cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            launch_all();
+            rc = launch_all();
             e = cudaStreamEndCapture(s, &graph);  // always leave capture mode
+            if (rc != WTRI_OK && e == cudaSuccess) {
+                cudaGraphDestroy(graph);
+                return rc;
+            }
         }
         cudaGraphExec_t exec = nullptr;
         if (e == cudaSuccess) {
@@ -441,9 +414,9 @@ int batch_plan_launch(BatchPlan* P, void* dbuf, cudaStream_t s, int use_graph) {
         if (graph) cudaGraphDestroy(graph);
         if (e != cudaSuccess) rc = cuda_error(e, "batch graph", __FILE__, __LINE__);
     } else {
-        launch_all();
+        rc = launch_all();
         cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) rc = cuda_error(e, "batch launch", __FILE__, __LINE__);
+        if (rc == WTRI_OK && e != cudaSuccess) rc = cuda_error(e, "batch launch", __FILE__, __LINE__);
     }
     return rc;
 }
@@ -523,7 +496,7 @@ int topk_batch(const wtri_graph* const* gs, const int32_t* pcodes, const int32_t
         cudaEventDestroy(ev);
         WTRI_CUDA(e);
     }
-    BatchPlan* P = batch_plan_create(gs, pcodes, ks, nq);
+    BatchPlan* P = batch_plan_create(gs, pcodes, ks, nq, false);
     if (!P) return set_error(WTRI_ENOMEM, "host allocation failed");
     void* buf = nullptr;
     if (cudaMallocAsync(&buf, P->bytes, s) != cudaSuccess) {

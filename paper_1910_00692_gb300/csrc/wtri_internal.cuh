@@ -99,7 +99,7 @@ struct wtri_batch_plan;  // defined in wtri_batch.cu
 
 namespace wtri {
 // Query schedule: rounds over [0, first_round), then ranges growing by
-// `growth`; threads scan t_short wedges inline before deferring.
+// `growth`; a warp scans up to t_short wedges of an edge itself.
 struct Tune {
     int64_t first_round = 64;
     int32_t growth = 8;
@@ -155,8 +155,9 @@ int topk_batch(const wtri_graph* const* gs, const int32_t* pcodes, const int32_t
 // scratch block (bytes from batch_plan_bytes), collect (synchronizes).
 typedef ::wtri_batch_plan BatchPlan;
 uint32_t batch_query_cap(int32_t k, int64_t m);
+// served: the plan's scratch keeps to the bytes a server's admission counts.
 BatchPlan* batch_plan_create(const wtri_graph* const* gs, const int32_t* pcodes, const int32_t* ks,
-                             int32_t nq);
+                             int32_t nq, bool served);
 size_t batch_plan_bytes(const BatchPlan* P);
 int batch_plan_launch(BatchPlan* P, void* dbuf, cudaStream_t s, int use_graph);
 int batch_plan_collect(BatchPlan* P, void* dbuf, cudaStream_t s);

@@ -1,5 +1,6 @@
 // Shared device machinery of the top-k query, the edge sampler and the
-// batched form (included by wtri_topk.cu and wtri_batch.cu).
+// batched form (included by wtri_topk.cu, wtri_batch.cu, wtri_wedge.cu and
+// wtri_clique.cu).
 //
 // Exact top-k weighted triangles: heavy-first enumeration with a running
 // threshold.
@@ -17,23 +18,35 @@
 //    threshold argument with one monotone cursor in place of two pointers.
 //  * Per edge, the entries of x and y after r are suffixes of their
 //    weight-sorted lists; their first entries bound the other two weights
-//    (edge bound), and scanning x's suffix in weight order gives a wedge bound
-//    K(w_r, w_xc, max_y) that only decreases, so the scan stops at the first
-//    wedge below tau.  The closing edge (y, c) is found by binary search in
-//    the oriented (degree-ordered) lists.
+//    (edge bound), and the wedge bound K(w_r, w_xc, max_y) only decreases
+//    along x's suffix, so the wedges that can reach tau are a prefix of it,
+//    the live range, found by search.  The shorter of the two live ranges is
+//    scanned; the closing edge (y, c) is found by search in the oriented
+//    (degree-ordered) lists.
 //  * tau is the key of the k-th best of k distinct triangles found so far, a
 //    valid lower bound on the true k-th key; pruning is strict (< tau), so
 //    triangles tied with the k-th key are still enumerated and the triple
 //    tie-break decides them.
 //
-// Schedule: the edge order is processed in rounds of geometrically growing
-// ranges [lo, hi).  Each round is three launches: k_round (thread per edge,
-// short scans inline, long scans deferred), k_long (block per deferred scan,
-// the closing-edge lookups go to the y row staged in shared memory by a bulk
-// copy), and k_select (one block: radix select of the k-th candidate under
-// the total order, in-place compaction, new tau).  Rounds after the stop
-// return at once, so the launch sequence depends only on (m, k) and can be
-// captured in a CUDA graph.
+// Schedule: one kernel runs the whole sweep.  Its threads form a team: every
+// block of a cooperative launch (one block per SM, a grid barrier between
+// phases), or one block alone (the batched form, many small graphs at once).
+// The edge order is processed in rounds of geometrically growing ranges, each
+// in three phases with a team barrier after each:
+//   A  edges: the checks and searches of every edge of the round (a warp per
+//      edge in small rounds, a thread per edge in large ones); an edge with
+//      a long live range leaves it as an item, with the running number of
+//      wedges before it;
+//   B  wedges: the items' wedges, numbered through, are dealt to the team 32
+//      at a time, whatever the items' lengths;
+//   C  select (one block): the k-th key, in-place compaction, the new tau,
+//      and the next round's range, cut where the edge bound falls below tau.
+// After the last round the same kernel ranks the k best and writes the
+// outputs.  What bounds a query is latency (binary searches over a pruned
+// set) and the launches: with a launch per phase a query on the 2e7-edge
+// graph spent about 75 of its 330 us in the launches of rounds after the
+// stop, 104 us on the 64 items of the first round (one block each), and 75 us
+// on selects whose histogram one thread scanned.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -46,32 +59,36 @@
 namespace wtri {
 namespace {
 
-constexpr int RBLK = 256;          // k_round block
-constexpr int LBLK = 256;          // k_long block
-constexpr int SBLK = 1024;         // k_select block
-constexpr int STAGE_MAX = 24576;   // ids of a y row staged in shared memory (96 KB)
-constexpr int64_t FIRST_ROUND = 64;  // batch schedule (single queries use the graph's tune)
-constexpr int ROUND_GROWTH = 8;
-constexpr uint32_t WAIT_LIMIT = 1u << 24;  // bounded mbarrier polling
-constexpr uint32_t STOP_NONE = 0x7fffffffu; // edge positions are below 2^31
+constexpr int TGRID = 1024;         // threads of a block of the grid team (one block per SM)
+constexpr int SORT_MAX = 2048;      // largest k ranked by a sort in shared memory
+constexpr uint32_t WAIT_LIMIT = 1u << 26;  // bounded polling of the grid barrier
+constexpr int64_t ITEM_CAP = 1 << 18;      // edges of one round (at most one item each)
+constexpr int64_t WARP_EDGES = 4096;       // largest round that takes a warp per edge
+constexpr int64_t MIN_FLAT = 8192;         // largest p = -inf round that numbers its entries through
 
+// State of one query (zeroed before it starts).
 struct QState {
-    unsigned long long tau;   // keys below tau are pruned; 0 = no bound yet
-    uint32_t stop_rev;        // STOP_NONE - (first edge whose bound fell below tau); 0 = none
-    uint32_t err;             // DEV_ERR_* bits
-    uint32_t count;           // candidates appended (may exceed capacity)
-    uint32_t long_count;      // deferred scans
-    uint32_t selected;        // count right after the last compaction
-    uint32_t pad[3];
+    unsigned long long tau;       // keys below tau are pruned; 0 = no bound yet
+    uint32_t err;                 // DEV_ERR_* bits
+    uint32_t count;               // candidates appended (may exceed capacity)
+    uint32_t selected;            // count right after the last compaction
+    uint32_t bar;                 // arrivals at the grid barrier
+    unsigned long long items[2];  // items of a phase (high 20 bits) and their wedges, by step parity
+    long long lo, hi, size;       // the next round and its uncut size (published by the selecting block)
+    uint32_t kept;                // candidates left for the ranking
+    uint32_t pad;
 };
 
-struct LongItem {
+// The wedges of one edge left to phase B.
+struct __align__(16) Item {
     int32_t r;      // owning edge (position in the edge order)
-    int32_t x, y;   // scanned endpoint, probed endpoint
-    int32_t w;      // w_r
-    int32_t ymax;   // first weight of y's suffix
-    int32_t pad;    // query index within a batch
-    int64_t j0, j1; // remaining suffix of x's weight-sorted list
+    int32_t x, y;   // scanned endpoint, probed endpoint (p = -inf: the edge's endpoints)
+    uint32_t w;     // w_r
+    int64_t j0;     // first wedge's position in x's list (p = -inf: in the scanned oriented row)
+    int64_t lb;     // y's oriented row (p = -inf: the searched row)
+    int32_t ln;     // its length
+    int32_t dy;     // y's degree
+    int32_t pad[2];
 };
 
 struct Query {
@@ -79,24 +96,27 @@ struct Query {
     unsigned long long* ckey;
     int4* ctri;
     uint32_t cap;
-    LongItem* longs;
-    uint32_t long_cap;
+    Item* items;                // item_cap items
+    unsigned long long* ibase;  // wedges before each item
+    int64_t item_cap;
     int32_t k;
+    // Sweep: edges (or drawn positions: *total_dev of them, known on the
+    // device only), first round, growth.
+    int64_t total;
+    const int64_t* total_dev;
+    int64_t first;
+    int32_t growth;
     // Sampled mode (edge sampling): bitmap of drawn edges by edge-order
     // position, and the drawn positions in ascending order.
     const uint32_t* smark;
     const int32_t* slist;
-    // Deferred-scan list counter (the query's own, or one shared by a batch)
-    // and the query's index in a batch (stored in deferred items).
-    uint32_t* long_count;
-    int32_t qid;
     // Sharding (multi-GPU split of one query): this query owns the edges
     // whose chunk (position >> SHARD_SHIFT) is congruent to shard modulo
     // nshards; nshards <= 1 means every edge.
     int32_t shard;
     int32_t nshards;
-    // Wedges an edge's thread scans before deferring the rest to a block (the
-    // boundary between the short-list and long-list strategies).
+    // Wedges an edge's warp scans itself before leaving them to phase B
+    // (rounded up to a multiple of 32).
     int32_t t_short;
     // Instrumented run: bytes of the adjacency loads are added here (null:
     // no counting).
@@ -106,9 +126,17 @@ struct Query {
     // Weights are positive fp32 bit patterns (a float-weight graph), not
     // integers: the means and reported values read them as floats.
     int32_t fw;
-    // Polls of the first wait for a staged row (WAIT_LIMIT in production;
-    // tests lower it to take the timeout path).
+    // Polls of the first grid-barrier wait (WAIT_LIMIT in production; tests
+    // lower it to take the timeout path).
     uint32_t wait_first;
+};
+
+// Where a query's results go.
+struct Out {
+    wtri_tri* tri;
+    double* w;
+    int32_t* count;
+    unsigned long long* key;  // may be null
 };
 
 // Bytes of adjacency loads issued by one thread (instrumented runs only).
@@ -149,7 +177,7 @@ __device__ __forceinline__ bool owns(const Query& q, int32_t r, int32_t rxc, int
 // ascending order (equal multisets give equal bits), scaled by the largest
 // (p > 0) or the smallest (p < 0) so that no power overflows:
 //   m_p = s * (((a/s)^p + (b/s)^p + (c/s)^p) / 3)^(1/p).
-__device__ __forceinline__ double general_mean(double p, uint32_t a, uint32_t b, uint32_t c, bool fw = false) {
+__device__ __noinline__ double general_mean(double p, uint32_t a, uint32_t b, uint32_t c, bool fw = false) {
     uint32_t t;
     if (a > b) { t = a; a = b; b = t; }
     if (b > c) { t = b; b = c; c = t; }
@@ -201,25 +229,6 @@ __device__ __forceinline__ unsigned long long ld_volatile_u64(const unsigned lon
     return *(volatile const unsigned long long*)p;
 }
 
-// Position just after edge r's own entry in x's weight-sorted list
-// [lo, hi) (x's row).
-__device__ __forceinline__ int64_t suffix_start(const DevGraph& G, int64_t lo, int64_t hi, int32_t r,
-                                                uint32_t* err, Tally& tb) {
-    const int64_t end = hi;
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        tb.add(4);
-        if (__ldg(G.wrk + mid) < r) lo = mid + 1;
-        else hi = mid;
-    }
-    tb.add(4);
-    if (lo >= end || __ldg(G.wrk + lo) != r) {
-        atomicOr(err, DEV_ERR_INTERNAL);
-        return end;
-    }
-    return lo + 1;
-}
-
 // Closing edge (y, c) in the oriented lists: stored once, at the endpoint of
 // lower (degree, id) rank, rows ascending by id (row s at
 // [orowptr[s], orowptr[s+1])).  y_owns: whether y is that endpoint.
@@ -257,18 +266,144 @@ __device__ __forceinline__ bool probe_oriented(const DevGraph& G, int32_t y, int
                                    : search_oriented(G, c, y, wyc, ryc, tb);
 }
 
-// Warp-aggregated append: the active lanes appending to the same query
-// (a batched launch mixes queries within a warp) take one atomic together.
-__device__ __forceinline__ void append(const Query& q, unsigned long long key, int32_t a, int32_t b,
-                                       int32_t c) {
+// ---------------------------------------------------------------------------
+// Pruning against tau along a list of non-increasing weights: fails(x) only
+// if no triangle with weights w, y and x (or less) reaches tau.
+//
+// The exact keys compare the bound itself.  For P_GEN (other finite p, and
+// real weights) the fp64 mean costs four pow per wedge on a chip whose fp64
+// rate is a sixty-fourth of its fp32 rate, so the smallest weight that can
+// reach tau is found once per edge in fp32 instead: with t = tau (1 - 1e-4)
+// and R = 3 - (w/t)^p - (y/t)^p, the mean reaches t iff (x/t)^p >= R (p > 0)
+// or <= R (p < 0), i.e. x >= t R^(1/p).  The 1e-4 leaves R a slack of
+// 3e-4 |p| while fp32 rounding moves it by less than 4e-6 (1 + |p|) wherever
+// R > 0, so for |p| >= 0.05 a weight is only pruned when the exact bound
+// prunes it too; smaller |p| keeps the fp64 bound.  Survivors are decided by
+// their fp64 key.
+// ---------------------------------------------------------------------------
+template <int P>
+struct Line {
+    unsigned long long tau;
+    uint32_t w, y;
+    double gp;
+    bool fw;
+    bool use_cut;
+    uint32_t cut;
+
+    __device__ __forceinline__ Line(const Query& q, unsigned long long tau_, uint32_t w_, uint32_t y_)
+        : tau(tau_), w(w_), y(y_), gp(q.gp), fw(q.fw != 0), use_cut(false), cut(0) {
+        if constexpr (P == P_GEN) {
+            const float p = (float)gp;
+            if (tau != 0 && ((fabsf(p) >= 0.05f && fabsf(p) <= 1000.0f) || p == 0.0f)) {
+                use_cut = true;
+                const float t = (float)__longlong_as_double((long long)tau) * (1.0f - 1e-4f);
+                const float a = fw ? __uint_as_float(w) : (float)w, b = fw ? __uint_as_float(y) : (float)y;
+                float x;
+                if (p == 0.0f) {  // geometric mean: x >= t^3 / (a b)
+                    x = exp2f(3.0f * log2f(t) - log2f(a) - log2f(b));
+                } else {
+                    const float R = 3.0f - exp2f(p * log2f(a / t)) - exp2f(p * log2f(b / t));
+                    if (R > 0.0f) x = t * exp2f(log2f(R) / p);
+                    else x = p > 0.0f ? 0.0f : __int_as_float(0x7f800000);
+                }
+                x *= 1.0f - 1e-6f;
+                if (!(x >= 0.0f)) x = 0.0f;  // no usable bound
+                if (fw) cut = __float_as_uint(x);
+                else cut = x >= 4294967040.0f ? 0xffffffffu : (uint32_t)x;
+            }
+        }
+    }
+    __device__ __forceinline__ bool fails(uint32_t x) const {
+        if (P == P_GEN && tau == 0) return false;
+        if (P == P_GEN && use_cut) return x < cut;
+        return boundof<P>(w, x, y, gp, fw) < tau;
+    }
+};
+
+// Whether every triangle of edges no heavier than w is below tau.
+template <int P>
+__device__ __forceinline__ bool edge_below(const Query& q, uint32_t w, unsigned long long tau) {
+    if (P == P_GEN) {
+        const double x = q.fw ? (double)__uint_as_float(w) : (double)w;
+        return (unsigned long long)__double_as_longlong(x * (1.0 + 1e-12)) < tau;
+    }
+    return boundof<P>(w, w, w) < tau;
+}
+
+__device__ __forceinline__ uint32_t lanemask_below() {
+    uint32_t m;
+    asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
+    return m;
+}
+
+// First position of [lo, hi) where `below` is false (true on a prefix), found
+// by groups of W lanes (16 or 32), each group with its own range and
+// predicate: W probes a step, so a list of 35,000 takes four dependent loads
+// instead of fifteen.  All 32 lanes call it.
+template <int W, class Pred>
+__device__ __forceinline__ int64_t group_search(int64_t lo, int64_t hi, const Pred& below) {
+    const int lane = threadIdx.x & 31, gl = lane & (W - 1), sh = lane & ~(W - 1);
+    const uint32_t gm = W == 32 ? 0xffffffffu : ((1u << W) - 1u);
+    for (;;) {
+        const int64_t n = hi - lo;
+        if (__all_sync(0xffffffffu, n <= 0)) break;
+        const int64_t step = (n + W) / (W + 1);
+        const int64_t pos = lo + (int64_t)(gl + 1) * step - 1;
+        const bool b = n > 0 && pos < hi && below(pos);
+        const int cnt = __popc((__ballot_sync(0xffffffffu, b) >> sh) & gm);
+        if (n > 0) {
+            const int64_t nlo = lo + cnt * step;
+            if (cnt < W) hi = min(hi, lo + (int64_t)(cnt + 1) * step - 1);
+            lo = nlo;
+        }
+    }
+    return lo;
+}
+
+// First position of the oriented ids [lo, lo + n) not below t (three probes a
+// step: half the dependent loads of a binary search).
+__device__ __forceinline__ int64_t search_ids(const int32_t* __restrict__ ids, int64_t lo, int32_t n, int32_t t,
+                                              Tally& tb) {
+    while (n > 4) {
+        const int32_t s = n >> 2;
+        const int32_t a = __ldg(ids + lo + s), b = __ldg(ids + lo + 2 * s), c = __ldg(ids + lo + 3 * s);
+        tb.add(12);
+        if (b < t) {
+            if (c < t) {
+                lo += 3 * s + 1;
+                n -= 3 * s + 1;
+            } else {
+                lo += 2 * s + 1;
+                n = s - 1;
+            }
+        } else if (a < t) {
+            lo += s + 1;
+            n = s - 1;
+        } else {
+            n = s;
+        }
+    }
+    while (n > 0) {
+        const int32_t s = n >> 1;
+        tb.add(4);
+        if (__ldg(ids + lo + s) < t) {
+            lo += s + 1;
+            n -= s + 1;
+        } else {
+            n = s;
+        }
+    }
+    return lo;
+}
+
+// Appends a candidate: the active lanes take one atomic together.
+__device__ __forceinline__ void append(const Query& q, unsigned long long key, int32_t a, int32_t b, int32_t c) {
     const uint32_t active = __activemask();
-    const uint32_t peers = __match_any_sync(active, (unsigned long long)(uintptr_t)q.st);
-    const int lane = threadIdx.x & 31;
-    const int leader = __ffs(peers) - 1;
+    const int lane = threadIdx.x & 31, leader = __ffs(active) - 1;
     uint32_t base = 0;
-    if (lane == leader) base = atomicAdd(&q.st->count, (uint32_t)__popc(peers));
-    base = __shfl_sync(peers, base, leader);
-    const uint32_t idx = base + __popc(peers & ((1u << lane) - 1u));
+    if (lane == leader) base = atomicAdd(&q.st->count, (uint32_t)__popc(active));
+    base = __shfl_sync(active, base, leader);
+    const uint32_t idx = base + __popc(active & ((1u << lane) - 1u));
     if (idx < q.cap) {
         q.ckey[idx] = key;
         q.ctri[idx] = make_int4(a, b, c, 0);
@@ -278,862 +413,809 @@ __device__ __forceinline__ void append(const Query& q, unsigned long long key, i
 }
 
 // ---------------------------------------------------------------------------
-// Round: threads stride over the edges of [lo, hi).
+// Teams.  sync() is a barrier of the whole team; false: give up (a grid
+// barrier whose bounded wait ran out for good).
 // ---------------------------------------------------------------------------
-template <int P, bool SAMPLED>
-__device__ __forceinline__ void scan_wedges(const DevGraph& G, const Query& q,
-                                            unsigned long long tau, int32_t r, uint32_t w,
-                                            int32_t x, int32_t y, int64_t dy, uint32_t ymax,
-                                            int64_t& j, int64_t jstop, bool& done, Tally& tb) {
-    for (; j < jstop; j++) {
-        const uint32_t wxc = (uint32_t)__ldg(G.wwt + j);
-        tb.add(4);
-        if (boundof<P>(w, wxc, ymax, q.gp, q.fw != 0) < tau) {  // wedge bound, non-increasing along the list
-            done = true;
-            return;
-        }
-        const int32_t c = __ldg(G.wcol + j);
-        tb.add(4);
-        if (SAMPLED && c == y) continue;  // the edge itself (full rows in sampled mode)
-        int32_t wyc, ryc;
-        if (probe_oriented(G, y, dy, c, wyc, ryc, tb) &&
-            (tb.add(4), owns<SAMPLED>(q, r, __ldg(G.wrk + j), ryc))) {
-            const unsigned long long key = keyof<P>(w, wxc, (uint32_t)wyc, q.gp, q.fw != 0);
-            if (key >= tau) {
-                int32_t a = x, b = y, cc = c;
-                sort3(a, b, cc);
-                append(q, key, a, b, cc);
-            }
-        }
+// TB threads of a block that work through the one-block phases together:
+// the whole block, or one of its parts of TB threads (each with a named
+// barrier of its own).
+template <int TB>
+struct Part {
+    __device__ __forceinline__ int tid() const { return (int)(threadIdx.x % TB); }
+    __device__ __forceinline__ void sync() const {
+        asm volatile("barrier.cta.sync %0, %1;" ::"r"(1 + (int)(threadIdx.x / TB)), "n"(TB) : "memory");
     }
-}
-
-// Returns false once this edge's bound is below tau (and so is every later
-// edge's).
-template <int P, bool SAMPLED>
-__device__ __forceinline__ bool process_edge(const DevGraph& G, const Query& q,
-                                             unsigned long long tau, int32_t idx, Tally& tb) {
-    const int32_t r = SAMPLED ? __ldg(q.slist + idx) : idx;
-    const uint32_t w = (uint32_t)__ldg(G.ord_w + r);
-    tb.add(4);
-    if (!SAMPLED && boundof<P>(w, w, w, q.gp, q.fw != 0) < tau) {
-        // every later edge has a bound no larger: record the first such edge
-        atomicMax(&q.st->stop_rev, STOP_NONE - (uint32_t)r);
-        return false;
-    }
-    if (!SAMPLED && q.nshards > 1 &&
-        (int32_t)(((uint32_t)r >> SHARD_SHIFT) % (uint32_t)q.nshards) != q.shard)
-        return true;  // owned by another shard
-    const int32_t u = __ldg(G.ord_u + r), v = __ldg(G.ord_v + r);
-    const int64_t bu = __ldg(G.rowptr + u), eu = __ldg(G.rowptr + u + 1);
-    const int64_t bv = __ldg(G.rowptr + v), ev = __ldg(G.rowptr + v + 1);
-    tb.add(40);
-    // Exact mode scans what comes after r in each list; sampled mode scans
-    // whole lists (the other two edges may be heavier than a drawn edge).
-    const int64_t su = SAMPLED ? bu : suffix_start(G, bu, eu, r, &q.st->err, tb);
-    const int64_t sv = SAMPLED ? bv : suffix_start(G, bv, ev, r, &q.st->err, tb);
-    if (su >= eu || sv >= ev) return true;  // no edge after r on one side: owns nothing
-    const uint32_t umax = (uint32_t)__ldg(G.wwt + su), vmax = (uint32_t)__ldg(G.wwt + sv);
-    tb.add(8);
-    if (boundof<P>(w, umax, vmax, q.gp, q.fw != 0) < tau) return true;  // edge bound
-    // Scan the shorter suffix; probe the other endpoint.
-    const bool xu = (eu - su) <= (ev - sv);
-    const int32_t x = xu ? u : v, y = xu ? v : u;
-    const int64_t sx = xu ? su : sv, ex = xu ? eu : ev;
-    const uint32_t ymax = xu ? vmax : umax;
-    const int64_t dy = xu ? ev - bv : eu - bu;
-    int64_t j = sx;
-    bool done = false;
-    scan_wedges<P, SAMPLED>(G, q, tau, r, w, x, y, dy, ymax, j, min(ex, sx + (int64_t)q.t_short),
-                            done, tb);
-    if (!done && j < ex) {
-        const uint32_t slot = atomicAdd(q.long_count, 1u);
-        if (slot < q.long_cap) {
-            LongItem it;
-            it.r = r;
-            it.x = x;
-            it.y = y;
-            it.w = (int32_t)w;
-            it.ymax = (int32_t)ymax;
-            it.pad = q.qid;
-            it.j0 = j;
-            it.j1 = ex;
-            q.longs[slot] = it;
-        } else {
-            // Deferred list full: finish the scan here.
-            scan_wedges<P, SAMPLED>(G, q, tau, r, w, x, y, dy, ymax, j, ex, done, tb);
-        }
-    }
-    return true;
-}
-
-template <int P, bool SAMPLED = false>
-__global__ void __launch_bounds__(RBLK) k_round(DevGraph G, Query q, int64_t lo, int64_t hi) {
-    // Blocks run in any order, so an edge is skipped only once an edge at or
-    // before it has failed its bound (all later edges have no larger bound).
-    const volatile uint32_t* stop_rev = &q.st->stop_rev;
-    if (lo >= (int64_t)(STOP_NONE - *stop_rev)) return;
-    if (*(volatile const uint32_t*)&q.st->err) return;  // the query has already failed
-    const unsigned long long tau = ld_volatile_u64(&q.st->tau);
-    const int64_t stride = (int64_t)gridDim.x * RBLK;
-    Tally tb;
-    tb.on = q.qbytes != nullptr;
-    for (int64_t r64 = lo + (int64_t)blockIdx.x * RBLK + threadIdx.x; r64 < hi; r64 += stride) {
-        if (r64 >= (int64_t)(STOP_NONE - *stop_rev)) break;
-        if (!process_edge<P, SAMPLED>(G, q, tau, (int32_t)r64, tb)) break;
-    }
-    flush_tally(q, tb);
-}
-
-// Grid of a round: a few resident blocks per SM, striding over the range.
-inline unsigned round_grid(int64_t edges) {
-    const int64_t cap = (int64_t)sm_count() * 8;
-    return (unsigned)std::max<int64_t>(1, std::min<int64_t>(cap, (edges + RBLK - 1) / RBLK));
-}
-
-// ---------------------------------------------------------------------------
-// Round at p = -inf by NodeIterator++ over the degree order (Section 5.2):
-// one warp per edge r = {a, b}, a the endpoint of lower (degree, id) rank.
-// A triangle a < b < c in that order is found exactly once, from its edge
-// {a, b}, as c in N+(a) ∩ N+(b) (the oriented rows): the shorter row is
-// scanned and each c binary-searched in the other.  Its key min(w_ab, w_ac,
-// w_bc) is at most w_r, so the heavy-first stop of the sweep holds: once
-// w_r < tau no later edge can close a triangle that enters the top-k, and
-// entries lighter than tau are skipped before the search.  Every edge of a
-// qualifying triangle is at least tau, which is why this replaces the
-// weight-sorted scan (whose wedge bound prunes little at p = -inf) for the
-// unsampled, unsharded query.
-// ---------------------------------------------------------------------------
-constexpr int MIN_WARPS = RBLK / 32;
-#ifndef WTRI_MIN_STAGE
-#define WTRI_MIN_STAGE 512
-#endif
-// Longest searched row staged in shared memory (per warp; 0: never staged).
-constexpr int MIN_STAGE = WTRI_MIN_STAGE;
-
-__global__ void __launch_bounds__(RBLK) k_round_min(DevGraph G, Query q, int64_t lo, int64_t hi) {
-    const volatile uint32_t* stop_rev = &q.st->stop_rev;
-    if (lo >= (int64_t)(STOP_NONE - *stop_rev)) return;
-    if (*(volatile const uint32_t*)&q.st->err) return;  // the query has already failed
-    const unsigned long long tau = ld_volatile_u64(&q.st->tau);
-    const int lane = threadIdx.x & 31;
-    const int64_t nwarps = (int64_t)gridDim.x * MIN_WARPS;
-    __shared__ int32_t stage_all[MIN_WARPS][MIN_STAGE > 0 ? MIN_STAGE : 1];
-    int32_t* srow = stage_all[threadIdx.x >> 5];
-    Tally tb;
-    tb.on = q.qbytes != nullptr;
-    // The warp's next edge is fetched while this one is scanned: its weight
-    // and endpoints at the top of the iteration, its degrees once this
-    // edge's oriented-row bounds are issued.
-    int64_t r = lo + (int64_t)blockIdx.x * MIN_WARPS + (threadIdx.x >> 5);
-    uint32_t w_nx = 0;
-    int32_t u_nx = 0, v_nx = 0;
-    int64_t du_nx = 0, dv_nx = 0;
-    if (r < hi) {
-        w_nx = (uint32_t)__ldg(G.ord_w + r);
-        u_nx = __ldg(G.ord_u + r);
-        v_nx = __ldg(G.ord_v + r);
-        du_nx = __ldg(G.rowptr + u_nx + 1) - __ldg(G.rowptr + u_nx);
-        dv_nx = __ldg(G.rowptr + v_nx + 1) - __ldg(G.rowptr + v_nx);
-    }
-    for (; r < hi; r += nwarps) {
-        const uint32_t w = w_nx;
-        const int32_t u = u_nx, v = v_nx;
-        const int64_t du = du_nx, dv = dv_nx;
-        const int64_t rn = r + nwarps;
-        const bool more = rn < hi;
-        if (more) {
-            w_nx = (uint32_t)__ldg(G.ord_w + rn);
-            u_nx = __ldg(G.ord_u + rn);
-            v_nx = __ldg(G.ord_v + rn);
-        }
-        if (r >= (int64_t)(STOP_NONE - *stop_rev)) break;
-        if (w < tau) {
-            // every later edge is lighter: record the first such edge
-            if (lane == 0) atomicMax(&q.st->stop_rev, STOP_NONE - (uint32_t)r);
-            break;
-        }
-        const bool ua = du < dv || (du == dv && u < v);
-        const int32_t a = ua ? u : v, b = ua ? v : u;
-        const int64_t ab = __ldg(G.orowptr + a), ae = __ldg(G.orowptr + a + 1);
-        const int64_t bb = __ldg(G.orowptr + b), be = __ldg(G.orowptr + b + 1);
-        if (more) {
-            du_nx = __ldg(G.rowptr + u_nx + 1) - __ldg(G.rowptr + u_nx);
-            dv_nx = __ldg(G.rowptr + v_nx + 1) - __ldg(G.rowptr + v_nx);
-        }
-        if (lane == 0) tb.add(12 + 32 + 32);
-        const bool as = (ae - ab) <= (be - bb);
-        const int64_t sb = as ? ab : bb, se = as ? ae : be;  // scanned row
-        const int64_t lb = as ? bb : ab, le = as ? be : ae;  // searched row
-        // The searched row goes to shared memory (coalesced, once per edge)
-        // as soon as a chunk of the scanned row holds an entry >= tau: one
-        // latency step instead of a global binary search per entry.
-        const int64_t llen = le - lb;
-        bool staged = false;
-        for (int64_t base = sb; base < se; base += 32) {
-            const int64_t j = base + lane;
-            const uint32_t wsc = j < se ? (uint32_t)__ldg(G.owt + j) : 0u;
-            if (j < se) tb.add(4);
-            const bool heavy = j < se && wsc >= tau;
-            if (__ballot_sync(0xffffffffu, heavy) == 0) continue;
-            if (!staged && llen <= MIN_STAGE) {
-                for (int t = lane; t < llen; t += 32) srow[t] = __ldg(G.ocol + lb + t);
-                tb.add((uint32_t)(lane < llen ? 4 * ((llen - lane + 31) / 32) : 0));
-                __syncwarp();
-                staged = true;
-            }
-            if (!heavy) continue;
-            const int32_t c = __ldg(G.ocol + j);
-            tb.add(4);
-            int64_t l0, found_at = -1;
-            if (staged) {
-                int s0 = 0, s1 = (int)llen;
-                while (s0 < s1) {
-                    const int mid = (s0 + s1) >> 1;
-                    if (srow[mid] < c) s0 = mid + 1;
-                    else s1 = mid;
-                }
-                if (s0 < llen && srow[s0] == c) found_at = lb + s0;
-            } else {
-                int64_t l1 = le;
-                l0 = lb;
-                while (l0 < l1) {
-                    const int64_t mid = (l0 + l1) >> 1;
-                    tb.add(4);
-                    if (__ldg(G.ocol + mid) < c) l0 = mid + 1;
-                    else l1 = mid;
-                }
-                if (l0 < le && (tb.add(4), __ldg(G.ocol + l0) == c)) found_at = l0;
-            }
-            if (found_at >= 0) {
-                const uint32_t wlc = (uint32_t)__ldg(G.owt + found_at);
-                tb.add(4);
-                const unsigned long long key = keyof<P_MIN>(w, wsc, wlc);
-                if (key >= tau) {
-                    int32_t x = a, y = b, z = c;
-                    sort3(x, y, z);
-                    append(q, key, x, y, z);
-                }
-            }
-        }
-        __syncwarp();  // the staged row is reused by the warp's next edge
-    }
-    flush_tally(q, tb);
-}
-
-inline unsigned round_grid_warps(int64_t edges) {
-    const int64_t cap = (int64_t)sm_count() * 8;
-    return (unsigned)std::max<int64_t>(1, std::min<int64_t>(cap, (edges + MIN_WARPS - 1) / MIN_WARPS));
-}
-
-// ---------------------------------------------------------------------------
-// Round with one warp per edge, for the small early rounds (up to
-// WTRI_WARP_ROUND_MAX edges), where a thread per edge leaves the GPU almost
-// idle and each thread scans its entries one dependent search after another.
-// Same sweep as k_round: the edge checks and the two suffix searches once
-// per warp (lanes 0 and 1 search u's and v's lists at once), then the first
-// t_short entries (rounded up to a multiple of 32) of the shorter suffix,
-// one entry and one probe per lane; the rest is deferred to k_long.  The
-// wedge bound does not increase along a list, so the lanes that pass it are
-// exactly the entries a serial scan would reach.
-// ---------------------------------------------------------------------------
-#ifndef WTRI_WARP_ROUND_MAX
-#define WTRI_WARP_ROUND_MAX 4096
-#endif
-constexpr int64_t WARP_ROUND_MAX = WTRI_WARP_ROUND_MAX;
-
-// Scans [jb, je) of x's list, 32 entries per step; true once an entry fails
-// the wedge bound (and so does every later one).  Warp-uniform result.
-template <int P>
-__device__ __forceinline__ bool scan_wedges_warp(const DevGraph& G, const Query& q, unsigned long long tau,
-                                                 int32_t r, uint32_t w, int32_t x, int32_t y, int64_t dy,
-                                                 uint32_t ymax, int64_t jb, int64_t je, Tally& tb) {
-    const int lane = threadIdx.x & 31;
-    for (int64_t base = jb; base < je; base += 32) {
-        const int64_t j = base + lane;
-        const bool live = j < je;
-        uint32_t wxc = 0;
-        if (live) {
-            wxc = (uint32_t)__ldg(G.wwt + j);
-            tb.add(4);
-        }
-        const bool fail = live && boundof<P>(w, wxc, ymax, q.gp, q.fw != 0) < tau;
-        const bool stop = __any_sync(0xffffffffu, fail);
-        if (live && !fail) {
-            const int32_t c = __ldg(G.wcol + j);
-            tb.add(4);
-            int32_t wyc, ryc;
-            if (probe_oriented(G, y, dy, c, wyc, ryc, tb) &&
-                (tb.add(4), owns<false>(q, r, __ldg(G.wrk + j), ryc))) {
-                const unsigned long long key = keyof<P>(w, wxc, (uint32_t)wyc, q.gp, q.fw != 0);
-                if (key >= tau) {
-                    int32_t a = x, b = y, cc = c;
-                    sort3(a, b, cc);
-                    append(q, key, a, b, cc);
-                }
-            }
-        }
-        if (stop) return true;
-    }
-    return false;
-}
-
-// process_edge with the warp: false once the edge's bound is below tau.
-// tu counts the warp's shared loads once (lane 0).
-template <int P>
-__device__ __forceinline__ bool process_edge_warp(const DevGraph& G, const Query& q, unsigned long long tau,
-                                                  int32_t r, Tally& tb, Tally& tu) {
-    const int lane = threadIdx.x & 31;
-    const uint32_t w = (uint32_t)__ldg(G.ord_w + r);
-    tu.add(4);
-    if (boundof<P>(w, w, w, q.gp, q.fw != 0) < tau) {
-        if (lane == 0) atomicMax(&q.st->stop_rev, STOP_NONE - (uint32_t)r);
-        return false;
-    }
-    if (q.nshards > 1 && (int32_t)(((uint32_t)r >> SHARD_SHIFT) % (uint32_t)q.nshards) != q.shard)
-        return true;  // owned by another shard
-    const int32_t u = __ldg(G.ord_u + r), v = __ldg(G.ord_v + r);
-    const int64_t bu = __ldg(G.rowptr + u), eu = __ldg(G.rowptr + u + 1);
-    const int64_t bv = __ldg(G.rowptr + v), ev = __ldg(G.rowptr + v + 1);
-    tu.add(40);
-    Tally ts;  // lanes 0 and 1 count their own search; the others repeat lane 0's
-    ts.on = tb.on && lane < 2;
-    const bool side_v = lane == 1;
-    const int64_t s1 = suffix_start(G, side_v ? bv : bu, side_v ? ev : eu, r, &q.st->err, ts);
-    tb.n += ts.n;
-    const int64_t su = __shfl_sync(0xffffffffu, s1, 0), sv = __shfl_sync(0xffffffffu, s1, 1);
-    if (su >= eu || sv >= ev) return true;  // no edge after r on one side: owns nothing
-    const uint32_t umax = (uint32_t)__ldg(G.wwt + su), vmax = (uint32_t)__ldg(G.wwt + sv);
-    tu.add(8);
-    if (boundof<P>(w, umax, vmax, q.gp, q.fw != 0) < tau) return true;  // edge bound
-    const bool xu = (eu - su) <= (ev - sv);
-    const int32_t x = xu ? u : v, y = xu ? v : u;
-    const int64_t sx = xu ? su : sv, ex = xu ? eu : ev;
-    const uint32_t ymax = xu ? vmax : umax;
-    const int64_t dy = xu ? ev - bv : eu - bu;
-    const int64_t budget = q.t_short > 32 ? ((int64_t)q.t_short + 31) / 32 * 32 : 32;
-    const int64_t jlim = ex < sx + budget ? ex : sx + budget;
-    if (scan_wedges_warp<P>(G, q, tau, r, w, x, y, dy, ymax, sx, jlim, tb) || jlim >= ex) return true;
-    uint32_t slot = 0;
-    if (lane == 0) slot = atomicAdd(q.long_count, 1u);
-    slot = __shfl_sync(0xffffffffu, slot, 0);
-    if (slot < q.long_cap) {
-        if (lane == 0) {
-            LongItem it;
-            it.r = r;
-            it.x = x;
-            it.y = y;
-            it.w = (int32_t)w;
-            it.ymax = (int32_t)ymax;
-            it.pad = q.qid;
-            it.j0 = jlim;
-            it.j1 = ex;
-            q.longs[slot] = it;
-        }
-    } else {
-        // Deferred list full: finish the scan here.
-        scan_wedges_warp<P>(G, q, tau, r, w, x, y, dy, ymax, jlim, ex, tb);
-    }
-    return true;
-}
-
-template <int P>
-__global__ void __launch_bounds__(RBLK) k_round_warp(DevGraph G, Query q, int64_t lo, int64_t hi) {
-    const volatile uint32_t* stop_rev = &q.st->stop_rev;
-    if (lo >= (int64_t)(STOP_NONE - *stop_rev)) return;
-    if (*(volatile const uint32_t*)&q.st->err) return;  // the query has already failed
-    const unsigned long long tau = ld_volatile_u64(&q.st->tau);
-    const int lane = threadIdx.x & 31;
-    const int64_t nwarps = (int64_t)gridDim.x * MIN_WARPS;
-    Tally tb, tu;
-    tb.on = q.qbytes != nullptr;
-    tu.on = tb.on && lane == 0;
-    for (int64_t r = lo + (int64_t)blockIdx.x * MIN_WARPS + (threadIdx.x >> 5); r < hi; r += nwarps) {
-        uint32_t sr = 0;
-        if (lane == 0) sr = *stop_rev;
-        sr = __shfl_sync(0xffffffffu, sr, 0);  // one reading for the whole warp
-        if (r >= (int64_t)(STOP_NONE - sr)) break;
-        if (!process_edge_warp<P>(G, q, tau, (int32_t)r, tb, tu)) break;
-    }
-    tb.n += tu.n;
-    flush_tally(q, tb);
-}
-
-// ---------------------------------------------------------------------------
-// Deferred long scans: one block per item.  y's oriented row (ids) is
-// staged in shared memory with a bulk async copy completed on an mbarrier;
-// closing edges that y owns are binary searches there, the others searches
-// of the neighbour's oriented row in global memory.  Oriented rows longer
-// than STAGE_MAX are searched in global memory too.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count)
-                 : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-                 "r"(bytes)
-                 : "memory");
-}
-
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_u32(dst)),
-        "l"(src), "r"(bytes), "r"(smem_u32(bar))
-        : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t phase) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(phase)
-        : "memory");
-    return ok != 0;
-}
-
-// Stages y's oriented row (ids; beg = orowptr[y], len entries) in shared
-// memory with one bulk copy (bounded wait: at most `limit` polls; a limit of
-// 0 does not wait at all, which tests use to take the timeout path on
-// purpose).  Returns false if the wait ran out (error recorded); the copy in
-// flight is then drained with the full WAIT_LIMIT before the block goes on,
-// so no copy outlives its block.
-__device__ __forceinline__ bool stage_row(const DevGraph& G, int64_t beg, int32_t len, int32_t* srow,
-                                          uint64_t* bar, uint32_t& phase, int32_t& off, uint32_t* err,
-                                          int* timed_out, uint32_t limit) {
-    // 16-byte aligned source: round the start down, the size up (the id
-    // array has 16 bytes of slack after its end).
-    const int64_t a0 = beg & ~int64_t(3);
-    off = (int32_t)(beg - a0);
-    const uint32_t bytes = (uint32_t)(((off + len) * 4 + 15) & ~15);
-    if (threadIdx.x == 0) {
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_expect_tx(bar, bytes);
-        bulk_g2s(srow, G.ocol + a0, bytes, bar);
-    }
-    bool landed = false;
-    for (uint32_t spins = 0; spins < limit; spins++) {
-        if (mbar_try_wait(bar, phase)) {
-            landed = true;
-            break;
-        }
-    }
-    if (!landed) {
-        atomicOr(err, DEV_ERR_TIMEOUT);
-        *timed_out = 1;
-    }
-    const uint32_t cur = phase;
-    phase ^= 1u;
-    __syncthreads();
-    if (*timed_out) {
-        uint32_t s2 = 0;
-        while (!mbar_try_wait(bar, cur) && ++s2 < WAIT_LIMIT) {
-        }
-        return false;
-    }
-    return true;
-}
-
-// One deferred scan, all threads of the block.  Warps take 32-entry chunks
-// in order; the wedge bound only decreases along the list, so a warp whose
-// chunk fails entirely stops.
-template <int P, bool SAMPLED>
-__device__ __forceinline__ void long_scan(const DevGraph& G, const Query& q, unsigned long long tau,
-                                          const LongItem& item, const int32_t* srow, int32_t off,
-                                          int64_t obeg, int32_t ody, int64_t dy, bool staged, Tally& tb) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const uint32_t w = (uint32_t)item.w, ymax = (uint32_t)item.ymax;
-    const int32_t x = item.x, y = item.y, r = item.r;
-    for (int64_t base = item.j0 + (int64_t)wid * 32; base < item.j1; base += LBLK) {
-        const int64_t j = base + lane;
-        bool live = false;
-        uint32_t wxc = 0;
-        if (j < item.j1) {
-            wxc = (uint32_t)__ldg(G.wwt + j);
-            tb.add(4);
-            live = boundof<P>(w, wxc, ymax, q.gp, q.fw != 0) >= tau;
-        }
-        if (__ballot_sync(0xffffffffu, live) == 0) break;
-        int32_t c = 0;
-        if (live) {
-            c = __ldg(G.wcol + j);
-            tb.add(4);
-            if (SAMPLED && c == y) live = false;  // the edge itself
-        }
-        if (live) {
-            int32_t wyc = 0, ryc = -1;
-            bool found = false;
-            if (y_owns(G, y, dy, c, tb)) {
-                if (staged) {
-                    int lo = 0, hi = ody;
-                    while (lo < hi) {
-                        const int mid = (lo + hi) >> 1;
-                        if (srow[off + mid] < c) lo = mid + 1;
-                        else hi = mid;
-                    }
-                    if (lo < ody && srow[off + lo] == c) {
-                        found = true;
-                        wyc = __ldg(G.owt + obeg + lo);
-                        ryc = __ldg(G.ork + obeg + lo);
-                        tb.add(8);
-                    }
-                } else {
-                    found = search_oriented(G, y, c, wyc, ryc, tb);
-                }
-            } else {
-                found = search_oriented(G, c, y, wyc, ryc, tb);
-            }
-            if (found && (tb.add(4), owns<SAMPLED>(q, r, __ldg(G.wrk + j), ryc))) {
-                const unsigned long long key = keyof<P>(w, wxc, (uint32_t)wyc, q.gp, q.fw != 0);
-                if (key >= tau) {
-                    int32_t a = x, b = y, cc = c;
-                    sort3(a, b, cc);
-                    append(q, key, a, b, cc);
-                }
-            }
-        }
-    }
-}
-
-// Deferred long scans: one block per item.  y's oriented row (ids) is
-// staged in shared memory with a bulk async copy completed on an mbarrier;
-// closing edges that y owns are binary searches there, the others searches
-// of the neighbour's oriented row in global memory.  Oriented rows longer
-// than STAGE_MAX are searched in global memory too.
-template <int P, bool SAMPLED = false>
-__global__ void __launch_bounds__(LBLK) k_long(DevGraph G, Query q);
-
-// Dynamic shared memory of k_long: one staged row plus 16 bytes of rounding.
-constexpr size_t LONG_SMEM = (size_t)STAGE_MAX * 4 + 16;
-
-// Opts k_long<P, SAMPLED> in to LONG_SMEM bytes of dynamic shared memory on
-// the current device (once per device).
-template <int P, bool SAMPLED>
-int long_optin() {
-    static std::atomic<uint64_t> done{0};
-    return smem_optin((const void*)k_long<P, SAMPLED>, (int)LONG_SMEM, done);
-}
-
-template <int P, bool SAMPLED>
-__global__ void __launch_bounds__(LBLK) k_long(DevGraph G, Query q) {
-    extern __shared__ __align__(128) unsigned char lsm[];
-    int32_t* srow = reinterpret_cast<int32_t*>(lsm);
-    __shared__ __align__(8) uint64_t bar;
-    __shared__ int timed_out;
-    const uint32_t n_items = min(*(volatile const uint32_t*)q.long_count, q.long_cap);
-    if (blockIdx.x >= n_items) return;
-    if (*(volatile const uint32_t*)&q.st->err) return;  // the query has already failed
-    const unsigned long long tau = ld_volatile_u64(&q.st->tau);
-    if (threadIdx.x == 0) {
-        mbar_init(&bar, 1);
-        timed_out = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncthreads();
-    uint32_t phase = 0;
-    Tally tb;
-    tb.on = q.qbytes != nullptr;
-    for (uint32_t it = blockIdx.x; it < n_items; it += gridDim.x) {
-        const LongItem item = q.longs[it];
-        const int64_t dy = __ldg(G.rowptr + item.y + 1) - __ldg(G.rowptr + item.y);
-        const int64_t obeg = __ldg(G.orowptr + item.y);
-        const int32_t ody = (int32_t)(__ldg(G.orowptr + item.y + 1) - obeg);
-        const bool staged = ody > 0 && ody <= STAGE_MAX;
-        int32_t off = 0;
-        if (staged && !stage_row(G, obeg, ody, srow, &bar, phase, off, &q.st->err, &timed_out,
-                                 q.wait_first))
-            break;
-        if (staged && threadIdx.x == 0) tb.add((uint32_t)ody * 4u + 32u);  // offsets, the staged row
-        long_scan<P, SAMPLED>(G, q, tau, item, srow, off, obeg, ody, dy, staged, tb);
-        __syncthreads();  // the staged row is reused by the next item
-    }
-    flush_tally(q, tb);
-}
-
-// ---------------------------------------------------------------------------
-// Selection under the total order (key desc, a asc, b asc, c asc).
-// Each candidate maps to a 5-word tuple where smaller is better:
-//   (~key_hi, ~key_lo, a, b, c).  An MSB-first radix select over its 20
-// bytes finds the prefix P such that exactly K candidates have tuple
-// prefix <= P; those are kept (compacted in place).
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t tuple_word(unsigned long long key, int4 t, int wi) {
-    switch (wi) {
-        case 0: return ~(uint32_t)(key >> 32);
-        case 1: return ~(uint32_t)key;
-        case 2: return (uint32_t)t.x;
-        case 3: return (uint32_t)t.y;
-        default: return (uint32_t)t.z;
-    }
-}
-
-// Compare the first 'depth' bytes of a candidate's tuple with the prefix
-// (pw = prefix words).  Returns <0, 0, >0.
-__device__ __forceinline__ int cmp_prefix(unsigned long long key, int4 t, const uint32_t* pw,
-                                          int depth) {
-    const int full = depth >> 2, rem = depth & 3;
-    for (int wi = 0; wi < full; wi++) {
-        const uint32_t a = tuple_word(key, t, wi);
-        if (a != pw[wi]) return a < pw[wi] ? -1 : 1;
-    }
-    if (rem) {
-        const uint32_t mask = 0xffffffffu << (32 - 8 * rem);
-        const uint32_t a = tuple_word(key, t, full) & mask;
-        const uint32_t b = pw[full] & mask;
-        if (a != b) return a < b ? -1 : 1;
-    }
-    return 0;
-}
-
-struct SelectSmem {
-    unsigned long long prefix;   // key-only select: chosen high bytes
-    unsigned long long maxkey;
-    uint32_t need;               // key-only select: remaining rank
-    uint32_t hist[256];
-    uint32_t pw[5];
-    uint32_t below;   // candidates strictly better than the prefix
-    uint32_t eq;      // candidates equal to the prefix
-    uint32_t done;
-    uint32_t warp_cnt[SBLK / 32];
-    uint32_t kept;
-    unsigned long long minkey;
 };
 
-// Keeps exactly K = min(K_want, n) best candidates at the front; returns the
-// kept count and sets *minkey_out to their smallest key.
-__device__ uint32_t select_and_compact(unsigned long long* ckey, int4* ctri, uint32_t n,
-                                       uint32_t K, SelectSmem& S,
-                                       unsigned long long* minkey_out) {
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    if (tid < 5) S.pw[tid] = 0;
-    if (tid == 0) {
-        S.below = 0;
-        S.eq = n;
-        S.done = (n <= K) ? 1u : 0u;
-        S.minkey = ~0ull;
+template <int TB_>
+struct BlockTeam {
+    static constexpr int TB = TB_;
+    static constexpr bool GRID = false;
+    Part<TB_> part;
+    __device__ __forceinline__ int64_t thread() const { return part.tid(); }
+    __device__ __forceinline__ int64_t threads() const { return TB; }
+    __device__ __forceinline__ int64_t warp() const { return part.tid() >> 5; }
+    __device__ __forceinline__ int64_t warps() const { return TB / 32; }
+    __device__ __forceinline__ bool leader() const { return true; }
+    __device__ __forceinline__ bool sync(const Query&) {
+        part.sync();
+        return true;
     }
-    __syncthreads();
-    int depth = 0;  // bytes fixed in the prefix
-    while (!S.done && depth < 20) {
-        for (int i = tid; i < 256; i += SBLK) S.hist[i] = 0;
-        __syncthreads();
-        const int wi = depth >> 2, sh = 24 - 8 * (depth & 3);
-        for (uint32_t base = 0; base < n; base += SBLK) {
-            const uint32_t i = base + tid;
-            uint32_t d = 256;
-            if (i < n) {
-                const unsigned long long kk = ckey[i];
-                const int4 t = ctri[i];
-                if (cmp_prefix(kk, t, S.pw, depth) == 0) d = (tuple_word(kk, t, wi) >> sh) & 255u;
-            }
-            const uint32_t peers = __match_any_sync(0xffffffffu, d);
-            if (d < 256 && (__ffs(peers) - 1) == lane) atomicAdd(&S.hist[d], __popc(peers));
-        }
-        __syncthreads();
-        if (tid == 0) {
-            // Need the K-th overall: K - below among the prefix-equal ones.
-            const uint32_t need = K - S.below;
-            uint32_t acc = 0, dsel = 0;
-            for (uint32_t d = 0; d < 256; d++) {
-                const uint32_t h = S.hist[d];
-                if (acc + h >= need) {
-                    dsel = d;
-                    break;
-                }
-                acc += h;
-            }
-            S.below += acc;
-            S.eq = S.hist[dsel];
-            S.pw[wi] |= dsel << sh;
-            if (S.below + S.eq == K) S.done = 1;
-        }
-        __syncthreads();
-        depth++;
-    }
-    const int final_depth = depth;
-    // Compact in place: keep tuple prefix <= P (or everything if n <= K).
-    const bool keep_all = (n <= K);
-    uint32_t out = 0;
-    unsigned long long mk = ~0ull;
-    for (uint32_t base = 0; base < n; base += SBLK) {
-        const uint32_t i = base + tid;
-        bool keep = false;
-        unsigned long long kk = 0;
-        int4 t = make_int4(0, 0, 0, 0);
-        if (i < n) {
-            kk = ckey[i];
-            t = ctri[i];
-            keep = keep_all || cmp_prefix(kk, t, S.pw, final_depth) <= 0;
-        }
-        const uint32_t b = __ballot_sync(0xffffffffu, keep);
-        if (lane == 0) S.warp_cnt[wid] = __popc(b);
-        __syncthreads();
-        if (tid == 0) {
-            uint32_t acc = 0;
-            for (int wv = 0; wv < SBLK / 32; wv++) {
-                const uint32_t c = S.warp_cnt[wv];
-                S.warp_cnt[wv] = acc;
-                acc += c;
-            }
-            S.kept = acc;
-        }
-        __syncthreads();
-        if (keep) {
-            const uint32_t p = out + S.warp_cnt[wid] + __popc(b & ((1u << lane) - 1u));
-            ckey[p] = kk;  // p <= i: writes never overtake unread entries
-            ctri[p] = t;
-            mk = kk < mk ? kk : mk;
-        }
-        out += S.kept;
-        __syncthreads();
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long y = __shfl_xor_sync(0xffffffffu, mk, o);
-        mk = y < mk ? y : mk;
-    }
-    if (lane == 0) atomicMin(&S.minkey, mk);
-    __syncthreads();
-    *minkey_out = S.minkey;
-    return out;
-}
+};
 
-// The K-th largest key among n candidates (one block, MSB-first over the
-// significant bytes only).
-__device__ unsigned long long kth_key(const unsigned long long* ckey, uint32_t n, uint32_t K,
-                                      SelectSmem& S) {
-    const int tid = threadIdx.x, lane = tid & 31;
-    unsigned long long mx = 0;
-    for (uint32_t i = tid; i < n; i += SBLK) mx = max(mx, ckey[i]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long y = __shfl_xor_sync(0xffffffffu, mx, o);
-        mx = y > mx ? y : mx;
+// nblk blocks of a cooperative launch (all resident), from block blk0 on.  A
+// barrier: every block's
+// first thread arrives at a counter in the query's state and polls it up to
+// a limit.  The first limit is the query's wait_first; when it runs out the
+// query is marked timed out and the block waits on with the full limit, so
+// that the blocks stay in step; only when that runs out too does it leave.
+template <int TB_>
+struct GridTeam {
+    static constexpr int TB = TB_;
+    static constexpr bool GRID = true;
+    Part<TB_> part;
+    uint32_t target = 0;
+    uint32_t limit;
+    uint32_t blk0, nblk;
+    int* gone;  // shared
+    __device__ __forceinline__ int64_t thread() const { return (int64_t)(blockIdx.x - blk0) * TB + threadIdx.x; }
+    __device__ __forceinline__ int64_t threads() const { return (int64_t)nblk * TB; }
+    __device__ __forceinline__ int64_t warp() const { return thread() >> 5; }
+    __device__ __forceinline__ int64_t warps() const { return threads() >> 5; }
+    __device__ __forceinline__ bool leader() const { return blockIdx.x == blk0; }
+    __device__ __forceinline__ uint32_t arrivals(const Query& q) const {
+        uint32_t v;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&q.st->bar) : "memory");
+        return v;
     }
-    if (tid == 0) {
-        S.prefix = 0;
-        S.maxkey = 0;
-        S.need = K;
-    }
-    __syncthreads();
-    if (lane == 0) atomicMax(&S.maxkey, mx);
-    __syncthreads();
-    int nbytes = 0;
-    for (unsigned long long t = S.maxkey; t; t >>= 8) nbytes++;
-    for (int byte = nbytes - 1; byte >= 0; byte--) {
-        const int shift = 8 * byte;
-        const unsigned long long hi_mask = (shift + 8 >= 64) ? 0ull : (~0ull << (shift + 8));
-        for (int i = tid; i < 256; i += SBLK) S.hist[i] = 0;
+    __device__ __forceinline__ bool sync(const Query& q) {
+        target += nblk;
         __syncthreads();
-        const unsigned long long prefix = S.prefix;
-        for (uint32_t base = 0; base < n; base += SBLK) {
-            const uint32_t i = base + tid;
-            uint32_t d = 256;
-            if (i < n) {
-                const unsigned long long kk = ckey[i];
-                if ((kk & hi_mask) == (prefix & hi_mask)) d = (uint32_t)(kk >> shift) & 255u;
+        if (threadIdx.x == 0) {
+            __threadfence();
+            atomicAdd(&q.st->bar, 1u);
+            bool there = false;
+            for (uint32_t i = 0; i < limit && !there; i++) there = (int32_t)(arrivals(q) - target) >= 0;
+            if (!there) {
+                atomicOr(&q.st->err, DEV_ERR_TIMEOUT);
+                for (uint32_t i = 0; i < WAIT_LIMIT && !there; i++) there = (int32_t)(arrivals(q) - target) >= 0;
             }
-            const uint32_t peers = __match_any_sync(0xffffffffu, d);
-            if (d < 256 && (__ffs(peers) - 1) == lane) atomicAdd(&S.hist[d], __popc(peers));
+            limit = WAIT_LIMIT;
+            if (!there) *gone = 1;
+            __threadfence();
         }
         __syncthreads();
-        if (tid == 0) {
-            const uint32_t need = S.need;
-            uint32_t acc = 0;
-            int dsel = 0;
-            for (int d = 255; d >= 0; d--) {
-                const uint32_t h = S.hist[d];
-                if (acc + h >= need) {
-                    dsel = d;
-                    break;
-                }
-                acc += h;
-            }
-            S.need = need - acc;
-            S.prefix = prefix | ((unsigned long long)dsel << shift);
-        }
-        __syncthreads();
+        return *gone == 0;
     }
-    const unsigned long long T = S.prefix;
-    __syncthreads();
-    return T;
-}
+};
 
-// Keeps candidates with key >= T at the front (in place); returns how many.
-__device__ uint32_t compact_ge(unsigned long long* ckey, int4* ctri, uint32_t n,
-                               unsigned long long T, SelectSmem& S) {
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    uint32_t out = 0;
-    for (uint32_t base = 0; base < n; base += SBLK) {
-        const uint32_t i = base + tid;
-        bool keep = false;
-        unsigned long long kk = 0;
-        int4 t = make_int4(0, 0, 0, 0);
-        if (i < n) {
-            kk = ckey[i];
-            keep = kk >= T;
-            if (keep) t = ctri[i];
-        }
-        const uint32_t b = __ballot_sync(0xffffffffu, keep);
-        if (lane == 0) S.warp_cnt[wid] = __popc(b);
-        __syncthreads();
-        if (tid == 0) {
-            uint32_t acc = 0;
-            for (int wv = 0; wv < SBLK / 32; wv++) {
-                const uint32_t c = S.warp_cnt[wv];
-                S.warp_cnt[wv] = acc;
-                acc += c;
-            }
-            S.kept = acc;
-        }
-        __syncthreads();
-        if (keep) {
-            const uint32_t p = out + S.warp_cnt[wid] + __popc(b & ((1u << lane) - 1u));
-            ckey[p] = kk;  // p <= i: writes never overtake unread entries
-            ctri[p] = t;
-        }
-        out += S.kept;
-        __syncthreads();
-    }
-    return out;
-}
+// ---------------------------------------------------------------------------
+// Items.
+// ---------------------------------------------------------------------------
+constexpr int ITEM_SHIFT = 44;  // item count above, wedge count below (both fit: at most 2^18 items)
+constexpr unsigned long long WEDGE_MASK = (1ull << ITEM_SHIFT) - 1;
 
-// After each round: tau = the k-th largest key among the candidates (a
-// lower bound on the final k-th key, since they are k distinct triangles),
-// and candidates below tau are dropped.  Ties with tau stay; the final step
-// resolves them by the vertex triple.
-__device__ void select_round(const Query& q, SelectSmem& S) {
-    const uint32_t err = *(volatile uint32_t*)&q.st->err;
-    if (err) return;
-    const uint32_t n = min(*(volatile uint32_t*)&q.st->count, q.cap);
-    if (n == q.st->selected || n < (uint32_t)q.k) {
-        if (threadIdx.x == 0) *q.long_count = 0;
+__device__ __forceinline__ void put_item(const Query& q, uint32_t slot, unsigned long long base, const Item& it) {
+    if (slot >= (uint32_t)q.item_cap) {
+        atomicOr(&q.st->err, DEV_ERR_INTERNAL);
         return;
     }
-    const unsigned long long T = kth_key(q.ckey, n, (uint32_t)q.k, S);
-    const uint32_t kept = compact_ge(q.ckey, q.ctri, n, T, S);
-    if (threadIdx.x == 0) {
-        q.st->count = kept;
-        q.st->selected = kept;
-        *q.long_count = 0;
-        if (T > q.st->tau) q.st->tau = T;
+    q.items[slot] = it;
+    q.ibase[slot] = base;
+}
+
+// Every lane of a warp: the lanes with len > 0 leave their item.
+__device__ __forceinline__ void push_items(const Query& q, int par, int64_t len, const Item& it) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t has = __ballot_sync(0xffffffffu, len > 0);
+    if (!has) return;
+    unsigned long long inc = len > 0 ? (unsigned long long)len : 0ull;
+    const unsigned long long mine = inc;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    unsigned long long old = 0;
+    if (lane == 31) old = atomicAdd(&q.st->items[par], ((unsigned long long)__popc(has) << ITEM_SHIFT) + inc);
+    old = __shfl_sync(0xffffffffu, old, 31);
+    if (len > 0)
+        put_item(q, (uint32_t)(old >> ITEM_SHIFT) + __popc(has & lanemask_below()), (old & WEDGE_MASK) + inc - mine,
+                 it);
+}
+
+// ---------------------------------------------------------------------------
+// One wedge (entry j of x's weight-sorted list) of edge r = {x, y}.  The
+// neighbour's degree and both its row bounds are loaded together: one step
+// of latency before the search.
+// ---------------------------------------------------------------------------
+template <int P, bool SAMPLED>
+__device__ __forceinline__ void wedge(const DevGraph& G, const Query& q, unsigned long long tau, int32_t r, uint32_t w,
+                                      int32_t x, int32_t y, int64_t dy, int64_t yb, int32_t yn, int64_t j, Tally& tb) {
+    const int32_t c = __ldg(G.wcol + j);
+    const uint32_t wxc = (uint32_t)__ldg(G.wwt + j);
+    const int32_t rxc = __ldg(G.wrk + j);
+    if (SAMPLED && c == y) return;  // the edge itself (full rows in sampled mode)
+    const int64_t c0 = __ldg(G.rowptr + c), c1 = __ldg(G.rowptr + c + 1);
+    const int64_t o0 = __ldg(G.orowptr + c), o1 = __ldg(G.orowptr + c + 1);
+    tb.add(12 + 32);
+    const int64_t dc = c1 - c0;
+    const bool yo = dy < dc || (dy == dc && y < c);  // the edge lies in the row of the lower-ranked endpoint
+    const int64_t lb = yo ? yb : o0;
+    const int32_t ln = yo ? yn : (int32_t)(o1 - o0), t = yo ? c : y;
+    const int64_t at = search_ids(G.ocol, lb, ln, t, tb);
+    if (at >= lb + ln) return;
+    tb.add(4);
+    if (__ldg(G.ocol + at) != t) return;
+    const uint32_t wyc = (uint32_t)__ldg(G.owt + at);
+    tb.add(8);
+    if (!owns<SAMPLED>(q, r, rxc, __ldg(G.ork + at))) return;
+    if (P == P_GEN && Line<P>(q, tau, w, wxc).fails(wyc)) return;  // surely below: no fp64 key
+    const unsigned long long key = keyof<P>(w, wxc, wyc, q.gp, q.fw != 0);
+    if (key >= tau) {
+        int32_t a = x, b = y, cc = c;
+        sort3(a, b, cc);
+        append(q, key, a, b, cc);
     }
 }
 
-__global__ void __launch_bounds__(SBLK) k_select(Query q) {
-    __shared__ SelectSmem S;
-    select_round(q, S);
+// Entry j of the scanned oriented row of the edge {a, b} at p = -inf; the
+// third vertex is searched in the other row [lb, lb + ln).
+__device__ __forceinline__ void min_entry(const DevGraph& G, const Query& q, unsigned long long tau, uint32_t w,
+                                          int32_t a, int32_t b, int64_t lb, int32_t ln, int64_t j, uint32_t wsc,
+                                          Tally& tb) {
+    const int32_t c = __ldg(G.ocol + j);
+    tb.add(4);
+    const int64_t at = search_ids(G.ocol, lb, ln, c, tb);
+    if (at >= lb + ln) return;
+    tb.add(4);
+    if (__ldg(G.ocol + at) != c) return;
+    const uint32_t wlc = (uint32_t)__ldg(G.owt + at);
+    tb.add(4);
+    const unsigned long long key = keyof<P_MIN>(w, wsc, wlc);
+    if (key >= tau) {
+        int32_t x = a, y = b, z = c;
+        sort3(x, y, z);
+        append(q, key, x, y, z);
+    }
 }
 
-// Final ranking: candidate i's rank is the number of kept candidates before
-// it in the total order.
+// ---------------------------------------------------------------------------
+// Phase A, heavy-first sweep.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ bool other_shard(const Query& q, int32_t r) {
+    return q.nshards > 1 && (int32_t)(((uint32_t)r >> SHARD_SHIFT) % (uint32_t)q.nshards) != q.shard;
+}
+
+// A warp per edge: lanes 0-15 search u's list, lanes 16-31 v's.
+template <int P, bool SAMPLED, class Team>
+__device__ __forceinline__ void edges_by_warp(const DevGraph& G, const Query& q, unsigned long long tau, int64_t lo,
+                                              int64_t hi, int par, const Team& T, Tally& tb) {
+    const int lane = threadIdx.x & 31;
+    const bool sv_ = lane >= 16;
+    for (int64_t idx = lo + T.warp(); idx < hi; idx += T.warps()) {
+        const int32_t r = SAMPLED ? __ldg(q.slist + idx) : (int32_t)idx;
+        if (!SAMPLED && other_shard(q, r)) continue;
+        const int32_t u = __ldg(G.ord_u + r), v = __ldg(G.ord_v + r);
+        const uint32_t w = (uint32_t)__ldg(G.ord_w + r);
+        const int32_t me = sv_ ? v : u;
+        const int64_t b = __ldg(G.rowptr + me), e = __ldg(G.rowptr + me + 1);
+        const int64_t ob = __ldg(G.orowptr + me), oe = __ldg(G.orowptr + me + 1);
+        if ((lane & 15) == 0) tb.add(6 + 32);
+        // Exact mode scans what comes after r in each list; sampled mode scans
+        // whole lists (the other two edges may be heavier than a drawn edge).
+        int64_t s = b;
+        bool bad = false;
+        if (!SAMPLED) {
+            s = group_search<16>(b, e, [&](int64_t p) {
+                tb.add(4);
+                return __ldg(G.wrk + p) < r;
+            });
+            bad = s >= e || __ldg(G.wrk + s) != r;
+            s++;
+        }
+        if (__any_sync(0xffffffffu, bad)) {
+            if (bad) atomicOr(&q.st->err, DEV_ERR_INTERNAL);
+            continue;
+        }
+        if (__any_sync(0xffffffffu, s >= e)) continue;  // no edge after r on one side: owns nothing
+        const uint32_t top = (uint32_t)__ldg(G.wwt + s);
+        const uint32_t oth = __shfl_xor_sync(0xffffffffu, top, 16);
+        const Line<P> line(q, tau, w, oth);
+        if (__any_sync(0xffffffffu, line.fails(top))) continue;  // edge bound
+        int64_t end = e;
+        if (tau != 0)
+            end = group_search<16>(s, e, [&](int64_t p) {
+                tb.add(4);
+                return !line.fails((uint32_t)__ldg(G.wwt + p));
+            });
+        const int64_t len = end - s, olen = __shfl_xor_sync(0xffffffffu, len, 16);
+        // x: the endpoint of the shorter live range (u on a tie)
+        const bool x_me = sv_ ? len < olen : len <= olen;
+        const int src = __ffs(__ballot_sync(0xffffffffu, x_me)) - 1, dst = src ^ 16;
+        const int64_t j0 = __shfl_sync(0xffffffffu, s, src), n = __shfl_sync(0xffffffffu, len, src);
+        const int32_t x = __shfl_sync(0xffffffffu, me, src), y = __shfl_sync(0xffffffffu, me, dst);
+        const int64_t dy = __shfl_sync(0xffffffffu, e - b, dst);
+        const int64_t yb = __shfl_sync(0xffffffffu, ob, dst);
+        const int32_t yn = (int32_t)__shfl_sync(0xffffffffu, oe - ob, dst);
+        const int64_t budget = q.t_short > 32 ? ((int64_t)q.t_short + 31) / 32 * 32 : 32;
+        if (n <= budget) {
+            for (int64_t j = j0 + lane; j < j0 + n; j += 32)
+                wedge<P, SAMPLED>(G, q, tau, r, w, x, y, dy, yb, yn, j, tb);
+            __syncwarp();
+        } else if (lane == 0) {
+            const unsigned long long old =
+                atomicAdd(&q.st->items[par], (1ull << ITEM_SHIFT) + (unsigned long long)n);
+            put_item(q, (uint32_t)(old >> ITEM_SHIFT), old & WEDGE_MASK,
+                     Item{r, x, y, w, j0, yb, yn, (int32_t)dy, {0, 0}});
+        }
+        __syncwarp();
+    }
+}
+
+// A thread per edge: large rounds, where most edges fail the edge bound.
+template <int P, bool SAMPLED, class Team>
+__device__ __forceinline__ void edges_by_thread(const DevGraph& G, const Query& q, unsigned long long tau, int64_t lo,
+                                                int64_t hi, int par, const Team& T, Tally& tb) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t i0 = lo + T.warp() * 32; i0 < hi; i0 += T.warps() * 32) {
+        const int64_t idx = i0 + lane;
+        int64_t n = 0;
+        Item it{};
+        if (idx < hi) {
+            const int32_t r = SAMPLED ? __ldg(q.slist + idx) : (int32_t)idx;
+            if (SAMPLED || !other_shard(q, r)) {
+                const int32_t u = __ldg(G.ord_u + r), v = __ldg(G.ord_v + r);
+                const uint32_t w = (uint32_t)__ldg(G.ord_w + r);
+                const int64_t bu = __ldg(G.rowptr + u), eu = __ldg(G.rowptr + u + 1);
+                const int64_t bv = __ldg(G.rowptr + v), ev = __ldg(G.rowptr + v + 1);
+                tb.add(44);
+                int64_t su = bu, sv = bv;
+                bool bad = false;
+                if (!SAMPLED) {  // both suffix searches step together
+                    int64_t hu = eu, hv = ev;
+                    while (su < hu || sv < hv) {
+                        const int64_t mu = (su + hu) >> 1, mv = (sv + hv) >> 1;
+                        const int32_t ku = su < hu ? __ldg(G.wrk + mu) : 0, kv = sv < hv ? __ldg(G.wrk + mv) : 0;
+                        tb.add(8);
+                        if (su < hu) {
+                            if (ku < r) su = mu + 1;
+                            else hu = mu;
+                        }
+                        if (sv < hv) {
+                            if (kv < r) sv = mv + 1;
+                            else hv = mv;
+                        }
+                    }
+                    bad = su >= eu || sv >= ev || __ldg(G.wrk + su) != r || __ldg(G.wrk + sv) != r;
+                    if (bad) atomicOr(&q.st->err, DEV_ERR_INTERNAL);
+                    su++;
+                    sv++;
+                }
+                if (!bad && su < eu && sv < ev) {
+                    const uint32_t umax = (uint32_t)__ldg(G.wwt + su), vmax = (uint32_t)__ldg(G.wwt + sv);
+                    tb.add(8);
+                    const Line<P> lu(q, tau, w, vmax);  // along u's list
+                    if (!lu.fails(umax)) {
+                        int64_t nu = eu - su, nv = ev - sv;
+                        if (tau != 0) {  // both live ranges
+                            const Line<P> lv(q, tau, w, umax);
+                            int64_t pu = su + 1, hu = eu, pv = sv + 1, hv = ev;
+                            while (pu < hu || pv < hv) {
+                                const int64_t mu = (pu + hu) >> 1, mv = (pv + hv) >> 1;
+                                const uint32_t ku = pu < hu ? (uint32_t)__ldg(G.wwt + mu) : 0u;
+                                const uint32_t kv = pv < hv ? (uint32_t)__ldg(G.wwt + mv) : 0u;
+                                tb.add(8);
+                                if (pu < hu) {
+                                    if (!lu.fails(ku)) pu = mu + 1;
+                                    else hu = mu;
+                                }
+                                if (pv < hv) {
+                                    if (!lv.fails(kv)) pv = mv + 1;
+                                    else hv = mv;
+                                }
+                            }
+                            nu = pu - su;
+                            nv = pv - sv;
+                        }
+                        const bool xu = nu <= nv;
+                        n = xu ? nu : nv;
+                        it.r = r;
+                        it.x = xu ? u : v;
+                        it.y = xu ? v : u;
+                        it.w = w;
+                        it.j0 = xu ? su : sv;
+                        it.lb = __ldg(G.orowptr + it.y);
+                        it.ln = (int32_t)(__ldg(G.orowptr + it.y + 1) - it.lb);
+                        it.dy = (int32_t)(xu ? ev - bv : eu - bu);
+                        tb.add(16);
+                    }
+                }
+            }
+        }
+        push_items(q, par, n, it);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Phase A at p = -inf by NodeIterator++ over the degree order (Section 5.2):
+// for each edge r = {a, b}, a the endpoint of lower (degree, id) rank, a
+// triangle a < b < c in that order is found exactly once, as c in N+(a) and
+// N+(b) (the oriented rows): the shorter row is scanned and each c searched
+// in the other.  Its key min(w_ab, w_ac, w_bc) is at most w_r, so the
+// heavy-first stop of the sweep holds, and entries lighter than tau are
+// skipped before the search.  Every edge of a qualifying triangle is at
+// least tau, which is why this replaces the weight-sorted scan (whose wedge
+// bound prunes little at p = -inf) for the unsampled, unsharded query.
+// ---------------------------------------------------------------------------
+struct MinRows {
+    int32_t a, b;
+    int64_t sb, se, lb;  // scanned row, searched row
+    int32_t ln;
+};
+
+__device__ __forceinline__ MinRows min_rows(int32_t u, int32_t v, int64_t du, int64_t dv, int64_t u0, int64_t u1,
+                                            int64_t v0, int64_t v1) {
+    MinRows R;
+    const bool ua = du < dv || (du == dv && u < v);
+    R.a = ua ? u : v;
+    R.b = ua ? v : u;
+    const bool us = (u1 - u0) < (v1 - v0) || ((u1 - u0) == (v1 - v0) && ua);
+    R.sb = us ? u0 : v0;
+    R.se = us ? u1 : v1;
+    R.lb = us ? v0 : u0;
+    R.ln = (int32_t)(us ? v1 - v0 : u1 - u0);
+    return R;
+}
+
+// Small rounds: every edge leaves its scanned row as an item.
+template <class Team>
+__device__ __forceinline__ void min_edges_items(const DevGraph& G, const Query& q, int64_t lo, int64_t hi, int par,
+                                                const Team& T, Tally& tb) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t i0 = lo + T.warp() * 32; i0 < hi; i0 += T.warps() * 32) {
+        const int64_t r = i0 + lane;
+        int64_t n = 0;
+        Item it{};
+        if (r < hi) {
+            const int32_t u = __ldg(G.ord_u + r), v = __ldg(G.ord_v + r);
+            const int64_t du = __ldg(G.rowptr + u + 1) - __ldg(G.rowptr + u);
+            const int64_t dv = __ldg(G.rowptr + v + 1) - __ldg(G.rowptr + v);
+            const MinRows R = min_rows(u, v, du, dv, __ldg(G.orowptr + u), __ldg(G.orowptr + u + 1),
+                                       __ldg(G.orowptr + v), __ldg(G.orowptr + v + 1));
+            tb.add(12 + 64);
+            it = Item{(int32_t)r, R.a, R.b, (uint32_t)__ldg(G.ord_w + r), R.sb, R.lb, R.ln, 0, {0, 0}};
+            n = R.ln > 0 ? R.se - R.sb : 0;
+        }
+        push_items(q, par, n, it);
+    }
+}
+
+// Large rounds, where few entries reach tau: GL lanes per edge read its
+// scanned row 4 GL weights at a time (16-byte loads, the next ones in flight
+// while these are compared), 32 / GL edges to a warp, the endpoints of the
+// edges two steps ahead and the row bounds of the next step's edges loaded
+// while this step scans.  The entries that reach tau wait in the warp's queue
+// until 32 of them are there, and are then searched one per lane.
+struct MinProbe {
+    int64_t j, lb;
+    int32_t ln;
+    uint32_t w;
+    int32_t a, b;
+};
+constexpr int64_t MIN_WIDE = 12;  // edges per vertex from which a scanned row gets eight lanes, not four
+constexpr int MINQ = 64;  // a step of at most 32 entries on top of at most 31 waiting
+
+template <int GL, class Team>
+__device__ __forceinline__ void min_edges_filtered(const DevGraph& G, const Query& q, unsigned long long tau,
+                                                   int64_t lo, int64_t hi, const Team& T, MinProbe* queue, Tally& tb) {
+    constexpr int EPW = 32 / GL;  // edges per warp and step
+    const int lane = threadIdx.x & 31, gl = lane & (GL - 1);
+    const uint32_t lt = lanemask_below();
+    const int64_t first = lo + T.warp() * EPW, stride = T.warps() * EPW;
+    const int32_t* ord = gl == 0 ? G.ord_u : (gl == 1 ? G.ord_v : G.ord_w);
+    auto triple = [&](int64_t r) { return gl < 3 && r < hi ? __ldg(ord + r) : 0; };
+    struct Bounds {
+        int64_t row, orow;
+    };
+    auto bounds = [&](int64_t r, int32_t t) {  // lane gl: bound gl & 1 of the rows of u or v (gl & 2)
+        const int32_t u = __shfl_sync(0xffffffffu, t, 0, GL), v = __shfl_sync(0xffffffffu, t, 1, GL);
+        Bounds x{0, 0};
+        if (r < hi) {
+            const int64_t i = (int64_t)(gl & 2 ? v : u) + (gl & 1);
+            x.row = __ldg(G.rowptr + i);
+            x.orow = __ldg(G.orowptr + i);
+        }
+        return x;
+    };
+    int qn = 0;
+    auto probe = [&](int n) {  // the queue's last n entries, one per lane
+        __syncwarp();
+        if (lane < n) {
+            const MinProbe e = queue[qn - n + lane];
+            min_entry(G, q, tau, e.w, e.a, e.b, e.lb, e.ln, e.j, (uint32_t)__ldg(G.owt + e.j), tb);
+        }
+        __syncwarp();
+        qn -= n;
+    };
+    int64_t r = first + lane / GL;
+    if (first >= hi) return;
+    int32_t t0 = triple(r), t1 = triple(r + stride);
+    Bounds b0 = bounds(r, t0);
+    for (int64_t base = first; base < hi; base += stride, r += stride) {
+        const int32_t t2 = triple(r + 2 * stride);
+        const Bounds b1 = bounds(r + stride, t1);
+        const int32_t u = __shfl_sync(0xffffffffu, t0, 0, GL), v = __shfl_sync(0xffffffffu, t0, 1, GL);
+        const uint32_t w = (uint32_t)__shfl_sync(0xffffffffu, t0, 2, GL);
+        int64_t x[4], ox[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            x[k] = __shfl_sync(0xffffffffu, b0.row, k, GL);
+            ox[k] = __shfl_sync(0xffffffffu, b0.orow, k, GL);
+        }
+        const MinRows R = min_rows(u, v, x[1] - x[0], x[3] - x[2], ox[0], ox[1], ox[2], ox[3]);
+        const int64_t se = r < hi && R.ln > 0 ? R.se : R.sb;
+        if (gl == 0) tb.add(12 + 64);
+        int64_t j = (R.sb & ~int64_t(3)) + 4 * gl;
+        int4 nx = j < se ? __ldg(reinterpret_cast<const int4*>(G.owt + j)) : make_int4(0, 0, 0, 0);
+        while (__any_sync(0xffffffffu, j < se)) {
+            const int4 cur = nx;
+            const int64_t jc = j;
+            j += 4 * GL;
+            nx = j < se ? __ldg(reinterpret_cast<const int4*>(G.owt + j)) : make_int4(0, 0, 0, 0);
+            const uint32_t cw[4] = {(uint32_t)cur.x, (uint32_t)cur.y, (uint32_t)cur.z, (uint32_t)cur.w};
+            if (jc < se) tb.add(16);
+            bool heavy[4], some = false;
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                heavy[k] = jc + k >= R.sb && jc + k < se && cw[k] >= tau;
+                some |= heavy[k];
+            }
+            if (!__any_sync(0xffffffffu, some)) continue;
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                const uint32_t m = __ballot_sync(0xffffffffu, heavy[k]);
+                if (heavy[k]) queue[qn + __popc(m & lt)] = MinProbe{jc + k, R.lb, R.ln, w, R.a, R.b};
+                qn += __popc(m);
+                if (qn >= 32) probe(32);
+            }
+        }
+        t0 = t1;
+        t1 = t2;
+        b0 = b1;
+    }
+    if (qn > 0) probe(qn);
+}
+
+// ---------------------------------------------------------------------------
+// Phase B: the items' wedges, numbered through.  Each warp takes a contiguous
+// share, 32 at a time; a lane finds its wedge's item among the next 32 items
+// (each has at least one wedge).
+// ---------------------------------------------------------------------------
+template <int P, bool SAMPLED, bool ORIENTED, class Team>
+__device__ __forceinline__ void item_wedges(const DevGraph& G, const Query& q, unsigned long long tau, int par,
+                                            const Team& T, Tally& tb) {
+    const unsigned long long ctr = *(volatile const unsigned long long*)&q.st->items[par];
+    const int64_t cnt = (int64_t)(ctr >> ITEM_SHIFT), tot = (int64_t)(ctr & WEDGE_MASK);
+    if (cnt > q.item_cap) return;
+    const int lane = threadIdx.x & 31;
+    const int64_t chunks = (tot + 31) >> 5, per = (chunks + T.warps() - 1) / T.warps();
+    const int64_t beg = T.warp() * per * 32, end = min(tot, beg + per * 32);
+    if (beg >= end) return;
+    const unsigned long long* ib = q.ibase;
+    int64_t it0 = group_search<32>(0, cnt, [&](int64_t p) { return (int64_t)ib[p] <= beg; }) - 1;
+    for (int64_t e0 = beg; e0 < end; e0 += 32) {
+        // where item it0 + lane ends, relative to e0
+        const int64_t nxt = it0 + 1 + lane;
+        const int64_t rel = (nxt < cnt ? (int64_t)ib[nxt] : tot) - e0;
+        const int stop = rel > 64 ? 64 : (int)rel;
+        int k = 0;
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1) {
+            const int v = __shfl_sync(0xffffffffu, stop, (k + s - 1) & 31);
+            if (v <= lane) k += s;
+        }
+        const int64_t i = it0 + k;
+        if (e0 + lane < end) {
+            const int4* p = reinterpret_cast<const int4*>(q.items + i);
+            const int4 a = p[0], b = p[1], c = p[2];
+            const int64_t j0 = ((int64_t)(uint32_t)b.y << 32) | (uint32_t)b.x;
+            const int64_t lb = ((int64_t)(uint32_t)b.w << 32) | (uint32_t)b.z;
+            const int64_t j = j0 + (e0 + lane - (int64_t)ib[i]);
+            if constexpr (ORIENTED) {
+                const uint32_t wsc = (uint32_t)__ldg(G.owt + j);
+                tb.add(4);
+                if (wsc >= tau) min_entry(G, q, tau, (uint32_t)a.w, a.y, a.z, lb, c.x, j, wsc, tb);
+            } else {
+                wedge<P, SAMPLED>(G, q, tau, a.x, (uint32_t)a.w, a.y, a.z, c.y, lb, c.x, j, tb);
+            }
+        }
+        __syncwarp();
+        const int k31 = __shfl_sync(0xffffffffu, k, 31);
+        const int s31 = __shfl_sync(0xffffffffu, stop, k31);
+        it0 += k31 + (s31 <= 32 ? 1 : 0);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Selection under the total order (key desc, a asc, b asc, c asc), one block.
+// Radix selects take digits of 11 bits from the highest bit in which the
+// candidates differ; the whole block scans a histogram's bins (a serial scan
+// by one thread cost 4 us per digit, half of every select).
+// ---------------------------------------------------------------------------
+constexpr int SEL_BITS = 11;
+constexpr int SEL_BINS = 1 << SEL_BITS;
+
+struct SelectSmem {
+    uint32_t hist[SEL_BINS];
+    uint32_t wsum[32];
+    unsigned long long mn, mx;
+    uint32_t bin, above, taken;
+    int gone;  // a grid barrier gave up
+};
+
+// The ranking's shared arrays (aliases the p = -inf queues of phase A).
+struct SortSmem {
+    unsigned long long key[SORT_MAX];
+    int32_t tri[3][SORT_MAX];
+    uint16_t id[SORT_MAX];
+};
+
+// First bin (in bin order) at which the running count reaches need (>= 1,
+// at most the histogram's sum): S.bin, and the count before it in S.above.
+template <int TB>
+__device__ __forceinline__ void pick_bin(const Part<TB>& B, SelectSmem& S, uint32_t need) {
+    constexpr int PER = SEL_BINS / TB;
+    const int tid = B.tid(), lane = tid & 31, wid = tid >> 5;
+    uint32_t h[PER], sum = 0;
+#pragma unroll
+    for (int i = 0; i < PER; i++) {
+        h[i] = S.hist[tid * PER + i];
+        sum += h[i];
+    }
+    uint32_t inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    if (lane == 31) S.wsum[wid] = inc;
+    B.sync();
+    uint32_t before = 0;
+#pragma unroll
+    for (int k = 0; k < TB / 32; k++) before += k < wid ? S.wsum[k] : 0u;
+    uint32_t acc = before + inc - sum;
+    if (acc < need && need <= acc + sum) {
+#pragma unroll
+        for (int i = 0; i < PER; i++) {
+            if (acc < need && need <= acc + h[i]) {
+                S.bin = (uint32_t)(tid * PER + i);
+                S.above = acc;
+            }
+            acc += h[i];
+        }
+    }
+    B.sync();
+}
+
+template <int TB>
+__device__ __forceinline__ void clear_hist(const Part<TB>& B, SelectSmem& S) {
+    for (int i = B.tid(); i < SEL_BINS; i += TB) S.hist[i] = 0;
+    B.sync();
+}
+
+// Counts d (< SEL_BINS; larger: nothing): the lanes of one bin add together.
+__device__ __forceinline__ void count_bin(SelectSmem& S, uint32_t d) {
+    const uint32_t peers = __match_any_sync(0xffffffffu, d);
+    if (d < SEL_BINS && (int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&S.hist[d], __popc(peers));
+}
+
+// The K-th largest of n keys (K <= n).
+template <int TB>
+__device__ unsigned long long kth_key(const Part<TB>& B, const unsigned long long* ckey, uint32_t n, uint32_t K, SelectSmem& S) {
+    const int tid = B.tid(), lane = tid & 31;
+    unsigned long long mx = 0, mn = ~0ull;
+#pragma unroll 4
+    for (uint32_t i = tid; i < n; i += TB) {
+        const unsigned long long x = ckey[i];
+        mx = x > mx ? x : mx;
+        mn = x < mn ? x : mn;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long a = __shfl_xor_sync(0xffffffffu, mx, o), b = __shfl_xor_sync(0xffffffffu, mn, o);
+        mx = a > mx ? a : mx;
+        mn = b < mn ? b : mn;
+    }
+    if (tid == 0) {
+        S.mx = 0;
+        S.mn = ~0ull;
+    }
+    B.sync();
+    if (lane == 0) {
+        atomicMax(&S.mx, mx);
+        atomicMin(&S.mn, mn);
+    }
+    B.sync();
+    mx = S.mx;
+    mn = S.mn;
+    if (mx == mn) return mx;
+    int shift = 64 - __clzll((long long)(mx ^ mn));  // the bits that differ
+    unsigned long long prefix = shift >= 64 ? 0ull : (mx >> shift) << shift;
+    uint32_t need = K;
+    while (shift > 0) {
+        const int bits = shift < SEL_BITS ? shift : SEL_BITS, hi = shift;
+        shift -= bits;
+        const uint32_t mask = (1u << bits) - 1u;
+        clear_hist<TB>(B, S);
+#pragma unroll 4
+        for (uint32_t base = 0; base < n; base += TB) {
+            const uint32_t i = base + tid;
+            uint32_t d = SEL_BINS;
+            if (i < n) {
+                const unsigned long long x = ckey[i];
+                if (hi >= 64 || (x >> hi) == (prefix >> hi)) d = mask - ((uint32_t)(x >> shift) & mask);  // descending
+            }
+            count_bin(S, d);
+        }
+        B.sync();
+        pick_bin<TB>(B, S, need);
+        prefix |= (unsigned long long)(mask - S.bin) << shift;
+        need -= S.above;
+        B.sync();
+    }
+    return prefix;
+}
+
+// Keeps the candidates for which keep(key, triple) holds at the front, in any
+// order, in place: a step's entries are in registers before any is written,
+// and no more are written than were read.  Returns how many.
+template <int TB, class Keep>
+__device__ uint32_t compact(const Part<TB>& B, unsigned long long* ckey, int4* ctri, uint32_t n, const Keep& keep, SelectSmem& S) {
+    constexpr int U = 2;
+    const int tid = B.tid(), lane = tid & 31;
+    if (tid == 0) S.taken = 0;
+    for (uint32_t base = 0; base < n; base += U * TB) {
+        unsigned long long k[U];
+        int4 t[U];
+        bool on[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const uint32_t i = base + u * TB + tid;
+            on[u] = false;
+            if (i < n) {
+                k[u] = ckey[i];
+                t[u] = ctri[i];
+                on[u] = keep(k[u], t[u]);
+            }
+        }
+        B.sync();
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const uint32_t b = __ballot_sync(0xffffffffu, on[u]);
+            uint32_t at = 0;
+            if (lane == 0 && b) at = atomicAdd(&S.taken, (uint32_t)__popc(b));
+            at = __shfl_sync(0xffffffffu, at, 0) + __popc(b & lanemask_below());
+            if (on[u]) {
+                ckey[at] = k[u];
+                ctri[at] = t[u];
+            }
+        }
+    }
+    B.sync();
+    const uint32_t got = S.taken;
+    B.sync();
+    return got;
+}
+
+__device__ __forceinline__ uint32_t tri_word(const int4& t, int i) {
+    return (uint32_t)(i == 0 ? t.x : (i == 1 ? t.y : t.z));
+}
+
+// Candidates all >= T: keeps those above T and the first of those equal to T
+// in triple order, K in all (n > K; fewer than K lie above T).
+template <int TB>
+__device__ uint32_t keep_first_ties(const Part<TB>& B, unsigned long long* ckey, int4* ctri, uint32_t n, uint32_t K,
+                                    unsigned long long T, SelectSmem& S) {
+    const int tid = B.tid();
+    if (tid == 0) S.taken = 0;
+    B.sync();
+    uint32_t mine = 0;
+    for (uint32_t i = tid; i < n; i += TB) mine += ckey[i] > T ? 1u : 0u;
+    if (mine) atomicAdd(&S.taken, mine);
+    B.sync();
+    uint32_t need = K - S.taken;
+    B.sync();
+    // limit: the need-th smallest triple among the ties, word by word
+    uint32_t lim[3] = {0u, 0u, 0u};
+    for (int wi = 0; wi < 3; wi++) {
+        int shift = 32;
+        while (shift > 0) {
+            const int bits = shift < SEL_BITS ? shift : SEL_BITS, hi = shift;
+            shift -= bits;
+            const uint32_t mask = (1u << bits) - 1u;
+            clear_hist<TB>(B, S);
+            for (uint32_t base = 0; base < n; base += TB) {
+                const uint32_t i = base + tid;
+                uint32_t d = SEL_BINS;
+                if (i < n && ckey[i] == T) {
+                    const int4 t = ctri[i];
+                    bool same = true;
+                    for (int k = 0; k < wi; k++) same = same && tri_word(t, k) == lim[k];
+                    const uint32_t x = tri_word(t, wi);
+                    if (same && (hi >= 32 || (x >> hi) == (lim[wi] >> hi))) d = (x >> shift) & mask;
+                }
+                count_bin(S, d);
+            }
+            B.sync();
+            pick_bin<TB>(B, S, need);
+            lim[wi] |= S.bin << shift;
+            need -= S.above;
+            B.sync();
+        }
+    }
+    const uint32_t l0 = lim[0], l1 = lim[1], l2 = lim[2];
+    return compact<TB>(B, ckey, ctri, n,
+                       [=](unsigned long long k, const int4& t) {
+                           if (k != T) return k > T;
+                           if ((uint32_t)t.x != l0) return (uint32_t)t.x < l0;
+                           if ((uint32_t)t.y != l1) return (uint32_t)t.y < l1;
+                           return (uint32_t)t.z <= l2;
+                       },
+                       S);
+}
+
+// After a round: tau = the k-th largest key among the candidates (a lower
+// bound on the final k-th key, since they are k distinct triangles), and
+// candidates below tau are dropped.  Ties with tau stay; the final step
+// resolves them by the vertex triple.  Returns how much larger the next round
+// may be: `growth`, or less where rounds as productive as this one would
+// fill half of the free candidate slots (small buffers: a batched query at
+// p = -inf overflowed its 16,384 slots at a fixed growth of 8).
+template <int TB>
+__device__ int64_t select_round(const Part<TB>& B, const Query& q, SelectSmem& S) {
+    const int64_t growth = q.growth;
+    if (*(volatile uint32_t*)&q.st->err) return growth;
+    const uint32_t n = min(*(volatile uint32_t*)&q.st->count, q.cap);
+    const uint32_t old = *(volatile uint32_t*)&q.st->selected;
+    B.sync();  // `selected` is rewritten below
+    if (n == old) return growth;
+    const int64_t added = n - old;
+    if (n < (uint32_t)q.k) {
+        if (B.tid() == 0) *(volatile uint32_t*)&q.st->selected = n;  // all of them stay
+        return max(int64_t(1), min(growth, (int64_t)(q.cap - n) / (2 * added)));
+    }
+    const unsigned long long T = kth_key<TB>(B, q.ckey, n, (uint32_t)q.k, S);
+    const uint32_t kept = compact<TB>(B, q.ckey, q.ctri, n, [=](unsigned long long k, const int4&) { return k >= T; }, S);
+    if (B.tid() == 0) {
+        *(volatile uint32_t*)&q.st->count = kept;
+        *(volatile uint32_t*)&q.st->selected = kept;
+        if (T > q.st->tau) *(volatile unsigned long long*)&q.st->tau = T;
+    }
+    B.sync();
+    return max(int64_t(1), min(growth, (int64_t)(q.cap - kept) / (2 * added)));
+}
+
+// The next round's range: [lo, lo + size) cut at the first edge whose bound
+// is below tau (the edges' weights do not increase).
+template <int P, bool SAMPLED>
+__device__ __forceinline__ void next_range(int tid, const DevGraph& G, const Query& q, int64_t lo, int64_t size, int64_t total) {
+    if (tid >= 32) return;
+    const bool failed = *(volatile uint32_t*)&q.st->err != 0;
+    const unsigned long long tau = ld_volatile_u64(&q.st->tau);
+    int64_t hi = failed ? lo : min(total, lo + size);
+    if (!SAMPLED && tau != 0)
+        hi = group_search<32>(lo, hi, [&](int64_t p) { return !edge_below<P>(q, (uint32_t)__ldg(G.ord_w + p), tau); });
+    if (tid == 0) {
+        *(volatile long long*)&q.st->lo = lo;
+        *(volatile long long*)&q.st->hi = hi;
+        *(volatile long long*)&q.st->size = size;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Ranking and outputs.
+// ---------------------------------------------------------------------------
 __device__ __forceinline__ bool before(unsigned long long ka, int4 a, unsigned long long kb, int4 b) {
     if (ka != kb) return ka > kb;
     if (a.x != b.x) return a.x < b.x;
@@ -1141,68 +1223,247 @@ __device__ __forceinline__ bool before(unsigned long long ka, int4 a, unsigned l
     return a.z < b.z;
 }
 
-// Candidate i's rank is the number of kept candidates before it in the
-// total order; one warp per candidate.  Also writes the status word.
 template <int P>
-__device__ __forceinline__ void rank_one(const Query& q, uint32_t i, wtri_tri* out_tri,
-                                         double* out_w, int32_t* out_count,
-                                         unsigned long long* out_key = nullptr) {
-    const uint32_t err = *(volatile uint32_t*)&q.st->err;
-    const uint32_t n = min(*(volatile uint32_t*)&q.st->count, q.cap);
-    const int lane = threadIdx.x & 31;
-    if (i == 0 && lane == 0) {
-        // a timeout first: it stops the per-round compaction, so a buffer
-        // overflow that follows it is its consequence, not the cause
-        int32_t status = (int32_t)n;
-        if (err & DEV_ERR_TIMEOUT) status = WTRI_ETIMEOUT;
-        else if (err & DEV_ERR_OVERFLOW) status = WTRI_ENOMEM;
-        else if (err) status = WTRI_ECUDA;
-        *out_count = status;
+__device__ __forceinline__ void write_rank(const Query& q, const Out& o, uint32_t rank, unsigned long long key,
+                                           int32_t a, int32_t b, int32_t c) {
+    o.tri[rank].a = a;
+    o.tri[rank].b = b;
+    o.tri[rank].c = c;
+    double val;
+    if (P == P_ONE) val = (double)key / 3.0;
+    else if (P == P_TWO) val = sqrt((double)key / 3.0);
+    else if (P == P_GEO) val = cbrt((double)key);
+    else if (P == P_GEN) val = __longlong_as_double((long long)key);
+    else val = q.fw ? (double)__uint_as_float((uint32_t)key) : (double)key;  // min, max
+    o.w[rank] = val;
+    if (o.key) o.key[rank] = key;
+}
+
+// Sorts n <= SORT_MAX candidates in shared memory (bitonic over positions)
+// and writes the first k.
+template <int P, int TB>
+__device__ __forceinline__ void sort_and_write(const Part<TB>& B, const Query& q, const Out& o, uint32_t n, SortSmem& R) {
+    uint32_t N = 2;
+    while (N < n) N <<= 1;
+    for (uint32_t i = B.tid(); i < N; i += TB) {
+        R.key[i] = i < n ? q.ckey[i] : 0ull;  // keys are positive: padding ranks last
+        const int4 t = i < n ? q.ctri[i] : make_int4(INT32_MAX, INT32_MAX, INT32_MAX, 0);
+        R.tri[0][i] = t.x;
+        R.tri[1][i] = t.y;
+        R.tri[2][i] = t.z;
+        R.id[i] = (uint16_t)i;
     }
-    if (err || i >= n) return;
-    const unsigned long long ki = q.ckey[i];
-    const int4 ti = q.ctri[i];
-    uint32_t rank = 0;
-    for (uint32_t j = lane; j < n; j += 32) rank += before(q.ckey[j], q.ctri[j], ki, ti) ? 1u : 0u;
+    B.sync();
+    auto first = [&](uint32_t a, uint32_t b) {  // candidate a ranks before b
+        if (R.key[a] != R.key[b]) return R.key[a] > R.key[b];
+        if (R.tri[0][a] != R.tri[0][b]) return R.tri[0][a] < R.tri[0][b];
+        if (R.tri[1][a] != R.tri[1][b]) return R.tri[1][a] < R.tri[1][b];
+        return R.tri[2][a] < R.tri[2][b];
+    };
+    for (uint32_t size = 2; size <= N; size <<= 1)
+        for (uint32_t d = size >> 1; d > 0; d >>= 1) {
+            for (uint32_t t = B.tid(); t < N / 2; t += TB) {
+                const uint32_t i = 2 * t - (t & (d - 1)), j = i + d;
+                const uint32_t a = R.id[i], b = R.id[j];
+                if ((i & size) == 0 ? first(b, a) : first(a, b)) {
+                    R.id[i] = (uint16_t)b;
+                    R.id[j] = (uint16_t)a;
+                }
+            }
+            B.sync();
+        }
+    for (uint32_t i = B.tid(); i < min(n, (uint32_t)q.k); i += TB) {
+        const uint32_t c = R.id[i];
+        write_rank<P>(q, o, i, R.key[c], R.tri[0][c], R.tri[1][c], R.tri[2][c]);
+    }
+}
+
+// The k best candidates in order, and the status word.  k <= SORT_MAX: one
+// block sorts them; above, every warp of the team ranks candidates by
+// counting those before them (a grid team).
+template <int P, class Team>
+__device__ void finish(const Query& q, const Out& o, Team& T, SelectSmem& S, SortSmem& R) {
+    const uint32_t K = (uint32_t)q.k;
+    const Part<Team::TB>& B = T.part;
+    if (T.leader()) {
+        const uint32_t err = *(volatile uint32_t*)&q.st->err;
+        uint32_t n = min(*(volatile uint32_t*)&q.st->count, q.cap);
+        B.sync();
+        if (err) n = 0;
+        if (n > K) {
+            unsigned long long T0 = ld_volatile_u64(&q.st->tau);
+            if (n != *(volatile uint32_t*)&q.st->selected) {
+                T0 = kth_key<Team::TB>(B, q.ckey, n, K, S);
+                n = compact<Team::TB>(B, q.ckey, q.ctri, n, [=](unsigned long long k, const int4&) { return k >= T0; }, S);
+            }
+            if (n > K && (n > SORT_MAX || K > SORT_MAX)) n = keep_first_ties<Team::TB>(B, q.ckey, q.ctri, n, K, T0, S);
+        }
+        if (B.tid() == 0) {
+            // a timeout first: an overflow that follows it is its consequence
+            int32_t status = (int32_t)min(n, K);
+            if (err & DEV_ERR_TIMEOUT) status = WTRI_ETIMEOUT;
+            else if (err & DEV_ERR_OVERFLOW) status = WTRI_ENOMEM;
+            else if (err) status = WTRI_ECUDA;
+            *o.count = status;
+            *(volatile uint32_t*)&q.st->kept = n;
+        }
+        if (K <= SORT_MAX) sort_and_write<P, Team::TB>(B, q, o, n, R);
+    }
+    if (Team::GRID && K > SORT_MAX) {
+        if (!T.sync(q)) return;
+        const uint32_t n = *(volatile uint32_t*)&q.st->kept;
+        const int lane = threadIdx.x & 31;
+        for (int64_t i = T.warp(); i < (int64_t)n; i += T.warps()) {
+            const unsigned long long ki = q.ckey[i];
+            const int4 ti = q.ctri[i];
+            uint32_t rank = 0;
+            for (uint32_t j = lane; j < n; j += 32) rank += before(q.ckey[j], q.ctri[j], ki, ti) ? 1u : 0u;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
-    if (lane == 0) {
-        out_tri[rank].a = ti.x;
-        out_tri[rank].b = ti.y;
-        out_tri[rank].c = ti.z;
-        double val;
-        if (P == P_ONE) val = (double)ki / 3.0;
-        else if (P == P_TWO) val = sqrt((double)ki / 3.0);
-        else if (P == P_GEO) val = cbrt((double)ki);
-        else if (P == P_GEN) val = __longlong_as_double((long long)ki);
-        else val = q.fw ? (double)__uint_as_float((uint32_t)ki) : (double)ki;  // min, max
-        out_w[rank] = val;
-        if (out_key) out_key[rank] = ki;
+            for (int s = 16; s > 0; s >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, s);
+            if (lane == 0) write_rank<P>(q, o, rank, ki, ti.x, ti.y, ti.z);
+        }
     }
 }
 
+// ---------------------------------------------------------------------------
+// The whole sweep.
+// ---------------------------------------------------------------------------
+template <int TB>
+struct SweepSmem {
+    SelectSmem sel;
+    union {
+        SortSmem sort;
+        MinProbe queue[TB / 32][MINQ];
+    };
+};
+
+template <int P, bool SAMPLED, class Team>
+__device__ void sweep(const DevGraph& G, const Query& q, const Out& o, Team& T, SweepSmem<Team::TB>& S) {
+    const bool oriented = P == P_MIN && !SAMPLED && q.nshards <= 1;
+    const int64_t total = q.total_dev ? __ldg(q.total_dev) : q.total;
+    // rounds of at most item_cap edges (an item each); the filtered p = -inf
+    // rounds leave none
+    const int64_t cap = oriented ? INT64_MAX / 16 : q.item_cap;
+    int64_t size = min(q.first, min(cap, q.item_cap)), lo = 0, hi = min(total, size);
+    unsigned long long tau = 0;
+    Tally tb;
+    tb.on = q.qbytes != nullptr;
+    for (int par = 0; lo < hi; par ^= 1) {
+        bool items = true;
+        if constexpr (P == P_MIN && !SAMPLED) {
+            if (oriented) {
+                items = hi - lo <= min(MIN_FLAT, q.item_cap);
+                if (items) min_edges_items(G, q, lo, hi, par, T, tb);
+                else if (G.m < MIN_WIDE * G.n) min_edges_filtered<4>(G, q, tau, lo, hi, T, S.queue[T.part.tid() >> 5], tb);
+                else min_edges_filtered<8>(G, q, tau, lo, hi, T, S.queue[T.part.tid() >> 5], tb);
+            }
+        }
+        if (!oriented) {
+            if (hi - lo <= min(WARP_EDGES, T.warps() * 4)) edges_by_warp<P, SAMPLED>(G, q, tau, lo, hi, par, T, tb);
+            else edges_by_thread<P, SAMPLED>(G, q, tau, lo, hi, par, T, tb);
+        }
+        if (!T.sync(q)) return;
+        if (items) {
+            if constexpr (P == P_MIN && !SAMPLED) {
+                if (oriented) item_wedges<P, false, true>(G, q, tau, par, T, tb);
+            }
+            if (!oriented) item_wedges<P, SAMPLED, false>(G, q, tau, par, T, tb);
+            if (!T.sync(q)) return;
+        }
+        if (T.leader()) {
+            if (T.part.tid() == 0) *(volatile unsigned long long*)&q.st->items[par ^ 1] = 0;
+            const int64_t grow = select_round<Team::TB>(T.part, q, S.sel);
+            next_range<P, SAMPLED>(T.part.tid(), G, q, hi, min(size * grow, cap), total);
+        }
+        if (!T.sync(q)) return;
+        size = *(volatile long long*)&q.st->size;
+        tau = ld_volatile_u64(&q.st->tau);
+        lo = *(volatile long long*)&q.st->lo;
+        hi = *(volatile long long*)&q.st->hi;
+    }
+    flush_tally(q, tb);
+    finish<P>(q, o, T, S.sel, S.sort);
+}
+
+template <int P, bool SAMPLED>
+__global__ void __launch_bounds__(TGRID, 1) k_sweep(DevGraph G, Query q, Out o) {
+    extern __shared__ __align__(16) unsigned char sweep_smem[];
+    SweepSmem<TGRID>& S = *reinterpret_cast<SweepSmem<TGRID>*>(sweep_smem);
+    GridTeam<TGRID> T;
+    T.limit = q.wait_first;
+    T.blk0 = 0;
+    T.nblk = gridDim.x;
+    T.gone = &S.sel.gone;
+    if (threadIdx.x == 0) S.sel.gone = 0;
+    __syncthreads();
+    sweep<P, SAMPLED>(G, q, o, T, S);
+}
+
+// Launches the sweep of one query on the whole GPU (a cooperative launch:
+// its blocks wait for one another, so all must be resident).
+template <int P, bool SAMPLED>
+int launch_sweep(const DevGraph& G, const Query& q, const Out& o, cudaStream_t s) {
+    static std::atomic<uint64_t> done{0};
+    const void* fn = (const void*)k_sweep<P, SAMPLED>;
+    const size_t smem = sizeof(SweepSmem<TGRID>);
+    WTRI_TRY(smem_optin(fn, (int)smem, done));
+    DevGraph g = G;
+    Query qq = q;
+    Out oo = o;
+    void* args[] = {&g, &qq, &oo};
+    WTRI_CUDA(cudaLaunchCooperativeKernel(fn, dim3((unsigned)sm_count()), dim3(TGRID), args, smem, s));
+    return WTRI_OK;
+}
+
+// The ranking alone, of candidates already collected (k <= SORT_MAX): one
+// block, no other has to be resident.
 template <int P>
-__global__ void __launch_bounds__(256) k_rank_scatter(Query q, wtri_tri* out_tri, double* out_w,
-                                                      int32_t* out_count,
-                                                      unsigned long long* out_key) {
-    const uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (i >= (uint32_t)max(q.k, 1)) return;
-    rank_one<P>(q, i, out_tri, out_w, out_count, out_key);
+__global__ void __launch_bounds__(TGRID, 1) k_finish(Query q, Out o) {
+    extern __shared__ __align__(16) unsigned char sweep_smem[];
+    SweepSmem<TGRID>& S = *reinterpret_cast<SweepSmem<TGRID>*>(sweep_smem);
+    BlockTeam<TGRID> T;
+    finish<P>(q, o, T, S.sel, S.sort);
 }
 
-__device__ void final_select(const Query& q, SelectSmem& S) {
-    const uint32_t err = *(volatile uint32_t*)&q.st->err;
-    if (err) return;
-    const uint32_t n = min(*(volatile uint32_t*)&q.st->count, q.cap);
-    unsigned long long mk;
-    const uint32_t kept = select_and_compact(q.ckey, q.ctri, n, (uint32_t)q.k, S, &mk);
-    if (threadIdx.x == 0) q.st->count = kept;
+template <int P>
+int launch_finish(const DevGraph& G, const Query& q, const Out& o, cudaStream_t s) {
+    if (q.k > SORT_MAX) return launch_sweep<P, false>(G, q, o, s);  // (no rounds: q.total = 0)
+    static std::atomic<uint64_t> done{0};
+    const size_t smem = sizeof(SweepSmem<TGRID>);
+    WTRI_TRY(smem_optin((const void*)k_finish<P>, (int)smem, done));
+    k_finish<P><<<1, TGRID, smem, s>>>(q, o);
+    WTRI_CUDA(cudaGetLastError());
+    return WTRI_OK;
 }
 
-__global__ void __launch_bounds__(SBLK) k_final_select(Query q) {
-    __shared__ SelectSmem S;
-    final_select(q, S);
+// Scratch of one query: bytes, and the pieces carved from a 256-byte aligned
+// block (every piece starts 256-byte aligned).
+inline size_t query_scratch_bytes(uint32_t cap, int64_t item_cap) {
+    auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    return al(sizeof(QState)) + al((size_t)cap * 8) + al((size_t)cap * 16) + al((size_t)item_cap * sizeof(Item)) +
+           al((size_t)item_cap * 8);
 }
+inline char* query_carve(Query& q, char* p, uint32_t cap, int64_t item_cap) {
+    auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    q = Query{};
+    q.st = (QState*)p;
+    p += al(sizeof(QState));
+    q.ckey = (unsigned long long*)p;
+    p += al((size_t)cap * 8);
+    q.ctri = (int4*)p;
+    p += al((size_t)cap * 16);
+    q.items = (Item*)p;
+    p += al((size_t)item_cap * sizeof(Item));
+    q.ibase = (unsigned long long*)p;
+    p += al((size_t)item_cap * 8);
+    q.cap = cap;
+    q.item_cap = item_cap;
+    q.nshards = 1;
+    q.wait_first = WAIT_LIMIT;
+    return p;
+}
+// Items of a graph's query: at most one per edge of a round.
+inline int64_t query_items(int64_t m) { return std::min<int64_t>(ITEM_CAP, std::max<int64_t>(m, 256)); }
 
 }  // namespace
 }  // namespace wtri

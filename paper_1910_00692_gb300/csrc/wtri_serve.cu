@@ -37,7 +37,7 @@ namespace {
 
 constexpr int WORKER_STREAMS = 4;
 constexpr int MAX_BATCH = 256;
-constexpr size_t BATCH_FIXED_BYTES = (size_t(1) << 18) * 40 + (1u << 16);  // deferred list + slack
+constexpr size_t BATCH_FIXED_BYTES = (size_t(1) << 18) * 40 + (1u << 16);  // a batch's items + slack
 
 double now_s() {
     return std::chrono::duration<double>(std::chrono::steady_clock::now().time_since_epoch()).count();
@@ -185,7 +185,7 @@ void launch_batch(wtri_server* S, std::vector<std::shared_ptr<Request>>& reqs, i
     int rc = WTRI_OK;
     // the plan's scratch is at most the sum of its requests' estimates
     // (one of them asked for the group's largest k), so admission holds
-    f.plan = batch_plan_create(gs.data(), pc.data(), ks.data(), (int32_t)gs.size());
+    f.plan = batch_plan_create(gs.data(), pc.data(), ks.data(), (int32_t)gs.size(), true);
     if (!f.plan) rc = WTRI_ENOMEM;
     if (rc == WTRI_OK && cudaMallocAsync(&f.dbuf, batch_plan_bytes(f.plan), s) != cudaSuccess) {
         cudaGetLastError();

@@ -7,95 +7,51 @@
 namespace wtri {
 namespace {
 
-// First-wait poll limit of the long-scan kernel's row staging (a test hook
-// lowers it; see wtri_debug_set_wait_limit).
+// Poll limit of a sweep's first grid-barrier wait (a test hook lowers it; see
+// wtri_debug_set_wait_limit).
 std::atomic<uint32_t> g_stage_wait{WAIT_LIMIT};
 uint32_t stage_wait_limit() { return g_stage_wait.load(std::memory_order_relaxed); }
+
+// The fields of a query's sweep that come from its graph and call.
+void set_sweep(Query& q, const wtri_graph* g, int32_t k) {
+    q.k = k;
+    q.total = g->d.m;
+    q.first = g->tune.first_round;
+    q.growth = g->tune.growth;
+    q.t_short = g->tune.t_short;
+    q.fw = g->d.fw;
+    q.wait_first = stage_wait_limit();
+}
 
 template <int P>
 int run_query(const wtri_graph* g, int32_t k, wtri_tri* d_tris, double* d_weight, int32_t* d_count,
               cudaStream_t s, int scale, int shard, int nshards, unsigned long long* d_keys,
               double gp) {
-    const DevGraph& G = g->d;
-    const int64_t m = G.m;
     const uint32_t cap = (uint32_t)std::min<int64_t>(
         (int64_t(1) << 20) * scale + 16 * (int64_t)k, (int64_t(1) << 31) - 1);
-    const uint32_t long_cap = (uint32_t)((1u << 16) * scale);
-    const size_t bytes = sizeof(QState) + 256 + (size_t)cap * (8 + 16) + 256 +
-                         (size_t)long_cap * sizeof(LongItem) + 256;
+    const int64_t item_cap = query_items(g->d.m);
     void* buf = nullptr;
-    cudaError_t e = cudaMallocAsync(&buf, bytes, s);
+    cudaError_t e = cudaMallocAsync(&buf, query_scratch_bytes(cap, item_cap), s);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return set_error(WTRI_ENOMEM, "query scratch allocation failed");
     }
-    char* p = (char*)buf;
     Query q;
-    q.st = (QState*)p;
-    p += 256;
-    q.ckey = (unsigned long long*)p;
-    p += (size_t)cap * 8;
-    q.ctri = (int4*)p;
-    p += (size_t)cap * 16;
-    p = (char*)(((uintptr_t)p + 255) & ~(uintptr_t)255);
-    q.longs = (LongItem*)p;
-    q.cap = cap;
-    q.long_cap = long_cap;
-    q.k = k;
-    q.smark = nullptr;
-    q.slist = nullptr;
-    q.long_count = &q.st->long_count;
-    q.qid = 0;
+    query_carve(q, (char*)buf, cap, item_cap);
+    set_sweep(q, g, k);
     q.shard = shard;
     q.nshards = nshards;
-    q.t_short = g->tune.t_short;
     q.qbytes = query_bytes_on() ? query_bytes_counter() : nullptr;
     q.gp = gp;
-    q.fw = g->d.fw;
-    q.wait_first = stage_wait_limit();
-    WTRI_CUDA(cudaMemsetAsync(q.st, 0, sizeof(QState), s));
-
-    const size_t lsmem = LONG_SMEM;
-    WTRI_TRY((long_optin<P, false>()));
-    const int long_grid = sm_count() * 2;
-    ProfScope whole(query_name(P), s, 0.0, 0);
-    // p = -inf on one shard: NodeIterator++ rounds (no deferred scans)
-    const bool oriented = P == P_MIN && nshards == 1;
-    int64_t lo = 0, size = g->tune.first_round;
-    while (lo < m) {
-        const int64_t hi = std::min(m, lo + size);
-        if (oriented) {
-            ProfScope ps("topk_round_min", s, 0.0, 1);
-            k_round_min<<<round_grid_warps(hi - lo), RBLK, 0, s>>>(G, q, lo, hi);
-        } else {
-            {
-                ProfScope ps("topk_round", s, 0.0, 1);
-                if (hi - lo <= WARP_ROUND_MAX)  // small early rounds: a warp per edge
-                    k_round_warp<P><<<round_grid_warps(hi - lo), RBLK, 0, s>>>(G, q, lo, hi);
-                else
-                    k_round<P><<<round_grid(hi - lo), RBLK, 0, s>>>(G, q, lo, hi);
-            }
-            {
-                ProfScope ps("topk_long", s, 0.0, 1);
-                k_long<P><<<long_grid, LBLK, lsmem, s>>>(G, q);
-            }
-        }
-        {
-            ProfScope ps("topk_select", s, 0.0, 1);
-            k_select<<<1, SBLK, 0, s>>>(q);
-        }
-        lo = hi;
-        size *= g->tune.growth;
+    int rc = WTRI_OK;
+    e = cudaMemsetAsync(q.st, 0, sizeof(QState), s);
+    if (e != cudaSuccess) rc = cuda_error(e, "query state", __FILE__, __LINE__);
+    if (rc == WTRI_OK) {
+        ProfScope whole(query_name(P), s, 0.0, 1);
+        rc = launch_sweep<P, false>(g->d, q, Out{d_tris, d_weight, d_count, d_keys}, s);
     }
-    {
-        ProfScope ps("topk_final", s, 0.0, 2);
-        k_final_select<<<1, SBLK, 0, s>>>(q);
-        k_rank_scatter<P><<<ceil_div_u(std::max(k, 1), 8), 256, 0, s>>>(q, d_tris, d_weight, d_count,
-                                                                        d_keys);
-    }
-    WTRI_CUDA(cudaGetLastError());
-    WTRI_CUDA(cudaFreeAsync(buf, s));
-    return WTRI_OK;
+    cudaFreeAsync(buf, s);
+    return rc;
 }
 
 // ---------------------------------------------------------------------------
@@ -294,26 +250,17 @@ int run_sample(const wtri_graph* g, int32_t k, int64_t nsamples, uint64_t seed, 
     const int64_t m = G.m, words = (m + 31) / 32;
     const uint32_t cap = (uint32_t)std::min<int64_t>(
         (int64_t(1) << 20) * scale + 16 * (int64_t)k, (int64_t(1) << 31) - 1);
-    const uint32_t long_cap = (uint32_t)((1u << 16) * scale);
-    const size_t qbytes = 256 + (size_t)cap * 24 + 256 + (size_t)long_cap * sizeof(LongItem) + 256;
+    const int64_t item_cap = query_items(m);
+    const size_t qbytes = query_scratch_bytes(cap, item_cap);
     const size_t sbytes = 4 * (size_t)words + 8 * (size_t)(words + 1) + 4 * (size_t)words + 4 * (size_t)m + 256;
     void* buf = nullptr;
     if (cudaMallocAsync(&buf, qbytes + sbytes, s) != cudaSuccess) {
         cudaGetLastError();
         return set_error(WTRI_ENOMEM, "sampling query scratch allocation failed");
     }
-    char* p = (char*)buf;
     Query q;
-    q.st = (QState*)p;
-    p += 256;
-    q.ckey = (unsigned long long*)p;
-    p += (size_t)cap * 8;
-    q.ctri = (int4*)p;
-    p += (size_t)cap * 16;
-    p = (char*)(((uintptr_t)p + 255) & ~(uintptr_t)255);
-    q.longs = (LongItem*)p;
-    p += (size_t)long_cap * sizeof(LongItem);
-    p = (char*)(((uintptr_t)p + 255) & ~(uintptr_t)255);
+    char* p = query_carve(q, (char*)buf, cap, item_cap);
+    set_sweep(q, g, k);
     uint32_t* mark = (uint32_t*)p;
     p += 4 * (size_t)words;
     p = (char*)(((uintptr_t)p + 7) & ~(uintptr_t)7);
@@ -322,62 +269,26 @@ int run_sample(const wtri_graph* g, int32_t k, int64_t nsamples, uint64_t seed, 
     int32_t* pc = (int32_t*)p;
     p += 4 * (size_t)words;
     int32_t* list = (int32_t*)p;
-    q.cap = cap;
-    q.long_cap = long_cap;
-    q.k = k;
     q.smark = mark;
     q.slist = list;
-    q.long_count = &q.st->long_count;
-    q.qid = 0;
-    q.shard = 0;
-    q.nshards = 1;
-    q.t_short = g->tune.t_short;
-    q.qbytes = nullptr;
-    q.gp = 0.0;
-    q.fw = 0;
-    q.wait_first = stage_wait_limit();
-    WTRI_CUDA(cudaMemsetAsync(q.st, 0, sizeof(QState), s));
-    ProfScope whole(P == P_ONE ? "sample_p=1" : (P == P_TWO ? "sample_p=2" : "sample_p=0"), s, 0.0, 0);
-    WTRI_TRY(draw_samples<P>(g, nsamples, seed, mark, s));
-    {
-        ProfScope ps("sample_compact", s, 8.0 * words, 2);
-        k_mark_popc<<<grid_of(words), 256, 0, s>>>(words, mark, pc);
-        WTRI_TRY(exclusive_scan_i32_to_i64(pc, off, words, s));
-        k_mark_list<<<grid_of(words), 256, 0, s>>>(words, mark, off, list);
-    }
-    int64_t nlist = 0;
-    WTRI_CUDA(cudaMemcpyAsync(&nlist, off + words, 8, cudaMemcpyDeviceToHost, s));
-    WTRI_CUDA(cudaStreamSynchronize(s));
-    const size_t lsmem = LONG_SMEM;
-    WTRI_TRY((long_optin<P, true>()));
-    const int long_grid = sm_count() * 2;
-    int64_t lo = 0, size = g->tune.first_round;
-    while (lo < nlist) {
-        const int64_t hi = std::min(nlist, lo + size);
+    q.total_dev = off + words;  // the number of drawn edges stays on the device
+    auto run = [&]() -> int {
+        WTRI_CUDA(cudaMemsetAsync(q.st, 0, sizeof(QState), s));
+        ProfScope whole(P == P_ONE ? "sample_p=1" : (P == P_TWO ? "sample_p=2" : "sample_p=0"), s, 0.0, 0);
+        WTRI_TRY(draw_samples<P>(g, nsamples, seed, mark, s));
         {
-            ProfScope ps("sample_round", s, 0.0, 1);
-            k_round<P, true><<<round_grid(hi - lo), RBLK, 0, s>>>(G, q, lo, hi);
+            ProfScope ps("sample_compact", s, 8.0 * words, 2);
+            k_mark_popc<<<grid_of(words), 256, 0, s>>>(words, mark, pc);
+            WTRI_TRY(exclusive_scan_i32_to_i64(pc, off, words, s));
+            k_mark_list<<<grid_of(words), 256, 0, s>>>(words, mark, off, list);
+            WTRI_CUDA(cudaGetLastError());
         }
-        {
-            ProfScope ps("sample_long", s, 0.0, 1);
-            k_long<P, true><<<long_grid, LBLK, lsmem, s>>>(G, q);
-        }
-        {
-            ProfScope ps("topk_select", s, 0.0, 1);
-            k_select<<<1, SBLK, 0, s>>>(q);
-        }
-        lo = hi;
-        size *= g->tune.growth;
-    }
-    {
-        ProfScope ps("topk_final", s, 0.0, 2);
-        k_final_select<<<1, SBLK, 0, s>>>(q);
-        k_rank_scatter<P><<<ceil_div_u(std::max(k, 1), 8), 256, 0, s>>>(q, d_tris, d_weight, d_count,
-                                                                    nullptr);
-    }
-    WTRI_CUDA(cudaGetLastError());
-    WTRI_CUDA(cudaFreeAsync(buf, s));
-    return WTRI_OK;
+        ProfScope ps("sample_sweep", s, 0.0, 1);
+        return launch_sweep<P, true>(G, q, Out{d_tris, d_weight, d_count, nullptr}, s);
+    };
+    const int rc = run();
+    cudaFreeAsync(buf, s);
+    return rc;
 }
 
 }  // namespace
@@ -410,7 +321,7 @@ int topk_device(const wtri_graph* g, int pcode, int32_t k, wtri_tri* d_tris, dou
 // for example a server whose device memory is all handed to its own caching
 // allocator at start-up, or a latency-critical loop that must never wait on
 // the allocator.  The query's scratch (status word, candidate buffer,
-// deferred-scan list) lives in one fixed array compiled into the library.
+// items) lives in one fixed array compiled into the library.
 // Every GPU that loads the library keeps this array (NOALLOC_BYTES, about
 // 26 MB) until the process exits.  All calls share it: the status word is
 // cleared at the start of each call, and calls that overlap on the GPU (on
@@ -420,14 +331,13 @@ namespace wtri {
 namespace {
 
 constexpr uint32_t NOALLOC_CAP = 1u << 20;     // candidates
-constexpr uint32_t NOALLOC_LONG = 1u << 16;    // deferred scans
+constexpr int64_t NOALLOC_ITEMS = 46592;       // edges of a round (an item each)
 constexpr int32_t NOALLOC_K_MAX = 16384;
-constexpr size_t NOALLOC_CAND_OFF = 256;
-constexpr size_t NOALLOC_TRI_OFF = NOALLOC_CAND_OFF + (size_t)NOALLOC_CAP * 8;
-constexpr size_t NOALLOC_LONG_OFF = NOALLOC_TRI_OFF + (size_t)NOALLOC_CAP * 16;
-constexpr size_t NOALLOC_BYTES = NOALLOC_LONG_OFF + (size_t)NOALLOC_LONG * sizeof(LongItem);
-static_assert(sizeof(QState) <= NOALLOC_CAND_OFF, "status word fits its slot");
-static_assert(NOALLOC_LONG_OFF % 256 == 0, "aligned deferred list");
+// state, keys, triples, items and the wedges before each item, as query_carve lays them out
+constexpr size_t NOALLOC_BYTES =
+    256 + (size_t)NOALLOC_CAP * 24 + (size_t)NOALLOC_ITEMS * (sizeof(Item) + sizeof(unsigned long long));
+static_assert(sizeof(QState) <= 256, "the state fits its slot");
+static_assert(NOALLOC_ITEMS % 32 == 0, "every piece is a multiple of 256 bytes");
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_BYTES];
 
@@ -460,61 +370,17 @@ int noalloc_scratch(void** out) {
 template <int P>
 int run_query_noalloc(const wtri_graph* g, int32_t k, wtri_tri* d_tris, double* d_weight,
                       int32_t* d_count, cudaStream_t s, double gp) {
-    const DevGraph& G = g->d;
-    const int64_t m = G.m;
     void* base = nullptr;
     WTRI_TRY(noalloc_scratch(&base));
-    char* p = (char*)base;
     Query q;
-    q.st = (QState*)p;
-    q.ckey = (unsigned long long*)(p + NOALLOC_CAND_OFF);
-    q.ctri = (int4*)(p + NOALLOC_TRI_OFF);
-    q.longs = (LongItem*)(p + NOALLOC_LONG_OFF);
-    q.cap = NOALLOC_CAP;
-    q.long_cap = NOALLOC_LONG;
-    q.k = k;
-    q.smark = nullptr;
-    q.slist = nullptr;
-    q.long_count = &q.st->long_count;
-    q.qid = 0;
-    q.shard = 0;
-    q.nshards = 1;
-    q.t_short = g->tune.t_short;
-    q.qbytes = nullptr;
+    query_carve(q, (char*)base, NOALLOC_CAP, NOALLOC_ITEMS);
+    set_sweep(q, g, k);
     q.gp = gp;
-    q.fw = g->d.fw;
-    q.wait_first = stage_wait_limit();
-    // The array keeps the previous call's contents: reset the status word
-    // (counters, threshold, stop flag, error bits).
+    // The array keeps the previous call's contents: reset the state
+    // (counters, threshold, barrier, error bits).
     WTRI_CUDA(cudaMemsetAsync(q.st, 0, sizeof(QState), s));
-
-    const size_t lsmem = LONG_SMEM;
-    WTRI_TRY((long_optin<P, false>()));
-    const int long_grid = sm_count() * 2;
-    int64_t lo = 0, size = g->tune.first_round;
-    while (lo < m) {
-        const int64_t hi = std::min(m, lo + size);
-        if (P == P_MIN) {  // NodeIterator++ rounds, as in run_query
-            k_round_min<<<round_grid_warps(hi - lo), RBLK, 0, s>>>(G, q, lo, hi);
-            count_launches(1);
-        } else {
-            if (hi - lo <= WARP_ROUND_MAX)
-                k_round_warp<P><<<round_grid_warps(hi - lo), RBLK, 0, s>>>(G, q, lo, hi);
-            else
-                k_round<P><<<round_grid(hi - lo), RBLK, 0, s>>>(G, q, lo, hi);
-            k_long<P><<<long_grid, LBLK, lsmem, s>>>(G, q);
-            count_launches(2);
-        }
-        k_select<<<1, SBLK, 0, s>>>(q);
-        count_launches(1);
-        lo = hi;
-        size *= g->tune.growth;
-    }
-    k_final_select<<<1, SBLK, 0, s>>>(q);
-    k_rank_scatter<P><<<ceil_div_u(std::max(k, 1), 8), 256, 0, s>>>(q, d_tris, d_weight, d_count,
-                                                                    nullptr);
-    count_launches(2);
-    WTRI_CUDA(cudaGetLastError());
+    WTRI_TRY((launch_sweep<P, false>(g->d, q, Out{d_tris, d_weight, d_count, nullptr}, s)));
+    count_launches(1);
     return WTRI_OK;
 }
 

@@ -402,7 +402,7 @@ int run_wedge_topk(const wtri_graph* g, int32_t k, int64_t nsamples, uint64_t se
     while (tcap < 2 * (uint64_t)nsamples) tcap <<= 1;
     const uint32_t cap = (uint32_t)std::min<int64_t>(std::max<int64_t>(nsamples, k), (int64_t(1) << 31) - 1);
     const size_t wsb = ws_bytes(g) + 512;
-    const size_t qb = 256 + (size_t)cap * 24 + 512 + 16 * sizeof(LongItem);
+    const size_t qb = query_scratch_bytes(cap, 0);
     const size_t hb = 8 * (size_t)tcap;
     void* buf = nullptr;
     if (cudaMallocAsync(&buf, wsb + qb + hb, s) != cudaSuccess) {
@@ -413,31 +413,8 @@ int run_wedge_topk(const wtri_graph* g, int32_t k, int64_t nsamples, uint64_t se
     WsScratch W = ws_carve(g, p);
     p += wsb;
     Query q;
-    q.st = (QState*)p;
-    p += 256;
-    q.ckey = (unsigned long long*)p;
-    p += (size_t)cap * 8;
-    p = (char*)(((uintptr_t)p + 15) & ~(uintptr_t)15);  // 16-byte triples: cap may be odd
-    q.ctri = (int4*)p;
-    p += (size_t)cap * 16;
-    p = (char*)(((uintptr_t)p + 255) & ~(uintptr_t)255);
-    q.longs = (LongItem*)p;
-    p += 16 * sizeof(LongItem);
-    unsigned long long* table = (unsigned long long*)p;
-    q.cap = cap;
-    q.long_cap = 16;
+    unsigned long long* table = (unsigned long long*)query_carve(q, p, cap, 0);
     q.k = k;
-    q.smark = nullptr;
-    q.slist = nullptr;
-    q.long_count = &q.st->long_count;
-    q.qid = 0;
-    q.shard = 0;
-    q.nshards = 1;
-    q.t_short = g->tune.t_short;
-    q.qbytes = nullptr;
-    q.gp = 0.0;
-    q.fw = 0;
-    q.wait_first = WAIT_LIMIT;
     WTRI_CUDA(cudaMemsetAsync(q.st, 0, sizeof(QState), s));
     WTRI_CUDA(cudaMemsetAsync(W.err, 0, 4, s));
     WTRI_CUDA(cudaMemsetAsync(table, 0xff, hb, s));
@@ -455,11 +432,12 @@ int run_wedge_topk(const wtri_graph* g, int32_t k, int64_t nsamples, uint64_t se
                                                        tcap - 1);
     }
     {
-        ProfScope ps("topk_final", s, 0.0, 3);
-        k_select<<<1, SBLK, 0, s>>>(q);
-        k_final_select<<<1, SBLK, 0, s>>>(q);
-        k_rank_scatter<P><<<ceil_div_u(std::max(k, 1), 8), 256, 0, s>>>(q, d_tris, d_weight, d_count,
-                                                                        nullptr);
+        ProfScope ps("topk_final", s, 0.0, 1);
+        const int rc = launch_finish<P>(G, q, Out{d_tris, d_weight, d_count, nullptr}, s);
+        if (rc != WTRI_OK) {
+            cudaFreeAsync(buf, s);
+            return rc;
+        }
     }
     WTRI_CUDA(cudaGetLastError());
     // a row sum above 64 bits: report it through the status word

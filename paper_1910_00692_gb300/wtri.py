@@ -466,7 +466,7 @@ def sample_edges(g: Graph, p: float, nsamples: int, seed: int) -> np.ndarray:
 
 def debug_set_wait_limit(polls: int):
     """wtri_debug_set_wait_limit: fault injection for tests (polls of the
-    long-scan kernel's first bounded wait; 0: every staged wait times out;
+    query kernel's first grid-barrier wait; 0: it times out at once;
     negative: the default)."""
     _check(lib().wtri_debug_set_wait_limit(int(polls)))
 
