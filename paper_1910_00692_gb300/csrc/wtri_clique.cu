@@ -8,17 +8,25 @@
 // edge (Section 4.5); with every edge taken instead of draws the answer is
 // the exact top-k.
 //
-// Per drawn edge {u, v} (one block): the common neighbours c of u and v,
-// with the weights and edge ranks of {u, c} and {v, c}, go to shared memory
-// (the shorter weight-sorted row is scanned, the other endpoint looked up
-// in the oriented rows).  q = 4: each pair of common neighbours joined by an
-// edge closes a 4-clique.  q = 5: the adjacency among the common neighbours
-// becomes a bit matrix in shared memory; an adjacent pair (i, j) and each
-// l above j adjacent to both close a 5-clique.  A clique is reported by its
-// first drawn edge in the edge order (no other of its edges is drawn and
-// earlier), so the candidates hold each clique once.  One block then keeps
-// exactly the k best under (key desc, sorted vertex tuple asc) by an
-// MSB-first radix select over the tuple, and a rank pass orders them.
+// A clique is reported by its first drawn edge in the edge order.  Per drawn
+// edge r = {u, v} (one block), the common neighbours c of u and v (the shorter
+// weight-sorted row is scanned, the other endpoint looked up in the oriented
+// rows) are kept unless {u, c} or {v, c} is drawn and earlier than r: a clique
+// through such a c belongs to that edge.  Likewise for the edges among them,
+// so every clique formed from what is left is reported, once, unchecked.  The
+// edges among the kept neighbours come from their oriented rows, scanned once
+// against a hash table of the kept ids in shared memory (a search per pair
+// took eight dependent loads each, twice, and cost 18.3 ms for the 10,000
+// draws of the 979-vertex graph at q = 5; now 0.22 ms for the
+// whole enumeration).  q = 4: each such edge closes a
+// clique.  q = 5: the edges go to a bit matrix and a list; for each edge
+// (i, j) of the list, each l above j adjacent to both closes a clique.  Edges
+// that keep more than 128 neighbours go to a second kernel with larger tables,
+// those that keep more than 256 to a third that looks pairs up one by one.  The whole GPU then selects the candidates that reach the
+// k-th key (a histogram per digit of the key, one grid barrier each), one
+// block keeps exactly the k best of those under (key desc, sorted vertex
+// tuple asc) by an MSB-first radix select over the tuple, and a rank pass
+// orders them.
 #include "wtri_query.cuh"
 
 #include <algorithm>
@@ -33,6 +41,7 @@ constexpr int QMAX = 5;
 constexpr int CSB = 1024;            // threads of the select block
 constexpr uint32_t CERR_CAND = 1u;   // the candidate buffer filled up
 constexpr uint32_t CERR_NBR = 2u;    // a common neighbourhood above CNB
+constexpr uint32_t CERR_WAIT = 4u;   // a bounded wait of the selection ran out
 constexpr uint32_t CLIQUE_CAP = 1u << 23;
 
 struct CliqueRun {
@@ -44,7 +53,9 @@ struct CliqueRun {
     uint32_t* count;
     uint32_t cap;
     uint32_t* err;
-    int32_t* cursor;       // next bitmap word
+    int32_t* cursor;       // next group of bitmap bits
+    int32_t* list[2];      // edges left to k_cliques_mid, to k_cliques_big
+    uint32_t* nlist;       // their numbers
 };
 
 // Shared memory of a clique block; the q = 5 bit matrix (CNB rows of CNW
@@ -52,7 +63,7 @@ struct CliqueRun {
 struct CliqueSmem {
     int32_t cid[CNB], cdg[CNB], cwu[CNB], cwv[CNB], cru[CNB], crv[CNB];
     int32_t n;
-    int32_t word;
+    int32_t item;
 };
 
 __device__ __forceinline__ bool drawn(const uint32_t* mark, int32_t r) {
@@ -181,24 +192,238 @@ __device__ void clique_edge(const DevGraph& G, const CliqueRun& C, CliqueSmem& S
     __syncthreads();  // the shared lists are reused by the next edge
 }
 
-// Blocks take words of the drawn-edge bitmap and handle their edges in turn.
-__global__ void __launch_bounds__(CB) k_cliques(DevGraph G, CliqueRun C) {
+// The edges that keep more common neighbours than the tables of k_cliques_mid.
+__global__ void __launch_bounds__(CB) k_cliques_big(DevGraph G, CliqueRun C) {
     extern __shared__ __align__(16) unsigned char csm[];
     CliqueSmem& S = *reinterpret_cast<CliqueSmem*>(csm);
     uint32_t* bits = reinterpret_cast<uint32_t*>(csm + sizeof(CliqueSmem));
     Tally tb;
-    for (;;) {
-        if (threadIdx.x == 0) S.word = atomicAdd(C.cursor, 1);
-        __syncthreads();
-        const int32_t wi = S.word;
-        __syncthreads();
-        if (wi >= C.words) break;
-        uint32_t mw = __ldg(C.mark + wi);
-        while (mw) {
-            const int32_t r = wi * 32 + __ffs(mw) - 1;
-            mw &= mw - 1;
-            clique_edge(G, C, S, bits, r, tb);
+    const uint32_t n = C.nlist[1];
+    for (uint32_t i = blockIdx.x; i < n; i += gridDim.x) clique_edge(G, C, S, bits, C.list[1][i], tb);
+}
+
+// ---- edges with at most FNB kept neighbours --------------------------------
+// Two sizes: FNB = 128 (58 KB of shared memory: three 256-thread blocks per
+// SM), and FNB = 256 (208 KB: one 1,024-thread block) for the few edges that
+// keep more.
+constexpr int FGROUP = 4;          // bitmap bits taken at a time
+
+template <int FNB>
+struct FastSmem {
+    static constexpr int HASH = 4 * FNB;    // slots of the id table (at most a quarter used)
+    uint32_t wm[FNB * (FNB - 1) / 2];       // q = 5: weight of the edge (i, j), i < j, at j (j - 1) / 2 + i;
+                                            // q = 4: weight of each edge of the list
+    uint16_t pair[FNB * (FNB - 1) / 2];     // the edges, i << 8 | j
+    uint32_t bits[FNB][FNB / 32];           // row i: adjacent j > i
+    int32_t hid[HASH];                      // ids (-1: free) and their places
+    uint8_t hix[HASH];
+    int32_t cid[FNB], cwu[FNB], cwv[FNB];
+    uint32_t wsum[32];
+    uint32_t base;
+    int32_t all, n, np, item;
+};
+
+// The key with another edge: acc with w added (minimum, sum, squares, maximum).
+template <int PC>
+__device__ __forceinline__ unsigned long long more(unsigned long long acc, uint32_t w) {
+    const unsigned long long x = w;
+    if (PC == P_MIN) return x < acc ? x : acc;
+    if (PC == P_ONE) return acc + x;
+    if (PC == P_TWO) return acc + x * x;
+    return x > acc ? x : acc;
+}
+
+// Candidate idx of a clique that is known to belong to the edge at hand.
+__device__ __forceinline__ void put(const CliqueRun& C, uint32_t idx, int32_t a, int32_t b, int32_t c, int32_t d,
+                                    int32_t e, int q, unsigned long long key) {
+    if (idx >= C.cap) {
+        atomicOr(C.err, CERR_CAND);
+        return;
+    }
+    auto sw = [](int32_t& x, int32_t& y) {
+        const int32_t lo = min(x, y), hi = max(x, y);
+        x = lo;
+        y = hi;
+    };
+    if (q == 5) {  // sorting networks
+        sw(a, d), sw(b, e), sw(a, c), sw(b, d), sw(a, b), sw(c, e), sw(b, c), sw(d, e), sw(c, d);
+    } else {
+        sw(a, c), sw(b, d), sw(a, b), sw(c, d), sw(b, c);
+    }
+    C.ckey[idx] = key;
+    int32_t* o = C.cids + (size_t)idx * QMAX;
+    o[0] = a;
+    o[1] = b;
+    o[2] = c;
+    o[3] = d;
+    o[4] = q == 5 ? e : 0;
+}
+
+template <int Q, int PC, int FNB, int NTH>
+__device__ __forceinline__ void fast_edge(const DevGraph& G, const CliqueRun& C, FastSmem<FNB>& S, int32_t r,
+                                          int32_t* left, uint32_t* nleft) {
+    constexpr int HASH = FastSmem<FNB>::HASH, HSHIFT = FNB == 128 ? 23 : 22, FNW = FNB / 32;
+    static_assert(HASH == 1 << (32 - HSHIFT), "the hash fills the table");
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    Tally tb;
+    const int32_t u = __ldg(G.ord_u + r), v = __ldg(G.ord_v + r);
+    const uint32_t wuv = (uint32_t)__ldg(G.ord_w + r);
+    const int64_t bu = __ldg(G.rowptr + u), eu = __ldg(G.rowptr + u + 1);
+    const int64_t bv = __ldg(G.rowptr + v), ev = __ldg(G.rowptr + v + 1);
+    const bool xu = (eu - bu) <= (ev - bv);  // scan the shorter row
+    const int32_t y = xu ? v : u;
+    const int64_t bx = xu ? bu : bv, ex = xu ? eu : ev;
+    const int64_t dy = xu ? ev - bv : eu - bu;
+    if (threadIdx.x == 0) S.all = S.n = S.np = 0;
+    for (int t = threadIdx.x; t < HASH; t += NTH) S.hid[t] = -1;
+    if (Q == 5)
+        for (int t = threadIdx.x; t < FNB * FNW; t += NTH) (&S.bits[0][0])[t] = 0u;
+    __syncthreads();
+    for (int64_t j = bx + threadIdx.x; j < ex; j += NTH) {
+        const int32_t c = __ldg(G.wcol + j);
+        if (c == y) continue;
+        int32_t wyc, ryc;
+        if (!probe_oriented(G, y, dy, c, wyc, ryc, tb)) continue;
+        atomicAdd(&S.all, 1);
+        const int32_t rxc = __ldg(G.wrk + j);
+        if ((rxc < r && drawn(C.mark, rxc)) || (ryc < r && drawn(C.mark, ryc))) continue;
+        const int i = atomicAdd(&S.n, 1);
+        if (i >= FNB) continue;
+        const int32_t wxc = __ldg(G.wwt + j);
+        S.cid[i] = c;
+        S.cwu[i] = xu ? wxc : wyc;
+        S.cwv[i] = xu ? wyc : wxc;
+        uint32_t h = ((uint32_t)c * 2654435761u) >> HSHIFT;
+        while (atomicCAS(&S.hid[h], -1, c) != -1) h = (h + 1) & (HASH - 1);  // ids are distinct
+        S.hix[h] = (uint8_t)i;
+    }
+    __syncthreads();
+    const int nc = S.n;
+    if (S.all > CNB) {  // recorded as an error; the call fails
+        if (threadIdx.x == 0) atomicOr(C.err, CERR_NBR);
+        return;
+    }
+    if (nc > FNB) {
+        if (threadIdx.x == 0) left[atomicAdd(nleft, 1u)] = r;
+        return;
+    }
+    if (nc < Q - 2) return;
+    auto edge = [&](int i, int j, int64_t at) {  // an edge among the kept neighbours, entry `at`
+        const int32_t rij = __ldg(G.ork + at);
+        if (rij < r && drawn(C.mark, rij)) return;
+        const uint32_t wij = (uint32_t)__ldg(G.owt + at);
+        const int a = min(i, j), b = max(i, j), t = atomicAdd(&S.np, 1);
+        S.pair[t] = (uint16_t)(a << 8 | b);
+        if constexpr (Q == 4) {
+            S.wm[t] = wij;
+        } else {
+            S.wm[b * (b - 1) / 2 + a] = wij;
+            atomicOr(&S.bits[a][b >> 5], 1u << (b & 31));
         }
+    };
+    for (int i = wid; i < nc; i += NTH / 32) {  // a warp per kept neighbour
+        const int32_t c = S.cid[i];
+        const int64_t ob = __ldg(G.orowptr + c), oe = __ldg(G.orowptr + c + 1);
+        if (oe - ob <= 64 + 8 * (int64_t)nc) {  // its row against the table
+            for (int64_t at = ob + lane; at < oe; at += 32) {
+                const int32_t x = __ldg(G.ocol + at);
+                uint32_t h = ((uint32_t)x * 2654435761u) >> HSHIFT;
+                int32_t id = S.hid[h];
+                while (id != -1 && id != x) id = S.hid[h = (h + 1) & (HASH - 1)];
+                if (id == x) edge(i, S.hix[h], at);
+            }
+        } else {  // a long row: each kept neighbour searched in it
+            for (int j = lane; j < nc; j += 32) {
+                const int64_t at = search_ids(G.ocol, ob, (int32_t)(oe - ob), S.cid[j], tb);
+                if (at < oe && __ldg(G.ocol + at) == S.cid[j]) edge(i, j, at);
+            }
+        }
+    }
+    __syncthreads();
+    // every thread counts its cliques, the block takes their places at once
+    // (an atomic round trip per clique made the heaviest edge the tail)
+    const int np = S.np;
+    auto common = [&](int i, int j, int wd) { return S.bits[i][wd] & S.bits[j][wd]; };  // (row j holds l > j only)
+    uint32_t mine = 0;
+    for (int t = threadIdx.x; t < np; t += NTH) {
+        if (Q == 4) {
+            mine++;
+        } else {
+            const int i = S.pair[t] >> 8, j = S.pair[t] & 255;
+            for (int wd = j >> 5; wd < FNW; wd++) mine += __popc(common(i, j, wd));
+        }
+    }
+    uint32_t inc = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t x = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += x;
+    }
+    if (lane == 31) S.wsum[wid] = inc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t acc = 0;
+        for (int k = 0; k < NTH / 32; k++) {
+            const uint32_t c = S.wsum[k];
+            S.wsum[k] = acc;
+            acc += c;
+        }
+        if (acc) S.base = atomicAdd(C.count, acc);
+    }
+    __syncthreads();
+    uint32_t idx = S.base + S.wsum[wid] + inc - mine;
+    const unsigned long long k0 = more<PC>(PC == P_MIN ? ~0ull : 0ull, wuv);
+    for (int t = threadIdx.x; t < np; t += NTH) {
+        const int i = S.pair[t] >> 8, j = S.pair[t] & 255;
+        unsigned long long kij = more<PC>(more<PC>(k0, S.cwu[i]), S.cwv[i]);
+        kij = more<PC>(more<PC>(kij, S.cwu[j]), S.cwv[j]);
+        if constexpr (Q == 4) {
+            put(C, idx++, u, v, S.cid[i], S.cid[j], 0, 4, more<PC>(kij, S.wm[t]));
+        } else {
+            kij = more<PC>(kij, S.wm[j * (j - 1) / 2 + i]);
+            for (int wd = j >> 5; wd < FNW; wd++) {
+                uint32_t both = common(i, j, wd);
+                while (both) {
+                    const int l = wd * 32 + __ffs(both) - 1;
+                    both &= both - 1;
+                    unsigned long long k = more<PC>(more<PC>(kij, S.cwu[l]), S.cwv[l]);
+                    k = more<PC>(more<PC>(k, S.wm[l * (l - 1) / 2 + i]), S.wm[l * (l - 1) / 2 + j]);
+                    put(C, idx++, u, v, S.cid[i], S.cid[j], S.cid[l], 5, k);
+                }
+            }
+        }
+    }
+}
+
+// The drawn edges, a few bitmap bits at a time.
+template <int Q, int PC>
+__global__ void __launch_bounds__(CB, 3) k_cliques(DevGraph G, CliqueRun C) {
+    extern __shared__ __align__(16) unsigned char csm[];
+    FastSmem<128>& S = *reinterpret_cast<FastSmem<128>*>(csm);
+    const int64_t m = G.m;
+    for (;;) {
+        if (threadIdx.x == 0) S.item = atomicAdd(C.cursor, 1);
+        __syncthreads();
+        const int64_t r0 = (int64_t)S.item * FGROUP;
+        __syncthreads();
+        if (r0 >= m) break;
+        for (int64_t r = r0; r < min(m, r0 + FGROUP); r++) {
+            if (!drawn(C.mark, (int32_t)r)) continue;
+            fast_edge<Q, PC, 128, CB>(G, C, S, (int32_t)r, C.list[0], C.nlist);
+            __syncthreads();  // the shared lists are reused by the next edge
+        }
+    }
+}
+
+// The edges that keep more than 128.
+template <int Q, int PC>
+__global__ void __launch_bounds__(1024, 1) k_cliques_mid(DevGraph G, CliqueRun C) {
+    extern __shared__ __align__(16) unsigned char csm[];
+    FastSmem<256>& S = *reinterpret_cast<FastSmem<256>*>(csm);
+    const uint32_t n = C.nlist[0];
+    for (uint32_t i = blockIdx.x; i < n; i += gridDim.x) {
+        fast_edge<Q, PC, 256, 1024>(G, C, S, C.list[0][i], C.list[1], C.nlist + 1);
+        __syncthreads();
     }
 }
 
@@ -213,6 +438,102 @@ __global__ void k_mark_all(int64_t m, uint32_t* mark) {
 }
 
 // ---- selection of the k best candidates ------------------------------------
+// The candidates whose key reaches the K-th largest (ties included), by the
+// whole GPU: their indices to ix, their number to *nix.  hist: SEL_BINS
+// counters per digit, and lim[2] (largest key, complement of the smallest),
+// all zero at the start.
+struct CliqueSelect {
+    Query q;  // barrier state
+    const unsigned long long* ckey;
+    const uint32_t* count;
+    uint32_t cap, K;
+    uint32_t* err;
+    uint32_t* hist;
+    unsigned long long* lim;
+    uint32_t* ix;
+    uint32_t* nix;
+};
+
+__global__ void __launch_bounds__(TGRID, 1) k_clique_reach(CliqueSelect A) {
+    __shared__ SelectSmem S;
+    if (*(volatile const uint32_t*)A.err) return;  // set before this launch: every block sees the same
+    const uint32_t n = min(*(volatile const uint32_t*)A.count, A.cap);
+    const int tid = threadIdx.x, lane = tid & 31;
+    GridTeam<TGRID> T;
+    T.limit = A.q.wait_first;
+    T.blk0 = 0;
+    T.nblk = gridDim.x;
+    T.gone = &S.gone;
+    if (tid == 0) S.gone = 0;
+    __syncthreads();
+    const uint32_t step = (uint32_t)T.threads();
+    auto wait = [&]() {
+        if (T.sync(A.q)) return true;
+        if (tid == 0) atomicOr(A.err, CERR_WAIT);
+        return false;
+    };
+    unsigned long long reach = 0;  // n <= K: all of them
+    if (n > A.K) {
+        unsigned long long mx = 0, mn = ~0ull;
+        for (uint32_t i = (uint32_t)T.thread(); i < n; i += step) {
+            const unsigned long long x = A.ckey[i];
+            mx = x > mx ? x : mx;
+            mn = x < mn ? x : mn;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long a = __shfl_xor_sync(0xffffffffu, mx, o), b = __shfl_xor_sync(0xffffffffu, mn, o);
+            mx = a > mx ? a : mx;
+            mn = b < mn ? b : mn;
+        }
+        if (lane == 0 && mx) {
+            atomicMax(A.lim, mx);
+            atomicMax(A.lim + 1, ~mn);
+        }
+        if (!wait()) return;
+        mx = ld_volatile_u64(A.lim);
+        mn = ~ld_volatile_u64(A.lim + 1);
+        int shift = mx == mn ? 0 : 64 - __clzll((long long)(mx ^ mn));
+        reach = shift >= 64 ? 0ull : (mx >> shift) << shift;
+        uint32_t need = A.K;
+        for (int dig = 0; shift > 0; dig++) {
+            const int bits = shift < SEL_BITS ? shift : SEL_BITS, hi = shift;
+            shift -= bits;
+            const uint32_t mask = (1u << bits) - 1u;
+            uint32_t* gh = A.hist + dig * SEL_BINS;
+            clear_hist<TGRID>(T.part, S);
+            for (uint32_t base = (uint32_t)(T.thread() - lane); base < n; base += step) {
+                const uint32_t i = base + lane;
+                uint32_t d = SEL_BINS;
+                if (i < n) {
+                    const unsigned long long x = A.ckey[i];
+                    if (hi >= 64 || (x >> hi) == (reach >> hi)) d = mask - ((uint32_t)(x >> shift) & mask);
+                }
+                count_bin(S, d);
+            }
+            __syncthreads();
+            for (int b = tid; b < SEL_BINS; b += TGRID)
+                if (S.hist[b]) atomicAdd(gh + b, S.hist[b]);
+            if (!wait()) return;
+            for (int b = tid; b < SEL_BINS; b += TGRID) S.hist[b] = *(volatile uint32_t*)(gh + b);
+            __syncthreads();
+            pick_bin<TGRID>(T.part, S, need);
+            reach |= (unsigned long long)(mask - S.bin) << shift;
+            need -= S.above;
+            __syncthreads();
+        }
+    }
+    for (uint32_t base = (uint32_t)(T.thread() - lane); base < n; base += step) {
+        const uint32_t i = base + lane;
+        const bool on = i < n && A.ckey[i] >= reach;
+        const uint32_t b = __ballot_sync(0xffffffffu, on);
+        uint32_t at = 0;
+        if (lane == 0 && b) at = atomicAdd(A.nix, (uint32_t)__popc(b));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (on) A.ix[at + __popc(b & lanemask_below())] = i;
+    }
+}
+
 // Tuple of a candidate, smaller is better: (~key_hi, ~key_lo, id_0 .. id_{q-1}).
 __device__ __forceinline__ uint32_t cword(const unsigned long long* ckey, const int32_t* cids, uint32_t i,
                                           int wi) {
@@ -244,14 +565,15 @@ __device__ __forceinline__ int cmp_cprefix(const unsigned long long* ckey, const
     return 0;
 }
 
-// Keeps exactly min(K, n) best candidates at the front (tuples are unique:
-// every clique appears once), n = *count; *kept receives their number.
-__global__ void __launch_bounds__(CSB) k_clique_select(unsigned long long* ckey, int32_t* cids,
-                                                       const uint32_t* count, uint32_t cap, int q, uint32_t K,
+// Keeps the indices of exactly min(K, n) best candidates at the front of ix
+// (tuples are unique: every clique appears once), n = *nix; *kept receives
+// their number.
+__global__ void __launch_bounds__(CSB) k_clique_select(const unsigned long long* ckey, const int32_t* cids,
+                                                       uint32_t* ix, const uint32_t* nix, int q, uint32_t K,
                                                        const uint32_t* err, uint32_t* kept) {
     __shared__ CSelSmem S;
     if (*(volatile const uint32_t*)err) return;
-    const uint32_t n = min(*(volatile const uint32_t*)count, cap);
+    const uint32_t n = *(volatile const uint32_t*)nix;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int nbytes = 4 * (2 + q);
     if (tid < 2 + QMAX) S.pw[tid] = 0;
@@ -266,24 +588,39 @@ __global__ void __launch_bounds__(CSB) k_clique_select(unsigned long long* ckey,
         for (int i = tid; i < 256; i += CSB) S.hist[i] = 0;
         __syncthreads();
         const int wi = depth >> 2, sh = 24 - 8 * (depth & 3);
-        for (uint32_t i = tid; i < n; i += CSB)
+        for (uint32_t t = tid; t < n; t += CSB) {
+            const uint32_t i = ix[t];
             if (cmp_cprefix(ckey, cids, i, S.pw, depth) == 0)
                 atomicAdd(&S.hist[(cword(ckey, cids, i, wi) >> sh) & 255u], 1u);
+        }
         __syncthreads();
-        if (tid == 0) {
+        if (wid == 0) {  // the bin where the running count reaches what is needed: eight bins a lane
             const uint32_t need = K - S.below;
-            uint32_t acc = 0, dsel = 0;
-            for (uint32_t d = 0; d < 256; d++) {
-                if (acc + S.hist[d] >= need) {
-                    dsel = d;
-                    break;
-                }
-                acc += S.hist[d];
+            uint32_t h[8], sum = 0;
+#pragma unroll
+            for (int b = 0; b < 8; b++) sum += h[b] = S.hist[8 * lane + b];
+            uint32_t acc = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, acc, o);
+                if (lane >= o) acc += y;
             }
-            S.below += acc;
-            S.eq = S.hist[dsel];
-            S.pw[wi] |= dsel << sh;
-            if (S.below + S.eq == K) S.done = 1;
+            acc -= sum;
+            __syncwarp();
+            if (acc < need && need <= acc + sum) {
+                bool hit = false;
+#pragma unroll
+                for (int b = 0; b < 8; b++) {
+                    if (!hit && need <= acc + h[b]) {
+                        hit = true;
+                        S.below += acc;
+                        S.eq = h[b];
+                        S.pw[wi] |= (uint32_t)(8 * lane + b) << sh;
+                        if (S.below + S.eq == K) S.done = 1;
+                    }
+                    acc += h[b];
+                }
+            }
         }
         __syncthreads();
         depth++;
@@ -291,14 +628,12 @@ __global__ void __launch_bounds__(CSB) k_clique_select(unsigned long long* ckey,
     const bool keep_all = n <= K;
     uint32_t out = 0;
     for (uint32_t base = 0; base < n; base += CSB) {
-        const uint32_t i = base + tid;
+        const uint32_t t = base + tid;
         bool keep = false;
-        unsigned long long kk = 0;
-        int32_t t[QMAX] = {0, 0, 0, 0, 0};
-        if (i < n) {
+        uint32_t i = 0;
+        if (t < n) {
+            i = ix[t];
             keep = keep_all || cmp_cprefix(ckey, cids, i, S.pw, depth) <= 0;
-            kk = ckey[i];
-            for (int a = 0; a < QMAX; a++) t[a] = cids[(size_t)i * QMAX + a];
         }
         const uint32_t b = __ballot_sync(0xffffffffu, keep);
         if (lane == 0) S.warp_cnt[wid] = __popc(b);
@@ -315,8 +650,7 @@ __global__ void __launch_bounds__(CSB) k_clique_select(unsigned long long* ckey,
         __syncthreads();
         if (keep) {
             const uint32_t p = out + S.warp_cnt[wid] + __popc(b & ((1u << lane) - 1u));
-            ckey[p] = kk;  // p <= i: this chunk was read before the barrier
-            for (int a = 0; a < QMAX; a++) cids[(size_t)p * QMAX + a] = t[a];
+            ix[p] = i;  // p <= t: this chunk was read before the barrier
         }
         out += S.kept;
         __syncthreads();
@@ -337,16 +671,18 @@ __device__ __forceinline__ bool cbefore(const unsigned long long* ckey, const in
 
 // One warp per kept candidate: its rank among the kept ones, then the
 // outputs at that rank (ids, fp64 mean, key).
-__global__ void k_clique_rank(const unsigned long long* ckey, const int32_t* cids, const uint32_t* kept,
+__global__ void k_clique_rank(const unsigned long long* ckey, const int32_t* cids, const uint32_t* ix,
+                              const uint32_t* kept,
                               const uint32_t* err, int q, int pcode, uint32_t kmax, int32_t* ids_out,
                               double* w_out, unsigned long long* key_out) {
     if (*(volatile const uint32_t*)err) return;
     const uint32_t K = *kept;
-    const uint32_t i = (uint32_t)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
+    const uint32_t at = (uint32_t)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
-    if (i >= K) return;
+    if (at >= K) return;
+    const uint32_t i = ix[at];
     uint32_t rank = 0;
-    for (uint32_t j = lane; j < K; j += 32) rank += cbefore(ckey, cids, j, i, q) ? 1u : 0u;
+    for (uint32_t j = lane; j < K; j += 32) rank += cbefore(ckey, cids, ix[j], i, q) ? 1u : 0u;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
     if (lane == 0 && rank < kmax) {
@@ -367,8 +703,13 @@ int clique_topk_host(const wtri_graph* g, int q, int pcode, int32_t k, int64_t n
     const int64_t words = (m + 31) / 32;
     const uint32_t cap = CLIQUE_CAP;
     cudaStream_t s = g->stream;
-    const size_t bytes = 4 * (size_t)words + 256 + (size_t)cap * 8 + (size_t)cap * 4 * QMAX + 256 +
-                         (size_t)k * (4 * q + 16) + 256 + 64;
+    auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    // cleared at the start: counters, key limits, barrier state, histograms
+    // (six digits of a 64-bit key)
+    const size_t small_bytes = 256 + 256 + al(sizeof(QState)) + 6 * SEL_BINS * 4;
+    const int64_t big_cap = nsamples < 0 ? m : std::min(m, nsamples);  // at most the drawn edges
+    const size_t bytes = al(4 * (size_t)words) + al((size_t)cap * 8) + al((size_t)cap * 4 * QMAX) +
+                         al((size_t)k * (4 * q + 16)) + al((size_t)cap * 4) + 2 * al(4 * (size_t)big_cap) + small_bytes;
     void* buf = nullptr;
     if (cudaMallocAsync(&buf, bytes, s) != cudaSuccess) {
         cudaGetLastError();
@@ -376,22 +717,26 @@ int clique_topk_host(const wtri_graph* g, int q, int pcode, int32_t k, int64_t n
     }
     char* p = (char*)buf;
     uint32_t* mark = (uint32_t*)p;
-    p += (4 * (size_t)words + 255) & ~(size_t)255;
+    p += al(4 * (size_t)words);
     unsigned long long* ckey = (unsigned long long*)p;
-    p += (size_t)cap * 8;
+    p += al((size_t)cap * 8);
     int32_t* cids = (int32_t*)p;
-    p += ((size_t)cap * 4 * QMAX + 255) & ~(size_t)255;
+    p += al((size_t)cap * 4 * QMAX);
     unsigned long long* okey = (unsigned long long*)p;
     double* ow = (double*)(okey + k);
     int32_t* oids = (int32_t*)(ow + k);
-    p += ((size_t)k * (4 * q + 16) + 255) & ~(size_t)255;
-    uint32_t* small = (uint32_t*)p;  // count, err, cursor, kept
+    p += al((size_t)k * (4 * q + 16));
+    uint32_t* ix = (uint32_t*)p;
+    p += al((size_t)cap * 4);
+    int32_t* big = (int32_t*)p;
+    p += 2 * al(4 * (size_t)big_cap);
+    uint32_t* small = (uint32_t*)p;  // count, err, cursor, kept, nix, nbig
     auto done = [&](int rc) {
         cudaFreeAsync(buf, s);
         cudaStreamSynchronize(s);
         return rc;
     };
-    if (cudaMemsetAsync(small, 0, 64, s) != cudaSuccess)
+    if (cudaMemsetAsync(small, 0, small_bytes, s) != cudaSuccess)
         return done(cuda_error(cudaGetLastError(), "memset", __FILE__, __LINE__));
     if (nsamples >= 0) {
         int rc = sample_edges_device(g, pcode, nsamples, seed, mark, s);
@@ -411,20 +756,59 @@ int clique_topk_host(const wtri_graph* g, int q, int pcode, int32_t k, int64_t n
     C.cap = cap;
     C.err = small + 1;
     C.cursor = (int32_t*)(small + 2);
-    const int smem = (int)sizeof(CliqueSmem) + (q == 5 ? CNB * CNW * 4 : 0);
-    static std::atomic<uint64_t> optin{0};
+    C.list[0] = big;
+    C.list[1] = (int32_t*)((char*)big + al(4 * (size_t)big_cap));
+    C.nlist = small + 5;
+    const int big_smem = (int)sizeof(CliqueSmem) + (q == 5 ? CNB * CNW * 4 : 0);
     {
-        int rc = smem_optin((const void*)k_cliques, (int)sizeof(CliqueSmem) + CNB * CNW * 4, optin);
+        static std::atomic<uint64_t> optin{0};
+        int rc = smem_optin((const void*)k_cliques_big, (int)sizeof(CliqueSmem) + CNB * CNW * 4, optin);
+        if (rc != WTRI_OK) return done(rc);
+    }
+    auto enumerate = [&](auto kern, auto mid, std::atomic<uint64_t>* optin) -> int {
+        WTRI_TRY(smem_optin((const void*)kern, (int)sizeof(FastSmem<128>), optin[0]));
+        WTRI_TRY(smem_optin((const void*)mid, (int)sizeof(FastSmem<256>), optin[1]));
+        kern<<<sm_count() * 3, CB, sizeof(FastSmem<128>), s>>>(G, C);
+        mid<<<sm_count(), 1024, sizeof(FastSmem<256>), s>>>(G, C);
+        k_cliques_big<<<sm_count() * (q == 5 ? 1 : 4), CB, big_smem, s>>>(G, C);
+        return WTRI_OK;
+    };
+    {
+        ProfScope ps("cliques_enumerate", s, 0.0, 3);
+        static std::atomic<uint64_t> optin[8][2];
+        int rc = WTRI_OK;
+        switch (pcode + (q == 5 ? 4 : 0)) {
+            case P_MIN: rc = enumerate(k_cliques<4, P_MIN>, k_cliques_mid<4, P_MIN>, optin[0]); break;
+            case P_ONE: rc = enumerate(k_cliques<4, P_ONE>, k_cliques_mid<4, P_ONE>, optin[1]); break;
+            case P_TWO: rc = enumerate(k_cliques<4, P_TWO>, k_cliques_mid<4, P_TWO>, optin[2]); break;
+            case P_MAX: rc = enumerate(k_cliques<4, P_MAX>, k_cliques_mid<4, P_MAX>, optin[3]); break;
+            case 4 + P_MIN: rc = enumerate(k_cliques<5, P_MIN>, k_cliques_mid<5, P_MIN>, optin[4]); break;
+            case 4 + P_ONE: rc = enumerate(k_cliques<5, P_ONE>, k_cliques_mid<5, P_ONE>, optin[5]); break;
+            case 4 + P_TWO: rc = enumerate(k_cliques<5, P_TWO>, k_cliques_mid<5, P_TWO>, optin[6]); break;
+            default: rc = enumerate(k_cliques<5, P_MAX>, k_cliques_mid<5, P_MAX>, optin[7]); break;
+        }
         if (rc != WTRI_OK) return done(rc);
     }
     {
-        ProfScope ps("cliques_enumerate", s, 0.0, 1);
-        k_cliques<<<sm_count() * (q == 5 ? 1 : 4), CB, smem, s>>>(G, C);
-    }
-    {
-        ProfScope ps("cliques_select", s, 0.0, 2);
-        k_clique_select<<<1, CSB, 0, s>>>(ckey, cids, small, cap, q, (uint32_t)k, small + 1, small + 3);
-        k_clique_rank<<<ceil_div_u(k, 8), 256, 0, s>>>(ckey, cids, small + 3, small + 1, q, pcode,
+        ProfScope ps("cliques_select", s, 0.0, 3);
+        CliqueSelect A{};
+        A.lim = (unsigned long long*)((char*)small + 256);
+        A.q.st = (QState*)((char*)small + 512);
+        A.q.wait_first = WAIT_LIMIT;
+        A.hist = (uint32_t*)((char*)small + 512 + al(sizeof(QState)));
+        A.ckey = ckey;
+        A.count = small;
+        A.cap = cap;
+        A.K = (uint32_t)k;
+        A.err = small + 1;
+        A.ix = ix;
+        A.nix = small + 4;
+        void* args[] = {&A};
+        cudaError_t le = cudaLaunchCooperativeKernel((const void*)k_clique_reach, dim3((unsigned)sm_count()),
+                                                     dim3(TGRID), args, 0, s);
+        if (le != cudaSuccess) return done(cuda_error(le, "clique select", __FILE__, __LINE__));
+        k_clique_select<<<1, CSB, 0, s>>>(ckey, cids, ix, small + 4, q, (uint32_t)k, small + 1, small + 3);
+        k_clique_rank<<<ceil_div_u(k, 8), 256, 0, s>>>(ckey, cids, ix, small + 3, small + 1, q, pcode,
                                                         (uint32_t)k, oids, ow, okey);
     }
     if (cudaGetLastError() != cudaSuccess)
@@ -433,6 +817,7 @@ int clique_topk_host(const wtri_graph* g, int q, int pcode, int32_t k, int64_t n
     cudaError_t e = cudaMemcpyAsync(hs, small, sizeof(hs), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return done(cuda_error(e, "clique results", __FILE__, __LINE__));
+    if (hs[1] & CERR_WAIT) return done(set_error(WTRI_ETIMEOUT, "a bounded wait of the clique selection ran out"));
     if (hs[1] & CERR_NBR)
         return done(set_error(WTRI_EUNSUPPORTED, "a drawn edge has more than " + std::to_string(CNB) +
                                                      " common neighbours"));
