@@ -214,6 +214,7 @@ struct EdgeLoader {
     __device__ __forceinline__ const void* tile_src(int a, int64_t tbase) const {
         return (a == 0 ? w : (a == 1 ? u : v)) + tbase;
     }
+    __device__ __forceinline__ uint32_t skey(const uint32_t* in, int li) const { return ~in[li]; }
     __device__ __forceinline__ uint4 srec(const uint32_t* in, int li, int64_t) const {
         return make_uint4(~in[li], in[TT + li], in[2 * TT + li], 0u);
     }
@@ -249,6 +250,9 @@ struct OrderEntryLoader {
     const int32_t* ow;
     __device__ __forceinline__ const void* tile_src(int a, int64_t tbase) const {
         return (a == 0 ? ou : (a == 1 ? ov : ow)) + (tbase >> 1);
+    }
+    __device__ __forceinline__ uint32_t skey(const uint32_t* in, int li) const {
+        return in[(li & 1 ? TT : 0) + (li >> 1)];
     }
     __device__ __forceinline__ uint4 srec(const uint32_t* in, int li, int64_t tbase) const {
         const int e = li >> 1, side = li & 1;

@@ -13,7 +13,8 @@
 //   Loader: static NARR, TILE_WORDS     source arrays copied per tile, words each
 //           static REC_BYTES            bytes read per record
 //           const void* tile_src(int a, int64_t tbase)
-//           uint4 srec(const uint32_t* in, int li, int64_t tbase)   from a copied tile
+//           uint32_t skey(const uint32_t* in, int li)               from a copied tile
+//           uint4 srec(const uint32_t* in, int li, int64_t tbase)
 //           uint4 grec(int64_t i)       from global memory
 //           uint32_t key(int64_t i)     (first-pass histogram)
 //           bool tma_ok()               sources 16-byte aligned
@@ -31,12 +32,24 @@
 // Three kernels per pass: per-chunk digit histograms (upsweep), a per-digit
 // scan over chunks, and the scatter.  The scatter streams its chunk tile by
 // tile; the next tile's sources arrive by bulk asynchronous copies
-// (cp.async.bulk, one mbarrier per half of a double buffer) while the
-// current one is ranked (per-warp peer masks built by shared-memory
-// atomicOr, per-warp counters; stable), staged in
-// digit order in the same shared-memory buffer it was read from, and written
-// out so that consecutive threads store consecutive positions of one
-// digit's run.
+// (cp.async.bulk, one mbarrier per buffer) while the current one is ranked
+// (ballots over the digit's bits give a strip's equal digits, per-warp
+// counters the ones before; stable).  The ranks give each place of the
+// digit order its record's place in the tile (2 bytes); the records
+// themselves stay where the copy put them, are read once, in digit order,
+// and go straight out, consecutive threads storing consecutive positions of
+// one digit's run.
+//
+// What bounds the scatter: the runs (TT / bins records) begin and end inside
+// lines, and the time follows the write requests that reach L2, 59 per ns
+// (9-bit digits: 37 million for 62 million records, 2/5 of them for the
+// digits), while DRAM is 45 % busy.  So one CTA per SM with the largest tile
+// that shared memory holds twice: with two CTAs of half the tile the phases
+// overlap (ranking on votes and arithmetic, writing on shared memory), yet
+// the 1e9-edge build's scatters take 86.9 ms instead of 68.9.  Keeping the
+// records in place instead of staging them (and with the ballots, which left
+// the registers they need) allowed 5,632 records a tile instead of 5,376:
+// 71.3 -> 68.9 ms.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -51,29 +64,22 @@ namespace radix {
 constexpr int MAX_BITS = 10;               // widest digit of a pass
 constexpr int MAX_BINS = 1 << MAX_BITS;
 #ifndef WTRI_RADIX_NT
-#define WTRI_RADIX_NT 256
-#endif
-constexpr int NT = WTRI_RADIX_NT;          // threads of the histogram and scatter CTAs
-constexpr int NW = NT / 32;
-// Ranking within a warp: peer masks built by shared-memory atomicOr, one
-// word per (warp, digit) (1), or ballots over the digit's bits (0).
-#ifndef WTRI_RANK_SMEM
-#define WTRI_RANK_SMEM 1
+#define WTRI_RADIX_NT 512
 #endif
 #ifndef WTRI_RADIX_IT
-#if WTRI_RANK_SMEM
-#define WTRI_RADIX_IT (WTRI_RADIX_NT == 512 ? 9 : 21)  // tiles, counters, masks and staging fit 227 KB
-#else
-#define WTRI_RADIX_IT (WTRI_RADIX_NT == 512 ? 11 : 24)  // the tiles, counters and staging fit 227 KB
-#endif
+#define WTRI_RADIX_IT 11
 #endif
 #ifndef WTRI_RADIX_CTAS
 #define WTRI_RADIX_CTAS 1
 #endif
+constexpr int NT = WTRI_RADIX_NT;          // threads of the histogram and scatter CTAs
+constexpr int NW = NT / 32;
 constexpr int IT = WTRI_RADIX_IT;          // records per thread per tile
 constexpr int TT = NT * IT;                // records per tile
 constexpr int CTAS_PER_SM = WTRI_RADIX_CTAS;
+constexpr int NBUF = 2;                    // tile buffers of a scatter CTA
 constexpr int DPT = MAX_BINS / NT;         // digits owned by a thread in the tile scan
+constexpr int MIN_CHUNK = 1024;            // records
 constexpr int UP_SPLIT = 8;                // histogram blocks per chunk
 constexpr int UNT = 256;                   // threads of a histogram block
 constexpr int UNW = UNT / 32;
@@ -120,7 +126,7 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t x, uint32_t* w
 
 struct PassGeom {
     int64_t n;        // records
-    int64_t chunk;    // records per chunk (whole tiles)
+    int64_t chunk;    // records per chunk
     int chunks;       // G
     int shift;
     int bins;         // 1 << digit bits
@@ -278,66 +284,33 @@ __device__ __forceinline__ bool bar_try_wait(uint64_t* bar, uint32_t parity) {
 }
 
 struct ScatterSmem {
-    uint4 buf[2][TT];              // a tile's sources, then its records in digit order
-    uint16_t cnt[NW][MAX_BINS];    // per (warp, digit): count, then staging offset
-#if WTRI_RANK_SMEM
-    uint32_t match[NW][MAX_BINS];  // per (warp, digit): lanes of the current strip; zero between strips
-#endif
-    uint32_t delta[MAX_BINS];      // output position of a staged record = delta[d] + index
+    uint4 buf[NBUF][TT];           // tiles' sources
+    uint16_t src[TT];              // tile place of the record at each place of the digit order
+    uint16_t cnt[NW][MAX_BINS];    // per (warp, digit): count, then offset in the digit order
+    uint32_t delta[MAX_BINS];      // output position of digit-order place p = delta[digit] + p
     uint32_t warp_tot[32];
     uint32_t total;
     int timed_out;
-    uint64_t bar[2];
+    uint64_t bar[NBUF];
 };
+static_assert(TT <= 65536, "a tile place fits 16 bits");
 
 __device__ __forceinline__ uint32_t lo16(uint32_t x) { return x & 0xffffu; }
-
-#ifndef WTRI_RANK_BALLOT
-#define WTRI_RANK_BALLOT 1
-#endif
-#ifndef WTRI_PEERS_ALL_BITS
-#define WTRI_PEERS_ALL_BITS 0
-#endif
-#ifndef WTRI_FULL_TILES
-#define WTRI_FULL_TILES 0
-#endif
-// Lanes of the warp holding the same digit as this lane (digits of 'bits'
-// bits; lanes with valid == false group only among themselves): one ballot
-// per digit bit.
-template <bool FULL>
-__device__ __forceinline__ uint32_t digit_peers(uint32_t d, int bits, bool valid) {
-#if WTRI_RANK_BALLOT
-    uint32_t p = 0xffffffffu;  // a full tile: every lane holds a record
-    if (!FULL) {
-        const uint32_t vb = __ballot_sync(0xffffffffu, valid);
-        p = valid ? vb : ~vb;
-    }
-#if WTRI_PEERS_ALL_BITS
-    // digits are below 1 << bits, so the ballots of the bits above are all
-    // zero and leave p unchanged: no per-bit test
-    (void)bits;
-#pragma unroll
-    for (int k = 0; k < MAX_BITS; k++) {
-        const bool bit = (d >> k) & 1u;
-        const uint32_t b = __ballot_sync(0xffffffffu, bit);
-        p &= bit ? b : ~b;
-    }
-#else
-#pragma unroll
-    for (int k = 0; k < MAX_BITS; k++) {
-        if (k < bits) {
-            const bool bit = (d >> k) & 1u;
-            const uint32_t b = __ballot_sync(0xffffffffu, bit);
-            p &= bit ? b : ~b;
-        }
-    }
-#endif
-    return p;
-#else
-    return __match_any_sync(0xffffffffu, valid ? d : 0xffffffffu);
-#endif
-}
 __device__ __forceinline__ uint32_t hi16(uint32_t x) { return x >> 16; }
+
+// Lanes of the warp holding the same digit (of BITS bits) as this lane; lanes
+// without a record group among themselves.
+template <int BITS>
+__device__ __forceinline__ uint32_t digit_peers(uint32_t d, bool valid) {
+    const uint32_t vb = __ballot_sync(0xffffffffu, valid);
+    uint32_t p = valid ? vb : ~vb;
+#pragma unroll
+    for (int k = 0; k < BITS; k++) {
+        const uint32_t b = __ballot_sync(0xffffffffu, (d >> k) & 1u);
+        p &= b ^ (((d >> k) & 1u) - 1u);  // the ballot, or its complement
+    }
+    return p;
+}
 
 // A thread's DPT consecutive 16-bit counters as one 4- or 8-byte word.
 __device__ __forceinline__ void load_counts(const uint16_t* p, uint32_t (&c)[DPT]) {
@@ -361,70 +334,55 @@ __device__ __forceinline__ void store_counts(uint16_t* p, const uint32_t (&s)[DP
     }
 }
 
-// Rank, stage and write one tile of tcount <= TT records held in registers.
-// Item j of warp w, lane l is record w * 32 * IT + j * 32 + l of the tile;
-// ranking strips in order and warps in order keeps equal digits stable.
-// run[] holds this thread's digits' next output positions (digits
-// threadIdx.x * DPT + i).
-template <bool FULL, class Storer>
-__device__ __forceinline__ void scatter_tile(const uint4 (&rec)[IT], int tcount, uint4* stage,
-                                             const Storer& st, const PassGeom& g,
-                                             uint32_t (&run)[DPT], ScatterSmem& S) {
+// Ranks a tile's digits within each warp: rk[j] = digit | rank << 16, and the
+// per-(warp, digit) counts.  Item j of warp w, lane l is record
+// (w * strips + j) * 32 + l of the tile, strips = IT in a full tile; strips in
+// order and warps in order keep equal digits stable.
+template <int BITS, bool FULL>
+__device__ __forceinline__ void rank_strips(uint32_t (&rk)[IT], int strips, int tcount, ScatterSmem& S) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t lt = lanemask_lt();
-    // 1. zero the counters of the used digits (16-byte words, 8 digits each)
-    const int zw = (g.bins + 7) >> 3;  // at least one word, so digits 0..3 always start at zero
-    for (int q = threadIdx.x; q < zw; q += NT) {
+    uint16_t* cnt = S.cnt[w];
+    auto valid = [&](int j) { return FULL || (j < strips && (w * strips + j) * 32 + lane < tcount); };
+    uint32_t peers[IT];
 #pragma unroll
-        for (int k = 0; k < NW; k++) reinterpret_cast<uint4*>(&S.cnt[k][0])[q] = make_uint4(0, 0, 0, 0);
+    for (int j = 0; j < IT; j++) {  // independent across strips
+        if (!FULL && j >= strips) break;
+        peers[j] = digit_peers<BITS>(rk[j], valid(j));
     }
+#pragma unroll
+    for (int j = 0; j < IT; j++) {
+        if (!FULL && j >= strips) break;
+        const uint32_t d = rk[j];
+        const uint32_t b = valid(j) ? (uint32_t)cnt[d] : 0u;
+        rk[j] = d | ((b + __popc(peers[j] & lt)) << 16);
+        __syncwarp();
+        if (valid(j) && (peers[j] & lt) == 0) cnt[d] = (uint16_t)(b + __popc(peers[j]));
+        __syncwarp();
+    }
+}
+
+// Ranks and writes one tile of tcount <= TT records.  key(li), rec(li): the
+// tile's records, in shared memory.  On entry the counters are zero and the
+// tile visible to every thread.  run[] holds this thread's digits' next
+// output positions (digits threadIdx.x * DPT + i).
+template <bool FULL, class Key, class Rec, class Storer>
+__device__ __forceinline__ void scatter_tile(const Key& key, const Rec& rec, int tcount, const Storer& st,
+                                             const PassGeom& g, uint32_t (&run)[DPT], ScatterSmem& S) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int strips = FULL ? IT : (tcount + NT - 1) / NT;
+    // 1. rank within the warp
+    uint32_t rk[IT];
+#pragma unroll
+    for (int j = 0; j < IT; j++) {
+        const int li = (w * strips + j) * 32 + lane;
+        rk[j] = FULL || (j < strips && li < tcount) ? (key(li) >> g.shift) & g.mask : 0u;
+    }
+    if (g.bits > 9) rank_strips<10, FULL>(rk, strips, tcount, S);
+    else if (g.bits == 9) rank_strips<9, FULL>(rk, strips, tcount, S);
+    else rank_strips<8, FULL>(rk, strips, tcount, S);
     __syncthreads();
-    uint32_t rank[IT];
-#if WTRI_RANK_SMEM
-    // 2. rank within the warp, strip by strip: each lane sets its bit in its
-    //    digit's mask word, reads the word back (its peers), and the lowest
-    //    peer advances the digit's counter and clears the word
-    uint32_t* mm = S.match[w];
-#pragma unroll
-    for (int j = 0; j < IT; j++) {
-        const int li = w * 32 * IT + j * 32 + lane;
-        const bool valid = FULL || li < tcount;
-        const uint32_t d = (rec[j].x >> g.shift) & g.mask;
-        if (valid) atomicOr(&mm[d], 1u << lane);
-        __syncwarp();
-        const uint32_t peers = valid ? mm[d] : 0u;
-        const uint32_t b = valid ? (uint32_t)S.cnt[w][d] : 0u;
-        rank[j] = b + __popc(peers & lt);
-        __syncwarp();
-        if (valid && lane == __ffs(peers) - 1) {
-            S.cnt[w][d] = (uint16_t)(b + __popc(peers));
-            mm[d] = 0u;
-        }
-        __syncwarp();
-    }
-#else
-    // 2. rank within the warp: first every item's peers (ballots, independent
-    //    across strips), then the running per-warp counters strip by strip
-#pragma unroll
-    for (int j = 0; j < IT; j++) {
-        const int li = w * 32 * IT + j * 32 + lane;
-        rank[j] = digit_peers<FULL>((rec[j].x >> g.shift) & g.mask, g.bits, FULL || li < tcount);
-    }
-#pragma unroll
-    for (int j = 0; j < IT; j++) {
-        const int li = w * 32 * IT + j * 32 + lane;
-        const bool valid = FULL || li < tcount;
-        const uint32_t d = (rec[j].x >> g.shift) & g.mask;
-        const uint32_t peers = rank[j];
-        const uint32_t b = valid ? (uint32_t)S.cnt[w][d] : 0u;
-        rank[j] = b + __popc(peers & lt);
-        __syncwarp();
-        if (valid && lane == __ffs(peers) - 1) S.cnt[w][d] = (uint16_t)(b + __popc(peers));
-        __syncwarp();
-    }
-#endif
-    __syncthreads();
-    // 3. per digit: offsets of each warp, tile start, output delta.  Thread t
+    // 2. per digit: offsets of each warp, tile start, output delta.  Thread t
     //    owns digits DPT t .. DPT t + DPT - 1: one word of each warp's counters.
     {
         const int d0 = threadIdx.x * DPT;
@@ -444,8 +402,18 @@ __device__ __forceinline__ void scatter_tile(const uint4 (&rec)[IT], int tcount,
         uint32_t sum = 0;
 #pragma unroll
         for (int i = 0; i < DPT; i++) sum += tot[i];
-        const uint32_t start = block_exclusive_scan<NT>(sum, S.warp_tot, &S.total);
+        uint32_t inc = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        if (lane == 31) S.warp_tot[w] = inc;
+        __syncthreads();
         if (mine) {
+            uint32_t start = inc - sum;
+#pragma unroll
+            for (int k = 0; k < NW; k++) start += k < w ? S.warp_tot[k] : 0u;
             uint32_t s[DPT];
             s[0] = start;
 #pragma unroll
@@ -466,30 +434,31 @@ __device__ __forceinline__ void scatter_tile(const uint4 (&rec)[IT], int tcount,
         }
     }
     __syncthreads();
-    // 4. stage in digit order (the tile's sources were read by every thread
-    //    before the barriers above)
+    // 3. the digit order
 #pragma unroll
     for (int j = 0; j < IT; j++) {
-        const int li = w * 32 * IT + j * 32 + lane;
-        if (FULL || li < tcount) {
-            const uint32_t d = (rec[j].x >> g.shift) & g.mask;
-            stage[rank[j] + S.cnt[w][d]] = rec[j];
-        }
+        const int li = (w * strips + j) * 32 + lane;
+        if (FULL || (j < strips && li < tcount)) S.src[S.cnt[w][lo16(rk[j])] + hi16(rk[j])] = (uint16_t)li;
     }
     __syncthreads();
-    // 5. write: consecutive threads, consecutive positions of one digit's run
+    // 4. write: consecutive threads, consecutive positions of one digit's run
 #pragma unroll
     for (int i = 0; i < IT; i++) {
         const int p = i * NT + threadIdx.x;
         if (FULL || p < tcount) {
-            const uint4 r = stage[p];
+            const uint4 r = rec((int)S.src[p]);
             const uint32_t d = (r.x >> g.shift) & g.mask;
             st.store((int64_t)S.delta[d] + p, r);
         }
     }
-    // generic accesses to the buffer are ordered before the next bulk copy into it
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
+}
+
+// The counters of the used digits, zeroed (16-byte words, 8 digits each; at
+// least one word).
+__device__ __forceinline__ void zero_counts(const PassGeom& g, ScatterSmem& S) {
+    const int zw = (g.bins + 7) >> 3;
+    for (int q = threadIdx.x; q < zw * NW; q += NT)
+        reinterpret_cast<uint4*>(&S.cnt[q / zw][0])[q % zw] = make_uint4(0, 0, 0, 0);
 }
 
 // One CTA per chunk; whole tiles arrive by bulk copies when USE_BULK (sources
@@ -527,18 +496,15 @@ __global__ void __launch_bounds__(NT, CTAS_PER_SM) k_scatter(Loader ld, Storer s
     const int64_t nfull = USE_BULK && end > beg ? (end - beg) / TT : 0;
     constexpr uint32_t ARR_BYTES = Loader::TILE_WORDS * 4u;
     static_assert(Loader::NARR * Loader::TILE_WORDS <= 4 * TT, "a tile's sources fit one buffer");
-#if WTRI_RANK_SMEM
-    for (int t = threadIdx.x; t < NW * MAX_BINS; t += NT) (&S.match[0][0])[t] = 0u;
-#endif
     if (threadIdx.x == 0) {
-        bar_init(&S.bar[0]);
-        bar_init(&S.bar[1]);
+        for (int b = 0; b < NBUF; b++) bar_init(&S.bar[b]);
         S.timed_out = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
     const uint64_t policy = evict_first_policy();
-    auto issue = [&](int64_t t, int b) {
+    auto issue = [&](int64_t t) {
+        const int b = (int)(t % NBUF);
         const int64_t tbase = beg + t * TT;
         bar_expect(&S.bar[b], ARR_BYTES * Loader::NARR);
         uint32_t* dst = reinterpret_cast<uint32_t*>(&S.buf[b][0]);
@@ -546,13 +512,12 @@ __global__ void __launch_bounds__(NT, CTAS_PER_SM) k_scatter(Loader ld, Storer s
         for (int a = 0; a < Loader::NARR; a++)
             bulk_load(dst + (size_t)a * TT, ld.tile_src(a, tbase), ARR_BYTES, &S.bar[b], policy);
     };
-    if (threadIdx.x == 0 && nfull > 0) issue(0, 0);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (threadIdx.x == 0)
+        for (int64_t t = 0; t < NBUF - 1 && t < nfull; t++) issue(t);
     for (int64_t t = 0; t < nfull; t++) {
-        const int b = (int)(t & 1);
-        // the other buffer was last used by tile t-1, released at its closing barrier
-        if (threadIdx.x == 0 && t + 1 < nfull) issue(t + 1, b ^ 1);
-        const uint32_t parity = (uint32_t)((t >> 1) & 1);
+        const int b = (int)(t % NBUF);
+        const uint32_t parity = (uint32_t)((t / NBUF) & 1);
+        zero_counts(g, S);  // last read before the previous tile's write
         uint32_t spins = 0;
         while (!bar_try_wait(&S.bar[b], parity)) {
             if (++spins >= WAIT_LIMIT) {
@@ -563,29 +528,28 @@ __global__ void __launch_bounds__(NT, CTAS_PER_SM) k_scatter(Loader ld, Storer s
         __syncthreads();
         if (S.timed_out) {
             if (threadIdx.x == 0) atomicOr(err, DEV_ERR_TIMEOUT);
-            for (int bb = 0; bb < 2; bb++) {
+            for (int bb = 0; bb < NBUF; bb++) {
                 uint32_t s2 = 0;
                 while (!bar_try_wait(&S.bar[bb], parity) && ++s2 < WAIT_LIMIT) {
                 }
             }
             return;
         }
+        // the buffer of tile t - 1 was read up to the barrier above
+        if (threadIdx.x == 0 && t + NBUF - 1 < nfull) issue(t + NBUF - 1);
         const int64_t tbase = beg + t * TT;
         const uint32_t* in = reinterpret_cast<const uint32_t*>(&S.buf[b][0]);
-        uint4 rec[IT];
-#pragma unroll
-        for (int j = 0; j < IT; j++) rec[j] = ld.srec(in, w * 32 * IT + j * 32 + lane, tbase);
-        scatter_tile<WTRI_FULL_TILES != 0>(rec, TT, &S.buf[b][0], st, g, run, S);
+        scatter_tile<true>([&](int li) { return ld.skey(in, li); }, [&](int li) { return ld.srec(in, li, tbase); }, TT,
+                           st, g, run, S);
     }
     for (int64_t tbase = beg + nfull * TT; tbase < end; tbase += TT) {
         const int tcount = (int)min((int64_t)TT, end - tbase);
-        uint4 rec[IT];
-#pragma unroll
-        for (int j = 0; j < IT; j++) {
-            const int li = w * 32 * IT + j * 32 + lane;
-            rec[j] = li < tcount ? ld.grec(tbase + li) : make_uint4(0, 0, 0, 0);
-        }
-        scatter_tile<false>(rec, tcount, &S.buf[0][0], st, g, run, S);
+        __syncthreads();  // the tile before is written
+        zero_counts(g, S);
+        uint4* in = S.buf[0];
+        for (int li = threadIdx.x; li < tcount; li += NT) in[li] = ld.grec(tbase + li);
+        __syncthreads();
+        scatter_tile<false>([&](int li) { return in[li].x; }, [&](int li) { return in[li]; }, tcount, st, g, run, S);
     }
 }
 
@@ -597,6 +561,7 @@ struct AosLoader {
     const uint4* r;
     __device__ __forceinline__ uint32_t key(int64_t i) const { return __ldg(&r[i].x); }
     __device__ __forceinline__ const void* tile_src(int, int64_t tbase) const { return r + tbase; }
+    __device__ __forceinline__ uint32_t skey(const uint32_t* in, int li) const { return in[4 * li]; }
     __device__ __forceinline__ uint4 srec(const uint32_t* in, int li, int64_t) const {
         return reinterpret_cast<const uint4*>(in)[li];
     }
@@ -640,18 +605,15 @@ struct SwitchStorer {
 };
 
 // ---- host side ------------------------------------------------------------------
-// Chunking: CTAS_PER_SM chunks per SM at most, each a whole number of tiles.
+// Chunking: CTAS_PER_SM chunks per SM at most, equal shares of at least
+// MIN_CHUNK records (a multiple of 32, so that every source stays 16-byte
+// aligned); the tiles of a chunk are whole but the last.
 inline PassGeom make_geom(int64_t n, int shift, int bits) {
     PassGeom g;
     g.n = n;
-    const int64_t tiles = (n + TT - 1) / TT;
-    int64_t want = (int64_t)sm_count() * CTAS_PER_SM;
-    if (want > tiles) want = tiles;
-    if (want < 1) want = 1;
-    const int64_t tiles_per = (tiles + want - 1) / want;
-    g.chunk = tiles_per * TT;
-    g.chunks = (int)((n + g.chunk - 1) / g.chunk);
-    if (g.chunks < 1) g.chunks = 1;
+    const int64_t want = (int64_t)sm_count() * CTAS_PER_SM, per = (n + want - 1) / want;
+    g.chunk = std::max<int64_t>(MIN_CHUNK, (per + 31) / 32 * 32);
+    g.chunks = (int)std::max<int64_t>(1, (n + g.chunk - 1) / g.chunk);
     g.shift = shift;
     g.bins = 1 << bits;
     g.bits = bits;
@@ -662,10 +624,11 @@ inline PassGeom make_geom(int64_t n, int shift, int bits) {
     return g;
 }
 
-// Scratch for counts: MAX_BINS * chunks + MAX_BINS (uint32).
+// Scratch for the counts of any sort of at most n records: MAX_BINS * chunks +
+// MAX_BINS (uint32).
 inline size_t scratch_words(int64_t n) {
-    PassGeom g = make_geom(n, 0, MAX_BITS);
-    return (size_t)MAX_BINS * g.chunks + MAX_BINS;
+    const int64_t chunks = std::min<int64_t>((int64_t)sm_count() * CTAS_PER_SM, n / MIN_CHUNK + 1);
+    return (size_t)MAX_BINS * (size_t)chunks + MAX_BINS;
 }
 
 // Whether whole tiles use bulk copies (WTRI_RADIX_TMA=0 turns them off).
