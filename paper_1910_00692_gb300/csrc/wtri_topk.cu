@@ -89,19 +89,151 @@ __device__ __forceinline__ uint64_t philox_word0(uint64_t c0, uint64_t k0) {
     return c0;
 }
 
-// Class starts: position r starts a class when its weight differs from r-1.
-__global__ void k_class_flags(int64_t m, const int32_t* __restrict__ ow, int32_t* __restrict__ flag) {
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < m;
-         r += (int64_t)gridDim.x * blockDim.x)
-        flag[r] = (r == 0 || __ldg(ow + r) != __ldg(ow + r - 1)) ? 1 : 0;
+// Ordered compactions (the class starts of the edge order, the drawn
+// positions of the bitmap) in three launches: each block counts what it will
+// write of its contiguous share, one block scans the counts, each block
+// reads its share again and writes.  Both are sparse, so a step without any
+// costs its loads and one barrier; an exclusive scan over all positions
+// first wrote and read 20 bytes each (160 us at 2e7 edges; now 27).
+constexpr int CB_T = 256;
+
+inline unsigned compact_blocks(int64_t work) {  // work: positions or words
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)sm_count() * 8, (work + 1023) / 1024));
 }
 
-__global__ void k_class_starts(int64_t m, const int32_t* __restrict__ flag,
-                               const int64_t* __restrict__ cls, int64_t* __restrict__ cstart) {
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < m;
-         r += (int64_t)gridDim.x * blockDim.x)
-        if (flag[r]) cstart[cls[r]] = r;
-    if (blockIdx.x == 0 && threadIdx.x == 0) cstart[cls[m]] = m;  // sentinel
+// Exclusive scan over a CB_T block; *total receives the sum.
+__device__ __forceinline__ uint32_t cb_scan(uint32_t x, uint32_t* wsum, uint32_t* total) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t inc = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    if (lane == 31) wsum[w] = inc;
+    __syncthreads();
+    uint32_t before = 0, all = 0;
+#pragma unroll
+    for (int k = 0; k < CB_T / 32; k++) {
+        before += k < w ? wsum[k] : 0u;
+        all += wsum[k];
+    }
+    *total = all;
+    __syncthreads();
+    return before + inc - x;
+}
+
+// Exclusive scan of the blocks' counts in place (one block); *total = sum.
+__global__ void __launch_bounds__(1024) k_block_offsets(uint32_t* cnt, int blocks, int64_t* total, int64_t* sentinel,
+                                                        int64_t sentinel_value) {
+    __shared__ uint32_t wsum[32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t carry = 0;
+    for (int base = 0; base < blocks; base += 1024) {
+        const int i = base + threadIdx.x;
+        const uint32_t x = i < blocks ? cnt[i] : 0u;
+        uint32_t inc = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        if (lane == 31) wsum[w] = inc;
+        __syncthreads();
+        uint32_t before = carry;
+        for (int k = 0; k < 32; k++) {
+            before += k < w ? wsum[k] : 0u;
+            carry += wsum[k];
+        }
+        if (i < blocks) cnt[i] = before + inc - x;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        *total = carry;
+        if (sentinel) sentinel[carry] = sentinel_value;
+    }
+}
+
+// The class starts among four positions from r on: bit i set when position
+// r + i's weight differs from the one before.
+__device__ __forceinline__ uint32_t class_starts4(const int32_t* __restrict__ ow, int64_t r, int64_t m) {
+    if (r >= m) return 0u;
+    int32_t prev = r > 0 ? __ldg(ow + r - 1) : 0;  // weights are positive
+    int4 x;
+    if (r + 4 <= m) {
+        x = __ldg(reinterpret_cast<const int4*>(ow + r));  // r is a multiple of 4, ow 256-byte aligned
+    } else {
+        x.x = __ldg(ow + r);
+        x.y = r + 1 < m ? __ldg(ow + r + 1) : x.x;
+        x.z = r + 2 < m ? __ldg(ow + r + 2) : x.y;
+        x.w = x.z;
+    }
+    return (x.x != prev ? 1u : 0u) | (x.y != x.x ? 2u : 0u) | (x.z != x.y ? 4u : 0u) | (x.w != x.z ? 8u : 0u);
+}
+
+// Items of a compaction: four positions' class starts, or a bitmap word.
+struct ClassBits {
+    static constexpr int PER = 4;  // positions per item
+    const int32_t* ow;
+    int64_t m;
+    __device__ __forceinline__ uint32_t get(int64_t item) const { return class_starts4(ow, 4 * item, m); }
+};
+struct DrawnBits {
+    static constexpr int PER = 32;
+    const uint32_t* mark;
+    int64_t words;
+    __device__ __forceinline__ uint32_t get(int64_t item) const { return item < words ? __ldg(mark + item) : 0u; }
+};
+
+template <class Bits>
+__global__ void __launch_bounds__(CB_T) k_compact_count(Bits B, int64_t items, uint32_t* cnt) {
+    __shared__ uint32_t wsum[CB_T / 32];
+    const int64_t per = ((items + gridDim.x - 1) / gridDim.x + CB_T - 1) / CB_T * CB_T;
+    const int64_t beg = (int64_t)blockIdx.x * per, end = min(items, beg + per);
+    uint32_t c = 0, total;
+#pragma unroll 4
+    for (int64_t i = beg + threadIdx.x; i < end; i += CB_T) c += __popc(B.get(i));
+    cb_scan(c, wsum, &total);
+    if (threadIdx.x == 0) cnt[blockIdx.x] = total;
+}
+
+template <class Bits, class T>
+__global__ void __launch_bounds__(CB_T) k_compact_write(Bits B, int64_t items, const uint32_t* cnt, T* out) {
+    __shared__ uint32_t wsum[CB_T / 32];
+    const int64_t per = ((items + gridDim.x - 1) / gridDim.x + CB_T - 1) / CB_T * CB_T;
+    const int64_t beg = (int64_t)blockIdx.x * per, end = min(items, beg + per);
+    int64_t off = cnt[blockIdx.x];
+    constexpr int U = 4;
+    for (int64_t i0 = beg; i0 < end; i0 += U * CB_T) {
+        uint32_t b[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int64_t i = i0 + u * CB_T + threadIdx.x;
+            b[u] = i < end ? B.get(i) : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            if (!__syncthreads_or(b[u] != 0u)) continue;
+            uint32_t total;
+            int64_t o = off + cb_scan((uint32_t)__popc(b[u]), wsum, &total);
+            const int64_t first = (i0 + u * CB_T + threadIdx.x) * Bits::PER;
+            for (uint32_t x = b[u]; x; x &= x - 1) out[o++] = (T)(first + __ffs(x) - 1);
+            off += total;
+        }
+    }
+}
+
+// The positions of the set bits, ascending, to out; their number to *total
+// (and `end` after the last one when sentinel is set).  cnt: compact_blocks.
+template <class Bits, class T>
+int ordered_compact(const Bits& B, int64_t items, uint32_t* cnt, T* out, int64_t* total, int64_t* sentinel, int64_t end,
+                    cudaStream_t s) {
+    const unsigned g = compact_blocks(items);
+    k_compact_count<Bits><<<g, CB_T, 0, s>>>(B, items, cnt);
+    k_block_offsets<<<1, 1024, 0, s>>>(cnt, (int)g, total, sentinel, end);
+    k_compact_write<Bits, T><<<g, CB_T, 0, s>>>(B, items, cnt, out);
+    WTRI_CUDA(cudaGetLastError());
+    return WTRI_OK;
 }
 
 // Inclusive prefix of class masses count * w^p, one block (classes are few:
@@ -150,6 +282,9 @@ __global__ void __launch_bounds__(1024) k_class_mass(const int64_t* __restrict__
     }
 }
 
+// (class masses below 2^64 in all, the usual case: 64-bit products and
+// divisions; the 128-bit division is a subroutine of hundreds of
+// instructions)
 template <int P>
 __global__ void k_draw(int64_t nsamples, uint64_t seed, const int64_t* __restrict__ cls_total,
                        const int64_t* __restrict__ cstart, const int32_t* __restrict__ ow,
@@ -157,41 +292,38 @@ __global__ void k_draw(int64_t nsamples, uint64_t seed, const int64_t* __restric
     const int64_t nc = *cls_total;
     const u128 Z = cmass[nc - 1];
     const uint64_t zl = (uint64_t)Z, zh = (uint64_t)(Z >> 64);
+    const uint64_t* low = reinterpret_cast<const uint64_t*>(cmass);  // low words at even places
     for (int64_t sidx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; sidx < nsamples;
          sidx += (int64_t)gridDim.x * blockDim.x) {
         const uint64_t x = philox_word0((uint64_t)sidx, seed);
-        const u128 t = (u128)x * zh + (u128)__umul64hi(x, zl);  // floor(x * Z / 2^64)
-        int64_t lo = 0, hi = nc;                                   // first class with mass > t
-        while (lo < hi) {
-            const int64_t mid = (lo + hi) >> 1;
-            if (cmass[mid] > t) hi = mid;
-            else lo = mid + 1;
+        int64_t lo = 0, hi = nc;  // first class with mass > t = floor(x * Z / 2^64)
+        uint64_t place;
+        if (zh == 0) {
+            const uint64_t t = __umul64hi(x, zl);
+            while (lo < hi) {
+                const int64_t mid = (lo + hi) >> 1;
+                if (__ldg(low + 2 * mid) > t) hi = mid;
+                else lo = mid + 1;
+            }
+            const uint64_t prev = lo > 0 ? __ldg(low + 2 * lo - 2) : 0ull;
+            const uint64_t wv = (uint64_t)__ldg(ow + __ldg(cstart + lo));
+            place = (t - prev) / (P == P_TWO ? wv * wv : (P == P_GEO ? 1ull : wv));
+        } else {
+            const u128 t = (u128)x * zh + (u128)__umul64hi(x, zl);
+            while (lo < hi) {
+                const int64_t mid = (lo + hi) >> 1;
+                if (cmass[mid] > t) hi = mid;
+                else lo = mid + 1;
+            }
+            const u128 prev = lo > 0 ? cmass[lo - 1] : (u128)0;
+            const u128 wv = (u128)(uint64_t)__ldg(ow + cstart[lo]);
+            place = (uint64_t)((t - prev) / (P == P_TWO ? wv * wv : (P == P_GEO ? (u128)1 : wv)));
         }
-        const u128 prev = lo > 0 ? cmass[lo - 1] : (u128)0;
-        const u128 wv = (u128)(uint64_t)__ldg(ow + cstart[lo]);
-        const u128 wp = P == P_TWO ? wv * wv : (P == P_GEO ? (u128)1 : wv);
-        const int64_t r = cstart[lo] + (int64_t)((t - prev) / wp);
-        atomicOr(mark + (r >> 5), 1u << (r & 31));
-    }
-}
-
-__global__ void k_mark_popc(int64_t words, const uint32_t* __restrict__ mark, int32_t* __restrict__ pc) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words;
-         i += (int64_t)gridDim.x * blockDim.x)
-        pc[i] = __popc(mark[i]);
-}
-
-__global__ void k_mark_list(int64_t words, const uint32_t* __restrict__ mark,
-                            const int64_t* __restrict__ off, int32_t* __restrict__ list) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t b = mark[i];
-        int64_t o = off[i];
-        while (b) {
-            const int bit = __ffs(b) - 1;
-            list[o++] = (int32_t)(i * 32 + bit);
-            b &= b - 1;
-        }
+        const int64_t r = __ldg(cstart + lo) + (int64_t)place;
+        // heavy edges are drawn thousands of times: look before the atomic (a
+        // stale reading only repeats it)
+        const uint32_t bit = 1u << (r & 31);
+        if (!(__ldcg(mark + (r >> 5)) & bit)) atomicOr(mark + (r >> 5), bit);
     }
 }
 
@@ -201,42 +333,32 @@ inline unsigned grid_of(int64_t work) {
 }
 
 // Draws the samples into a bitmap over edge-order positions (words =
-// ceil(m/32), zeroed here).  Scratch: cls (m+1 int64), cstart (m+1 int64),
-// cmass (m u128), flags (m int32).
+// ceil(m/32), zeroed here).  Scratch: cmass (m u128), cstart (m+1 int64), the
+// number of classes, block counts.
 template <int P>
 int draw_samples(const wtri_graph* g, int64_t nsamples, uint64_t seed, uint32_t* mark,
                  cudaStream_t s) {
     const DevGraph& G = g->d;
-    const int64_t m = G.m, words = (m + 31) / 32;
-    const size_t bytes = 8 * (size_t)(m + 1) * 2 + 16 * (size_t)m + 4 * (size_t)m + 256;
+    const int64_t m = G.m, words = (m + 31) / 32, items = (m + 3) / 4;
+    const size_t bytes = 16 * (size_t)m + 8 * (size_t)(m + 2) + 4 * (size_t)compact_blocks(items) + 256;
     void* buf = nullptr;
     if (cudaMallocAsync(&buf, bytes, s) != cudaSuccess) {
         cudaGetLastError();
         return set_error(WTRI_ENOMEM, "sampling scratch allocation failed");
     }
-    char* p = (char*)buf;
-    int64_t* cls = (int64_t*)p;
-    p += 8 * (size_t)(m + 1);
-    int64_t* cstart = (int64_t*)p;
-    p += 8 * (size_t)(m + 1);
-    u128* cmass = (u128*)p;
-    p += 16 * (size_t)m;
-    int32_t* flag = (int32_t*)p;
+    u128* cmass = (u128*)buf;
+    int64_t* cstart = (int64_t*)(cmass + m);
+    int64_t* nc = cstart + m + 1;
+    uint32_t* cnt = (uint32_t*)(nc + 1);
     WTRI_CUDA(cudaMemsetAsync(mark, 0, 4 * (size_t)words, s));
     {
-        ProfScope ps("sample_classes", s, 4.0 * m + 4.0 * m, 1);
-        k_class_flags<<<grid_of(m), 256, 0, s>>>(m, G.ord_w, flag);
-    }
-    WTRI_TRY(exclusive_scan_i32_to_i64(flag, cls, m, s));  // cls[m] = number of classes
-    {
-        ProfScope ps("sample_class_table", s, 12.0 * m, 2);
-        k_class_starts<<<grid_of(m), 256, 0, s>>>(m, flag, cls, cstart);
-        k_class_mass<P><<<1, 1024, 0, s>>>(cls + m, cstart, G.ord_w, cmass);
+        ProfScope ps("sample_class_table", s, 12.0 * m, 4);
+        WTRI_TRY(ordered_compact(ClassBits{G.ord_w, m}, items, cnt, cstart, nc, cstart, m, s));
+        k_class_mass<P><<<1, 1024, 0, s>>>(nc, cstart, G.ord_w, cmass);
     }
     {
         ProfScope ps("sample_draw", s, 0.0, 1);
-        k_draw<P><<<grid_of(nsamples), 256, 0, s>>>(nsamples, seed, cls + m, cstart, G.ord_w, cmass,
-                                                    mark);
+        k_draw<P><<<grid_of(nsamples), 256, 0, s>>>(nsamples, seed, nc, cstart, G.ord_w, cmass, mark);
     }
     WTRI_CUDA(cudaGetLastError());
     WTRI_CUDA(cudaFreeAsync(buf, s));
@@ -252,7 +374,7 @@ int run_sample(const wtri_graph* g, int32_t k, int64_t nsamples, uint64_t seed, 
         (int64_t(1) << 20) * scale + 16 * (int64_t)k, (int64_t(1) << 31) - 1);
     const int64_t item_cap = query_items(m);
     const size_t qbytes = query_scratch_bytes(cap, item_cap);
-    const size_t sbytes = 4 * (size_t)words + 8 * (size_t)(words + 1) + 4 * (size_t)words + 4 * (size_t)m + 256;
+    const size_t sbytes = 4 * (size_t)words + 16 + 4 * (size_t)compact_blocks(words) + 4 * (size_t)m + 256;
     void* buf = nullptr;
     if (cudaMallocAsync(&buf, qbytes + sbytes, s) != cudaSuccess) {
         cudaGetLastError();
@@ -264,24 +386,21 @@ int run_sample(const wtri_graph* g, int32_t k, int64_t nsamples, uint64_t seed, 
     uint32_t* mark = (uint32_t*)p;
     p += 4 * (size_t)words;
     p = (char*)(((uintptr_t)p + 7) & ~(uintptr_t)7);
-    int64_t* off = (int64_t*)p;
-    p += 8 * (size_t)(words + 1);
-    int32_t* pc = (int32_t*)p;
-    p += 4 * (size_t)words;
+    int64_t* count = (int64_t*)p;
+    p += 8;
+    uint32_t* cnt = (uint32_t*)p;
+    p += 4 * (size_t)compact_blocks(words);
     int32_t* list = (int32_t*)p;
     q.smark = mark;
     q.slist = list;
-    q.total_dev = off + words;  // the number of drawn edges stays on the device
+    q.total_dev = count;  // the number of drawn edges stays on the device
     auto run = [&]() -> int {
         WTRI_CUDA(cudaMemsetAsync(q.st, 0, sizeof(QState), s));
         ProfScope whole(P == P_ONE ? "sample_p=1" : (P == P_TWO ? "sample_p=2" : "sample_p=0"), s, 0.0, 0);
         WTRI_TRY(draw_samples<P>(g, nsamples, seed, mark, s));
         {
-            ProfScope ps("sample_compact", s, 8.0 * words, 2);
-            k_mark_popc<<<grid_of(words), 256, 0, s>>>(words, mark, pc);
-            WTRI_TRY(exclusive_scan_i32_to_i64(pc, off, words, s));
-            k_mark_list<<<grid_of(words), 256, 0, s>>>(words, mark, off, list);
-            WTRI_CUDA(cudaGetLastError());
+            ProfScope ps("sample_compact", s, 8.0 * words, 3);
+            WTRI_TRY(ordered_compact(DrawnBits{mark, words}, words, cnt, list, count, (int64_t*)nullptr, 0, s));
         }
         ProfScope ps("sample_sweep", s, 0.0, 1);
         return launch_sweep<P, true>(G, q, Out{d_tris, d_weight, d_count, nullptr}, s);

@@ -55,6 +55,13 @@ __device__ __forceinline__ u128 mulhi_z(uint64_t x, u128 Z) {
     return (u128)x * zh + (u128)__umul64hi(x, zl);
 }
 
+// a / b; both below 2^64 in nearly every draw, where one 64-bit division does
+// (the 128-bit one is a subroutine of hundreds of instructions).
+__device__ __forceinline__ u128 div128(u128 a, u128 b) {
+    if (((uint64_t)(a >> 64) | (uint64_t)(b >> 64)) == 0) return (u128)((uint64_t)a / (uint64_t)b);
+    return a / b;
+}
+
 template <int P>
 __device__ __forceinline__ uint64_t wpow(int32_t w) {
     const uint64_t x = (uint64_t)(uint32_t)w;
@@ -64,31 +71,51 @@ __device__ __forceinline__ uint64_t wpow(int32_t w) {
 constexpr int WBLK = 256;
 constexpr unsigned long long HASH_EMPTY = ~0ull;
 
-// Per-row cumulative w^p (u64, one warp per row, a warp scan per 32
-// entries) and D(a); flags a row whose sum does not fit 64 bits.
+// Per-row cumulative w^p (u64, one warp per row: eight consecutive entries
+// per lane and step, one warp scan of their sums) and D(a); flags a row whose
+// sum does not fit 64 bits.  (With one entry per lane and step the longest
+// row's serial scans took 215 us on the 2e6-edge graph.)
 template <int P>
 __global__ void __launch_bounds__(WBLK) k_ws_rows(DevGraph G, uint64_t* __restrict__ cum,
                                                   uint64_t* __restrict__ D, uint32_t* err) {
+    constexpr int E = 8;
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = ((int64_t)gridDim.x * WBLK) >> 5;
     for (int64_t x = ((int64_t)blockIdx.x * WBLK + threadIdx.x) >> 5; x < G.n; x += nwarps) {
         const int64_t b0 = __ldg(G.rowptr + x), e0 = __ldg(G.rowptr + x + 1);
         uint64_t carry = 0;
         bool over = false;
-        for (int64_t base = b0; base < e0; base += 32) {
-            const int64_t j = base + lane;
-            uint64_t v = j < e0 ? wpow<P>(__ldg(G.wwt + j)) : 0;
+        // short rows: one entry per lane, so that a step is one coalesced load
+        const int per = e0 - b0 > 64 ? E : 1;
+        for (int64_t base = b0; base < e0; base += 32 * per) {
+            const int64_t j0 = base + (int64_t)lane * per;
+            uint64_t v[E], sum = 0;
+#pragma unroll
+            for (int i = 0; i < E; i++) {
+                const bool in = i < per && j0 + i < e0;
+                v[i] = in ? wpow<P>(__ldg(G.wwt + j0 + i)) : 0;
+            }
+#pragma unroll
+            for (int i = 0; i < E; i++) {
+                over |= sum + v[i] < sum;
+                sum += v[i];
+                v[i] = sum;
+            }
+            uint64_t inc = sum;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const uint64_t y = __shfl_up_sync(0xffffffffu, v, o);
+                const uint64_t y = __shfl_up_sync(0xffffffffu, inc, o);
                 if (lane >= o) {
-                    over |= v + y < v;
-                    v += y;
+                    over |= inc + y < inc;
+                    inc += y;
                 }
             }
-            const uint64_t s = carry + v;
+            const uint64_t s = carry + inc;
             over |= s < carry;
-            if (j < e0) cum[j] = s;
+            const uint64_t before = s - sum;
+#pragma unroll
+            for (int i = 0; i < E; i++)
+                if (i < per && j0 + i < e0) cum[j0 + i] = before + v[i];
             carry = __shfl_sync(0xffffffffu, s, 31);
         }
         if (__any_sync(0xffffffffu, over) && lane == 0) atomicOr(err, DEV_ERR_OVERFLOW);
@@ -198,7 +225,7 @@ __device__ __forceinline__ WsDraw ws_draw(const DevGraph& G, const uint64_t* __r
     const u128 dD = (u128)da * Da;
     const u128 t2 = mulhi_z(x[1], 2 * dD);
     if (t2 < dD) {
-        const uint64_t tp = (uint64_t)(t2 / da);
+        const uint64_t tp = (uint64_t)div128(t2, da);
         int64_t l2 = 0, h2 = (int64_t)da - 1;
         while (l2 < h2) {
             const int64_t mid = (l2 + h2) >> 1;
@@ -207,7 +234,7 @@ __device__ __forceinline__ WsDraw ws_draw(const DevGraph& G, const uint64_t* __r
         }
         r.jb = l2;
     } else {
-        r.jb = (int64_t)((t2 - dD) / Da);
+        r.jb = (int64_t)div128(t2 - dD, Da);
     }
     const u128 wab = wpow<P>(__ldg(G.wwt + b0 + r.jb));
     const u128 t3 = mulhi_z(x[2], Da + (u128)da * wab);
@@ -221,7 +248,7 @@ __device__ __forceinline__ WsDraw ws_draw(const DevGraph& G, const uint64_t* __r
         }
         r.jc = l2;
     } else {
-        r.jc = (int64_t)((t3 - Da) / wab);
+        r.jc = (int64_t)div128(t3 - Da, wab);
     }
     return r;
 }
