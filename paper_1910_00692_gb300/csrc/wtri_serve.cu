@@ -35,7 +35,12 @@
 namespace wtri {
 namespace {
 
-constexpr int WORKER_STREAMS = 4;
+// Micro-batches in flight: one on the device, one queued behind it.  A batch
+// holds the whole GPU (its kernel is one cooperative launch), so more would
+// only take requests out of the queue that can share a query with those
+// still to come: with four a burst of 512 requests went out as 10 batches and
+// took 6.3 ms.
+constexpr int WORKER_STREAMS = 2;
 constexpr int MAX_BATCH = 256;
 constexpr size_t BATCH_FIXED_BYTES = (size_t(1) << 18) * 40 + (1u << 16);  // a batch's items + slack
 
