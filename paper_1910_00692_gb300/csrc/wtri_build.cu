@@ -408,25 +408,29 @@ int sort_rows(const rows::RowsOut& R, unsigned long long* g0, unsigned long long
     const int sms = sm_count();
     {
         ProfScope ps("rows_sort_small", s, 0.0, 3);
-        rows::k_rows_small<8><<<sms * 8, rows::NT, 0, s>>>(R, rows::CLS_G8, gate);
-        rows::k_rows_small<16><<<sms * 8, rows::NT, 0, s>>>(R, rows::CLS_G16, gate);
-        rows::k_rows_small<32><<<sms * 8, rows::NT, 0, s>>>(R, rows::CLS_G32, gate);
+        auto launch = [&](auto packed, auto wide, int bits, int cls) {
+            // 32-bit keys where the id and the lane fit (nbits: of an id)
+            (nbits + bits <= 32 ? packed : wide)<<<sms * 8, rows::NT, 0, s>>>(R, cls, gate);
+        };
+        launch(rows::k_rows_small<8, true>, rows::k_rows_small<8, false>, 3, rows::CLS_G8);
+        launch(rows::k_rows_small<16, true>, rows::k_rows_small<16, false>, 4, rows::CLS_G16);
+        launch(rows::k_rows_small<32, true>, rows::k_rows_small<32, false>, 5, rows::CLS_G32);
     }
     {
         ProfScope ps("rows_sort_warp", s, 0.0, 4);
-        auto launch = [&](auto kern, int epl, int cls) -> int {
-            static std::atomic<uint64_t> done[6];
-            const int smem = rows::NWARPS * 32 * epl * 16;  // keys + weights + ranks
-            int slot = 0;
-            for (int e = epl; e > 2; e >>= 1) slot++;
-            WTRI_TRY(smem_optin((const void*)kern, smem, done[slot]));
+        static std::atomic<uint64_t> done[4][2];
+        auto launch = [&](auto packed, auto ids, int bits, int cls) -> int {
+            const int smem = rows::NWARPS * (1 << bits) * rows::WARP_ENTRY_BYTES;
+            const bool pack = nbits + bits <= 32;
+            auto kern = pack ? packed : ids;
+            WTRI_TRY(smem_optin((const void*)kern, smem, done[bits - 6][pack]));
             kern<<<sms * 4, rows::NT, smem, s>>>(R, cls, gate);
             return WTRI_OK;
         };
-        WTRI_TRY(launch(rows::k_rows_warp<2>, 2, rows::CLS_W2));
-        WTRI_TRY(launch(rows::k_rows_warp<4>, 4, rows::CLS_W4));
-        WTRI_TRY(launch(rows::k_rows_warp<8>, 8, rows::CLS_W8));
-        WTRI_TRY(launch(rows::k_rows_warp<16>, 16, rows::CLS_W16));
+        WTRI_TRY(launch(rows::k_rows_warp<2, true>, rows::k_rows_warp<2, false>, 6, rows::CLS_W2));
+        WTRI_TRY(launch(rows::k_rows_warp<4, true>, rows::k_rows_warp<4, false>, 7, rows::CLS_W4));
+        WTRI_TRY(launch(rows::k_rows_warp<8, true>, rows::k_rows_warp<8, false>, 8, rows::CLS_W8));
+        WTRI_TRY(launch(rows::k_rows_warp<16, true>, rows::k_rows_warp<16, false>, 9, rows::CLS_W16));
     }
     {
         ProfScope ps("rows_sort_block", s, 0.0, 1);

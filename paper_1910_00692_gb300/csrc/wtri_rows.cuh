@@ -15,12 +15,16 @@
 // forward entry's key (id << 32 | position in the weight-sorted row) into
 // the first odeg[x] slots of its row's range in scratch (unordered: one
 // atomic per row and warp).  A scan of odeg gives orowptr.  Rows are then
-// sorted by their oriented degree d, on 64-bit keys (id << 32 | index of the
-// key among the row's packed keys), unique within a row:
+// sorted by their oriented degree d, on the id and the index of the key among
+// the row's packed keys (unique within a row):
 //   d <= 32           sub-warp bitonic network in registers (groups of 8, 16
 //                     or 32 lanes, several rows per warp);
 //   32 < d <= 512     one warp per row: bitonic network over 2..16 keys per
 //                     lane in registers, transposed through shared memory;
+// both on 32-bit keys, id and index together, where they fit (a shuffle and
+// a minimum or maximum per exchange; on 64-bit keys, five instructions), else
+// d <= 32 on 64-bit keys and 32 < d on the ids alone, each entry's place then
+// found by a search of the sorted ids;
 //   512 < d           one block per row: stable LSD radix sort of the ids in
 //                     shared memory (digits of at most 9 bits, ranked by warp
 //                     ballots), slices of at most SR keys; rows above SR
@@ -329,9 +333,35 @@ __device__ __forceinline__ void gather_wr(const RowsOut& R, int64_t s, unsigned 
 // ---------------------------------------------------------------------------
 constexpr int SMALL_U = 4;  // rows per lane group and iteration (their loads issued together)
 
+// The sort key of a small row's entry: id and lane of the group.  PACK: in 32
+// bits (the id shifted by log2 G).  Padding is all ones: a real key equals it
+// only at the last lane of a full row, which has no padding.
+template <int G, bool PACK>
+struct SmallKey;
 template <int G>
+struct SmallKey<G, true> {
+    typedef uint32_t T;
+    static constexpr T NONE = ~0u;
+    static __device__ __forceinline__ T make(int32_t c, int gl) { return (uint32_t)c * G + (uint32_t)gl; }
+    static __device__ __forceinline__ int32_t col(T k) { return (int32_t)(k / G); }
+    static __device__ __forceinline__ int src(T k) { return (int)(k & (G - 1)); }
+};
+template <int G>
+struct SmallKey<G, false> {
+    typedef unsigned long long T;
+    static constexpr T NONE = ~0ull;
+    static __device__ __forceinline__ T make(int32_t c, int gl) {
+        return ((unsigned long long)(uint32_t)c << 32) | (uint32_t)gl;
+    }
+    static __device__ __forceinline__ int32_t col(T k) { return (int32_t)(k >> 32); }
+    static __device__ __forceinline__ int src(T k) { return (int)(k & (G - 1)); }
+};
+
+template <int G, bool PACK>
 __global__ void __launch_bounds__(NT) k_rows_small(RowsOut R, int cls, const uint32_t* gate) {
     if (rows_gate_closed(gate)) return;
+    typedef SmallKey<G, PACK> K;
+    typedef typename K::T T;
     const int lane = threadIdx.x & 31, gl = lane & (G - 1), grp = lane / G;
     constexpr int RPW = 32 / G;  // rows per warp and unrolled step
     const int64_t lo = R.cls_off[cls], hi = R.cls_off[cls + 1];
@@ -356,41 +386,43 @@ __global__ void __launch_bounds__(NT) k_rows_small(RowsOut R, int cls, const uin
                 ob[u] = __ldg(R.orowptr + x[u]);
             }
         }
-        unsigned long long key[SMALL_U];
+        unsigned long long pk[SMALL_U];
 #pragma unroll
-        for (int u = 0; u < SMALL_U; u++) key[u] = gl < d[u] ? __ldcs(R.pk + s[u] + gl) : KEY_NONE;
+        for (int u = 0; u < SMALL_U; u++) pk[u] = gl < d[u] ? __ldcs(R.pk + s[u] + gl) : KEY_NONE;
+        T key[SMALL_U];
         int32_t w[SMALL_U], rk[SMALL_U];
 #pragma unroll
         for (int u = 0; u < SMALL_U; u++) {
             w[u] = 0;
             rk[u] = 0;
+            key[u] = K::NONE;
             if (gl < d[u]) {
-                gather_wr(R, s[u], key[u], w[u], rk[u]);
-                key[u] = with_pos(key[u], gl);
+                gather_wr(R, s[u], pk[u], w[u], rk[u]);
+                key[u] = K::make(key_col(pk[u]), gl);
             }
         }
 #pragma unroll
         for (int k = 2; k <= G; k <<= 1) {
 #pragma unroll
             for (int j = k >> 1; j > 0; j >>= 1) {
-                const bool up = (gl & k) == 0, lower = (gl & j) == 0;
+                const bool least = ((gl & k) == 0) == ((gl & j) == 0);
 #pragma unroll
                 for (int u = 0; u < SMALL_U; u++) {
-                    const unsigned long long ok = __shfl_xor_sync(0xffffffffu, key[u], j, G);
-                    key[u] = (lower == up) ? (ok < key[u] ? ok : key[u]) : (ok > key[u] ? ok : key[u]);
+                    const T o = __shfl_xor_sync(0xffffffffu, key[u], j, G);
+                    key[u] = least ? min(o, key[u]) : max(o, key[u]);
                 }
             }
         }
 #pragma unroll
         for (int u = 0; u < SMALL_U; u++) {
-            const int src = (int)key_pos(key[u]) & (G - 1);
+            const int src = K::src(key[u]);
             const int32_t ws = __shfl_sync(0xffffffffu, w[u], src, G);
             const int32_t rks = __shfl_sync(0xffffffffu, rk[u], src, G);
-            const unsigned long long prev = __shfl_up_sync(0xffffffffu, key[u], 1, G);
+            const T prev = __shfl_up_sync(0xffffffffu, key[u], 1, G);
             if (gl < d[u]) {
-                const int32_t c = key_col(key[u]);
+                const int32_t c = K::col(key[u]);
                 write_orient(R, ob[u] + gl, c, ws, rks);
-                if (gl > 0 && key_col(prev) == c) flag_dup(R, x[u], c);
+                if (gl > 0 && K::col(prev) == c) flag_dup(R, x[u], c);
             }
         }
     }
@@ -400,34 +432,35 @@ __global__ void __launch_bounds__(NT) k_rows_small(RowsOut R, int cls, const uin
 // Bitonic network over the 32 * EPL keys of a warp, in registers: key i of
 // lane l is element l * EPL + i.  Stages with a partner distance below EPL
 // stay inside a lane; the others exchange with lane l ^ (distance / EPL).
-// Sorts ascending; keys must be distinct (KEY_NONE padding may repeat).
+// Sorts ascending.  Blocks that a merge sorts downwards hold their keys
+// complemented meanwhile, so every exchange is a plain minimum and maximum.
 // ---------------------------------------------------------------------------
-// Intra-lane compare-exchange stage at partner distance J (< EPL) of a
-// bitonic merge of blocks of `size` elements.
 template <int EPL, int J>
-__device__ __forceinline__ void bitonic_intra(unsigned long long (&k)[EPL], int lane, int size) {
+__device__ __forceinline__ void bitonic_intra(uint32_t (&k)[EPL]) {
 #pragma unroll
     for (int i = 0; i < EPL; i++) {
         const int p = i ^ J;
         if (p > i) {
-            const bool up = ((lane * EPL + i) & size) == 0;
-            const unsigned long long a = k[i], b = k[p];
-            if ((a > b) == up) {
-                k[i] = b;
-                k[p] = a;
-            }
+            const uint32_t a = min(k[i], k[p]), b = max(k[i], k[p]);
+            k[i] = a;
+            k[p] = b;
         }
     }
 }
 
 template <int EPL>
-__device__ __forceinline__ void warp_bitonic(unsigned long long (&k)[EPL]) {
-    // The stage loops stay rolled (a fully unrolled network of 32 keys per
-    // lane is tens of thousands of instructions, far beyond the instruction
-    // cache); the element loops are unrolled, so registers stay registers.
+__device__ __forceinline__ void warp_bitonic(uint32_t (&k)[EPL]) {
+    // The stage loops stay rolled (the unrolled network is far beyond the
+    // instruction cache); the element loops are unrolled, so registers stay
+    // registers.
     const int lane = threadIdx.x & 31;
 #pragma unroll 1
     for (int size = 2; size <= 32 * EPL; size <<= 1) {
+#pragma unroll
+        for (int i = 0; i < EPL; i++) {
+            const int e = lane * EPL + i;
+            if (((e & size) != 0) != (size > 2 && (e & (size >> 1)) != 0)) k[i] = ~k[i];
+        }
 #pragma unroll 1
         for (int j = size >> 1; j > 0; j >>= 1) {
             if (j >= EPL) {
@@ -435,18 +468,15 @@ __device__ __forceinline__ void warp_bitonic(unsigned long long (&k)[EPL]) {
                 const bool lower = (lane & lm) == 0;
 #pragma unroll
                 for (int i = 0; i < EPL; i++) {
-                    const unsigned long long o = __shfl_xor_sync(0xffffffffu, k[i], lm);
-                    const bool up = ((lane * EPL + i) & size) == 0;
-                    const bool keep_min = lower == up;
-                    k[i] = keep_min ? (o < k[i] ? o : k[i]) : (o > k[i] ? o : k[i]);
+                    const uint32_t o = __shfl_xor_sync(0xffffffffu, k[i], lm);
+                    k[i] = lower ? min(k[i], o) : max(k[i], o);
                 }
             } else {
                 switch (j) {
-                    case 16: if constexpr (EPL > 16) bitonic_intra<EPL, 16>(k, lane, size); break;
-                    case 8: if constexpr (EPL > 8) bitonic_intra<EPL, 8>(k, lane, size); break;
-                    case 4: if constexpr (EPL > 4) bitonic_intra<EPL, 4>(k, lane, size); break;
-                    case 2: if constexpr (EPL > 2) bitonic_intra<EPL, 2>(k, lane, size); break;
-                    default: if constexpr (EPL > 1) bitonic_intra<EPL, 1>(k, lane, size); break;
+                    case 8: if constexpr (EPL > 8) bitonic_intra<EPL, 8>(k); break;
+                    case 4: if constexpr (EPL > 4) bitonic_intra<EPL, 4>(k); break;
+                    case 2: if constexpr (EPL > 2) bitonic_intra<EPL, 2>(k); break;
+                    default: if constexpr (EPL > 1) bitonic_intra<EPL, 1>(k); break;
                 }
             }
         }
@@ -460,16 +490,21 @@ __device__ __forceinline__ int swz(int p) { return p ^ ((p >> 5) & 31); }
 // ---------------------------------------------------------------------------
 // Rows of 33..512 entries: one warp per row, 32 * EPL keys in registers
 // (EPL = 2, 4, 8, 16 by class), sorted, transposed through the warp's
-// shared memory (keys, and the row's weights and ranks by packed index).
+// shared memory.  PACK: the key is the id and the entry's packed index, which
+// finds its weight and rank.  Otherwise the ids are sorted alone, and each
+// entry searches its id among them and leaves its weight and rank there.
 // ---------------------------------------------------------------------------
-template <int EPL>
+constexpr int WARP_ENTRY_BYTES = 12;  // shared memory per entry: key, weight, rank
+
+template <int EPL, bool PACK>
 __global__ void __launch_bounds__(NT) k_rows_warp(RowsOut R, int cls, const uint32_t* gate) {
     if (rows_gate_closed(gate)) return;
-    extern __shared__ __align__(16) unsigned long long wsm[];
+    extern __shared__ __align__(16) uint32_t wsm[];
+    constexpr int N = 32 * EPL;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    unsigned long long* run = wsm + (size_t)wid * 2 * 32 * EPL;
-    int32_t* wv = reinterpret_cast<int32_t*>(run + 32 * EPL);  // weights by packed index
-    int32_t* rv = wv + 32 * EPL;                                 // ranks by packed index
+    uint32_t* run = wsm + (size_t)wid * 3 * N;
+    int32_t* wv = reinterpret_cast<int32_t*>(run + N);  // weights, by packed index (PACK) or place
+    int32_t* rv = wv + N;                               // ranks
     const int64_t lo = R.cls_off[cls], hi = R.cls_off[cls + 1];
     const int64_t nwarps = ((int64_t)gridDim.x * NT) >> 5;
     for (int64_t ri = lo + (((int64_t)blockIdx.x * NT + threadIdx.x) >> 5); ri < hi; ri += nwarps) {
@@ -477,28 +512,45 @@ __global__ void __launch_bounds__(NT) k_rows_warp(RowsOut R, int cls, const uint
         const int64_t s = __ldg(R.rowptr + x);
         const int d = __ldg(R.odeg + x);
         const int64_t ob = __ldg(R.orowptr + x);
-        unsigned long long k[EPL];
+        uint32_t k[EPL];
 #pragma unroll
         for (int i = 0; i < EPL; i++) {
             const int j = i * 32 + lane;  // coalesced loads; the network ignores input order
+            k[i] = ~0u;  // padding: a packed key equals it only in a full row
             if (j < d) {
-                const unsigned long long kk = __ldcs(R.pk + s + j);
-                gather_wr(R, s, kk, wv[j], rv[j]);
-                k[i] = with_pos(kk, j);
-            } else {
-                k[i] = KEY_NONE;
+                const unsigned long long kk = __ldg(R.pk + s + j);
+                k[i] = PACK ? (uint32_t)key_col(kk) * N + (uint32_t)j : (uint32_t)key_col(kk);
+                if (PACK) gather_wr(R, s, kk, wv[j], rv[j]);
             }
         }
         warp_bitonic<EPL>(k);
 #pragma unroll
         for (int i = 0; i < EPL; i++) run[swz(lane * EPL + i)] = k[i];
         __syncwarp();
+        if (!PACK) {
+#pragma unroll 4
+            for (int j = lane; j < d; j += 32) {  // (the keys again, from cache: not held across the network)
+                const unsigned long long kk = __ldg(R.pk + s + j);
+                int32_t w, rk;
+                gather_wr(R, s, kk, w, rk);
+                int p = 0;  // places below its id
+#pragma unroll
+                for (int h = N / 2; h > 0; h >>= 1)
+                    if (run[swz(p + h - 1)] < (uint32_t)key_col(kk)) p += h;
+                wv[p] = w;
+                rv[p] = rk;
+            }
+            __syncwarp();
+        }
         for (int j = lane; j < d; j += 32) {
-            const unsigned long long kk = run[swz(j)];
-            const int32_t c = key_col(kk);
-            const uint32_t src = key_pos(kk);
+            const uint32_t kk = run[swz(j)];
+            const int32_t c = (int32_t)(PACK ? kk / N : kk);
+            const int src = PACK ? (int)(kk & (N - 1)) : j;
             write_orient(R, ob + j, c, wv[src], rv[src]);
-            if (j > 0 && key_col(run[swz(j - 1)]) == c) flag_dup(R, x, c);
+            if (j > 0) {
+                const uint32_t pv = run[swz(j - 1)];
+                if ((int32_t)(PACK ? pv / N : pv) == c) flag_dup(R, x, c);
+            }
         }
         __syncwarp();
     }
