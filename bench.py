@@ -626,7 +626,7 @@ def prof_table(L):
 
 # Kernel families the phase timers name, by the kernels they launch.
 KERNEL_OF = {"radix_downsweep": "radix::k_scatter", "radix_upsweep": "radix::k_upsweep",
-             "radix_digit_scan": "radix::k_digit_scan",
+             "radix_digit_scan": "radix::k_col_scan",
              "rows_sort": "rows::k_rows_small/k_rows_warp/k_rows_block (per-row sort by id)"}
 
 

@@ -211,6 +211,12 @@ struct EdgeLoader {
     const int32_t* v;
     const int32_t* w;
     __device__ __forceinline__ uint32_t key(int64_t i) const { return ~(uint32_t)__ldg(w + i); }
+    __device__ __forceinline__ void keys8(int64_t i, uint32_t (&k)[8]) const {
+        const uint4* p = reinterpret_cast<const uint4*>(w + i);
+        const uint4 a = __ldg(p), b = __ldg(p + 1);
+        k[0] = ~a.x, k[1] = ~a.y, k[2] = ~a.z, k[3] = ~a.w;
+        k[4] = ~b.x, k[5] = ~b.y, k[6] = ~b.z, k[7] = ~b.w;
+    }
     __device__ __forceinline__ const void* tile_src(int a, int64_t tbase) const {
         return (a == 0 ? w : (a == 1 ? u : v)) + tbase;
     }
@@ -268,11 +274,18 @@ struct OrderEntryLoader {
     __device__ __forceinline__ uint32_t key(int64_t i) const {
         return (uint32_t)__ldg(((i & 1) ? ov : ou) + (i >> 1));
     }
+    __device__ __forceinline__ void keys8(int64_t i, uint32_t (&k)[8]) const {
+        const uint4 a = __ldg(reinterpret_cast<const uint4*>(ou + (i >> 1)));
+        const uint4 b = __ldg(reinterpret_cast<const uint4*>(ov + (i >> 1)));
+        k[0] = a.x, k[1] = b.x, k[2] = a.y, k[3] = b.y;
+        k[4] = a.z, k[5] = b.z, k[6] = a.w, k[7] = b.w;
+    }
     bool tma_ok() const { return (((uintptr_t)ou | (uintptr_t)ov | (uintptr_t)ow) & 15) == 0; }
 };
 
 // Final row-sorted output: row, col, weight, r.
 struct RowsStorer {
+    static constexpr int STREAMS = 4;
     __host__ __device__ double rec_bytes() const { return 16.0; }
     int32_t* row;
     int32_t* col;

@@ -17,6 +17,7 @@
 //           uint4 srec(const uint32_t* in, int li, int64_t tbase)
 //           uint4 grec(int64_t i)       from global memory
 //           uint32_t key(int64_t i)     (first-pass histogram)
+//           void keys8(int64_t i, uint32_t (&k)[8])   keys i .. i + 7 (i a multiple of 8, sources aligned)
 //           bool tma_ok()               sources 16-byte aligned
 //   Storer: void store(int64_t p, const uint4& rec); double rec_bytes();
 //           void prepare()          once per CTA before the first store
@@ -29,11 +30,12 @@
 // only known on the device launch the widest plan and skip the passes it
 // does not need.
 //
-// Three kernels per pass: per-chunk digit histograms (upsweep), a per-digit
-// scan over chunks, and the scatter.  The scatter streams its chunk tile by
-// tile; the next tile's sources arrive by bulk asynchronous copies
-// (cp.async.bulk, one mbarrier per buffer) while the current one is ranked
-// (ballots over the digit's bits give a strip's equal digits, per-warp
+// Per pass: digit histograms of the rows of a count table (upsweep), a scan
+// of the table's columns, and the scatter.  A CTA of the scatter streams its
+// share of the records tile by tile (or, see spread_pass, takes every
+// gridDim-th tile); the next tile's sources arrive by bulk asynchronous
+// copies (cp.async.bulk, one mbarrier per buffer) while the current one is
+// ranked (ballots over the digit's bits give a strip's equal digits, per-warp
 // counters the ones before; stable).  The ranks give each place of the
 // digit order its record's place in the tile (2 bytes); the records
 // themselves stay where the copy put them, are read once, in digit order,
@@ -41,15 +43,24 @@
 // one digit's run.
 //
 // What bounds the scatter: the runs (TT / bins records) begin and end inside
-// lines, and the time follows the write requests that reach L2, 59 per ns
-// (9-bit digits: 37 million for 62 million records, 2/5 of them for the
+// lines, and the time follows the write requests that reach L2, about 59 per
+// ns (9-bit digits: 37 million for 62 million records, 2/5 of them for the
 // digits), while DRAM is 45 % busy.  So one CTA per SM with the largest tile
-// that shared memory holds twice: with two CTAs of half the tile the phases
-// overlap (ranking on votes and arithmetic, writing on shared memory), yet
-// the 1e9-edge build's scatters take 86.9 ms instead of 68.9.  Keeping the
-// records in place instead of staging them (and with the ballots, which left
-// the registers they need) allowed 5,632 records a tile instead of 5,376:
-// 71.3 -> 68.9 ms.
+// that shared memory holds twice.  Overlapping a CTA's phases gains nothing:
+// two CTAs of 5,120 records without a second buffer take 77.0 ms where this
+// takes 69.9 (the 1e9-edge build's scatters), of 2,688 with one 86.9.  One
+// bulk copy per run from a tile staged in digit order: 66.3 without the
+// digits, plain stores 60.7 (and histograms that read the records instead
+// take back 10 ms).  Keeping the records in place instead of staging them
+// (and with the ballots, which left the registers they need) allowed 5,632
+// records a tile instead of 5,376: 71.3 -> 68.9 ms.
+//
+// One table for all: rows x bins, a row's counts written once by the block
+// that counts it (no clearing, no global atomics) and scanned by 128 threads
+// per column.  With counts per (digit, share) that eight blocks added into and
+// one block per digit scanned, a 20,000-edge build took 515 us, now 465; 1e6
+// edges 780, now 705; a 2e7-edge build 2.79 ms, now 2.51 (most of it the last
+// pass's spread tiles).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -79,8 +90,13 @@ constexpr int TT = NT * IT;                // records per tile
 constexpr int CTAS_PER_SM = WTRI_RADIX_CTAS;
 constexpr int NBUF = 2;                    // tile buffers of a scatter CTA
 constexpr int DPT = MAX_BINS / NT;         // digits owned by a thread in the tile scan
-constexpr int MIN_CHUNK = 1024;            // records
-constexpr int UP_SPLIT = 8;                // histogram blocks per chunk
+constexpr int MIN_SHARE = 1024;            // records
+constexpr int MIN_ROW = 2048;              // records, where a share has several rows
+constexpr int UP_SPLIT = 12;               // most table rows of a CTA's share (two full waves of the histogram's blocks)
+constexpr int64_t OPEN_BYTES = int64_t(64) << 20;  // lines that L2 keeps open for the runs (half of it)
+constexpr int SPREAD_TILES = 16;           // fewest tiles per CTA of a spread pass
+constexpr int SCAN_ROWS = 2048;            // most rows that one launch scans
+constexpr int SCAN_X = 8, SCAN_Y = 128;    // columns and row shares of a scan block
 constexpr int UNT = 256;                   // threads of a histogram block
 constexpr int UNW = UNT / 32;
 constexpr uint32_t WAIT_LIMIT = 1u << 24;  // bounded mbarrier polling
@@ -126,8 +142,10 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t x, uint32_t* w
 
 struct PassGeom {
     int64_t n;        // records
-    int64_t chunk;    // records per chunk
-    int chunks;       // G
+    int64_t share;    // records that a CTA takes at a time
+    int64_t row;      // records per row of the count table
+    int split;        // rows per share (the last may be shorter, or empty)
+    int64_t rows;
     int shift;
     int bins;         // 1 << digit bits
     int bits;
@@ -154,46 +172,54 @@ struct KeyDigits {  // first pass: the loader's keys
     Loader ld;
     int shift;
     uint32_t mask;
+    bool vec;  // the sources are 16-byte aligned
     __device__ __forceinline__ uint32_t digit(int64_t i) const { return (ld.key(i) >> shift) & mask; }
+    __device__ __forceinline__ void digits8(int64_t i, uint32_t (&d)[8]) const {
+        ld.keys8(i, d);
+#pragma unroll
+        for (int k = 0; k < 8; k++) d[k] = (d[k] >> shift) & mask;
+    }
 };
 struct StoredDigits {  // later passes: 16-bit digits written by the previous scatter
     static constexpr bool PACKED = true;
+    static constexpr bool vec = true;
     const uint16_t* d;
     __device__ __forceinline__ uint32_t digit(int64_t i) const { return __ldg(d + i); }
+    __device__ __forceinline__ void digits8(int64_t i, uint32_t (&x)[8]) const {
+        const uint4 r = __ldg(reinterpret_cast<const uint4*>(d + i));
+        x[0] = r.x & 0xffffu, x[1] = r.x >> 16, x[2] = r.y & 0xffffu, x[3] = r.y >> 16;
+        x[4] = r.z & 0xffffu, x[5] = r.z >> 16, x[6] = r.w & 0xffffu, x[7] = r.w >> 16;
+    }
 };
 
-// Digit histogram of each chunk.  UP_SPLIT blocks share a chunk (each a
-// slice of it, a multiple of 8 records) and add their counts into the
-// zeroed per-chunk histogram; each warp counts into its own shared copy.
-// Stored digits are read eight at a time (one 16-byte load).
+// Digit histograms of equal shares: row r of the table counts part r % split
+// of share r / split.  Each warp of a block counts into its own shared copy.
+// Eight digits per thread and step: one 16-byte load of stored digits, two of
+// sources.  1e9 and 2e9 keys take 710 and 1,580 us, 2e9 stored digits 830-900
+// (with counts added into one row per share: 640, 1,430 and 850-930); with
+// one key per load 730 and 1,650.
 template <class Dig>
-__global__ void __launch_bounds__(UNT) k_upsweep(Dig dg, PassGeom g, uint32_t* counts) {
+__global__ void __launch_bounds__(UNT) k_upsweep(Dig dg, PassGeom g, uint32_t* table) {
     if (pass_closed(g)) return;
     __shared__ uint32_t hist[UNW][MAX_BINS];
     const int w = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < UNW * MAX_BINS; i += UNT) (&hist[0][0])[i] = 0;
     __syncthreads();
     uint32_t* h = hist[w];
-    const int chunk = blockIdx.x / UP_SPLIT, part = blockIdx.x % UP_SPLIT;
-    const int64_t cbeg = (int64_t)chunk * g.chunk;
-    const int64_t cend = min(g.n, cbeg + g.chunk);
-    const int64_t slice = ((g.chunk + UP_SPLIT - 1) / UP_SPLIT + 7) & ~int64_t(7);
-    const int64_t beg = min(cend, cbeg + part * slice);
-    const int64_t end = min(cend, beg + slice);
+    const int share = blockIdx.x / g.split, part = blockIdx.x % g.split;
+    const int64_t sbeg = (int64_t)share * g.share;
+    const int64_t send = min(g.n, sbeg + g.share);
+    const int64_t beg = min(send, sbeg + part * g.row);
+    const int64_t end = min(send, beg + g.row);
     int64_t i0 = beg;
-    if constexpr (Dig::PACKED) {
+    if (dg.vec) {
         const int64_t nv = (end - beg) >> 3;  // whole groups of 8 (beg is a multiple of 8)
-        const uint4* v = reinterpret_cast<const uint4*>(dg.d + beg);
+#pragma unroll 2
         for (int64_t q = threadIdx.x; q < nv; q += UNT) {
-            const uint4 x = __ldg(v + q);
-            atomicAdd(&h[x.x & 0xffffu], 1u);
-            atomicAdd(&h[x.x >> 16], 1u);
-            atomicAdd(&h[x.y & 0xffffu], 1u);
-            atomicAdd(&h[x.y >> 16], 1u);
-            atomicAdd(&h[x.z & 0xffffu], 1u);
-            atomicAdd(&h[x.z >> 16], 1u);
-            atomicAdd(&h[x.w & 0xffffu], 1u);
-            atomicAdd(&h[x.w >> 16], 1u);
+            uint32_t d[8];
+            dg.digits8(beg + (q << 3), d);
+#pragma unroll
+            for (int k = 0; k < 8; k++) atomicAdd(&h[d[k]], 1u);
         }
         i0 = beg + (nv << 3);
     } else {
@@ -212,26 +238,128 @@ __global__ void __launch_bounds__(UNT) k_upsweep(Dig dg, PassGeom g, uint32_t* c
         uint32_t s = 0;
 #pragma unroll
         for (int k = 0; k < UNW; k++) s += hist[k][d];
-        if (s) atomicAdd(&counts[(int64_t)d * g.chunks + chunk], s);
+        table[(int64_t)blockIdx.x * g.bins + d] = s;
     }
 }
 
-// Block d: exclusive scan of counts[d][0..G) in place; totals[d] = sum.
-__global__ void __launch_bounds__(NT) k_digit_scan(uint32_t* counts, int chunks, uint32_t* totals,
+// The same where a share is one tile (a row each): a block takes every
+// gridDim-th tile.
+__global__ void __launch_bounds__(UNT) k_upsweep_tiles(const uint16_t* __restrict__ dig, PassGeom g, uint32_t* table) {
+    if (pass_closed(g)) return;
+    __shared__ uint32_t hist[UNW][MAX_BINS];
+    for (int i = threadIdx.x; i < UNW * MAX_BINS; i += UNT) (&hist[0][0])[i] = 0;
+    __syncthreads();
+    uint32_t* h = hist[threadIdx.x >> 5];
+    const StoredDigits dg{dig};
+    for (int64_t r = blockIdx.x; r < g.rows; r += gridDim.x) {
+        const int64_t beg = r * g.share, end = min(g.n, beg + g.share), nv = (end - beg) >> 3;
+        for (int64_t q = threadIdx.x; q < nv; q += UNT) {
+            uint32_t d[8];
+            dg.digits8(beg + (q << 3), d);
+#pragma unroll
+            for (int k = 0; k < 8; k++) atomicAdd(&h[d[k]], 1u);
+        }
+        for (int64_t i = beg + (nv << 3) + threadIdx.x; i < end; i += UNT) atomicAdd(&h[__ldg(dig + i)], 1u);
+        __syncthreads();
+        for (int d = threadIdx.x; d < g.bins; d += UNT) {
+            uint32_t s = 0;
+#pragma unroll
+            for (int k = 0; k < UNW; k++) {
+                s += hist[k][d];
+                hist[k][d] = 0;
+            }
+            table[r * g.bins + d] = s;
+        }
+        __syncthreads();
+    }
+}
+
+// Exclusive scan of the table's columns (rows x bins), in place; totals[d] =
+// column d's sum.  Up to SCAN_ROWS rows: k_col_scan alone.  More: in segments
+// of rows, whose sums k_seg_sum writes, k_col_scan scans and k_seg_apply
+// spreads over their rows.
+__global__ void __launch_bounds__(SCAN_X * SCAN_Y) k_col_scan(uint32_t* table, int64_t rows, uint32_t* totals,
+                                                              PassGeom g) {
+    if (pass_closed(g)) return;
+    __shared__ uint32_t part[SCAN_X][SCAN_Y + 1];
+    const int x = threadIdx.x % SCAN_X, y = threadIdx.x / SCAN_X, d = blockIdx.x * SCAN_X + x;
+    const int64_t per = (rows + SCAN_Y - 1) / SCAN_Y, beg = min(rows, y * per), end = min(rows, beg + per);
+    uint32_t s = 0;
+    if (d < g.bins) {
+#pragma unroll 8
+        for (int64_t r = beg; r < end; r++) s += table[r * g.bins + d];
+    }
+    part[x][y] = s;
+    __syncthreads();
+    const int lane = threadIdx.x & 31, c = threadIdx.x >> 5;
+    if (c < SCAN_X) {  // a warp per column
+        constexpr int PER = SCAN_Y / 32;
+        uint32_t v[PER], sum = 0;
+#pragma unroll
+        for (int i = 0; i < PER; i++) {
+            v[i] = part[c][lane * PER + i];
+            sum += v[i];
+        }
+        uint32_t inc = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t z = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += z;
+        }
+        uint32_t run = inc - sum;
+#pragma unroll
+        for (int i = 0; i < PER; i++) {
+            part[c][lane * PER + i] = run;
+            run += v[i];
+        }
+        if (lane == 31 && blockIdx.x * SCAN_X + c < g.bins) totals[blockIdx.x * SCAN_X + c] = run;
+    }
+    __syncthreads();
+    if (d >= g.bins) return;
+    uint32_t run = part[x][y];
+    constexpr int U = 8;
+    for (int64_t r0 = beg; r0 < end; r0 += U) {
+        uint32_t v[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) v[u] = r0 + u < end ? table[(r0 + u) * g.bins + d] : 0u;
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            if (r0 + u < end) table[(r0 + u) * g.bins + d] = run;
+            run += v[u];
+        }
+    }
+}
+
+__global__ void __launch_bounds__(UNT) k_seg_sum(const uint32_t* __restrict__ table, int seg,
+                                                 uint32_t* __restrict__ sums, PassGeom g) {
+    if (pass_closed(g)) return;
+    const int d = blockIdx.y * UNT + threadIdx.x;
+    if (d >= g.bins) return;
+    const int64_t beg = (int64_t)blockIdx.x * seg, end = min(g.rows, beg + seg);
+    uint32_t s = 0;
+#pragma unroll 8
+    for (int64_t r = beg; r < end; r++) s += __ldg(table + r * g.bins + d);
+    sums[(int64_t)blockIdx.x * g.bins + d] = s;
+}
+
+__global__ void __launch_bounds__(UNT) k_seg_apply(uint32_t* table, int seg, const uint32_t* __restrict__ sums,
                                                    PassGeom g) {
     if (pass_closed(g)) return;
-    __shared__ uint32_t warp_tot[NW];
-    __shared__ uint32_t tot;
-    uint32_t* c = counts + (int64_t)blockIdx.x * chunks;
-    uint32_t carry = 0;
-    for (int base = 0; base < chunks; base += NT) {
-        int i = base + threadIdx.x;
-        uint32_t x = i < chunks ? c[i] : 0;
-        uint32_t ex = block_exclusive_scan<NT>(x, warp_tot, &tot);
-        if (i < chunks) c[i] = carry + ex;
-        carry += tot;
+    const int d = blockIdx.y * UNT + threadIdx.x;
+    if (d >= g.bins) return;
+    const int64_t beg = (int64_t)blockIdx.x * seg, end = min(g.rows, beg + seg);
+    uint32_t run = sums[(int64_t)blockIdx.x * g.bins + d];
+    constexpr int U = 8;
+    for (int64_t r0 = beg; r0 < end; r0 += U) {
+        uint32_t v[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) v[u] = r0 + u < end ? table[(r0 + u) * g.bins + d] : 0u;
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            if (r0 + u < end) table[(r0 + u) * g.bins + d] = run;
+            run += v[u];
+        }
     }
-    if (threadIdx.x == 0) totals[blockIdx.x] = carry;
 }
 
 // ---- scatter -----------------------------------------------------------------
@@ -365,10 +493,12 @@ __device__ __forceinline__ void rank_strips(uint32_t (&rk)[IT], int strips, int 
 // Ranks and writes one tile of tcount <= TT records.  key(li), rec(li): the
 // tile's records, in shared memory.  On entry the counters are zero and the
 // tile visible to every thread.  run[] holds this thread's digits' next
-// output positions (digits threadIdx.x * DPT + i).
-template <bool FULL, class Key, class Rec, class Storer>
+// output positions (digits threadIdx.x * DPT + i); FRESH: they are base[] +
+// first[] (loads that may still be in flight on entry).
+template <bool FULL, bool FRESH, class Key, class Rec, class Storer>
 __device__ __forceinline__ void scatter_tile(const Key& key, const Rec& rec, int tcount, const Storer& st,
-                                             const PassGeom& g, uint32_t (&run)[DPT], ScatterSmem& S) {
+                                             const PassGeom& g, uint32_t (&run)[DPT], const uint32_t (&base)[DPT],
+                                             const uint32_t (&first)[DPT], ScatterSmem& S) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int strips = FULL ? IT : (tcount + NT - 1) / NT;
     // 1. rank within the warp
@@ -420,6 +550,7 @@ __device__ __forceinline__ void scatter_tile(const Key& key, const Rec& rec, int
             for (int i = 1; i < DPT; i++) s[i] = s[i - 1] + tot[i - 1];
 #pragma unroll
             for (int i = 0; i < DPT; i++) {
+                if (FRESH) run[i] = base[i] + first[i];
                 S.delta[d0 + i] = run[i] - s[i];
                 run[i] += tot[i];
             }
@@ -461,39 +592,37 @@ __device__ __forceinline__ void zero_counts(const PassGeom& g, ScatterSmem& S) {
         reinterpret_cast<uint4*>(&S.cnt[q / zw][0])[q % zw] = make_uint4(0, 0, 0, 0);
 }
 
-// One CTA per chunk; whole tiles arrive by bulk copies when USE_BULK (sources
-// 16-byte aligned), the last partial tile (and every tile otherwise) by plain
-// loads.  Waits are bounded: on timeout the pass sets DEV_ERR_TIMEOUT, gives
-// copies in flight a bounded chance to land and the CTA returns.
-template <class Loader, class Storer, bool USE_BULK>
+// CTA b takes share b, or, SPREAD (a share is one tile), the tiles b, b +
+// gridDim.x, ...  Whole tiles arrive by bulk copies when
+// USE_BULK (sources 16-byte aligned), the last partial tile of the last share
+// (and every tile otherwise) by plain loads.  Waits are bounded: on timeout
+// the pass sets DEV_ERR_TIMEOUT, gives copies in flight a bounded chance to
+// land and the CTA returns.
+template <class Loader, class Storer, bool USE_BULK, bool SPREAD>
 __global__ void __launch_bounds__(NT, CTAS_PER_SM) k_scatter(Loader ld, Storer st_in, PassGeom g,
-                                                           const uint32_t* counts,
-                                                           const uint32_t* totals, uint32_t* err) {
+                                                           const uint32_t* __restrict__ table,
+                                                           const uint32_t* __restrict__ totals, uint32_t* err) {
     if (pass_closed(g)) return;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     ScatterSmem& S = *reinterpret_cast<ScatterSmem*>(smem_raw);
     Storer st = st_in;
     st.prepare();
-    uint32_t run[DPT];
-    {   // global start of this chunk's records of each digit
+    const int d0 = threadIdx.x * DPT;
+    uint32_t base[DPT], run[DPT], first[DPT];
+    {   // where each digit's records start
         uint32_t t[DPT], sum = 0;
 #pragma unroll
         for (int i = 0; i < DPT; i++) {
-            const int d = threadIdx.x * DPT + i;
-            t[i] = d < g.bins ? totals[d] : 0u;
+            t[i] = d0 + i < g.bins ? totals[d0 + i] : 0u;
             sum += t[i];
+            run[i] = first[i] = 0;
         }
-        uint32_t base = block_exclusive_scan<NT>(sum, S.warp_tot, &S.total);
+        base[0] = block_exclusive_scan<NT>(sum, S.warp_tot, &S.total);
 #pragma unroll
-        for (int i = 0; i < DPT; i++) {
-            const int d = threadIdx.x * DPT + i;
-            run[i] = d < g.bins ? base + counts[(int64_t)d * g.chunks + blockIdx.x] : 0u;
-            base += t[i];
-        }
+        for (int i = 1; i < DPT; i++) base[i] = base[i - 1] + t[i - 1];
     }
-    const int64_t beg = (int64_t)blockIdx.x * g.chunk;
-    const int64_t end = min(g.n, beg + g.chunk);
-    const int64_t nfull = USE_BULK && end > beg ? (end - beg) / TT : 0;
+    int64_t pos = (int64_t)blockIdx.x * g.share;
+    int64_t end = min(g.n, pos + g.share);
     constexpr uint32_t ARR_BYTES = Loader::TILE_WORDS * 4u;
     static_assert(Loader::NARR * Loader::TILE_WORDS <= 4 * TT, "a tile's sources fit one buffer");
     if (threadIdx.x == 0) {
@@ -503,20 +632,28 @@ __global__ void __launch_bounds__(NT, CTAS_PER_SM) k_scatter(Loader ld, Storer s
     }
     __syncthreads();
     const uint64_t policy = evict_first_policy();
-    auto issue = [&](int64_t t) {
-        const int b = (int)(t % NBUF);
-        const int64_t tbase = beg + t * TT;
+    auto issue = [&](int64_t tbase, int b) {
         bar_expect(&S.bar[b], ARR_BYTES * Loader::NARR);
         uint32_t* dst = reinterpret_cast<uint32_t*>(&S.buf[b][0]);
 #pragma unroll
         for (int a = 0; a < Loader::NARR; a++)
             bulk_load(dst + (size_t)a * TT, ld.tile_src(a, tbase), ARR_BYTES, &S.bar[b], policy);
     };
-    if (threadIdx.x == 0)
-        for (int64_t t = 0; t < NBUF - 1 && t < nfull; t++) issue(t);
-    for (int64_t t = 0; t < nfull; t++) {
-        const int b = (int)(t % NBUF);
-        const uint32_t parity = (uint32_t)((t / NBUF) & 1);
+    auto load_first = [&](int64_t row) {
+#pragma unroll
+        for (int i = 0; i < DPT; i++)
+            if (d0 + i < g.bins) first[i] = __ldg(table + row * g.bins + d0 + i);
+    };
+    const int64_t step = (int64_t)gridDim.x * g.share;  // SPREAD: from a tile to the CTA's next
+    load_first((int64_t)blockIdx.x * g.split);
+    if (!SPREAD) {
+#pragma unroll
+        for (int i = 0; i < DPT; i++) run[i] = base[i] + first[i];
+    }
+    if (USE_BULK && threadIdx.x == 0 && pos + TT <= end) issue(pos, 0);
+    for (int64_t k = 0; USE_BULK && pos + TT <= end; k++) {
+        const int b = (int)(k % NBUF);
+        const uint32_t parity = (uint32_t)((k / NBUF) & 1);
         zero_counts(g, S);  // last read before the previous tile's write
         uint32_t spins = 0;
         while (!bar_try_wait(&S.bar[b], parity)) {
@@ -535,21 +672,32 @@ __global__ void __launch_bounds__(NT, CTAS_PER_SM) k_scatter(Loader ld, Storer s
             }
             return;
         }
-        // the buffer of tile t - 1 was read up to the barrier above
-        if (threadIdx.x == 0 && t + NBUF - 1 < nfull) issue(t + NBUF - 1);
-        const int64_t tbase = beg + t * TT;
+        const int64_t next = SPREAD ? pos + step : pos + TT, nend = SPREAD ? min(g.n, next + TT) : end;
+        // the buffer of the tile before was read up to the barrier above
+        if (threadIdx.x == 0 && next + TT <= nend) issue(next, (b + 1) % NBUF);
         const uint32_t* in = reinterpret_cast<const uint32_t*>(&S.buf[b][0]);
-        scatter_tile<true>([&](int li) { return ld.skey(in, li); }, [&](int li) { return ld.srec(in, li, tbase); }, TT,
-                           st, g, run, S);
+        scatter_tile<true, SPREAD>([&](int li) { return ld.skey(in, li); },
+                                   [&](int li) { return ld.srec(in, li, pos); }, TT, st, g, run, base, first, S);
+        if (SPREAD && next < g.n) load_first(next / TT);
+        pos = next;
+        end = nend;
     }
-    for (int64_t tbase = beg + nfull * TT; tbase < end; tbase += TT) {
-        const int tcount = (int)min((int64_t)TT, end - tbase);
+    while (pos < end) {
+        const int tcount = (int)min((int64_t)TT, end - pos);
         __syncthreads();  // the tile before is written
         zero_counts(g, S);
         uint4* in = S.buf[0];
-        for (int li = threadIdx.x; li < tcount; li += NT) in[li] = ld.grec(tbase + li);
+        for (int li = threadIdx.x; li < tcount; li += NT) in[li] = ld.grec(pos + li);
         __syncthreads();
-        scatter_tile<false>([&](int li) { return in[li].x; }, [&](int li) { return in[li]; }, tcount, st, g, run, S);
+        scatter_tile<false, SPREAD>([&](int li) { return in[li].x; }, [&](int li) { return in[li]; }, tcount, st, g, run,
+                                    base, first, S);
+        if (SPREAD) {
+            pos += step;
+            end = min(g.n, pos + TT);
+            if (pos < g.n) load_first(pos / TT);
+        } else {
+            pos += TT;
+        }
     }
 }
 
@@ -605,15 +753,21 @@ struct SwitchStorer {
 };
 
 // ---- host side ------------------------------------------------------------------
-// Chunking: CTAS_PER_SM chunks per SM at most, equal shares of at least
-// MIN_CHUNK records (a multiple of 32, so that every source stays 16-byte
-// aligned); the tiles of a chunk are whole but the last.
-inline PassGeom make_geom(int64_t n, int shift, int bits) {
+inline int64_t scatter_ctas() { return (int64_t)sm_count() * CTAS_PER_SM; }
+
+// Shares: one per CTA, equal (a multiple of 32 records, so that every source
+// stays 16-byte aligned; not of more, or the CTAs would all stand at the same
+// offset of the memory channels: 4 % slower scatters at 1e8 edges with shares
+// of 1,285 x 1,024 records), counted in up to UP_SPLIT rows; or, spread, one
+// tile each, dealt round-robin.
+inline PassGeom make_geom(int64_t n, int shift, int bits, bool spread = false) {
     PassGeom g;
     g.n = n;
-    const int64_t want = (int64_t)sm_count() * CTAS_PER_SM, per = (n + want - 1) / want;
-    g.chunk = std::max<int64_t>(MIN_CHUNK, (per + 31) / 32 * 32);
-    g.chunks = (int)std::max<int64_t>(1, (n + g.chunk - 1) / g.chunk);
+    const int64_t ctas = scatter_ctas(), per = (std::max<int64_t>(MIN_SHARE, (n + ctas - 1) / ctas) + 31) / 32 * 32;
+    g.share = spread ? TT : per;
+    g.split = spread ? 1 : (int)std::min<int64_t>(UP_SPLIT, std::max<int64_t>(1, per / MIN_ROW));
+    g.row = ((g.share + g.split - 1) / g.split + 31) / 32 * 32;
+    g.rows = std::max<int64_t>(1, (n + g.share - 1) / g.share * g.split);
     g.shift = shift;
     g.bins = 1 << bits;
     g.bits = bits;
@@ -624,11 +778,25 @@ inline PassGeom make_geom(int64_t n, int shift, int bits) {
     return g;
 }
 
-// Scratch for the counts of any sort of at most n records: MAX_BINS * chunks +
-// MAX_BINS (uint32).
+// Whether a pass into `streams` arrays deals its tiles round-robin.  With a
+// share each, every CTA keeps a line open for every digit and array; beyond
+// what L2 holds of them, lines are evicted half written (10-bit digits into
+// the four arrays of the rows: 80 MB; the pass takes 744 us at 2e7 edges, 539
+// spread).  Below, the spread tiles cost their counts and scans and gain
+// nothing: 10-bit digits into records and digits, 40 MB, 475 -> 404 us but 66
+// us more of counting; 9-bit ones at 1e9 edges 17.4 -> 19 ms.
+inline bool spread_pass(int64_t n, int bits, int streams) {
+    const int64_t ctas = scatter_ctas();
+    return n >= SPREAD_TILES * ctas * TT && (ctas * streams * 128 << bits) > OPEN_BYTES;
+}
+
+inline int64_t max_segs() { return (int64_t)sm_count() * 8; }
+
+// Scratch for the counts of any sort of at most n records: the table, its
+// totals, the segments' sums (uint32).
 inline size_t scratch_words(int64_t n) {
-    const int64_t chunks = std::min<int64_t>((int64_t)sm_count() * CTAS_PER_SM, n / MIN_CHUNK + 1);
-    return (size_t)MAX_BINS * (size_t)chunks + MAX_BINS;
+    const int64_t rows = std::max(std::min<int64_t>(scatter_ctas() * UP_SPLIT, n / MIN_SHARE + UP_SPLIT), n / TT + 1);
+    return (size_t)MAX_BINS * (size_t)(rows + 1 + (rows > SCAN_ROWS ? max_segs() : 0));
 }
 
 // Whether whole tiles use bulk copies (WTRI_RADIX_TMA=0 turns them off).
@@ -658,32 +826,50 @@ inline int pass_shift(int bits, int p) {
 // scatter's phase timer; histograms and scans declare none).  expected:
 // whether the pass is expected to run (a conditional pass that the widest
 // expected keys skip declares no moved bytes either).
-template <class Dig, class Loader, class Storer>
+template <bool SPREAD = false, class Dig, class Loader, class Storer>
 int run_pass(const Dig& dg, const Loader& ld, const Storer& st, const PassGeom& g, uint32_t* scratch,
              cudaStream_t s, uint32_t* err, double hist_bytes, double alg_bytes, bool expected = true) {
     const double mv = expected ? 1.0 : 0.0;
     if (g.n <= 0) return WTRI_OK;
-    uint32_t* counts = scratch;
-    uint32_t* totals = scratch + (size_t)MAX_BINS * g.chunks;
+    uint32_t* table = scratch;
+    uint32_t* totals = table + (size_t)MAX_BINS * g.rows;
     {
-        ProfScope ps("radix_upsweep", s, 0.0, 1, mv * (hist_bytes * (double)g.n + 4.0 * g.bins * g.chunks));
-        WTRI_CUDA(cudaMemsetAsync(counts, 0, sizeof(uint32_t) * (size_t)g.bins * g.chunks, s));
-        k_upsweep<Dig><<<g.chunks * UP_SPLIT, UNT, 0, s>>>(dg, g, counts);
+        ProfScope ps("radix_upsweep", s, 0.0, 1, mv * (hist_bytes * (double)g.n + 4.0 * g.bins * (double)g.rows));
+        if constexpr (SPREAD) {
+            static_assert(Dig::PACKED, "spread passes read stored digits");
+            k_upsweep_tiles<<<(unsigned)std::min<int64_t>(g.rows, sm_count() * 6), UNT, 0, s>>>(dg.d, g, table);
+        } else {
+            k_upsweep<Dig><<<(unsigned)g.rows, UNT, 0, s>>>(dg, g, table);
+        }
     }
     {
-        ProfScope ps("radix_digit_scan", s, 0.0, 1, mv * 8.0 * g.bins * g.chunks);
-        k_digit_scan<<<g.bins, NT, 0, s>>>(counts, g.chunks, totals, g);
+        const bool segmented = g.rows > SCAN_ROWS;
+        const unsigned cols = (unsigned)((g.bins + SCAN_X - 1) / SCAN_X);
+        ProfScope ps("radix_digit_scan", s, 0.0, segmented ? 3 : 1,
+                     mv * (segmented ? 12.0 : 8.0) * g.bins * (double)g.rows);
+        if (!segmented) {
+            k_col_scan<<<cols, SCAN_X * SCAN_Y, 0, s>>>(table, g.rows, totals, g);
+        } else {
+            uint32_t* sums = totals + MAX_BINS;
+            const int seg = (int)((g.rows + max_segs() - 1) / max_segs());
+            const unsigned segs = (unsigned)((g.rows + seg - 1) / seg);
+            const dim3 grid(segs, (unsigned)((g.bins + UNT - 1) / UNT));
+            k_seg_sum<<<grid, UNT, 0, s>>>(table, seg, sums, g);
+            k_col_scan<<<cols, SCAN_X * SCAN_Y, 0, s>>>(sums, segs, totals, g);
+            k_seg_apply<<<grid, UNT, 0, s>>>(table, seg, sums, g);
+        }
     }
     const size_t smem = sizeof(ScatterSmem);
+    const unsigned ctas = (unsigned)std::min<int64_t>(scatter_ctas(), (g.n + g.share - 1) / g.share);
     ProfScope ps("radix_downsweep", s, alg_bytes, 1, mv * (double)g.n * (Loader::REC_BYTES + st.rec_bytes()));
     if (bulk_enabled() && ld.tma_ok()) {
         static std::atomic<uint64_t> done{0};  // per instantiation and device
-        WTRI_TRY(smem_optin((const void*)k_scatter<Loader, Storer, true>, (int)smem, done));
-        k_scatter<Loader, Storer, true><<<g.chunks, NT, smem, s>>>(ld, st, g, counts, totals, err);
+        WTRI_TRY(smem_optin((const void*)k_scatter<Loader, Storer, true, SPREAD>, (int)smem, done));
+        k_scatter<Loader, Storer, true, SPREAD><<<ctas, NT, smem, s>>>(ld, st, g, table, totals, err);
     } else {
         static std::atomic<uint64_t> done{0};
-        WTRI_TRY(smem_optin((const void*)k_scatter<Loader, Storer, false>, (int)smem, done));
-        k_scatter<Loader, Storer, false><<<g.chunks, NT, smem, s>>>(ld, st, g, counts, totals, err);
+        WTRI_TRY(smem_optin((const void*)k_scatter<Loader, Storer, false, SPREAD>, (int)smem, done));
+        k_scatter<Loader, Storer, false, SPREAD><<<ctas, NT, smem, s>>>(ld, st, g, table, totals, err);
     }
     WTRI_CUDA(cudaGetLastError());
     return WTRI_OK;
@@ -704,7 +890,8 @@ int lsd_sort(const First& first, const Last& last, int64_t n, int bits, uint4* r
     uint4* cur = rec_a;
     uint4* nxt = rec_b;
     for (int p = 0; p < passes; p++) {
-        PassGeom g = make_geom(n, pass_shift(bits, p), pass_bits(bits, p));
+        const bool spread = p > 0 && p == passes - 1 && spread_pass(n, pass_bits(bits, p), Last::STREAMS);
+        PassGeom g = make_geom(n, pass_shift(bits, p), pass_bits(bits, p), spread);
         g.gerr = err;
         AosStorer as{nxt, dig, 0, 0u};
         if (p + 1 < passes) {
@@ -714,14 +901,15 @@ int lsd_sort(const First& first, const Last& last, int64_t n, int bits, uint4* r
         AosLoader al{cur};
         StoredDigits sd{dig};
         if (p == 0) {
-            KeyDigits<First> kd{first, g.shift, g.mask};
+            KeyDigits<First> kd{first, g.shift, g.mask, first.tma_ok()};
             if (passes == 1) {
                 WTRI_TRY(run_pass(kd, first, last, g, scratch, s, err, 4.0, alg));
             } else {
                 WTRI_TRY(run_pass(kd, first, as, g, scratch, s, err, 4.0, alg));
             }
         } else if (p == passes - 1) {
-            WTRI_TRY(run_pass(sd, al, last, g, scratch, s, err, 2.0, alg));
+            if (spread) WTRI_TRY(run_pass<true>(sd, al, last, g, scratch, s, err, 2.0, alg));
+            else WTRI_TRY(run_pass(sd, al, last, g, scratch, s, err, 2.0, alg));
         } else {
             WTRI_TRY(run_pass(sd, al, as, g, scratch, s, err, 2.0, alg));
         }
@@ -764,7 +952,7 @@ int lsd_sort_device_width(const First& first, const Last& last, int64_t n, int m
         const bool ex = p < expected_passes;
         const double a = ex ? alg : 0.0;
         if (p == 0) {
-            KeyDigits<First> kd{first, g.shift, g.mask};
+            KeyDigits<First> kd{first, g.shift, g.mask, first.tma_ok()};
             if (passes == 1) {
                 WTRI_TRY(run_pass(kd, first, last, g, scratch, s, err, 4.0, a, ex));
             } else {
