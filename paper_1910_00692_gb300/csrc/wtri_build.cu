@@ -572,7 +572,9 @@ int build_graph(int32_t n, int64_t m, const int32_t* u_in, const int32_t* v_in,
         const size_t rec_words = 4 * (size_t)n2 + 4;
         // (multiples of four words: wrow below starts 16-byte aligned)
         const size_t dig_words = align_up(((size_t)n2 + 1) / 2 + 4, 4);
-        const size_t cnt_words = align_up(radix::scratch_words(n2), 4);
+        const int nbits = std::max(1, radix::bit_length((uint64_t)(n - 1)));  // of a row key
+        const bool spread = radix::sort_spreads(n2, nbits, RowsStorer::STREAMS);
+        const size_t cnt_words = align_up(radix::scratch_words(n2, spread), 4);
         const size_t words = 2 * rec_words + dig_words + cnt_words + (size_t)n2 + (N1 + 1) / 2 + 4 +
                              N1 + 4 + N1 + 4 + 64;
         Scratch tmp(s);
@@ -609,7 +611,6 @@ int build_graph(int32_t n, int64_t m, const int32_t* u_in, const int32_t* v_in,
             if (rc != WTRI_OK) return fail(rc);
         }
         // 3. weight-sorted rows (row key kept in wrow)
-        const int nbits = std::max(1, radix::bit_length((uint64_t)(n - 1)));
         {
             OrderEntryLoader ol{ou, ov, ow};
             RowsStorer rs{wrow, wcol, wwt, wrk};

@@ -792,10 +792,11 @@ inline bool spread_pass(int64_t n, int bits, int streams) {
 
 inline int64_t max_segs() { return (int64_t)sm_count() * 8; }
 
-// Scratch for the counts of any sort of at most n records: the table, its
-// totals, the segments' sums (uint32).
-inline size_t scratch_words(int64_t n) {
-    const int64_t rows = std::max(std::min<int64_t>(scatter_ctas() * UP_SPLIT, n / MIN_SHARE + UP_SPLIT), n / TT + 1);
+// Scratch for the counts of any sort of at most n records, with or without a
+// spread pass: the table, its totals, the segments' sums (uint32).
+inline size_t scratch_words(int64_t n, bool spread) {
+    int64_t rows = std::min<int64_t>(scatter_ctas() * UP_SPLIT, n / MIN_SHARE + UP_SPLIT);
+    if (spread) rows = std::max(rows, n / TT + 1);
     return (size_t)MAX_BINS * (size_t)(rows + 1 + (rows > SCAN_ROWS ? max_segs() : 0));
 }
 
@@ -875,6 +876,12 @@ int run_pass(const Dig& dg, const Loader& ld, const Storer& st, const PassGeom& 
     return WTRI_OK;
 }
 
+// Whether lsd_sort spreads the last pass of n records over 'bits' key bits.
+inline bool sort_spreads(int64_t n, int bits, int streams) {
+    const int last = pass_count(bits) - 1;
+    return last > 0 && spread_pass(n, pass_bits(bits, last), streams);
+}
+
 // Full stable LSD sort of n records over 'bits' key bits: first pass from
 // 'first', middle passes through the 16-byte record buffers rec_a / rec_b
 // (n records each) with digits in 'dig' (n 16-bit words), last pass into
@@ -890,7 +897,7 @@ int lsd_sort(const First& first, const Last& last, int64_t n, int bits, uint4* r
     uint4* cur = rec_a;
     uint4* nxt = rec_b;
     for (int p = 0; p < passes; p++) {
-        const bool spread = p > 0 && p == passes - 1 && spread_pass(n, pass_bits(bits, p), Last::STREAMS);
+        const bool spread = p == passes - 1 && sort_spreads(n, bits, Last::STREAMS);
         PassGeom g = make_geom(n, pass_shift(bits, p), pass_bits(bits, p), spread);
         g.gerr = err;
         AosStorer as{nxt, dig, 0, 0u};
