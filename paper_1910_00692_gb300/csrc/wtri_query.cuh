@@ -275,11 +275,15 @@ __device__ __forceinline__ bool probe_oriented(const DevGraph& G, int32_t y, int
 // rate is a sixty-fourth of its fp32 rate, so the smallest weight that can
 // reach tau is found once per edge in fp32 instead: with t = tau (1 - 1e-4)
 // and R = 3 - (w/t)^p - (y/t)^p, the mean reaches t iff (x/t)^p >= R (p > 0)
-// or <= R (p < 0), i.e. x >= t R^(1/p).  The 1e-4 leaves R a slack of
-// 3e-4 |p| while fp32 rounding moves it by less than 4e-6 (1 + |p|) wherever
-// R > 0, so for |p| >= 0.05 a weight is only pruned when the exact bound
-// prunes it too; smaller |p| keeps the fp64 bound.  Survivors are decided by
-// their fp64 key.
+// or <= R (p < 0), i.e. x >= t R^(1/p) (p = 0: x >= t / ((w/t) (y/t))).  The
+// 1e-4 leaves R a slack of 3e-4 |p| while fp32 rounding moves it by less than
+// 4e-6 (1 + |p|) wherever R > 0, so for |p| >= 0.05 a weight is only pruned
+// when the exact bound prunes it too; smaller |p| keeps the fp64 bound.  All of
+// it holds in fp32's normal range only, which real weights may leave (they
+// reach down to 2^-149): t, both quotients and the power must lie well inside,
+// else the fp64 bound decides (a power below 2^-120: no bound; x itself may be
+// subnormal, as rounding to the weights' own grid passes none of them).
+// Survivors are decided by their fp64 key.
 // ---------------------------------------------------------------------------
 template <int P>
 struct Line {
@@ -294,23 +298,29 @@ struct Line {
         : tau(tau_), w(w_), y(y_), gp(q.gp), fw(q.fw != 0), use_cut(false), cut(0) {
         if constexpr (P == P_GEN) {
             const float p = (float)gp;
-            if (tau != 0 && ((fabsf(p) >= 0.05f && fabsf(p) <= 1000.0f) || p == 0.0f)) {
-                use_cut = true;
-                const float t = (float)__longlong_as_double((long long)tau) * (1.0f - 1e-4f);
-                const float a = fw ? __uint_as_float(w) : (float)w, b = fw ? __uint_as_float(y) : (float)y;
-                float x;
-                if (p == 0.0f) {  // geometric mean: x >= t^3 / (a b)
-                    x = exp2f(3.0f * log2f(t) - log2f(a) - log2f(b));
-                } else {
-                    const float R = 3.0f - exp2f(p * log2f(a / t)) - exp2f(p * log2f(b / t));
-                    if (R > 0.0f) x = t * exp2f(log2f(R) / p);
-                    else x = p > 0.0f ? 0.0f : __int_as_float(0x7f800000);
+            if (tau == 0 || !((fabsf(p) >= 0.05f && fabsf(p) <= 1000.0f) || p == 0.0f)) return;
+            const float t = (float)__longlong_as_double((long long)tau) * (1.0f - 1e-4f);
+            const float a = (fw ? __uint_as_float(w) : (float)w) / t, b = (fw ? __uint_as_float(y) : (float)y) / t;
+            auto inside = [](float x) { return x >= 0x1p-100f && x <= 0x1p100f; };
+            if (!inside(t) || !inside(a) || !inside(b)) return;
+            float e;  // log2 of the smallest x / t
+            if (p == 0.0f) {
+                e = -log2f(a) - log2f(b);
+            } else {
+                const float R = 3.0f - exp2f(p * log2f(a)) - exp2f(p * log2f(b));
+                use_cut = !(R > 0.0f);  // w and y alone reach t (p > 0), or keep any x from it
+                if (use_cut) {
+                    cut = p > 0.0f ? 0u : 0xffffffffu;
+                    return;
                 }
-                x *= 1.0f - 1e-6f;
-                if (!(x >= 0.0f)) x = 0.0f;  // no usable bound
-                if (fw) cut = __float_as_uint(x);
-                else cut = x >= 4294967040.0f ? 0xffffffffu : (uint32_t)x;
+                e = log2f(R) / p;
             }
+            if (!(e <= 120.0f)) return;
+            use_cut = true;
+            if (e < -120.0f) return;  // cut = 0
+            const float x = t * exp2f(e) * (1.0f - 1e-6f);
+            if (fw) cut = __float_as_uint(x);
+            else cut = x >= 4294967040.0f ? 0xffffffffu : (uint32_t)x;
         }
     }
     __device__ __forceinline__ bool fails(uint32_t x) const {
