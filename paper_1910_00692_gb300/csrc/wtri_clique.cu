@@ -456,9 +456,13 @@ struct CliqueSelect {
 
 __global__ void __launch_bounds__(TGRID, 1) k_clique_reach(CliqueSelect A) {
     __shared__ SelectSmem S;
-    if (*(volatile const uint32_t*)A.err) return;  // set before this launch: every block sees the same
-    const uint32_t n = min(*(volatile const uint32_t*)A.count, A.cap);
     const int tid = threadIdx.x, lane = tid & 31;
+    // one thread reads the error word: a block that gives up below sets it,
+    // maybe before this one has started
+    if (tid == 0) S.err = *(volatile const uint32_t*)A.err;
+    __syncthreads();
+    if (S.err) return;
+    const uint32_t n = min(*(volatile const uint32_t*)A.count, A.cap);
     GridTeam<TGRID> T;
     T.limit = A.q.wait_first;
     T.blk0 = 0;

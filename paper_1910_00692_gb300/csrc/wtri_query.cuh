@@ -961,8 +961,23 @@ struct SelectSmem {
     uint32_t wsum[32];
     unsigned long long mn, mx;
     uint32_t bin, above, taken;
+    uint32_t err, n, old;  // the query's error bits, candidates and `selected`, as one thread read them
     int gone;  // a grid barrier gave up
 };
+
+// The query's state for the whole selecting block.  One thread reads it: a
+// block whose first barrier wait runs out sets the timeout bit after its
+// arrival has been counted, so at any moment here, and threads that branched
+// around the block's barriers on readings of their own could part.
+template <int TB>
+__device__ __forceinline__ void read_state(const Part<TB>& B, const Query& q, SelectSmem& S) {
+    if (B.tid() == 0) {
+        S.err = *(volatile uint32_t*)&q.st->err;
+        S.n = min(*(volatile uint32_t*)&q.st->count, q.cap);
+        S.old = *(volatile uint32_t*)&q.st->selected;
+    }
+    B.sync();
+}
 
 // The ranking's shared arrays (aliases the p = -inf queues of phase A).
 struct SortSmem {
@@ -1185,11 +1200,9 @@ __device__ uint32_t keep_first_ties(const Part<TB>& B, unsigned long long* ckey,
 template <int TB>
 __device__ int64_t select_round(const Part<TB>& B, const Query& q, SelectSmem& S) {
     const int64_t growth = q.growth;
-    if (*(volatile uint32_t*)&q.st->err) return growth;
-    const uint32_t n = min(*(volatile uint32_t*)&q.st->count, q.cap);
-    const uint32_t old = *(volatile uint32_t*)&q.st->selected;
-    B.sync();  // `selected` is rewritten below
-    if (n == old) return growth;
+    read_state<TB>(B, q, S);
+    const uint32_t n = S.n, old = S.old;
+    if (S.err || n == old) return growth;
     const int64_t added = n - old;
     if (n < (uint32_t)q.k) {
         if (B.tid() == 0) *(volatile uint32_t*)&q.st->selected = n;  // all of them stay
@@ -1207,11 +1220,11 @@ __device__ int64_t select_round(const Part<TB>& B, const Query& q, SelectSmem& S
 }
 
 // The next round's range: [lo, lo + size) cut at the first edge whose bound
-// is below tau (the edges' weights do not increase).
+// is below tau (the edges' weights do not increase); empty after an error.
 template <int P, bool SAMPLED>
-__device__ __forceinline__ void next_range(int tid, const DevGraph& G, const Query& q, int64_t lo, int64_t size, int64_t total) {
+__device__ __forceinline__ void next_range(int tid, const DevGraph& G, const Query& q, int64_t lo, int64_t size,
+                                           int64_t total, bool failed) {
     if (tid >= 32) return;
-    const bool failed = *(volatile uint32_t*)&q.st->err != 0;
     const unsigned long long tau = ld_volatile_u64(&q.st->tau);
     int64_t hi = failed ? lo : min(total, lo + size);
     if (!SAMPLED && tau != 0)
@@ -1296,13 +1309,12 @@ __device__ void finish(const Query& q, const Out& o, Team& T, SelectSmem& S, Sor
     const uint32_t K = (uint32_t)q.k;
     const Part<Team::TB>& B = T.part;
     if (T.leader()) {
-        const uint32_t err = *(volatile uint32_t*)&q.st->err;
-        uint32_t n = min(*(volatile uint32_t*)&q.st->count, q.cap);
-        B.sync();
-        if (err) n = 0;
+        read_state<Team::TB>(B, q, S);
+        const uint32_t err = S.err;
+        uint32_t n = err ? 0 : S.n;
         if (n > K) {
             unsigned long long T0 = ld_volatile_u64(&q.st->tau);
-            if (n != *(volatile uint32_t*)&q.st->selected) {
+            if (n != S.old) {
                 T0 = kth_key<Team::TB>(B, q.ckey, n, K, S);
                 n = compact<Team::TB>(B, q.ckey, q.ctri, n, [=](unsigned long long k, const int4&) { return k >= T0; }, S);
             }
@@ -1383,7 +1395,7 @@ __device__ void sweep(const DevGraph& G, const Query& q, const Out& o, Team& T, 
         if (T.leader()) {
             if (T.part.tid() == 0) *(volatile unsigned long long*)&q.st->items[par ^ 1] = 0;
             const int64_t grow = select_round<Team::TB>(T.part, q, S.sel);
-            next_range<P, SAMPLED>(T.part.tid(), G, q, hi, min(size * grow, cap), total);
+            next_range<P, SAMPLED>(T.part.tid(), G, q, hi, min(size * grow, cap), total, S.sel.err != 0);
         }
         if (!T.sync(q)) return;
         size = *(volatile long long*)&q.st->size;
