@@ -469,15 +469,22 @@ WTRI_API int wtri_query_bytes(int on, int reset, unsigned long long* bytes);
 
 /*
  * Fault injection for tests (no counterpart in the paper).  The blocks of
- * an exact query's kernel wait for one another at a grid barrier with a
- * bounded number of polls; when the polls run out the query reports
- * WTRI_ETIMEOUT (the other blocks are still waited for, with the full bound,
- * so that all leave in step).  This sets the bound of each block's first
- * wait for queries started afterwards in this process: polls = 0 makes it
- * report a timeout at once; polls < 0 restores the default.  Nothing else
- * changes; a query after restoring the default is unaffected.
+ * a query's kernel wait for one another at a grid barrier with a bounded
+ * number of polls; when the polls run out the query reports WTRI_ETIMEOUT
+ * (the other blocks are still waited for, with the full bound, so that all
+ * leave in step; if that runs out too, the block leaves, the others follow
+ * at their next barrier, and the status stays WTRI_ETIMEOUT).  This sets the
+ * bound of each block's first wait for queries started afterwards in this
+ * process: polls = 0 makes it report a timeout at once; polls < 0 restores
+ * the default.  Nothing else changes; a query after restoring the default is
+ * unaffected.
+ *
+ * wtri_debug_set_wait_limits sets the bound of the first wait and of every
+ * later one, the waiting on after a timeout among them: with both 0 every
+ * block leaves at the first barrier.
  */
 WTRI_API int wtri_debug_set_wait_limit(int64_t polls);
+WTRI_API int wtri_debug_set_wait_limits(int64_t first, int64_t later);
 
 /* Thread-local message for the last failing call on this thread ("" if none). */
 WTRI_API const char* wtri_last_error(void);

@@ -17,6 +17,7 @@ from .wtri import (  # noqa: F401
     autotune_buckets,
     build_csr,
     debug_set_wait_limit,
+    debug_set_wait_limits,
     lib,
     lib_path,
     merge_topk,
@@ -33,6 +34,6 @@ from .wtri import (  # noqa: F401
 )
 
 __all__ = ["ARRAYS", "Graph", "Server", "WtriError", "WtriUnavailable", "autotune_buckets", "build_csr",
-           "debug_set_wait_limit", "lib", "lib_path", "merge_topk", "topk_shard",
+           "debug_set_wait_limit", "debug_set_wait_limits", "lib", "lib_path", "merge_topk", "topk_shard",
            "sample_cliques", "sample_edges", "sample_topk", "sample_wedges", "topk", "topk_batch", "topk_device",
            "topk_device_noalloc", "wedge_topk"]

@@ -125,6 +125,7 @@ int host_result_query(const wtri_graph* g, int32_t k, wtri_result* out, Launch l
         if (status == WTRI_ENOMEM && scale < 64) continue;  // bounded buffer overflowed: retry
         break;
     }
+    if (rc == WTRI_OK && status > k) status = WTRI_ECUDA;  // no count: not to be copied by
     if (rc == WTRI_OK && status < 0) {
         rc = set_error(status, status == WTRI_ENOMEM     ? "device candidate buffer overflow"
                                : status == WTRI_ETIMEOUT ? "bounded device wait ran out"

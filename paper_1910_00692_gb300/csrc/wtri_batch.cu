@@ -65,14 +65,14 @@ __device__ __noinline__ void sweep_part(PartSmem& S) {
 }
 
 template <int P>
-__device__ __noinline__ void sweep_team(const DevGraph& G, const Query& q, const Out& o, SweepSmem<TGRID>& S,
+__device__ __noinline__ bool sweep_team(const DevGraph& G, const Query& q, const Out& o, SweepSmem<TGRID>& S,
                                         uint32_t blk0, uint32_t nblk) {
     GridTeam<TGRID> T;
     T.limit = q.wait_first;
     T.blk0 = blk0;
     T.nblk = nblk;
     T.gone = &S.sel.gone;
-    sweep<P, false>(G, q, o, T, S);
+    return sweep<P, false>(G, q, o, T, S);
 }
 
 union BatchSmem {
@@ -101,13 +101,16 @@ __global__ void __launch_bounds__(TGRID, 1) k_sweep_batch(BatchDev B, TeamList L
             S.team.sel.gone = 0;
         }
         __syncthreads();
+        bool ok;
         switch (B.pcodes[qi]) {
-            case P_MIN: sweep_team<P_MIN>(G, q, o, S.team, blk0, nblk); break;
-            case P_ONE: sweep_team<P_ONE>(G, q, o, S.team, blk0, nblk); break;
-            case P_TWO: sweep_team<P_TWO>(G, q, o, S.team, blk0, nblk); break;
-            case P_GEO: sweep_team<P_GEO>(G, q, o, S.team, blk0, nblk); break;
-            default: sweep_team<P_MAX>(G, q, o, S.team, blk0, nblk); break;
+            case P_MIN: ok = sweep_team<P_MIN>(G, q, o, S.team, blk0, nblk); break;
+            case P_ONE: ok = sweep_team<P_ONE>(G, q, o, S.team, blk0, nblk); break;
+            case P_TWO: ok = sweep_team<P_TWO>(G, q, o, S.team, blk0, nblk); break;
+            case P_GEO: ok = sweep_team<P_GEO>(G, q, o, S.team, blk0, nblk); break;
+            default: ok = sweep_team<P_MAX>(G, q, o, S.team, blk0, nblk); break;
         }
+        // gave up: the other blocks may still be using this one's items
+        if (!ok) return;
         __syncthreads();
     }
     const int p = threadIdx.x / PT;
@@ -171,14 +174,15 @@ struct wtri_batch_plan {
     int32_t nq = 0;
     int64_t pool = 0;  // items
     std::vector<wtri::DevGraph> hg;
-    std::vector<int32_t> pcodes, ks, tshort;
+    std::vector<int32_t> pcodes;  // nq, and after them the statuses as they start: one upload
+    std::vector<int32_t> ks, tshort;
     std::vector<int32_t> alone;  // queries with a launch of their own (k above what a part ranks, no team left)
     std::vector<int32_t> order;  // the queries answered by parts, largest first
     wtri::TeamList teams;
     std::vector<uint32_t> caps;
     std::vector<int64_t> koffs;
     size_t cand_total = 0;
-    size_t o_st, o_key, o_tri, o_items, o_ibase, o_cur, o_g, o_q, o_o, o_pc, o_ord, o_otri, o_ow, o_stat, bytes;
+    size_t o_st, o_key, o_tri, o_items, o_ibase, o_cur, o_g, o_q, o_o, o_pc, o_ord, o_otri, o_ow, bytes;
     std::vector<int32_t> stat;
     std::vector<wtri_tri> otri;
     std::vector<double> ow;
@@ -239,6 +243,7 @@ BatchPlan* batch_plan_create(const wtri_graph* const* gs, const int32_t* pcodes,
     P->nq = nq;
     P->hg.resize((size_t)nq);
     P->pcodes.assign(pcodes, pcodes + nq);
+    P->pcodes.resize(2 * (size_t)nq, WTRI_ETIMEOUT);  // until a query is answered
     P->ks.assign(ks, ks + nq);
     P->caps.resize((size_t)nq);
     P->tshort.resize((size_t)nq);
@@ -267,11 +272,10 @@ BatchPlan* batch_plan_create(const wtri_graph* const* gs, const int32_t* pcodes,
     P->o_g = take(sizeof(DevGraph) * (size_t)nq);
     P->o_q = take(sizeof(Query) * (size_t)nq);
     P->o_o = take(sizeof(Out) * (size_t)nq);
-    P->o_pc = take(4 * (size_t)nq);
+    P->o_pc = take(8 * (size_t)nq);
     P->o_ord = take(4 * (size_t)nq);
     P->o_otri = take(sizeof(wtri_tri) * (size_t)P->koffs[(size_t)nq]);
     P->o_ow = take(8 * (size_t)P->koffs[(size_t)nq]);
-    P->o_stat = take(4 * (size_t)nq);
     P->bytes = off;
     return P;
 }
@@ -304,7 +308,7 @@ int batch_plan_launch(BatchPlan* P, void* dbuf, cudaStream_t s, int use_graph) {
     int4* ctri = (int4*)(B0 + P->o_tri);
     wtri_tri* d_otri = (wtri_tri*)(B0 + P->o_otri);
     double* d_ow = (double*)(B0 + P->o_ow);
-    int32_t* d_stat = (int32_t*)(B0 + P->o_stat);
+    int32_t* d_stat = (int32_t*)(B0 + P->o_pc) + nq;
     std::vector<Query> hq((size_t)nq);
     std::vector<Out> ho((size_t)nq);
     size_t c0 = 0;
@@ -322,7 +326,8 @@ int batch_plan_launch(BatchPlan* P, void* dbuf, cudaStream_t s, int use_graph) {
         q.growth = BATCH_GROWTH;
         q.nshards = 1;
         q.t_short = P->tshort[(size_t)i];
-        q.wait_first = WAIT_LIMIT;
+        q.wait_first = first_wait_limit();
+        q.wait_later = later_wait_limit();
         ho[(size_t)i] = Out{d_otri + P->koffs[(size_t)i], d_ow + P->koffs[(size_t)i], d_stat + i, nullptr};
         c0 += P->caps[(size_t)i];
     }
@@ -342,7 +347,7 @@ int batch_plan_launch(BatchPlan* P, void* dbuf, cudaStream_t s, int use_graph) {
     WTRI_CUDA(cudaMemcpyAsync((void*)Bd.graphs, P->hg.data(), sizeof(DevGraph) * nq, cudaMemcpyHostToDevice, s));
     WTRI_CUDA(cudaMemcpyAsync((void*)Bd.queries, hq.data(), sizeof(Query) * nq, cudaMemcpyHostToDevice, s));
     WTRI_CUDA(cudaMemcpyAsync((void*)Bd.outs, ho.data(), sizeof(Out) * nq, cudaMemcpyHostToDevice, s));
-    WTRI_CUDA(cudaMemcpyAsync((void*)Bd.pcodes, P->pcodes.data(), 4 * (size_t)nq, cudaMemcpyHostToDevice, s));
+    WTRI_CUDA(cudaMemcpyAsync((void*)Bd.pcodes, P->pcodes.data(), 8 * (size_t)nq, cudaMemcpyHostToDevice, s));
     if (!P->order.empty())
         WTRI_CUDA(cudaMemcpyAsync((void*)Bd.order, P->order.data(), 4 * P->order.size(), cudaMemcpyHostToDevice, s));
     static std::atomic<uint64_t> done{0};
@@ -428,11 +433,14 @@ int batch_plan_collect(BatchPlan* P, void* dbuf, cudaStream_t s) {
     P->stat.assign((size_t)nq, 0);
     P->otri.resize((size_t)P->koffs[(size_t)nq]);
     P->ow.resize((size_t)P->koffs[(size_t)nq]);
-    WTRI_CUDA(cudaMemcpyAsync(P->stat.data(), B0 + P->o_stat, 4 * (size_t)nq, cudaMemcpyDeviceToHost, s));
+    WTRI_CUDA(cudaMemcpyAsync(P->stat.data(), (int32_t*)(B0 + P->o_pc) + nq, 4 * (size_t)nq, cudaMemcpyDeviceToHost,
+                              s));
     WTRI_CUDA(cudaMemcpyAsync(P->otri.data(), B0 + P->o_otri, sizeof(wtri_tri) * P->otri.size(),
                               cudaMemcpyDeviceToHost, s));
     WTRI_CUDA(cudaMemcpyAsync(P->ow.data(), B0 + P->o_ow, 8 * P->ow.size(), cudaMemcpyDeviceToHost, s));
     WTRI_CUDA(cudaStreamSynchronize(s));
+    for (int i = 0; i < nq; i++)
+        if (P->stat[(size_t)i] > P->ks[(size_t)i]) P->stat[(size_t)i] = WTRI_ECUDA;  // no count: not to be copied by
     return WTRI_OK;
 }
 
@@ -459,6 +467,7 @@ int topk_retry_host(const wtri_graph* g, int pcode, int32_t k, cudaStream_t s, w
             if (e != cudaSuccess) rc = cuda_error(e, "retry", __FILE__, __LINE__);
         }
     }
+    if (rc == WTRI_OK && cnt > k) cnt = WTRI_ECUDA;
     if (rc == WTRI_OK && cnt < 0) rc = set_error(cnt, "query failed on retry with larger buffers");
     if (rc == WTRI_OK && cnt > 0) {
         cudaError_t e = cudaMemcpyAsync(htri, dt, sizeof(wtri_tri) * (size_t)cnt, cudaMemcpyDeviceToHost, s);

@@ -798,7 +798,8 @@ int clique_topk_host(const wtri_graph* g, int q, int pcode, int32_t k, int64_t n
         CliqueSelect A{};
         A.lim = (unsigned long long*)((char*)small + 256);
         A.q.st = (QState*)((char*)small + 512);
-        A.q.wait_first = WAIT_LIMIT;
+        A.q.wait_first = first_wait_limit();
+        A.q.wait_later = later_wait_limit();
         A.hist = (uint32_t*)((char*)small + 512 + al(sizeof(QState)));
         A.ckey = ckey;
         A.count = small;

@@ -191,6 +191,10 @@ struct ProfScope {
 bool query_bytes_on();
 unsigned long long* query_bytes_counter();  // device address for the current device
 
+// Poll limits of a grid barrier's first wait and of the later ones (wtri_topk.cu).
+uint32_t first_wait_limit();
+uint32_t later_wait_limit();
+
 // Shared launch helpers.
 inline unsigned int ceil_div_u(int64_t a, int64_t b) { return (unsigned int)((a + b - 1) / b); }
 int sm_count();  // of the current device

@@ -126,9 +126,10 @@ struct Query {
     // Weights are positive fp32 bit patterns (a float-weight graph), not
     // integers: the means and reported values read them as floats.
     int32_t fw;
-    // Polls of the first grid-barrier wait (WAIT_LIMIT in production; tests
-    // lower it to take the timeout path).
+    // Polls of the first grid-barrier wait and of every later one (WAIT_LIMIT
+    // in production; tests lower them to take the timeout paths).
     uint32_t wait_first;
+    uint32_t wait_later;
 };
 
 // Where a query's results go.
@@ -457,8 +458,9 @@ struct BlockTeam {
 // barrier: every block's
 // first thread arrives at a counter in the query's state and polls it up to
 // a limit.  The first limit is the query's wait_first; when it runs out the
-// query is marked timed out and the block waits on with the full limit, so
-// that the blocks stay in step; only when that runs out too does it leave.
+// query is marked timed out and the block waits on with the full limit
+// (wait_later), so that the blocks stay in step; only when that runs out too
+// does it leave.  From then on no barrier of the team can complete.
 template <int TB_>
 struct GridTeam {
     static constexpr int TB = TB_;
@@ -488,9 +490,9 @@ struct GridTeam {
             for (uint32_t i = 0; i < limit && !there; i++) there = (int32_t)(arrivals(q) - target) >= 0;
             if (!there) {
                 atomicOr(&q.st->err, DEV_ERR_TIMEOUT);
-                for (uint32_t i = 0; i < WAIT_LIMIT && !there; i++) there = (int32_t)(arrivals(q) - target) >= 0;
+                for (uint32_t i = 0; i < q.wait_later && !there; i++) there = (int32_t)(arrivals(q) - target) >= 0;
             }
-            limit = WAIT_LIMIT;
+            limit = q.wait_later;
             if (!there) *gone = 1;
             __threadfence();
         }
@@ -1303,11 +1305,13 @@ __device__ __forceinline__ void sort_and_write(const Part<TB>& B, const Query& q
 
 // The k best candidates in order, and the status word.  k <= SORT_MAX: one
 // block sorts them; above, every warp of the team ranks candidates by
-// counting those before them (a grid team).
+// counting those before them (a grid team), and the status is written after
+// one more barrier, when every rank is.  False: a barrier gave up.
 template <int P, class Team>
-__device__ void finish(const Query& q, const Out& o, Team& T, SelectSmem& S, SortSmem& R) {
+__device__ bool finish(const Query& q, const Out& o, Team& T, SelectSmem& S, SortSmem& R) {
     const uint32_t K = (uint32_t)q.k;
     const Part<Team::TB>& B = T.part;
+    int32_t status = 0;
     if (T.leader()) {
         read_state<Team::TB>(B, q, S);
         const uint32_t err = S.err;
@@ -1320,19 +1324,16 @@ __device__ void finish(const Query& q, const Out& o, Team& T, SelectSmem& S, Sor
             }
             if (n > K && (n > SORT_MAX || K > SORT_MAX)) n = keep_first_ties<Team::TB>(B, q.ckey, q.ctri, n, K, T0, S);
         }
-        if (B.tid() == 0) {
-            // a timeout first: an overflow that follows it is its consequence
-            int32_t status = (int32_t)min(n, K);
-            if (err & DEV_ERR_TIMEOUT) status = WTRI_ETIMEOUT;
-            else if (err & DEV_ERR_OVERFLOW) status = WTRI_ENOMEM;
-            else if (err) status = WTRI_ECUDA;
-            *o.count = status;
-            *(volatile uint32_t*)&q.st->kept = n;
-        }
+        // a timeout first: an overflow that follows it is its consequence
+        status = (int32_t)min(n, K);
+        if (err & DEV_ERR_TIMEOUT) status = WTRI_ETIMEOUT;
+        else if (err & DEV_ERR_OVERFLOW) status = WTRI_ENOMEM;
+        else if (err) status = WTRI_ECUDA;
+        if (B.tid() == 0) *(volatile uint32_t*)&q.st->kept = n;
         if (K <= SORT_MAX) sort_and_write<P, Team::TB>(B, q, o, n, R);
     }
     if (Team::GRID && K > SORT_MAX) {
-        if (!T.sync(q)) return;
+        if (!T.sync(q)) return false;
         const uint32_t n = *(volatile uint32_t*)&q.st->kept;
         const int lane = threadIdx.x & 31;
         for (int64_t i = T.warp(); i < (int64_t)n; i += T.warps()) {
@@ -1344,11 +1345,16 @@ __device__ void finish(const Query& q, const Out& o, Team& T, SelectSmem& S, Sor
             for (int s = 16; s > 0; s >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, s);
             if (lane == 0) write_rank<P>(q, o, rank, ki, ti.x, ti.y, ti.z);
         }
+        if (!T.sync(q)) return false;
     }
+    if (T.leader() && B.tid() == 0) *o.count = status;
+    return true;
 }
 
 // ---------------------------------------------------------------------------
-// The whole sweep.
+// The whole sweep.  The status says WTRI_ETIMEOUT until the answer is complete,
+// so a team whose blocks give up (false) leaves that; a block that gives up
+// has done its work up to that barrier, and the others cannot pass the next.
 // ---------------------------------------------------------------------------
 template <int TB>
 struct SweepSmem {
@@ -1360,7 +1366,8 @@ struct SweepSmem {
 };
 
 template <int P, bool SAMPLED, class Team>
-__device__ void sweep(const DevGraph& G, const Query& q, const Out& o, Team& T, SweepSmem<Team::TB>& S) {
+__device__ bool sweep(const DevGraph& G, const Query& q, const Out& o, Team& T, SweepSmem<Team::TB>& S) {
+    if (Team::GRID && T.leader() && T.part.tid() == 0) *o.count = WTRI_ETIMEOUT;
     const bool oriented = P == P_MIN && !SAMPLED && q.nshards <= 1;
     const int64_t total = q.total_dev ? __ldg(q.total_dev) : q.total;
     // rounds of at most item_cap edges (an item each); the filtered p = -inf
@@ -1384,27 +1391,27 @@ __device__ void sweep(const DevGraph& G, const Query& q, const Out& o, Team& T, 
             if (hi - lo <= min(WARP_EDGES, T.warps() * 4)) edges_by_warp<P, SAMPLED>(G, q, tau, lo, hi, par, T, tb);
             else edges_by_thread<P, SAMPLED>(G, q, tau, lo, hi, par, T, tb);
         }
-        if (!T.sync(q)) return;
+        if (!T.sync(q)) return false;
         if (items) {
             if constexpr (P == P_MIN && !SAMPLED) {
                 if (oriented) item_wedges<P, false, true>(G, q, tau, par, T, tb);
             }
             if (!oriented) item_wedges<P, SAMPLED, false>(G, q, tau, par, T, tb);
-            if (!T.sync(q)) return;
+            if (!T.sync(q)) return false;
         }
         if (T.leader()) {
             if (T.part.tid() == 0) *(volatile unsigned long long*)&q.st->items[par ^ 1] = 0;
             const int64_t grow = select_round<Team::TB>(T.part, q, S.sel);
             next_range<P, SAMPLED>(T.part.tid(), G, q, hi, min(size * grow, cap), total, S.sel.err != 0);
         }
-        if (!T.sync(q)) return;
+        if (!T.sync(q)) return false;
         size = *(volatile long long*)&q.st->size;
         tau = ld_volatile_u64(&q.st->tau);
         lo = *(volatile long long*)&q.st->lo;
         hi = *(volatile long long*)&q.st->hi;
     }
     flush_tally(q, tb);
-    finish<P>(q, o, T, S.sel, S.sort);
+    return finish<P>(q, o, T, S.sel, S.sort);
 }
 
 template <int P, bool SAMPLED>
@@ -1481,7 +1488,7 @@ inline char* query_carve(Query& q, char* p, uint32_t cap, int64_t item_cap) {
     q.cap = cap;
     q.item_cap = item_cap;
     q.nshards = 1;
-    q.wait_first = WAIT_LIMIT;
+    q.wait_first = q.wait_later = WAIT_LIMIT;
     return p;
 }
 // Items of a graph's query: at most one per edge of a round.

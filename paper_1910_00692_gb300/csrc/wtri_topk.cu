@@ -7,10 +7,13 @@
 namespace wtri {
 namespace {
 
-// Poll limit of a sweep's first grid-barrier wait (a test hook lowers it; see
-// wtri_debug_set_wait_limit).
-std::atomic<uint32_t> g_stage_wait{WAIT_LIMIT};
-uint32_t stage_wait_limit() { return g_stage_wait.load(std::memory_order_relaxed); }
+// Poll limits of a grid barrier's first wait and of the later ones (test hooks
+// lower them; see wtri_debug_set_wait_limits).
+std::atomic<uint32_t> g_wait_first{WAIT_LIMIT}, g_wait_later{WAIT_LIMIT};
+
+uint32_t poll_limit(int64_t polls) {
+    return polls < 0 ? WAIT_LIMIT : (uint32_t)std::min<int64_t>(polls, UINT32_MAX);
+}
 
 // The fields of a query's sweep that come from its graph and call.
 void set_sweep(Query& q, const wtri_graph* g, int32_t k) {
@@ -20,7 +23,8 @@ void set_sweep(Query& q, const wtri_graph* g, int32_t k) {
     q.growth = g->tune.growth;
     q.t_short = g->tune.t_short;
     q.fw = g->d.fw;
-    q.wait_first = stage_wait_limit();
+    q.wait_first = first_wait_limit();
+    q.wait_later = later_wait_limit();
 }
 
 template <int P>
@@ -412,6 +416,9 @@ int run_sample(const wtri_graph* g, int32_t k, int64_t nsamples, uint64_t seed, 
 
 }  // namespace
 
+uint32_t first_wait_limit() { return g_wait_first.load(std::memory_order_relaxed); }
+uint32_t later_wait_limit() { return g_wait_later.load(std::memory_order_relaxed); }
+
 int topk_device(const wtri_graph* g, int pcode, int32_t k, wtri_tri* d_tris, double* d_weight,
                 int32_t* d_count, cudaStream_t stream, int retry_scale, int shard, int nshards,
                 unsigned long long* d_keys, double gp) {
@@ -592,6 +599,11 @@ extern "C" WTRI_API int wtri_query_bytes(int on, int reset, unsigned long long* 
 }
 
 extern "C" WTRI_API int wtri_debug_set_wait_limit(int64_t polls) {
-    wtri::g_stage_wait.store(polls < 0 ? wtri::WAIT_LIMIT : (uint32_t)std::min<int64_t>(polls, UINT32_MAX));
+    return wtri_debug_set_wait_limits(polls, -1);
+}
+
+extern "C" WTRI_API int wtri_debug_set_wait_limits(int64_t first, int64_t later) {
+    wtri::g_wait_first.store(wtri::poll_limit(first));
+    wtri::g_wait_later.store(wtri::poll_limit(later));
     return WTRI_OK;
 }

@@ -442,6 +442,8 @@ int run_wedge_topk(const wtri_graph* g, int32_t k, int64_t nsamples, uint64_t se
     Query q;
     unsigned long long* table = (unsigned long long*)query_carve(q, p, cap, 0);
     q.k = k;
+    q.wait_first = first_wait_limit();
+    q.wait_later = later_wait_limit();
     WTRI_CUDA(cudaMemsetAsync(q.st, 0, sizeof(QState), s));
     WTRI_CUDA(cudaMemsetAsync(W.err, 0, 4, s));
     WTRI_CUDA(cudaMemsetAsync(table, 0xff, hb, s));

@@ -120,6 +120,8 @@ def lib():
                                     ctypes.POINTER(i32), ctypes.POINTER(u64), ctypes.POINTER(u64)]
     L.wtri_debug_set_wait_limit.argtypes = [i64]
     L.wtri_debug_set_wait_limit.restype = ctypes.c_int
+    L.wtri_debug_set_wait_limits.argtypes = [i64, i64]
+    L.wtri_debug_set_wait_limits.restype = ctypes.c_int
     L.wtri_server_set_option.argtypes = [vp, ctypes.c_int, i64]
     L.wtri_server_set_option.restype = ctypes.c_int
     L.wtri_server_free.argtypes = [vp]
@@ -469,6 +471,12 @@ def debug_set_wait_limit(polls: int):
     query kernel's first grid-barrier wait; 0: it times out at once;
     negative: the default)."""
     _check(lib().wtri_debug_set_wait_limit(int(polls)))
+
+
+def debug_set_wait_limits(first: int, later: int):
+    """wtri_debug_set_wait_limits: the polls of the first grid-barrier wait and
+    of every later one (0 and 0: every block leaves at the first barrier)."""
+    _check(lib().wtri_debug_set_wait_limits(int(first), int(later)))
 
 
 def p_values():

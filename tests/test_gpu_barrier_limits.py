@@ -54,3 +54,68 @@ def test_first_wait_of_a_few_polls(scaled, p, first):
         wt.debug_set_wait_limit(-1)
         d.set_tune(64, 8, 32)
     assert math.isinf(PS[0])
+
+
+def _calls(d, torch):
+    """Every call whose kernel has a grid barrier: name, the call."""
+    dev = torch.device("cuda:0")
+
+    def device(fn, k):
+        t = torch.zeros((k, 3), dtype=torch.int32, device=dev)
+        w = torch.zeros(k, dtype=torch.float64, device=dev)
+        c = torch.full((1,), 7, dtype=torch.int32, device=dev)  # what an earlier call left
+        fn(d, 1.0, k, t, w, c)
+        torch.cuda.synchronize()
+        if int(c.item()) < 0:
+            raise wt.WtriError(int(c.item()), "device status")
+        return t[:int(c.item())].cpu().numpy(), w[:int(c.item())].cpu().numpy()
+
+    def served(p, k):
+        s = wt.Server(8 << 30, 16)
+        try:
+            gid = s.add_graph(d)
+            ticket = s.submit(gid, p, k)
+            while True:
+                r = s.poll(ticket, k)
+                if r is not None:
+                    return r[:2]
+        finally:
+            s.free()
+
+    yield from ((f"topk p={p} k={k}", lambda p=p, k=k: d.topk(p, k)) for p in PS + [-1.0] for k in (100, 2100))
+    yield "device", lambda: device(wt.topk_device, 100)
+    yield "device, ranked by counting", lambda: device(wt.topk_device, 2100)
+    yield "noalloc", lambda: device(wt.topk_device_noalloc, 100)
+    yield "shard", lambda: wt.topk_shard(d, 1.0, 100, 1, 2)
+    yield "sampled", lambda: d.sample_topk(1.0, 100, 50_000, 3)
+    yield "wedges, ranked by counting", lambda: wt.wedge_topk(d, 1.0, 2100, 50_000, 3)
+    yield "batch", lambda: wt.topk_batch([d, d, d], [1.0, -math.inf, 2.0], [100, 100, 2100])[0]
+    yield "server", lambda: served(-math.inf, 100)
+    yield "cliques", lambda: wt.sample_cliques(d, 4, 1.0, 100, 20_000, 3)
+
+
+def test_waits_that_run_out_for_good(scaled):
+    """No block waits for another: each leaves at its first barrier (later
+    limit 0) or as soon as one is a few polls late.  The status says so,
+    whatever the count held, and the same call is exact afterwards."""
+    torch = pytest.importorskip("torch")
+    _, d, _ = scaled
+    for name, call in _calls(d, torch):
+        wt.debug_set_wait_limits(-1, -1)
+        before = call()
+        try:
+            wt.debug_set_wait_limits(0, 0)
+            with pytest.raises(wt.WtriError) as ei:
+                call()
+            assert ei.value.code == ETIMEOUT, name
+            for first, later in ((50, 0), (0, 50), (50, 50), (400, 400), (3000, 10)):
+                wt.debug_set_wait_limits(first, later)
+                try:
+                    got = call()
+                except wt.WtriError as e:
+                    assert e.code == ETIMEOUT, name
+                else:
+                    assert all((a == b).all() for a, b in zip(got, before)), name
+        finally:
+            wt.debug_set_wait_limits(-1, -1)
+        assert all((a == b).all() for a, b in zip(call(), before)), name
