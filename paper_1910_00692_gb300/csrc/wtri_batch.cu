@@ -20,10 +20,10 @@ namespace {
 
 constexpr int PT = 512;                   // threads of a part
 constexpr int PARTS = TGRID / PT;         // parts of a block
-// Items, shared evenly by the SMs: a round of a query takes at most its share
-// (edges).  A server's batches keep to the bytes its admission counts.
+// Items, shared evenly by the SMs: a query has those of its SMs.  A server's batches keep to the bytes its admission counts.
 constexpr int64_t POOL_SERVED = 180000;
 constexpr int64_t POOL_BATCH = 640000;
+static_assert(POOL_BATCH + (1 << 18) < (1 << (64 - ITEM_SHIFT)), "a team's items, and 32 more per warp, are counted in 20 bits");
 constexpr int TEAMS = 64;                 // most teams of a launch
 constexpr int64_t BATCH_FIRST = 64;       // first round of a batched query (edges)
 constexpr int32_t BATCH_GROWTH = 8;       // growth of its rounds

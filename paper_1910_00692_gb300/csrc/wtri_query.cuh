@@ -36,7 +36,8 @@
 //   A  edges: the checks and searches of every edge of the round (a warp per
 //      edge in small rounds, a thread per edge in large ones); an edge with
 //      a long live range leaves it as an item, with the running number of
-//      wedges before it;
+//      wedges before it (rounds of more edges than items, once the threshold
+//      hardly moves: most live ranges are scanned by their warp);
 //   B  wedges: the items' wedges, numbered through, are dealt to the team 32
 //      at a time, whatever the items' lengths;
 //   C  select (one block): the k-th key, in-place compaction, the new tau,
@@ -62,7 +63,7 @@ namespace {
 constexpr int TGRID = 1024;         // threads of a block of the grid team (one block per SM)
 constexpr int SORT_MAX = 2048;      // largest k ranked by a sort in shared memory
 constexpr uint32_t WAIT_LIMIT = 1u << 26;  // bounded polling of the grid barrier
-constexpr int64_t ITEM_CAP = 1 << 18;      // edges of one round (at most one item each)
+constexpr int64_t ITEM_CAP = 1 << 18;      // most items
 constexpr int64_t WARP_EDGES = 4096;       // largest round that takes a warp per edge
 constexpr int64_t MIN_FLAT = 8192;         // largest p = -inf round that numbers its entries through
 
@@ -504,7 +505,8 @@ struct GridTeam {
 // ---------------------------------------------------------------------------
 // Items.
 // ---------------------------------------------------------------------------
-constexpr int ITEM_SHIFT = 44;  // item count above, wedge count below (both fit: at most 2^18 items)
+constexpr int ITEM_SHIFT = 44;  // item count above (20 bits), wedge count below
+static_assert(ITEM_CAP + (1 << 18) < (1 << (64 - ITEM_SHIFT)), "the items and 32 more per warp are counted in 20 bits");
 constexpr unsigned long long WEDGE_MASK = (1ull << ITEM_SHIFT) - 1;
 
 __device__ __forceinline__ void put_item(const Query& q, uint32_t slot, unsigned long long base, const Item& it) {
@@ -516,7 +518,8 @@ __device__ __forceinline__ void put_item(const Query& q, uint32_t slot, unsigned
     q.ibase[slot] = base;
 }
 
-// Every lane of a warp: the lanes with len > 0 leave their item.
+// Every lane of a warp: the lanes with len > 0 leave their item.  (For rounds of
+// fewer edges than there are items.)
 __device__ __forceinline__ void push_items(const Query& q, int par, int64_t len, const Item& it) {
     const int lane = threadIdx.x & 31;
     const uint32_t has = __ballot_sync(0xffffffffu, len > 0);
@@ -534,6 +537,46 @@ __device__ __forceinline__ void push_items(const Query& q, int par, int64_t len,
     if (len > 0)
         put_item(q, (uint32_t)(old >> ITEM_SHIFT) + __popc(has & lanemask_below()), (old & WEDGE_MASK) + inc - mine,
                  it);
+}
+
+// Rounds of more edges than items: only live ranges above FLAT_SHORT are left
+// to phase B, while there is room, the others are scanned by their warp (see
+// scan_here).  The last slot stays free: whoever draws it leaves the wedges
+// before it there, the total of the items that were kept.  True: left.
+//
+// Such rounds are for sweeps that visit most of a graph.  Rounds cut to the
+// items' number, 2e8 edges at random on 5e7 vertices (86 triangles, k = 1,000)
+// took 764 rounds and 141 ms at p = 1, with the 46,592 items of the fixed
+// scratch 289; now 100 either way.  16, 64 or 256 as the limit: the same
+// there; on rows of 200 entries a shard takes 1.74, 1.62 and 2.83 ms.
+constexpr int64_t FLAT_SHORT = 64;
+
+__device__ __forceinline__ bool push_long(const Query& q, int par, int64_t len, const Item& it) {
+    const int lane = threadIdx.x & 31;
+    const bool lng = len > FLAT_SHORT;
+    const uint32_t has = __ballot_sync(0xffffffffu, lng);
+    if (!has) return false;
+    const uint32_t usable = (uint32_t)q.item_cap - 1;
+    unsigned long long old = 0;
+    if (lane == 0) old = ld_volatile_u64(&q.st->items[par]);
+    old = __shfl_sync(0xffffffffu, old, 0);
+    if ((uint32_t)(old >> ITEM_SHIFT) >= usable) return false;  // (a warp adds at most 32 past it: 20 bits hold the count)
+    unsigned long long inc = lng ? (unsigned long long)len : 0ull;
+    const unsigned long long mine = inc;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    if (lane == 31) old = atomicAdd(&q.st->items[par], ((unsigned long long)__popc(has) << ITEM_SHIFT) + inc);
+    old = __shfl_sync(0xffffffffu, old, 31);
+    const uint32_t slot = (uint32_t)(old >> ITEM_SHIFT) + __popc(has & lanemask_below());
+    const unsigned long long base = (old & WEDGE_MASK) + inc - mine;
+    if (!lng || slot > usable) return false;
+    q.ibase[slot] = base;
+    if (slot == usable) return false;
+    q.items[slot] = it;
+    return true;
 }
 
 // ---------------------------------------------------------------------------
@@ -569,6 +612,40 @@ __device__ __forceinline__ void wedge(const DevGraph& G, const Query& q, unsigne
         sort3(a, b, cc);
         append(q, key, a, b, cc);
     }
+}
+
+// The live ranges of a warp's 32 edges, scanned on the spot: their wedges
+// numbered through, 32 at a time.
+struct WarpItems {
+    Item it[32];
+    unsigned long long end[32];  // wedges up to and with each range
+};
+
+template <int P, bool SAMPLED>
+__device__ __forceinline__ void scan_here(const DevGraph& G, const Query& q, unsigned long long tau, int64_t len,
+                                          const Item& it, WarpItems& W, Tally& tb) {
+    const int lane = threadIdx.x & 31;
+    if (!__any_sync(0xffffffffu, len > 0)) return;
+    unsigned long long inc = (unsigned long long)len;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    const unsigned long long tot = __shfl_sync(0xffffffffu, inc, 31);
+    W.it[lane] = it;
+    W.end[lane] = inc;
+    __syncwarp();
+    for (unsigned long long e = lane; e < tot; e += 32) {
+        int k = 0;
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1)
+            if (W.end[k + s - 1] <= e) k += s;
+        const Item& x = W.it[k];
+        const int64_t j = x.j0 + (int64_t)(e - (k > 0 ? W.end[k - 1] : 0ull));
+        wedge<P, SAMPLED>(G, q, tau, x.r, x.w, x.x, x.y, x.dy, x.lb, x.ln, j, tb);
+    }
+    __syncwarp();
 }
 
 // Entry j of the scanned oriented row of the edge {a, b} at p = -inf; the
@@ -665,10 +742,11 @@ __device__ __forceinline__ void edges_by_warp(const DevGraph& G, const Query& q,
     }
 }
 
-// A thread per edge: large rounds, where most edges fail the edge bound.
+// A thread per edge: large rounds, where most edges fail the edge bound.  flat:
+// the round may have more live ranges than there are items.
 template <int P, bool SAMPLED, class Team>
 __device__ __forceinline__ void edges_by_thread(const DevGraph& G, const Query& q, unsigned long long tau, int64_t lo,
-                                                int64_t hi, int par, const Team& T, Tally& tb) {
+                                                int64_t hi, int par, bool flat, const Team& T, WarpItems& W, Tally& tb) {
     const int lane = threadIdx.x & 31;
     for (int64_t i0 = lo + T.warp() * 32; i0 < hi; i0 += T.warps() * 32) {
         const int64_t idx = i0 + lane;
@@ -705,10 +783,13 @@ __device__ __forceinline__ void edges_by_thread(const DevGraph& G, const Query& 
                     sv++;
                 }
                 if (!bad && su < eu && sv < ev) {
-                    const uint32_t umax = (uint32_t)__ldg(G.wwt + su), vmax = (uint32_t)__ldg(G.wwt + sv);
-                    tb.add(8);
+                    uint32_t umax = 0, vmax = 0;
+                    if (tau != 0) {  // (without a threshold nothing is bounded: two loads saved)
+                        umax = (uint32_t)__ldg(G.wwt + su), vmax = (uint32_t)__ldg(G.wwt + sv);
+                        tb.add(8);
+                    }
                     const Line<P> lu(q, tau, w, vmax);  // along u's list
-                    if (!lu.fails(umax)) {
+                    if (tau == 0 || !lu.fails(umax)) {
                         int64_t nu = eu - su, nv = ev - sv;
                         if (tau != 0) {  // both live ranges
                             const Line<P> lv(q, tau, w, umax);
@@ -745,7 +826,12 @@ __device__ __forceinline__ void edges_by_thread(const DevGraph& G, const Query& 
                 }
             }
         }
-        push_items(q, par, n, it);
+        if (!flat) {
+            push_items(q, par, n, it);
+        } else {
+            if (push_long(q, par, n, it)) n = 0;
+            scan_here<P, SAMPLED>(G, q, tau, n, it, W, tb);
+        }
     }
 }
 
@@ -906,10 +992,11 @@ __device__ __forceinline__ void min_edges_filtered(const DevGraph& G, const Quer
 // ---------------------------------------------------------------------------
 template <int P, bool SAMPLED, bool ORIENTED, class Team>
 __device__ __forceinline__ void item_wedges(const DevGraph& G, const Query& q, unsigned long long tau, int par,
-                                            const Team& T, Tally& tb) {
+                                            bool flat, const Team& T, Tally& tb) {
     const unsigned long long ctr = *(volatile const unsigned long long*)&q.st->items[par];
-    const int64_t cnt = (int64_t)(ctr >> ITEM_SHIFT), tot = (int64_t)(ctr & WEDGE_MASK);
-    if (cnt > q.item_cap) return;
+    const int64_t drawn_ = (int64_t)(ctr >> ITEM_SHIFT), cnt = min(drawn_, flat ? q.item_cap - 1 : q.item_cap);
+    const int64_t tot = cnt == drawn_ ? (int64_t)(ctr & WEDGE_MASK) : (int64_t)q.ibase[cnt];
+    if (!flat && cnt != drawn_) return;
     const int lane = threadIdx.x & 31;
     const int64_t chunks = (tot + 31) >> 5, per = (chunks + T.warps() - 1) / T.warps();
     const int64_t beg = T.warp() * per * 32, end = min(tot, beg + per * 32);
@@ -1198,17 +1285,24 @@ __device__ uint32_t keep_first_ties(const Part<TB>& B, unsigned long long* ckey,
 // resolves them by the vertex triple.  Returns how much larger the next round
 // may be: `growth`, or less where rounds as productive as this one would
 // fill half of the free candidate slots (small buffers: a batched query at
-// p = -inf overflowed its 16,384 slots at a fixed growth of 8).
+// p = -inf overflowed its 16,384 slots at a fixed growth of 8); and whether it
+// may have more edges than there are items: where the threshold hardly moved,
+// or there is none yet, a select earlier would prune little.
+struct Growth {
+    int64_t times;
+    bool wide;
+};
+
 template <int TB>
-__device__ int64_t select_round(const Part<TB>& B, const Query& q, SelectSmem& S) {
+__device__ Growth select_round(const Part<TB>& B, const Query& q, SelectSmem& S) {
     const int64_t growth = q.growth;
     read_state<TB>(B, q, S);
     const uint32_t n = S.n, old = S.old;
-    if (S.err || n == old) return growth;
+    if (S.err || n == old) return Growth{growth, true};
     const int64_t added = n - old;
     if (n < (uint32_t)q.k) {
         if (B.tid() == 0) *(volatile uint32_t*)&q.st->selected = n;  // all of them stay
-        return max(int64_t(1), min(growth, (int64_t)(q.cap - n) / (2 * added)));
+        return Growth{max(int64_t(1), min(growth, (int64_t)(q.cap - n) / (2 * added))), true};
     }
     const unsigned long long T = kth_key<TB>(B, q.ckey, n, (uint32_t)q.k, S);
     const uint32_t kept = compact<TB>(B, q.ckey, q.ctri, n, [=](unsigned long long k, const int4&) { return k >= T; }, S);
@@ -1218,7 +1312,7 @@ __device__ int64_t select_round(const Part<TB>& B, const Query& q, SelectSmem& S
         if (T > q.st->tau) *(volatile unsigned long long*)&q.st->tau = T;
     }
     B.sync();
-    return max(int64_t(1), min(growth, (int64_t)(q.cap - kept) / (2 * added)));
+    return Growth{max(int64_t(1), min(growth, (int64_t)(q.cap - kept) / (2 * added))), 8 * added <= q.k};
 }
 
 // The next round's range: [lo, lo + size) cut at the first edge whose bound
@@ -1362,6 +1456,7 @@ struct SweepSmem {
     union {
         SortSmem sort;
         MinProbe queue[TB / 32][MINQ];
+        WarpItems here[TB / 32];
     };
 };
 
@@ -1370,15 +1465,13 @@ __device__ bool sweep(const DevGraph& G, const Query& q, const Out& o, Team& T, 
     if (Team::GRID && T.leader() && T.part.tid() == 0) *o.count = WTRI_ETIMEOUT;
     const bool oriented = P == P_MIN && !SAMPLED && q.nshards <= 1;
     const int64_t total = q.total_dev ? __ldg(q.total_dev) : q.total;
-    // rounds of at most item_cap edges (an item each); the filtered p = -inf
-    // rounds leave none
-    const int64_t cap = oriented ? INT64_MAX / 16 : q.item_cap;
-    int64_t size = min(q.first, min(cap, q.item_cap)), lo = 0, hi = min(total, size);
+    int64_t size = min(q.first, q.item_cap), lo = 0, hi = min(total, size);
     unsigned long long tau = 0;
     Tally tb;
     tb.on = q.qbytes != nullptr;
     for (int par = 0; lo < hi; par ^= 1) {
         bool items = true;
+        const bool flat = hi - lo > q.item_cap;  // more edges than items
         if constexpr (P == P_MIN && !SAMPLED) {
             if (oriented) {
                 items = hi - lo <= min(MIN_FLAT, q.item_cap);
@@ -1389,20 +1482,21 @@ __device__ bool sweep(const DevGraph& G, const Query& q, const Out& o, Team& T, 
         }
         if (!oriented) {
             if (hi - lo <= min(WARP_EDGES, T.warps() * 4)) edges_by_warp<P, SAMPLED>(G, q, tau, lo, hi, par, T, tb);
-            else edges_by_thread<P, SAMPLED>(G, q, tau, lo, hi, par, T, tb);
+            else edges_by_thread<P, SAMPLED>(G, q, tau, lo, hi, par, flat, T, S.here[T.part.tid() >> 5], tb);
         }
         if (!T.sync(q)) return false;
         if (items) {
             if constexpr (P == P_MIN && !SAMPLED) {
-                if (oriented) item_wedges<P, false, true>(G, q, tau, par, T, tb);
+                if (oriented) item_wedges<P, false, true>(G, q, tau, par, false, T, tb);
             }
-            if (!oriented) item_wedges<P, SAMPLED, false>(G, q, tau, par, T, tb);
+            if (!oriented) item_wedges<P, SAMPLED, false>(G, q, tau, par, flat, T, tb);
             if (!T.sync(q)) return false;
         }
         if (T.leader()) {
             if (T.part.tid() == 0) *(volatile unsigned long long*)&q.st->items[par ^ 1] = 0;
-            const int64_t grow = select_round<Team::TB>(T.part, q, S.sel);
-            next_range<P, SAMPLED>(T.part.tid(), G, q, hi, min(size * grow, cap), total, S.sel.err != 0);
+            const Growth grow = select_round<Team::TB>(T.part, q, S.sel);
+            const int64_t cap = oriented || grow.wide ? INT64_MAX / 1024 : q.item_cap;
+            next_range<P, SAMPLED>(T.part.tid(), G, q, hi, min(size * grow.times, cap), total, S.sel.err != 0);
         }
         if (!T.sync(q)) return false;
         size = *(volatile long long*)&q.st->size;
