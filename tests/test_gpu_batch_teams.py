@@ -1,0 +1,53 @@
+"""How a batched call deals the SMs: equal queries that share them unevenly,
+more queries than one launch has teams (k above what a part of a block ranks
+needs one each), and both beside small ones; with the graph launch built anew
+and updated."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from wtri_testutil import PS, assert_topk_equal
+
+pytestmark = pytest.mark.gpu
+
+wt = pytest.importorskip("paper_1910_00692_gb300")
+
+SIZES = [(120, 500), (400, 3000), (1500, 12_000), (6000, 60_000)]
+
+
+@pytest.fixture(scope="module")
+def pool():
+    gs = [synth.scaled_mid_graph(n, m, seed=70 + i) for i, (n, m) in enumerate(SIZES)]
+    ds = [wt.build_csr(g.n, g.u, g.v, g.w) for g in gs]
+    wants = {(i, p): oracle.topk(g.n, g.u, g.v, g.w, p, 4100) for i, g in enumerate(gs) for p in PS}
+    yield ds, wants
+    for d in ds:
+        d.free()
+
+
+def _check(pool, queries):
+    ds, wants = pool
+    for call in range(2):
+        res = wt.topk_batch([ds[i] for i, _, _ in queries], [p for _, p, _ in queries], [k for _, _, k in queries])
+        for (i, p, k), (tris, wts) in zip(queries, res):
+            w = wants[i, p]
+            part = {"tri": w["tri"][:k], "value": w["value"][:k], "count": min(k, w["count"])}
+            assert_topk_equal(tris, wts, part, p, f"call={call} graph={i} p={p} k={k}")
+
+
+# one k each; then k above 2,048, so that every query has a team: fewer than
+# there are SMs, one too many for 64, two launches' worth and more
+@pytest.mark.parametrize("count", [1, 2, 16, 64, 65, 153, 330])
+@pytest.mark.parametrize("k", [500, 2100])
+def test_equal_queries(pool, count, k):
+    _check(pool, [(2, PS[count % 5], k)] * count)
+
+
+def test_more_teams_than_a_launch_has_beside_parts(pool):
+    rng = np.random.default_rng(8)
+    queries = [(i % 4, PS[i % 5], 2100) for i in range(70)]
+    queries += [(int(rng.integers(0, 4)), PS[int(rng.integers(0, 5))], int(rng.integers(1, 1001))) for _ in range(300)]
+    queries = [queries[i] for i in rng.permutation(len(queries))]
+    _check(pool, queries)
+    _check(pool, queries[:200] + [(3, p, 4100) for p in PS])
