@@ -25,7 +25,9 @@ constexpr int PARTS = TGRID / PT;         // parts of a block
 constexpr int64_t POOL_SERVED = 180000;
 constexpr int64_t POOL_BATCH = 640000;
 static_assert(POOL_BATCH + (1 << 18) < (1 << (64 - ITEM_SHIFT)), "a team's items, and 32 more per warp, are counted in 20 bits");
-constexpr int TEAMS = 64;                 // most teams of a launch
+// Most teams of a launch: one per SM.  (With 64, 100 equal queries left 36 to the
+// parts: 200,000 random edges each, p = 1, k = 1,000, 8.5 ms; now 5.4.)
+constexpr int TEAMS = 152;
 constexpr int64_t BATCH_FIRST = 64;       // first round of a batched query (edges)
 constexpr int32_t BATCH_GROWTH = 8;       // growth of its rounds
 
@@ -87,8 +89,12 @@ __global__ void __launch_bounds__(TGRID, 1) k_sweep_batch(BatchDev B, TeamList L
     __shared__ DevGraph G;
     __shared__ Query q;
     __shared__ Out o;
-    int t = 0;
-    while (t < L.n && (int)blockIdx.x >= L.blk[t + 1]) t++;
+    int t = 0;  // this block's team: the first that ends after it
+    for (int n = L.n; n > 0;) {
+        const int h = n / 2;
+        if ((int)blockIdx.x >= L.blk[t + h + 1]) t += h + 1, n -= h + 1;
+        else n = h;
+    }
     if (t < L.n) {
         const int32_t qi = L.qi[t];
         const uint32_t blk0 = (uint32_t)L.blk[t], nblk = (uint32_t)(L.blk[t + 1] - L.blk[t]);
@@ -154,10 +160,13 @@ __global__ void __launch_bounds__(TGRID, 1) k_sweep_batch(BatchDev B, TeamList L
 // its heaviest edges), 117 at 2e7; on 152 SMs 64-97.  The minimum reads the
 // rows of a share of all edges: 348 us on one SM at 1e4 edges, 1,151 at 5e4,
 // 1,289 at 2e5, 5,881 at 5e6, 13,990 at 2e7; on 152 SMs 298 at 2e7.
-double part_us(int pcode, int64_t m) {
-    const double x = (double)m;
-    if (pcode != P_MIN) return 150.0 + 100.0 * std::min(1.0, x / 2e5);
-    return 300.0 + 900.0 * std::min(1.0, x / 5e4) + 1200.0 * std::min(1.0, x / 2e5) + 1.3e-3 * x;
+// Above k = 2,048 (SORT_MAX) the selects and the ranking take about 1 us per
+// result more (304 queries of k = 1,000 / 4,096 / 8,192 on a part each: 1.1 /
+// 4.8 / 7.4 ms at p = 1, 4.3 / 9.1 / 13.9 at p = -inf).
+double part_us(int pcode, int64_t m, int32_t k) {
+    const double x = (double)m, rank = k > SORT_MAX ? (double)k : 0.0;
+    if (pcode != P_MIN) return 150.0 + 100.0 * std::min(1.0, x / 2e5) + rank;
+    return 300.0 + 900.0 * std::min(1.0, x / 5e4) + 1200.0 * std::min(1.0, x / 2e5) + 1.3e-3 * x + rank;
 }
 
 size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -177,7 +186,6 @@ struct wtri_batch_plan {
     std::vector<wtri::DevGraph> hg;
     std::vector<int32_t> pcodes;  // nq, and after them the statuses as they start: one upload
     std::vector<int32_t> ks, tshort;
-    std::vector<int32_t> alone;  // queries with a launch of their own (k above what a part ranks, no team left)
     std::vector<int32_t> order;  // the queries answered by parts, largest first
     wtri::TeamList teams;
     std::vector<uint32_t> caps;
@@ -200,8 +208,8 @@ uint32_t batch_query_cap(int32_t k, int64_t m) {
 }
 
 // Deals the SMs: a query whose expected time on one part is well above an even
-// share of the whole batch (or that has more results than a part ranks) gets
-// a team of SMs in proportion to its work, the rest are left to the parts.
+// share of the whole batch gets a team of SMs in proportion to its work, the
+// rest are left to the parts.
 // The teams' ends are the running sum of their shares, rounded: sizes rounded
 // up each gave 16 equal queries 15 teams of 10 SMs and one of two, and of 64
 // equal ones 50 teams of three, 14 left to the parts (200,000 random edges
@@ -210,13 +218,10 @@ static void plan_teams(BatchPlan* P) {
     const int nq = P->nq, sms = sm_count();
     std::vector<double> us((size_t)nq);
     double total = 0.0;
-    for (int i = 0; i < nq; i++) total += us[(size_t)i] = part_us(P->pcodes[(size_t)i], P->hg[(size_t)i].m);
+    for (int i = 0; i < nq; i++) total += us[(size_t)i] = part_us(P->pcodes[(size_t)i], P->hg[(size_t)i].m, P->ks[(size_t)i]);
     std::vector<int32_t> by((size_t)nq);
     for (int i = 0; i < nq; i++) by[(size_t)i] = i;
-    std::stable_sort(by.begin(), by.end(), [&](int32_t a, int32_t b) {
-        const bool ka = P->ks[(size_t)a] > SORT_MAX, kb = P->ks[(size_t)b] > SORT_MAX;
-        return ka != kb ? ka : us[(size_t)a] > us[(size_t)b];
-    });
+    std::stable_sort(by.begin(), by.end(), [&](int32_t a, int32_t b) { return us[(size_t)a] > us[(size_t)b]; });
     P->teams.n = 0;
     P->teams.blk[0] = 0;
     P->order.clear();
@@ -224,12 +229,7 @@ static void plan_teams(BatchPlan* P) {
     double end = 0.0;
     for (int32_t i : by) {
         const int t = P->teams.n, used = P->teams.blk[t];
-        const bool must = P->ks[(size_t)i] > SORT_MAX;
-        if (must || (us[(size_t)i] > 1.5 * share && us[(size_t)i] > 150.0 && t < TEAMS && used < sms)) {
-            if (t == TEAMS || used == sms) {  // no team left: a launch of its own
-                P->alone.push_back(i);
-                continue;
-            }
+        if (us[(size_t)i] > 1.5 * share && us[(size_t)i] > 150.0 && t < TEAMS && used < sms) {
             end += us[(size_t)i] / (PARTS * share);
             P->teams.qi[t] = i;
             P->teams.blk[t + 1] = (int16_t)std::min(sms, std::max(used + 1, (int)(end + 0.5)));
@@ -268,7 +268,7 @@ BatchPlan* batch_plan_create(const wtri_graph* const* gs, const int32_t* pcodes,
         off = al256(off + bytes);
         return o;
     };
-    P->o_st = take(sizeof(QState) * ((size_t)P->teams.n + P->alone.size() + 1));
+    P->o_st = take(sizeof(QState) * (size_t)(P->teams.n + 1));
     P->o_cur = take(64);  // cleared together with the states
     P->o_key = take(8 * P->cand_total);
     P->o_tri = take(16 * P->cand_total);
@@ -337,7 +337,6 @@ int batch_plan_launch(BatchPlan* P, void* dbuf, cudaStream_t s, int use_graph) {
         c0 += P->caps[(size_t)i];
     }
     for (int t = 0; t < P->teams.n; t++) hq[(size_t)P->teams.qi[t]].st = st + t;
-    for (size_t j = 0; j < P->alone.size(); j++) hq[(size_t)P->alone[j]].st = st + P->teams.n + j;
     BatchDev Bd;
     Bd.graphs = (const DevGraph*)(B0 + P->o_g);
     Bd.queries = (const Query*)(B0 + P->o_q);
@@ -357,36 +356,23 @@ int batch_plan_launch(BatchPlan* P, void* dbuf, cudaStream_t s, int use_graph) {
         WTRI_CUDA(cudaMemcpyAsync((void*)Bd.order, P->order.data(), 4 * P->order.size(), cudaMemcpyHostToDevice, s));
     static std::atomic<uint64_t> done{0};
     WTRI_TRY(smem_optin((const void*)k_sweep_batch, (int)sizeof(BatchSmem), done));
-    // the teams, then each query left over as a team of the whole GPU
-    std::vector<TeamList> launches;
-    launches.push_back(P->teams);
-    for (int32_t i : P->alone) {
-        TeamList L{};
-        L.n = 1;
-        L.qi[0] = i;
-        L.blk[1] = (int16_t)sm_count();
-        launches.push_back(L);
-    }
     const size_t clear = P->o_cur + 64 - P->o_st;  // states of the teams, cursor
     auto launch_all = [&]() -> int {
         WTRI_CUDA(cudaMemsetAsync(B0 + P->o_st, 0, clear, s));
-        for (TeamList& L : launches) {
-            void* args[] = {&Bd, &L};
-            WTRI_CUDA(cudaLaunchCooperativeKernel((const void*)k_sweep_batch, dim3((unsigned)sm_count()), dim3(TGRID),
-                                                  args, sizeof(BatchSmem), s));
-        }
+        void* args[] = {&Bd, &P->teams};
+        WTRI_CUDA(cudaLaunchCooperativeKernel((const void*)k_sweep_batch, dim3((unsigned)sm_count()), dim3(TGRID), args,
+                                              sizeof(BatchSmem), s));
         return WTRI_OK;
     };
     int rc = WTRI_OK;
-    ProfScope ps("topk_batch", s, 0.0, (int)launches.size());
+    ProfScope ps("topk_batch", s, 0.0, 1);
     if (use_graph) {
         // The descriptors must have landed before the captured work refers
         // to them only through device pointers: that holds, the copies are
         // ordered on s before the graph launch.  The instantiated graph is
         // kept (per thread and device) and refreshed with
-        // cudaGraphExecUpdate when the next batch has the same launch
-        // topology (the same kinds of launch), so a repeated batch
-        // shape is instantiated once.
+        // cudaGraphExecUpdate for the next batch (always one memset and one
+        // launch).
         cudaGraph_t graph = nullptr;
         cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {

@@ -51,3 +51,39 @@ def test_more_teams_than_a_launch_has_beside_parts(pool):
     queries = [queries[i] for i in rng.permutation(len(queries))]
     _check(pool, queries)
     _check(pool, queries[:200] + [(3, p, 4100) for p in PS])
+
+
+@pytest.fixture(scope="module")
+def ties():
+    """Weights 1..3 only: most candidates tie, the vertex triple decides."""
+    g = synth.scaled_mid_graph(8000, 90_000, seed=77)
+    g.w = (1 + np.random.default_rng(6).integers(0, 3, g.m)).astype(np.int32)
+    d = wt.build_csr(g.n, g.u, g.v, g.w)
+    yield d, {p: oracle.topk(g.n, g.u, g.v, g.w, p, 65_536) for p in PS}
+    d.free()
+
+
+# On both sides of a sorted run (2,048), of two candidates per warp of the
+# whole GPU (9,728), of 32 runs, and the largest k; alone, in a team of a few
+# SMs, and on a part of one.
+@pytest.mark.parametrize("p", PS)
+def test_rankings_of_many(ties, p):
+    d, wants = ties
+    w = wants[p]
+
+    def check(got, k, ctx):
+        part = {"tri": w["tri"][:k], "value": w["value"][:k], "count": min(k, w["count"])}
+        assert_topk_equal(*got, part, p, f"p={p} k={k} {ctx}")
+
+    assert w["count"] == 65_536
+    for k in (2049, 4096, 4097, 9727, 9728, 9729, 9730, 63_488, 65_535, 65_536):
+        check(d.topk(p, k), k, "alone")
+    for k in (2049, 4097, 20_000):
+        for got in wt.topk_batch([d] * 20, [p] * 20, [k] * 20):
+            check(got, k, "team")
+    for k in (2049, 4096, 6145):
+        for got in wt.topk_batch([d] * 310, [p] * 310, [k] * 310):
+            check(got, k, "part")
+    ks = [65_536] + [50] * 400
+    for k, got in zip(ks, wt.topk_batch([d] * len(ks), [p] * len(ks), ks)):
+        check(got, k, "beside small ones")
