@@ -176,15 +176,17 @@ WTRI_API int wtri_topk_device(const wtri_graph* g, double p, int32_t k, wtri_tri
  * of wtri_topk_device.
  *
  * Scratch comes from one fixed array inside the library: about 28 MB
- * (1,048,576 candidate triangles and the scans of 46,592 edges) that every GPU
- * loading the library keeps until the process exits.  k above 16384 is
+ * (1,048,576 candidate triangles and 46,592 scans left to the whole GPU) that
+ * every GPU loading the library keeps until the process exits.  k above 16384 is
  * rejected with WTRI_EINVAL.  If a query produces more candidates than the
  * array holds, d_count receives WTRI_ENOMEM; use wtri_topk_device then.
- * All calls share the array (its status word is cleared at the start of
- * each call), so calls that overlap on the GPU, on different streams or
- * from different host threads, race: serialize them.  The first call on a
- * device looks up the array's device address with that device current;
- * make that first call before any stream capture.
+ * All calls share the array (its state is cleared at the start of each call).
+ * The library runs them one after another on the device, whatever streams and
+ * host threads they come from, except calls captured into a graph: those must
+ * not overlap another call (each would clear the other's state, and their
+ * blocks could wait for a minute before they give up with WTRI_ETIMEOUT).
+ * The first call on a device looks up the array's device address with that
+ * device current; make that first call before any stream capture.
  */
 WTRI_API int wtri_topk_device_noalloc(const wtri_graph* g, double p, int32_t k, wtri_tri* d_tris,
                                       double* d_weight, int32_t* d_count, void* stream);

@@ -449,9 +449,11 @@ int topk_device(const wtri_graph* g, int pcode, int32_t k, wtri_tri* d_tris, dou
 // the allocator.  The query's scratch (status word, candidate buffer,
 // items) lives in one fixed array compiled into the library.
 // Every GPU that loads the library keeps this array (NOALLOC_BYTES, about
-// 26 MB) until the process exits.  All calls share it: the status word is
-// cleared at the start of each call, and calls that overlap on the GPU (on
-// different streams, or from several host threads) race on it.
+// 28 MB) until the process exits.  All calls share it: the state is cleared at
+// the start of each call.  A call that cleared it under a running sweep would
+// take the barrier's counter away from blocks that wait for it, so each call
+// waits on the device for the one before it (an event; captured calls, which
+// cannot wait for one outside their graph, are left to the caller).
 // ---------------------------------------------------------------------------
 namespace wtri {
 namespace {
@@ -468,18 +470,23 @@ static_assert(NOALLOC_ITEMS % 32 == 0, "every piece is a multiple of 256 bytes")
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_BYTES];
 
 constexpr int NOALLOC_MAX_DEVICES = 64;
-std::mutex g_noalloc_mu;
-void* g_noalloc_ptr[NOALLOC_MAX_DEVICES] = {};
+struct Noalloc {
+    std::mutex mu;  // held while a call is enqueued
+    void* ptr = nullptr;
+    cudaEvent_t last = nullptr;  // the end of the last call
+};
+Noalloc g_noalloc[NOALLOC_MAX_DEVICES];
 
-// Device address of the fixed array for the current device, looked up once
-// per device (with that device current).
-int noalloc_scratch(void** out) {
+// The fixed array of the current device (with that device current), its
+// address looked up once, locked for a call.
+int noalloc_scratch(Noalloc** out, std::unique_lock<std::mutex>* lock) {
     int dev = 0;
     WTRI_CUDA(cudaGetDevice(&dev));
     if (dev < 0 || dev >= NOALLOC_MAX_DEVICES)
         return set_error(WTRI_EUNSUPPORTED, "device index above 63");
-    std::lock_guard<std::mutex> lk(g_noalloc_mu);
-    if (!g_noalloc_ptr[dev]) {
+    Noalloc& N = g_noalloc[dev];
+    *lock = std::unique_lock<std::mutex>(N.mu);
+    if (!N.ptr) {
         void* p = nullptr;
         cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
         if (e != cudaSuccess || !p) {
@@ -487,25 +494,32 @@ int noalloc_scratch(void** out) {
             return cuda_error(e == cudaSuccess ? cudaErrorInvalidSymbol : e,
                               "cudaGetSymbolAddress(static query scratch)", __FILE__, __LINE__);
         }
-        g_noalloc_ptr[dev] = p;
+        if (!N.last) WTRI_CUDA(cudaEventCreateWithFlags(&N.last, cudaEventDisableTiming));
+        N.ptr = p;
     }
-    *out = g_noalloc_ptr[dev];
+    *out = &N;
     return WTRI_OK;
 }
 
 template <int P>
 int run_query_noalloc(const wtri_graph* g, int32_t k, wtri_tri* d_tris, double* d_weight,
                       int32_t* d_count, cudaStream_t s, double gp) {
-    void* base = nullptr;
-    WTRI_TRY(noalloc_scratch(&base));
+    Noalloc* N = nullptr;
+    std::unique_lock<std::mutex> lock;
+    WTRI_TRY(noalloc_scratch(&N, &lock));
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    WTRI_CUDA(cudaStreamIsCapturing(s, &capture));
+    const bool ordered = capture == cudaStreamCaptureStatusNone;
+    if (ordered) WTRI_CUDA(cudaStreamWaitEvent(s, N->last, 0));
     Query q;
-    query_carve(q, (char*)base, NOALLOC_CAP, NOALLOC_ITEMS);
+    query_carve(q, (char*)N->ptr, NOALLOC_CAP, NOALLOC_ITEMS);
     set_sweep(q, g, k);
     q.gp = gp;
     // The array keeps the previous call's contents: reset the state
     // (counters, threshold, barrier, error bits).
     WTRI_CUDA(cudaMemsetAsync(q.st, 0, sizeof(QState), s));
     WTRI_TRY((launch_sweep<P, false>(g->d, q, Out{d_tris, d_weight, d_count, nullptr}, s)));
+    if (ordered) WTRI_CUDA(cudaEventRecord(N->last, s));
     count_launches(1);
     return WTRI_OK;
 }
