@@ -22,11 +22,12 @@
 // clique.  q = 5: the edges go to a bit matrix and a list; for each edge
 // (i, j) of the list, each l above j adjacent to both closes a clique.  Edges
 // that keep more than 128 neighbours go to a second kernel with larger tables,
-// those that keep more than 256 to a third that looks pairs up one by one.  The whole GPU then selects the candidates that reach the
-// k-th key (a histogram per digit of the key, one grid barrier each), one
-// block keeps exactly the k best of those under (key desc, sorted vertex
-// tuple asc) by an MSB-first radix select over the tuple, and a rank pass
-// orders them.
+// those that keep more than 256 to a third that looks pairs up one by one.  On
+// large graphs a filter lists the drawn edges that may close a clique at all.
+// The whole GPU then selects the candidates that reach the k-th key (a
+// histogram per digit of the key, one grid barrier each), one block keeps
+// exactly the k best of those under (key desc, sorted vertex tuple asc) by an
+// MSB-first radix select over the tuple, and a rank pass orders them.
 #include "wtri_query.cuh"
 
 #include <algorithm>
@@ -46,14 +47,15 @@ constexpr uint32_t CLIQUE_CAP = 1u << 23;
 
 struct CliqueRun {
     const uint32_t* mark;  // drawn edges: bit r = the r-th edge of the edge order
-    int32_t words;
     int32_t q, pcode;
     unsigned long long* ckey;
     int32_t* cids;         // QMAX ids per candidate, ascending
     uint32_t* count;
     uint32_t cap;
     uint32_t* err;
-    int32_t* cursor;       // next group of bitmap bits
+    int32_t* cursor;       // next group of bitmap bits, or of the work list
+    int32_t* work;         // the drawn edges that may close a clique (null: the bitmap is walked)
+    uint32_t* nwork;
     int32_t* list[2];      // edges left to k_cliques_mid, to k_cliques_big
     uint32_t* nlist;       // their numbers
 };
@@ -63,7 +65,6 @@ struct CliqueRun {
 struct CliqueSmem {
     int32_t cid[CNB], cdg[CNB], cwu[CNB], cwv[CNB], cru[CNB], crv[CNB];
     int32_t n;
-    int32_t item;
 };
 
 __device__ __forceinline__ bool drawn(const uint32_t* mark, int32_t r) {
@@ -203,7 +204,7 @@ __global__ void __launch_bounds__(CB) k_cliques_big(DevGraph G, CliqueRun C) {
 }
 
 // ---- edges with at most FNB kept neighbours --------------------------------
-// Two sizes: FNB = 128 (58 KB of shared memory: three 256-thread blocks per
+// Two sizes: FNB = 128 (54 KB of shared memory: three 256-thread blocks per
 // SM), and FNB = 256 (208 KB: one 1,024-thread block) for the few edges that
 // keep more.
 constexpr int FGROUP = 4;          // bitmap bits taken at a time
@@ -395,21 +396,101 @@ __device__ __forceinline__ void fast_edge(const DevGraph& G, const CliqueRun& C,
     }
 }
 
-// The drawn edges, a few bitmap bits at a time.
+// Large graphs: the drawn edges with enough kept common neighbours for a clique,
+// to the work list.  A warp takes a word of the bitmap; the entries of its
+// edges' shorter rows are numbered through and looked up 32 at a time, as the
+// blocks below do it.  Rows above FILTER_ROW go to the list as they are (64: all
+// edges of the graph below take 32 ms).  Blocks that walk the bitmap a few bits
+// at a time and clear their tables for every drawn edge took 8.3 ms for 100 draws
+// from 2e7 edges on 2e6 vertices and 187 ms for all of them (q = 4, k = 1,000);
+// with the list 0.18 and 16.  Small graphs walk: q = 5, 10,000 draws from 29,000
+// edges 0.41 ms, 0.58 with the list; from 100,000 edges 0.45 and 0.57.
+constexpr int64_t WALK_MAX = 1 << 17;    // most edges whose bitmap is walked
+constexpr int64_t FILTER_ROW = 256;
+
+static_assert(3 * (sizeof(FastSmem<128>) + 1024) <= 228 * 1024, "three small-table blocks per SM");
+
+struct FilterWarp {
+    int64_t j0[32];
+    uint32_t end[32], cnt[32];  // entries up to and with each row; neighbours kept
+    int32_t r[32], y[32], dy[32];
+};
+
+template <int Q>
+__global__ void __launch_bounds__(CB) k_clique_edges(DevGraph G, CliqueRun C) {
+    __shared__ FilterWarp shared[CB / 32];
+    FilterWarp& W = shared[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    const int64_t words = (G.m + 31) / 32, nwarps = ((int64_t)gridDim.x * CB) >> 5;
+    Tally tb;
+    for (int64_t w = ((int64_t)blockIdx.x * CB + threadIdx.x) >> 5; w < words; w += nwarps) {
+        const uint32_t bits = __ldg(C.mark + w);
+        if (!bits) continue;
+        const int32_t r = (int32_t)(32 * w + lane);
+        int64_t n = 0;
+        W.cnt[lane] = 0;
+        W.r[lane] = r;
+        if ((bits >> lane) & 1u) {
+            const int32_t u = __ldg(G.ord_u + r), v = __ldg(G.ord_v + r);
+            const int64_t bu = __ldg(G.rowptr + u), eu = __ldg(G.rowptr + u + 1);
+            const int64_t bv = __ldg(G.rowptr + v), ev = __ldg(G.rowptr + v + 1);
+            const bool xu = (eu - bu) <= (ev - bv);  // scan the shorter row
+            n = xu ? eu - bu : ev - bv;
+            W.j0[lane] = xu ? bu : bv;
+            W.y[lane] = xu ? v : u;
+            W.dy[lane] = (int32_t)(xu ? ev - bv : eu - bu);
+        }
+        bool keep = n > FILTER_ROW;
+        uint32_t inc = keep || n < Q - 1 ? 0u : (uint32_t)n;  // (a clique takes Q - 1 entries of the row)
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t x = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += x;
+        }
+        W.end[lane] = inc;
+        const uint32_t tot = __shfl_sync(0xffffffffu, inc, 31);
+        __syncwarp();
+        for (uint32_t e = lane; e < tot; e += 32) {
+            int k = 0;
+#pragma unroll
+            for (int s = 16; s > 0; s >>= 1)
+                if (W.end[k + s - 1] <= e) k += s;
+            const int64_t j = W.j0[k] + (e - (k > 0 ? W.end[k - 1] : 0u));
+            const int32_t c = __ldg(G.wcol + j), y = W.y[k], rk = W.r[k];
+            int32_t wyc, ryc;
+            if (c == y || !probe_oriented(G, y, W.dy[k], c, wyc, ryc, tb)) continue;
+            const int32_t rxc = __ldg(G.wrk + j);
+            if ((rxc < rk && drawn(C.mark, rxc)) || (ryc < rk && drawn(C.mark, ryc))) continue;
+            atomicAdd(&W.cnt[k], 1u);
+        }
+        __syncwarp();
+        keep |= W.cnt[lane] >= Q - 2;
+        const uint32_t b = __ballot_sync(0xffffffffu, keep);
+        uint32_t at = 0;
+        if (lane == 0 && b) at = atomicAdd(C.nwork, (uint32_t)__popc(b));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (keep) C.work[at + __popc(b & lanemask_below())] = r;
+        __syncwarp();
+    }
+}
+
+// The drawn edges: the work list one by one, or a few bitmap bits at a time.
 template <int Q, int PC>
 __global__ void __launch_bounds__(CB, 3) k_cliques(DevGraph G, CliqueRun C) {
     extern __shared__ __align__(16) unsigned char csm[];
     FastSmem<128>& S = *reinterpret_cast<FastSmem<128>*>(csm);
-    const int64_t m = G.m;
+    const bool list = C.work != nullptr;
+    const int64_t n = list ? (int64_t)*C.nwork : G.m, group = list ? 1 : FGROUP;
     for (;;) {
         if (threadIdx.x == 0) S.item = atomicAdd(C.cursor, 1);
         __syncthreads();
-        const int64_t r0 = (int64_t)S.item * FGROUP;
+        const int64_t i0 = (int64_t)S.item * group;
         __syncthreads();
-        if (r0 >= m) break;
-        for (int64_t r = r0; r < min(m, r0 + FGROUP); r++) {
-            if (!drawn(C.mark, (int32_t)r)) continue;
-            fast_edge<Q, PC, 128, CB>(G, C, S, (int32_t)r, C.list[0], C.nlist);
+        if (i0 >= n) break;
+        for (int64_t i = i0; i < min(n, i0 + group); i++) {
+            const int32_t r = list ? C.work[i] : (int32_t)i;
+            if (!list && !drawn(C.mark, r)) continue;
+            fast_edge<Q, PC, 128, CB>(G, C, S, r, C.list[0], C.nlist);
             __syncthreads();  // the shared lists are reused by the next edge
         }
     }
@@ -734,7 +815,7 @@ int clique_topk_host(const wtri_graph* g, int q, int pcode, int32_t k, int64_t n
     p += al((size_t)cap * 4);
     int32_t* big = (int32_t*)p;
     p += 2 * al(4 * (size_t)big_cap);
-    uint32_t* small = (uint32_t*)p;  // count, err, cursor, kept, nix, nbig
+    uint32_t* small = (uint32_t*)p;  // count, err, cursor, kept, nix, nlist[2], nwork
     auto done = [&](int rc) {
         cudaFreeAsync(buf, s);
         cudaStreamSynchronize(s);
@@ -751,7 +832,6 @@ int clique_topk_host(const wtri_graph* g, int q, int pcode, int32_t k, int64_t n
     }
     CliqueRun C;
     C.mark = mark;
-    C.words = (int32_t)words;
     C.q = q;
     C.pcode = pcode;
     C.ckey = ckey;
@@ -763,6 +843,9 @@ int clique_topk_host(const wtri_graph* g, int q, int pcode, int32_t k, int64_t n
     C.list[0] = big;
     C.list[1] = (int32_t*)((char*)big + al(4 * (size_t)big_cap));
     C.nlist = small + 5;
+    // (the work list is read before k_cliques_mid fills list[1])
+    C.work = m > WALK_MAX ? C.list[1] : nullptr;
+    C.nwork = small + 7;
     const int big_smem = (int)sizeof(CliqueSmem) + (q == 5 ? CNB * CNW * 4 : 0);
     {
         static std::atomic<uint64_t> optin{0};
@@ -772,13 +855,18 @@ int clique_topk_host(const wtri_graph* g, int q, int pcode, int32_t k, int64_t n
     auto enumerate = [&](auto kern, auto mid, std::atomic<uint64_t>* optin) -> int {
         WTRI_TRY(smem_optin((const void*)kern, (int)sizeof(FastSmem<128>), optin[0]));
         WTRI_TRY(smem_optin((const void*)mid, (int)sizeof(FastSmem<256>), optin[1]));
+        if (C.work) {
+            const unsigned blocks = (unsigned)std::min<int64_t>(sm_count() * 8, (words + CB / 32 - 1) / (CB / 32));
+            if (q == 5) k_clique_edges<5><<<blocks, CB, 0, s>>>(G, C);
+            else k_clique_edges<4><<<blocks, CB, 0, s>>>(G, C);
+        }
         kern<<<sm_count() * 3, CB, sizeof(FastSmem<128>), s>>>(G, C);
         mid<<<sm_count(), 1024, sizeof(FastSmem<256>), s>>>(G, C);
         k_cliques_big<<<sm_count() * (q == 5 ? 1 : 4), CB, big_smem, s>>>(G, C);
         return WTRI_OK;
     };
     {
-        ProfScope ps("cliques_enumerate", s, 0.0, 3);
+        ProfScope ps("cliques_enumerate", s, 0.0, C.work ? 4 : 3);
         static std::atomic<uint64_t> optin[8][2];
         int rc = WTRI_OK;
         switch (pcode + (q == 5 ? 4 : 0)) {
