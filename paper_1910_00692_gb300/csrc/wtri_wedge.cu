@@ -71,55 +71,68 @@ __device__ __forceinline__ uint64_t wpow(int32_t w) {
 constexpr int WBLK = 256;
 constexpr unsigned long long HASH_EMPTY = ~0ull;
 
-// Per-row cumulative w^p (u64, one warp per row: eight consecutive entries
-// per lane and step, one warp scan of their sums) and D(a); flags a row whose
-// sum does not fit 64 bits.  (With one entry per lane and step the longest
-// row's serial scans took 215 us on the 2e6-edge graph.)
-template <int P>
-__global__ void __launch_bounds__(WBLK) k_ws_rows(DevGraph G, uint64_t* __restrict__ cum,
-                                                  uint64_t* __restrict__ D, uint32_t* err) {
-    constexpr int E = 8;
+// Per-row cumulative w^p (u64, one warp per row) and D(a); flags a row whose
+// sum does not fit 64 bits.  Rows above WS_SHORT: four consecutive entries per
+// lane and step, one warp scan of their sums (with one entry per lane the
+// longest row's serial scans took 215 us on the 2e6-edge graph); shorter ones:
+// one entry per lane, a step is one coalesced load.  Short rows are bound by
+// the warps in flight: 32 registers, eight blocks per SM.  A call with 100 draws
+// on 2e7 random edges (5e6 vertices) / on the skewed graph of 2e7: one loop of
+// eight predicated entries 1.77 / 0.54 ms, a loop each 1.27 / 0.46, four entries
+// 1.24 / 0.38, at 32 registers 0.97 / 0.40 (eight: 0.99 / 0.48).
+constexpr int64_t WS_SHORT = 64;
+constexpr int WS_E = 4;
+
+template <int P, int E>
+__device__ __forceinline__ uint64_t ws_row(const DevGraph& G, uint64_t* __restrict__ cum, int64_t b0, int64_t e0,
+                                           bool& over) {
     const int lane = threadIdx.x & 31;
+    uint64_t carry = 0;
+    for (int64_t base = b0; base < e0; base += 32 * E) {
+        const int64_t j0 = base + (int64_t)lane * E;
+        uint64_t v[E], sum = 0;
+#pragma unroll
+        for (int i = 0; i < E; i++) v[i] = j0 + i < e0 ? wpow<P>(__ldg(G.wwt + j0 + i)) : 0;
+#pragma unroll
+        for (int i = 0; i < E; i++) {
+            over |= sum + v[i] < sum;
+            sum += v[i];
+            v[i] = sum;
+        }
+        uint64_t inc = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint64_t y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) {
+                over |= inc + y < inc;
+                inc += y;
+            }
+        }
+        const uint64_t s = carry + inc;
+        over |= s < carry;
+        const uint64_t before = s - sum;
+#pragma unroll
+        for (int i = 0; i < E; i++)
+            if (j0 + i < e0) cum[j0 + i] = before + v[i];
+        carry = __shfl_sync(0xffffffffu, s, 31);
+    }
+    return carry;
+}
+
+template <int P>
+__global__ void __launch_bounds__(WBLK, 8) k_ws_rows(DevGraph G, uint64_t* __restrict__ cum, uint64_t* __restrict__ D,
+                                                     uint32_t* err) {
     const int64_t nwarps = ((int64_t)gridDim.x * WBLK) >> 5;
     for (int64_t x = ((int64_t)blockIdx.x * WBLK + threadIdx.x) >> 5; x < G.n; x += nwarps) {
         const int64_t b0 = __ldg(G.rowptr + x), e0 = __ldg(G.rowptr + x + 1);
-        uint64_t carry = 0;
         bool over = false;
-        // short rows: one entry per lane, so that a step is one coalesced load
-        const int per = e0 - b0 > 64 ? E : 1;
-        for (int64_t base = b0; base < e0; base += 32 * per) {
-            const int64_t j0 = base + (int64_t)lane * per;
-            uint64_t v[E], sum = 0;
-#pragma unroll
-            for (int i = 0; i < E; i++) {
-                const bool in = i < per && j0 + i < e0;
-                v[i] = in ? wpow<P>(__ldg(G.wwt + j0 + i)) : 0;
-            }
-#pragma unroll
-            for (int i = 0; i < E; i++) {
-                over |= sum + v[i] < sum;
-                sum += v[i];
-                v[i] = sum;
-            }
-            uint64_t inc = sum;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint64_t y = __shfl_up_sync(0xffffffffu, inc, o);
-                if (lane >= o) {
-                    over |= inc + y < inc;
-                    inc += y;
-                }
-            }
-            const uint64_t s = carry + inc;
-            over |= s < carry;
-            const uint64_t before = s - sum;
-#pragma unroll
-            for (int i = 0; i < E; i++)
-                if (i < per && j0 + i < e0) cum[j0 + i] = before + v[i];
-            carry = __shfl_sync(0xffffffffu, s, 31);
+        const uint64_t d =
+            e0 - b0 > WS_SHORT ? ws_row<P, WS_E>(G, cum, b0, e0, over) : ws_row<P, 1>(G, cum, b0, e0, over);
+        const bool any = __any_sync(0xffffffffu, over);
+        if ((threadIdx.x & 31) == 0) {
+            if (any) atomicOr(err, DEV_ERR_OVERFLOW);
+            D[x] = d;
         }
-        if (__any_sync(0xffffffffu, over) && lane == 0) atomicOr(err, DEV_ERR_OVERFLOW);
-        if (lane == 0) D[x] = carry;
     }
 }
 
