@@ -1398,16 +1398,28 @@ __device__ __forceinline__ void sort_ids(const Part<TB>& B, const unsigned long 
         }
 }
 
-// Ranks n > SORT_MAX candidates, all of them results.  False: a barrier gave up.
-// Up to two per warp: each warp counts the candidates before its own (k = 3,000
-// on the whole GPU: the query takes 208 us, 244 by runs).  More: sorted runs of
+// Whether the team ranks n candidates of a k above SORT_MAX together: more than
+// one block sorts, or few enough to count (1,333 results of k = 3,000 on 2e5 edges,
+// the whole query: 175 us, sorted by one block 194).
+template <class Team>
+__device__ __forceinline__ bool counts_ranks(const Team& T, uint32_t n) {
+    return Team::GRID && (int64_t)n <= 2 * T.warps();
+}
+template <class Team>
+__device__ __forceinline__ bool ranks_many(const Team& T, uint32_t n) {
+    return n > SORT_MAX || counts_ranks(T, n);
+}
+
+// Ranks candidates, all of them results.  False: a barrier gave up.  Up to two
+// per warp: each warp counts the candidates before its own (k = 3,000 on the
+// whole GPU: the query takes 208 us, 244 by runs).  More: sorted runs of
 // SORT_MAX, a block each, then every candidate's place is its place in its run
 // and, for each other run, the entries before it (a lane per run searches).  By
 // counting, k = 16,384 / 65,536 on the whole GPU 0.59 / 4.9 ms, by runs 0.42 /
 // 0.97; and 490 ms on one SM of a batch.
 template <int P, class Team>
 __device__ __forceinline__ bool rank_many(const Query& q, const Out& o, uint32_t n, Team& T, SortSmem& R) {
-    if (Team::GRID && (int64_t)n <= 2 * T.warps()) {
+    if (counts_ranks(T, n)) {
         for (int64_t i = T.warp(); i < (int64_t)n; i += T.warps()) {
             const unsigned long long ki = q.ckey[i];
             const int4 ti = q.ctri[i];
@@ -1483,7 +1495,7 @@ __device__ bool finish(const Query& q, const Out& o, Team& T, SelectSmem& S, Sor
         else if (err & DEV_ERR_OVERFLOW) status = WTRI_ENOMEM;
         else if (err) status = WTRI_ECUDA;
         if (B.tid() == 0) *(volatile uint32_t*)&q.st->kept = n;
-        if (n <= SORT_MAX) {
+        if (K <= SORT_MAX || !ranks_many(T, n)) {
             sort_ids<Team::TB>(B, q.ckey, q.ctri, n, R);
             for (uint32_t i = B.tid(); i < min(n, K); i += Team::TB) {
                 const uint32_t c = R.id[i];
@@ -1494,7 +1506,7 @@ __device__ bool finish(const Query& q, const Out& o, Team& T, SelectSmem& S, Sor
     if (K > SORT_MAX) {
         if (!T.sync(q)) return false;
         const uint32_t n = *(volatile uint32_t*)&q.st->kept;
-        if (n > SORT_MAX && !rank_many<P>(q, o, n, T, R)) return false;
+        if (ranks_many(T, n) && !rank_many<P>(q, o, n, T, R)) return false;
     }
     if (T.leader() && B.tid() == 0) *o.count = status;
     return true;

@@ -87,3 +87,22 @@ def test_rankings_of_many(ties, p):
     ks = [65_536] + [50] * 400
     for k, got in zip(ks, wt.topk_batch([d] * len(ks), [p] * len(ks), ks)):
         check(got, k, "beside small ones")
+
+
+@pytest.mark.parametrize("p", PS)
+def test_fewer_results_than_asked_for(p):
+    """k above 2,048 on graphs with fewer triangles: ranked by counting on the
+    whole GPU, by one block's sort on a few SMs and on a part."""
+    for n, m, seed in ((60, 400, 1), (2000, 20_000, 2)):
+        g = synth.scaled_mid_graph(n, m, seed=seed)
+        d = wt.build_csr(g.n, g.u, g.v, g.w)
+        try:
+            want = oracle.topk(g.n, g.u, g.v, g.w, p, 3000)
+            for k in (2049, 3000):
+                w = {"tri": want["tri"][:k], "value": want["value"][:k], "count": min(k, want["count"])}
+                assert_topk_equal(*d.topk(p, k), w, p, f"m={m} k={k}")
+                for count in (1, 40, 320):
+                    for got in wt.topk_batch([d] * count, [p] * count, [k] * count):
+                        assert_topk_equal(*got, w, p, f"m={m} k={k} batch of {count}")
+        finally:
+            d.free()
