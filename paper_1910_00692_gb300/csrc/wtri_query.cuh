@@ -66,6 +66,7 @@ constexpr uint32_t WAIT_LIMIT = 1u << 26;  // bounded polling of the grid barrie
 constexpr int64_t ITEM_CAP = 1 << 18;      // most items
 constexpr int64_t WARP_EDGES = 4096;       // largest round that takes a warp per edge
 constexpr int64_t MIN_FLAT = 8192;         // largest p = -inf round that numbers its entries through
+constexpr int64_t SMALL_M = 1 << 16;       // edges of a small graph (see sweep_blocks)
 
 // State of one query (zeroed before it starts).
 struct QState {
@@ -893,6 +894,30 @@ __device__ __forceinline__ void min_edges_items(const DevGraph& G, const Query& 
     }
 }
 
+// Small graphs: a warp scans its edge's row itself (of at most sqrt(2 SMALL_M)
+// entries), so that a round has no second phase.
+template <class Team>
+__device__ __forceinline__ void min_edges_by_warp(const DevGraph& G, const Query& q, unsigned long long tau, int64_t lo,
+                                                  int64_t hi, const Team& T, Tally& tb) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t r = lo + T.warp(); r < hi; r += T.warps()) {
+        const int32_t u = __ldg(G.ord_u + r), v = __ldg(G.ord_v + r);
+        const uint32_t w = (uint32_t)__ldg(G.ord_w + r);
+        const int64_t du = __ldg(G.rowptr + u + 1) - __ldg(G.rowptr + u);
+        const int64_t dv = __ldg(G.rowptr + v + 1) - __ldg(G.rowptr + v);
+        const MinRows R = min_rows(u, v, du, dv, __ldg(G.orowptr + u), __ldg(G.orowptr + u + 1),
+                                   __ldg(G.orowptr + v), __ldg(G.orowptr + v + 1));
+        if (lane == 0) tb.add(12 + 64);
+        if (R.ln == 0) continue;
+        for (int64_t j = R.sb + lane; j < R.se; j += 32) {
+            const uint32_t wsc = (uint32_t)__ldg(G.owt + j);
+            tb.add(4);
+            if (wsc >= tau) min_entry(G, q, tau, w, R.a, R.b, R.lb, R.ln, j, wsc, tb);
+        }
+        __syncwarp();
+    }
+}
+
 // Large rounds, where few entries reach tau: GL lanes per edge read its
 // scanned row 4 GL weights at a time (16-byte loads, the next ones in flight
 // while these are compared), 32 / GL edges to a warp, the endpoints of the
@@ -995,9 +1020,8 @@ __device__ __forceinline__ void min_edges_filtered(const DevGraph& G, const Quer
 // (each has at least one wedge).
 // ---------------------------------------------------------------------------
 template <int P, bool SAMPLED, bool ORIENTED, class Team>
-__device__ __forceinline__ void item_wedges(const DevGraph& G, const Query& q, unsigned long long tau, int par,
-                                            bool flat, const Team& T, Tally& tb) {
-    const unsigned long long ctr = *(volatile const unsigned long long*)&q.st->items[par];
+__device__ __forceinline__ void item_wedges(const DevGraph& G, const Query& q, unsigned long long tau,
+                                            unsigned long long ctr, bool flat, const Team& T, Tally& tb) {
     const int64_t drawn_ = (int64_t)(ctr >> ITEM_SHIFT), cnt = min(drawn_, flat ? q.item_cap - 1 : q.item_cap);
     const int64_t tot = cnt == drawn_ ? (int64_t)(ctr & WEDGE_MASK) : (int64_t)q.ibase[cnt];
     if (!flat && cnt != drawn_) return;
@@ -1541,8 +1565,10 @@ __device__ bool sweep(const DevGraph& G, const Query& q, const Out& o, Team& T, 
         const bool flat = hi - lo > q.item_cap;  // more edges than items
         if constexpr (P == P_MIN && !SAMPLED) {
             if (oriented) {
-                items = hi - lo <= min(MIN_FLAT, q.item_cap);
-                if (items) min_edges_items(G, q, lo, hi, par, T, tb);
+                const bool by_warp = G.m <= SMALL_M && hi - lo <= min(WARP_EDGES, T.warps() * 4);
+                items = !by_warp && hi - lo <= min(MIN_FLAT, q.item_cap);
+                if (by_warp) min_edges_by_warp(G, q, tau, lo, hi, T, tb);
+                else if (items) min_edges_items(G, q, lo, hi, par, T, tb);
                 else if (G.m < MIN_WIDE * G.n) min_edges_filtered<4>(G, q, tau, lo, hi, T, S.queue[T.part.tid() >> 5], tb);
                 else min_edges_filtered<8>(G, q, tau, lo, hi, T, S.queue[T.part.tid() >> 5], tb);
             }
@@ -1552,11 +1578,13 @@ __device__ bool sweep(const DevGraph& G, const Query& q, const Out& o, Team& T, 
             else edges_by_thread<P, SAMPLED>(G, q, tau, lo, hi, par, flat, T, S.here[T.part.tid() >> 5], tb);
         }
         if (!T.sync(q)) return false;
-        if (items) {
+        // (none: small rounds often scan every live range in the first phase)
+        const unsigned long long ctr = items ? ld_volatile_u64(&q.st->items[par]) : 0ull;
+        if (ctr != 0) {
             if constexpr (P == P_MIN && !SAMPLED) {
-                if (oriented) item_wedges<P, false, true>(G, q, tau, par, false, T, tb);
+                if (oriented) item_wedges<P, false, true>(G, q, tau, ctr, false, T, tb);
             }
-            if (!oriented) item_wedges<P, SAMPLED, false>(G, q, tau, par, flat, T, tb);
+            if (!oriented) item_wedges<P, SAMPLED, false>(G, q, tau, ctr, flat, T, tb);
             if (!T.sync(q)) return false;
         }
         if (T.leader()) {
@@ -1589,6 +1617,19 @@ __global__ void __launch_bounds__(TGRID, 1) k_sweep(DevGraph G, Query q, Out o) 
     sweep<P, SAMPLED>(G, q, o, T, S);
 }
 
+// Blocks of a query's sweep: the whole GPU, fewer on small graphs, whose rounds
+// have too few edges to fill them and pay for every block at the barriers
+// (random graphs of 300 / 3,000 / 20,000 edges, p = 1, k = 50: 56 / 84 / 89 us on
+// all SMs, now 40 / 62 / 76; p = -inf, k = 1,000, with the rounds of
+// min_edges_by_warp: 54 / 83 / 119, now 37 / 56 / 93).  The general means spend
+// their time in fp64 pow and take four times as many.
+template <int P>
+inline unsigned sweep_blocks(int64_t m) {
+    if (m > SMALL_M) return (unsigned)sm_count();
+    const int64_t fit = P == P_GEN ? (m + 15) / 16 : std::min<int64_t>(48, (m + 63) / 64);
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>(sm_count(), fit));
+}
+
 // Launches the sweep of one query on the whole GPU (a cooperative launch:
 // its blocks wait for one another, so all must be resident).
 template <int P, bool SAMPLED>
@@ -1601,7 +1642,7 @@ int launch_sweep(const DevGraph& G, const Query& q, const Out& o, cudaStream_t s
     Query qq = q;
     Out oo = o;
     void* args[] = {&g, &qq, &oo};
-    WTRI_CUDA(cudaLaunchCooperativeKernel(fn, dim3((unsigned)sm_count()), dim3(TGRID), args, smem, s));
+    WTRI_CUDA(cudaLaunchCooperativeKernel(fn, dim3(sweep_blocks<P>(G.m)), dim3(TGRID), args, smem, s));
     return WTRI_OK;
 }
 
