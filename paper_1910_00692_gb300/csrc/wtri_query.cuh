@@ -64,8 +64,12 @@ constexpr int TGRID = 1024;         // threads of a block of the grid team (one 
 constexpr int SORT_MAX = 2048;      // most candidates sorted in shared memory
 constexpr uint32_t WAIT_LIMIT = 1u << 26;  // bounded polling of the grid barrier
 constexpr int64_t ITEM_CAP = 1 << 18;      // most items
-constexpr int64_t WARP_EDGES = 4096;       // largest round that takes a warp per edge
-constexpr int64_t MIN_FLAT = 8192;         // largest p = -inf round that numbers its entries through
+// Largest round that takes a warp per edge (512, 4,096 or 32,768: the same to 1 %
+// at p = 1 and +inf on graphs of 5e6 to 6e7 edges).
+constexpr int64_t WARP_EDGES = 4096;
+// Largest p = -inf round that numbers its entries through (2e7 skewed edges, us at
+// 1,024 / 8,192 / 65,536: 381 / 357 / 369; 6e7 edges: 784 / 731 / 732).
+constexpr int64_t MIN_FLAT = 8192;
 constexpr int64_t SMALL_M = 1 << 16;       // edges of a small graph (see sweep_blocks)
 
 // State of one query (zeroed before it starts).
@@ -894,8 +898,9 @@ __device__ __forceinline__ void min_edges_items(const DevGraph& G, const Query& 
     }
 }
 
-// Small graphs: a warp scans its edge's row itself (of at most sqrt(2 SMALL_M)
-// entries), so that a round has no second phase.
+// A warp scans its edge's row itself: small graphs (rows of at most sqrt(2
+// SMALL_M) entries), whose rounds then have no second phase, and dense ones
+// before there is a threshold.
 template <class Team>
 __device__ __forceinline__ void min_edges_by_warp(const DevGraph& G, const Query& q, unsigned long long tau, int64_t lo,
                                                   int64_t hi, const Team& T, Tally& tb) {
@@ -930,7 +935,14 @@ struct MinProbe {
     uint32_t w;
     int32_t a, b;
 };
-constexpr int64_t MIN_WIDE = 12;  // edges per vertex from which a scanned row gets eight lanes, not four
+// Edges per vertex from which a scanned row gets eight lanes, not four (us with
+// four / eight: random graphs of 4 / 16 edges per vertex 2,370 / 3,230, 4,140 /
+// 4,860; skewed ones of 8 / 20 / 30: 280 / 276, 364 / 357, 261 / 254).
+constexpr int64_t MIN_WIDE = 12;
+// Edges per vertex from which a round without a threshold, whose entries all count,
+// takes a warp per edge and no queue (us, warp / queue: 100 edges per vertex, no
+// triangles, 1,539 / 1,694; 16 per vertex 9,990 / 4,870).
+constexpr int64_t MIN_DENSE = 64;
 constexpr int MINQ = 64;  // a step of at most 32 entries on top of at most 31 waiting
 
 template <int GL, class Team>
@@ -1565,7 +1577,8 @@ __device__ bool sweep(const DevGraph& G, const Query& q, const Out& o, Team& T, 
         const bool flat = hi - lo > q.item_cap;  // more edges than items
         if constexpr (P == P_MIN && !SAMPLED) {
             if (oriented) {
-                const bool by_warp = G.m <= SMALL_M && hi - lo <= min(WARP_EDGES, T.warps() * 4);
+                const bool by_warp = G.m <= SMALL_M ? hi - lo <= min(WARP_EDGES, T.warps() * 4)
+                                                    : tau == 0 && hi - lo > MIN_FLAT && G.m >= MIN_DENSE * G.n;
                 items = !by_warp && hi - lo <= min(MIN_FLAT, q.item_cap);
                 if (by_warp) min_edges_by_warp(G, q, tau, lo, hi, T, tb);
                 else if (items) min_edges_items(G, q, lo, hi, par, T, tb);
