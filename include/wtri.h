@@ -40,7 +40,10 @@
  * Device memory behind a wtri_graph is owned by the library and freed by
  * wtri_graph_free.  A graph is immutable after wtri_build_csr; queries on
  * one graph from several host threads are safe (each query uses its own
- * stream-ordered scratch).
+ * stream-ordered scratch).  A query, a batch and a clique selection hold the
+ * SMs they run on until they end (all of them, but for small graphs), so those
+ * of several streams run one after another: a short query issued behind a
+ * long one waits for it.
  */
 #ifndef WTRI_H
 #define WTRI_H
@@ -221,9 +224,9 @@ WTRI_API int wtri_merge_topk(int32_t nparts, const int32_t* counts, const wtri_t
  * Batched exact top-k: query i asks for the top-k[i] triangles of gs[i] at
  * p[i] (same problem and result format as wtri_topk, results in outs[i]).
  * All queries run in one launch sequence captured in a CUDA graph on the
- * first graph's stream: small graphs one block each, larger ones a share of
- * the SMs each, and each query keeps its own threshold and candidate buffer.  Graphs must be
- * on one device.  Returns after all results are in the host arrays.  No
+ * first graph's stream: most queries half an SM each, those of more expected
+ * work a share of the SMs, and each query keeps its own threshold and
+ * candidate buffer.  Graphs must be on one device.  Returns after all results are in the host arrays.  No
  * counterpart in the paper (whose algorithms answer one query at a time).
  */
 WTRI_API int wtri_topk_batch(const wtri_graph* const* gs, const double* p, const int32_t* k,

@@ -101,7 +101,7 @@ constexpr int UNT = 256;                   // threads of a histogram block
 constexpr int UNW = UNT / 32;
 constexpr uint32_t WAIT_LIMIT = 1u << 24;  // bounded mbarrier polling
 static_assert(TT % 16 == 0, "tiles are whole 16-byte lines of every source array");
-static_assert(DPT == 2 || DPT == 4, "a thread's digits are one 4- or 8-byte word of each warp's counters");
+static_assert(DPT == 2, "a thread's digits are one 4-byte word of each warp's counters");
 
 __device__ __forceinline__ uint32_t lanemask_lt() {
     uint32_t m;
@@ -440,26 +440,14 @@ __device__ __forceinline__ uint32_t digit_peers(uint32_t d, bool valid) {
     return p;
 }
 
-// A thread's DPT consecutive 16-bit counters as one 4- or 8-byte word.
+// A thread's DPT consecutive 16-bit counters as one word.
 __device__ __forceinline__ void load_counts(const uint16_t* p, uint32_t (&c)[DPT]) {
-    if constexpr (DPT == 4) {
-        const uint2 r = *reinterpret_cast<const uint2*>(p);
-        c[0] = lo16(r.x);
-        c[1] = hi16(r.x);
-        c[2] = lo16(r.y);
-        c[3] = hi16(r.y);
-    } else {
-        const uint32_t r = *reinterpret_cast<const uint32_t*>(p);
-        c[0] = lo16(r);
-        c[1] = hi16(r);
-    }
+    const uint32_t r = *reinterpret_cast<const uint32_t*>(p);
+    c[0] = lo16(r);
+    c[1] = hi16(r);
 }
 __device__ __forceinline__ void store_counts(uint16_t* p, const uint32_t (&s)[DPT]) {
-    if constexpr (DPT == 4) {
-        *reinterpret_cast<uint2*>(p) = make_uint2(s[0] | (s[1] << 16), s[2] | (s[3] << 16));
-    } else {
-        *reinterpret_cast<uint32_t*>(p) = s[0] | (s[1] << 16);
-    }
+    *reinterpret_cast<uint32_t*>(p) = s[0] | (s[1] << 16);
 }
 
 // Ranks a tile's digits within each warp: rk[j] = digit | rank << 16, and the

@@ -483,8 +483,8 @@ __device__ __forceinline__ void warp_bitonic(uint32_t (&k)[EPL]) {
     }
 }
 
-// Shared-memory index of element p of a warp's sorted run (lane-blocked
-// stores of 8-byte keys would all hit one bank: swizzle the low five bits).
+// Shared-memory index of element p of a warp's sorted run (lane-blocked stores
+// of 4-byte keys would meet in every EPL-th bank: swizzle the low five bits).
 __device__ __forceinline__ int swz(int p) { return p ^ ((p >> 5) & 31); }
 
 // ---------------------------------------------------------------------------
