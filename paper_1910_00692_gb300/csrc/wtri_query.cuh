@@ -1549,9 +1549,11 @@ __device__ bool finish(const Query& q, const Out& o, Team& T, SelectSmem& S, Sor
 }
 
 // ---------------------------------------------------------------------------
-// The whole sweep.  The status says WTRI_ETIMEOUT until the answer is complete,
-// so a team whose blocks give up (false) leaves that; a block that gives up
-// has done its work up to that barrier, and the others cannot pass the next.
+// The whole sweep.  False: a barrier gave up, and the leading block's caller
+// writes WTRI_ETIMEOUT for the status, which is written once, at the end, either
+// way.  A block that gives up has done its work up to that barrier, and the
+// others, the leading one among them, cannot pass the next: where there is none,
+// the answer is complete.
 // ---------------------------------------------------------------------------
 template <int TB>
 struct SweepSmem {
@@ -1565,7 +1567,6 @@ struct SweepSmem {
 
 template <int P, bool SAMPLED, class Team>
 __device__ bool sweep(const DevGraph& G, const Query& q, const Out& o, Team& T, SweepSmem<Team::TB>& S) {
-    if (Team::GRID && T.leader() && T.part.tid() == 0) *o.count = WTRI_ETIMEOUT;
     const bool oriented = P == P_MIN && !SAMPLED && q.nshards <= 1;
     const int64_t total = q.total_dev ? __ldg(q.total_dev) : q.total;
     int64_t size = min(q.first, q.item_cap), lo = 0, hi = min(total, size);
@@ -1627,7 +1628,7 @@ __global__ void __launch_bounds__(TGRID, 1) k_sweep(DevGraph G, Query q, Out o) 
     T.gone = &S.sel.gone;
     if (threadIdx.x == 0) S.sel.gone = 0;
     __syncthreads();
-    sweep<P, SAMPLED>(G, q, o, T, S);
+    if (!sweep<P, SAMPLED>(G, q, o, T, S) && T.leader() && threadIdx.x == 0) *o.count = WTRI_ETIMEOUT;
 }
 
 // Blocks of a query's sweep: the whole GPU, fewer on small graphs, whose rounds

@@ -119,3 +119,25 @@ def test_waits_that_run_out_for_good(scaled):
         finally:
             wt.debug_set_wait_limits(-1, -1)
         assert all((a == b).all() for a, b in zip(call(), before)), name
+
+
+def test_status_is_written_once(scaled):
+    """A count that the host reads while the query runs holds what it held, or
+    the answer: no status of a query that has not given up shows."""
+    torch = pytest.importorskip("torch")
+    _, d, _ = scaled
+    dev = torch.device("cuda:0")
+    t = torch.zeros((100, 3), dtype=torch.int32, device=dev)
+    w = torch.zeros(100, dtype=torch.float64, device=dev)
+    c = torch.zeros(1, dtype=torch.int32, pin_memory=True)  # the device writes host memory
+    seen = set()
+    for i in range(200):
+        c[0] = 7777
+        wt.topk_device(d, PS[i % 5], 100, t, w, c)
+        done = torch.cuda.Event()
+        done.record()
+        while not done.query():
+            seen.add(int(c[0]))
+        seen.add(int(c[0]))
+    torch.cuda.synchronize()
+    assert seen <= {7777, 100}, seen
