@@ -1091,7 +1091,8 @@ struct SelectSmem {
     unsigned long long mn, mx;
     uint32_t bin, above, taken;
     uint32_t err, n, old;  // the query's error bits, candidates and `selected`, as one thread read them
-    int gone;  // a grid barrier gave up
+    int narrow;  // a round of more edges than items filled the candidate buffer
+    int gone;    // a grid barrier gave up
 };
 
 // The query's state for the whole selecting block.  One thread reads it: a
@@ -1327,22 +1328,34 @@ __device__ uint32_t keep_first_ties(const Part<TB>& B, unsigned long long* ckey,
 // fill half of the free candidate slots (small buffers: a batched query at
 // p = -inf overflowed its 16,384 slots at a fixed growth of 8); and whether it
 // may have more edges than there are items: where the threshold hardly moved,
-// or there is none yet, a select earlier would prune little.
+// or there is none yet, a select earlier would prune little.  Such a round
+// (flat) may fill the candidate buffer where rounds of as many edges as items
+// would not: then its candidates are dropped and it is to be done again, and all
+// that follow, in those.
 struct Growth {
     int64_t times;
     bool wide;
+    bool again;
 };
 
 template <int TB>
-__device__ Growth select_round(const Part<TB>& B, const Query& q, SelectSmem& S) {
+__device__ Growth select_round(const Part<TB>& B, const Query& q, bool flat, SelectSmem& S) {
     const int64_t growth = q.growth;
     read_state<TB>(B, q, S);
     const uint32_t n = S.n, old = S.old;
-    if (S.err || n == old) return Growth{growth, true};
+    if (flat && S.err == DEV_ERR_OVERFLOW) {
+        if (B.tid() == 0) {
+            S.narrow = 1;
+            *(volatile uint32_t*)&q.st->count = old;
+            atomicAnd(&q.st->err, ~DEV_ERR_OVERFLOW);
+        }
+        return Growth{1, false, true};
+    }
+    if (S.err || n == old) return Growth{growth, true, false};
     const int64_t added = n - old;
     if (n < (uint32_t)q.k) {
         if (B.tid() == 0) *(volatile uint32_t*)&q.st->selected = n;  // all of them stay
-        return Growth{max(int64_t(1), min(growth, (int64_t)(q.cap - n) / (2 * added))), true};
+        return Growth{max(int64_t(1), min(growth, (int64_t)(q.cap - n) / (2 * added))), true, false};
     }
     const unsigned long long T = kth_key<TB>(B, q.ckey, n, (uint32_t)q.k, S);
     const uint32_t kept = compact<TB>(B, q.ckey, q.ctri, n, [=](unsigned long long k, const int4&) { return k >= T; }, S);
@@ -1352,7 +1365,7 @@ __device__ Growth select_round(const Part<TB>& B, const Query& q, SelectSmem& S)
         if (T > q.st->tau) *(volatile unsigned long long*)&q.st->tau = T;
     }
     B.sync();
-    return Growth{max(int64_t(1), min(growth, (int64_t)(q.cap - kept) / (2 * added))), 8 * added <= q.k};
+    return Growth{max(int64_t(1), min(growth, (int64_t)(q.cap - kept) / (2 * added))), 8 * added <= q.k, false};
 }
 
 // The next round's range: [lo, lo + size) cut at the first edge whose bound
@@ -1571,6 +1584,7 @@ __device__ bool sweep(const DevGraph& G, const Query& q, const Out& o, Team& T, 
     const int64_t total = q.total_dev ? __ldg(q.total_dev) : q.total;
     int64_t size = min(q.first, q.item_cap), lo = 0, hi = min(total, size);
     unsigned long long tau = 0;
+    if (T.part.tid() == 0) S.sel.narrow = 0;
     Tally tb;
     tb.on = q.qbytes != nullptr;
     for (int par = 0; lo < hi; par ^= 1) {
@@ -1603,9 +1617,11 @@ __device__ bool sweep(const DevGraph& G, const Query& q, const Out& o, Team& T, 
         }
         if (T.leader()) {
             if (T.part.tid() == 0) *(volatile unsigned long long*)&q.st->items[par ^ 1] = 0;
-            const Growth grow = select_round<Team::TB>(T.part, q, S.sel);
-            const int64_t cap = oriented || grow.wide ? INT64_MAX / 1024 : q.item_cap;
-            next_range<P, SAMPLED>(T.part.tid(), G, q, hi, min(size * grow.times, cap), total, S.sel.err != 0);
+            const Growth grow = select_round<Team::TB>(T.part, q, flat && !oriented, S.sel);
+            const int64_t cap = oriented || (grow.wide && !S.sel.narrow) ? INT64_MAX / 1024 : q.item_cap;
+            // (the state still holds this round's start)
+            next_range<P, SAMPLED>(T.part.tid(), G, q, grow.again ? *(volatile long long*)&q.st->lo : hi,
+                                   min(size * grow.times, cap), total, S.sel.err != 0 && !grow.again);
         }
         if (!T.sync(q)) return false;
         size = *(volatile long long*)&q.st->size;

@@ -77,3 +77,38 @@ def test_sweep_of_the_whole_graph(n, m, bipartite):
             assert_topk_equal(*d.sample_topk(p, 2000, 4 * u.size, 5), want, p, f"sampled p={p}")
     finally:
         d.free()
+
+
+def _late(heavy, m, n, seed):
+    """heavy triangle-free heavy edges, then a light random graph of m edges on n
+    vertices: every triangle lies in the last edges of the edge order."""
+    rng = np.random.default_rng(seed)
+    key = np.unique(rng.integers(0, 200_000, 2 * heavy) * 400_000 + rng.integers(200_000, 400_000, 2 * heavy))
+    key = rng.permutation(key)[:heavy]
+    a, b = rng.integers(0, n, 2 * m), rng.integers(0, n, 2 * m)
+    light = np.unique(np.minimum(a, b)[a != b] * n + np.maximum(a, b)[a != b])
+    light = rng.permutation(light)[:m]
+    u = np.concatenate([key // 400_000, 400_000 + light // n])
+    v = np.concatenate([key % 400_000, 400_000 + light % n])
+    w = np.concatenate([rng.integers(1000, 1100, key.size), rng.integers(1, 21, light.size)])
+    return 400_000 + n, u.astype(np.int32), v.astype(np.int32), w.astype(np.int32)
+
+
+@pytest.mark.parametrize("p", [0.0, 1.0, 2.0, np.inf])
+def test_wide_round_that_fills_the_candidates(p):
+    """1.3 million triangles in the edges of one wide round, more than the
+    1,048,576 candidates of the fixed scratch; rounds of as many edges as items
+    (46,592) hold them.  (p = -inf and the allocating device form take all these
+    edges in one round whatever the items, and report WTRI_ENOMEM.)"""
+    n, u, v, w = _late(600_000, 200_000, 2000, 3)
+    d = wt.build_csr(n, u, v, w)
+    try:
+        for k in (16_384, 3000):
+            want = oracle.topk(n, u, v, w, p, k)
+            assert want["ntri"] > 1 << 20
+            assert_topk_equal(*_device(wt.topk_device_noalloc, d, p, k), want, p, f"noalloc p={p} k={k}")
+            assert_topk_equal(*d.topk(p, k), want, p, f"host p={p} k={k}")
+            for got in wt.topk_batch([d] * 3, [p] * 3, [k] * 3):
+                assert_topk_equal(*got, want, p, f"batch p={p} k={k}")
+    finally:
+        d.free()
